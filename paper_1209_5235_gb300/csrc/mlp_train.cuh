@@ -1,0 +1,455 @@
+// mlp_train.cuh -- training steps of the candidate-proposal MLP as one persistent cooperative kernel
+// (included once, by mlp.cu).
+//
+// A minibatch of this network is little work -- 4096 rows are 0.17 GFLOP of GEMM -- and every step
+// needs the weights of the one before it, so training is bound by the length of a step's serial
+// chain, not by arithmetic.  As separate kernels per GEMM and elementwise pass a step was 26
+// launches and clears in a row, 186 us at 4096 rows on GB300; here all steps of an epoch are one
+// launch and a step takes 10.5 us (an epoch of 2^20 samples: 47.7 -> 2.82 ms with the loading of the
+// parameters before it and their reading back).  A step:
+//   forward and backward of the block's row tiles, every intermediate in registers or shared memory;
+//   partial gradients to global memory; grid barrier;
+//   each block sums the partials of its share of the parameters and updates them (Adam); grid barrier;
+//   reload of the weights' image (31 KB, from L2).
+//
+// A tile is 32 rows by all 64 hidden columns on 8 warps (2 row halves x 4 column groups of 16), so
+// that a minibatch of 4096 rows fills 128 SMs and a layer is a few mma.sync per warp.  Products are
+// mma.sync m16n8k16 (BF16 in, FP32 accumulation), the K chunks of an output in ascending order from a
+// zero accumulator, bias added afterwards.  tcgen05 tiles need 128 rows per CTA: a quarter of the SMs
+// and four times the elementwise work (erf, exp) per SM, on a chain that waits for latency anyway.
+// The weight-gradient products take their transposed operands from shared memory with ldmatrix.trans
+// and keep their 28 accumulators per lane in registers over all of a block's tiles.  Summation order
+// is fixed: results do not vary from run to run.
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include <cstdint>
+
+#include "mlp_device.cuh"
+
+namespace g4n {
+namespace mlp {
+
+constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kIn * kHid, kOffW2 = kOffB1 + kHid, kOffB2 = kOffW2 + kHid * kHid,
+              kOffW3 = kOffB2 + kHid, kOffB3 = kOffW3 + kHid * kOut;
+
+constexpr int kTrRows = 32, kTrThreads = 256;
+constexpr int kSOutB = 40;                       // padded row stride of 32 BF16 columns (16-byte rows for ldmatrix)
+constexpr unsigned kBarrierPolls = 1u << 22;     // polls of a grid barrier before it gives up (seconds)
+
+__device__ __forceinline__ float gelu_grad(float x, float e) {  // e = erf(x / sqrt 2)
+  return 0.5f * (1.0f + e) + x * 0.39894228040143268f * expf(-0.5f * x * x);
+}
+
+// Device control block of the kernel.
+struct TrainCtrl {
+  unsigned int arrived;   // grid barrier: blocks arrived, over all barriers of the launch
+  unsigned int failed;    // a barrier gave up
+  double loss;            // sum of the losses over the launch
+};
+
+struct TrainParams {
+  int64_t n;                        // samples
+  const float *feat;
+  const int32_t *label, *ncand;
+  int steps, batch;                 // minibatches of `batch` rows
+  bool permuted;                    // row r of step s is sample ((s batch + r) mod n * stride + offset) mod n, else s batch + r
+  uint64_t stride, offset;
+  float inv_scale;
+  float *P, *M, *V;                 // parameters and Adam moments; M null: gradients of one step into `grads` instead
+  float *grads;
+  float *part;                      // gridDim.x x kNParams partial gradients
+  double *part_loss;                // gridDim.x
+  const float2 *bias_corr;          // per step: Adam's 1 / (1 - beta^t)
+  float lr, b1, b2, eps;
+  TrainCtrl *ctrl;
+  struct TrainWeights *img;
+};
+
+// The weights as the products read them.  The blocks keep one image in global memory, each writing its share of the
+// parameters, and copy it to shared memory 16 bytes at a time.
+struct alignas(16) TrainWeights {
+  __nv_bfloat16 w1t[kHid * kSIn];    // [n][k]: B operands of the forward products (padding stays zero)
+  __nv_bfloat16 w2t[kHid * kSHid];
+  __nv_bfloat16 w3t[kOut * kSHid];
+  __nv_bfloat16 w2[kHid * kSHid];    // [k][n]: B operands of the backward products
+  __nv_bfloat16 w3[kHid * kSOutB];
+  float b1[kHid], b2[kHid], b3[kOut];
+};
+static_assert(sizeof(TrainWeights) % 16 == 0, "copied in 16-byte pieces");
+
+struct TrainSmem {
+  TrainWeights w;
+  __nv_bfloat16 x[kTrRows * kSIn], h1[kTrRows * kSHid], h2[kTrRows * kSHid];
+  __nv_bfloat16 d3[kTrRows * kSOutB], d2[kTrRows * kSHid], d1[kTrRows * kSHid];
+  float logits[kTrRows * kSOut];
+  float red[kTrThreads], colsum[2][kHid];
+  float lossw[kTrThreads / 32];
+  int32_t label[kTrRows], ncand[kTrRows];
+};
+
+__device__ __forceinline__ void ldsm4t(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, const __nv_bfloat16 *p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldsm2t(uint32_t &r0, uint32_t &r1, const __nv_bfloat16 *p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(a) : "memory");
+}
+
+// d[4] (+)= a row-major 16 x K tile of `in` (row stride SA, first row row0) times B from wt ([n][k], stride SB) at
+// columns n0 .. n0 + 7.
+template <int K, int SA, int SB>
+__device__ __forceinline__ void tile_mma(float d[4], const __nv_bfloat16 *in, int row0, const __nv_bfloat16 *wt, int n0) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const __nv_bfloat16 *a_lo = in + (row0 + g) * SA + 2 * q, *a_hi = a_lo + 8 * SA;
+  const __nv_bfloat16 *bp = wt + (n0 + g) * SB + 2 * q;
+#pragma unroll
+  for (int kt = 0; kt < K / 16; ++kt)
+    mma_bf16(d[0], d[1], d[2], d[3], ld_pair(a_lo + kt * 16), ld_pair(a_hi + kt * 16), ld_pair(a_lo + kt * 16 + 8),
+             ld_pair(a_hi + kt * 16 + 8), ld_pair(bp + kt * 16), ld_pair(bp + kt * 16 + 8));
+}
+
+// acc[NT][4] += (columns m0 .. m0 + 15 of `a`)^T (columns n0 .. of `b`) over the tile's 32 rows: NT n-tiles of 8.
+template <int NT, int SA, int SB>
+__device__ __forceinline__ void grad_mma(float acc[][4], const __nv_bfloat16 *a, int m0, const __nv_bfloat16 *b, int n0) {
+  const int lane = threadIdx.x & 31, r = lane & 7, mat = lane >> 3;
+#pragma unroll
+  for (int k = 0; k < kTrRows; k += 16) {
+    uint32_t a0, a1, a2, a3;
+    ldsm4t(a0, a1, a2, a3, a + (k + (mat >> 1) * 8 + r) * SA + m0 + (mat & 1) * 8);
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      uint32_t b0, b1;
+      ldsm2t(b0, b1, b + (k + (mat & 1) * 8 + r) * SB + n0 + t * 8);
+      mma_bf16(acc[t][0], acc[t][1], acc[t][2], acc[t][3], a0, a1, a2, a3, b0, b1);
+    }
+  }
+}
+
+// Parameter p of value v into the image.
+__device__ __forceinline__ void train_image(TrainWeights &W, int p, float v) {
+  const __nv_bfloat16 w = __float2bfloat16_rn(v);
+  if (p < kOffB1) {
+    W.w1t[(p & 63) * kSIn + (p >> 6)] = w;
+  } else if (p < kOffW2) {
+    W.b1[p - kOffB1] = v;
+  } else if (p < kOffB2) {
+    const int k = (p - kOffW2) >> 6, n = (p - kOffW2) & 63;
+    W.w2t[n * kSHid + k] = w;
+    W.w2[k * kSHid + n] = w;
+  } else if (p < kOffW3) {
+    W.b2[p - kOffB2] = v;
+  } else if (p < kOffB3) {
+    const int k = (p - kOffW3) >> 5, n = (p - kOffW3) & 31;
+    W.w3t[n * kSHid + k] = w;
+    W.w3[k * kSOutB + n] = w;
+  } else {
+    W.b3[p - kOffB3] = v;
+  }
+}
+
+// The image to shared memory (written by other blocks: read past the L1).
+__device__ __forceinline__ void train_load_weights(TrainWeights &S, const TrainWeights *img) {
+  const uint4 *src = reinterpret_cast<const uint4 *>(img);
+  uint4 *dst = reinterpret_cast<uint4 *>(&S);
+  constexpr int kVec = sizeof(TrainWeights) / 16;
+#pragma unroll
+  for (int i = 0; i < (kVec + kTrThreads - 1) / kTrThreads; ++i) {
+    const int e = threadIdx.x + i * kTrThreads;
+    if (e < kVec) dst[e] = __ldcg(src + e);
+  }
+}
+
+// Barrier number `k` (1, 2, ...) of the grid (cooperative launch: every block is resident).  A block that has polled
+// kBarrierPolls times sets `failed` and ends; the others see it at their next barrier (or while they poll) and end too.
+__device__ __forceinline__ bool grid_barrier(TrainCtrl *C, unsigned k) {
+  __shared__ bool ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&C->arrived, 1u);
+    const unsigned target = k * gridDim.x;
+    unsigned polls = 0, seen;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&C->arrived) : "memory");
+      if ((int)(seen - target) >= 0 || ++polls >= kBarrierPolls) break;
+      if ((polls & 1023u) == 0 && *(volatile unsigned int *)&C->failed) break;
+    }
+    if ((int)(seen - target) < 0) atomicExch(&C->failed, 1u);
+    ok = *(volatile unsigned int *)&C->failed == 0u;
+  }
+  __syncthreads();
+  return ok;
+}
+
+// One element of a tile's inputs: sample row r = e / 11, its nine features, label and candidate count.
+struct TrainFetch {
+  uint32_t bits[2];
+};
+
+__device__ __forceinline__ TrainFetch train_fetch(const TrainParams &T, int64_t step, int tile) {
+  TrainFetch f{{0u, 0u}};
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int e = threadIdx.x + j * kTrThreads;
+    const int r = e / (kIn + 2), k = e % (kIn + 2);
+    const int64_t row = (int64_t)tile * kTrRows + r;
+    if (r >= kTrRows || row >= T.batch || step >= T.steps) continue;
+    uint64_t at = (uint64_t)(step * T.batch + row);
+    if (T.permuted) at = ((at % (uint64_t)T.n) * T.stride + T.offset) % (uint64_t)T.n;
+    if (k < kIn) f.bits[j] = __float_as_uint(__ldg(T.feat + at * kIn + k));
+    else f.bits[j] = (uint32_t)__ldg((k == kIn ? T.label : T.ncand) + at);
+  }
+  return f;
+}
+
+__device__ __forceinline__ void train_put(TrainSmem &S, const TrainFetch &f) {
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int e = threadIdx.x + j * kTrThreads;
+    const int r = e / (kIn + 2), k = e % (kIn + 2);
+    if (r >= kTrRows) continue;
+    if (k < kIn) S.x[r * kSIn + k] = __float2bfloat16_rn(__uint_as_float(f.bits[j]));
+    else (k == kIn ? S.label : S.ncand)[r] = (int32_t)f.bits[j];
+  }
+}
+
+__global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  TrainSmem &S = *reinterpret_cast<TrainSmem *>(smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
+  const int wm = (warp & 1) * 16, wn = (warp >> 1) * 16;   // the warp's rows and hidden columns of a tile
+  const int tiles = (T.batch + kTrRows - 1) / kTrRows;
+  for (int e = tid; e < kTrRows * kSIn; e += kTrThreads) S.x[e] = __float2bfloat16_rn(0.f);   // columns 9 .. 15 stay zero
+  // the share of the parameters that this block updates
+  const int share = (kNParams + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int p0 = min(kNParams, (int)blockIdx.x * share), p1 = min(kNParams, p0 + share);
+  unsigned barriers = 0;
+  for (int p = p0 + tid; p < p1; p += kTrThreads) train_image(*T.img, p, T.P[p]);
+  if (!grid_barrier(T.ctrl, ++barriers)) return;
+  TrainFetch next = train_fetch(T, 0, blockIdx.x);
+#pragma unroll 1
+  for (int64_t step = 0; step < T.steps; ++step) {
+    __syncthreads();
+    train_load_weights(S.w, T.img);
+    float gw1[1][4] = {}, gw2[4][4] = {}, gw3[2][4] = {};   // weight gradients: the warp's tiles
+    float gb1[4] = {}, gb2[4] = {}, gb3[4] = {};            // bias gradients: the lane's columns
+    float loss = 0.f;
+#pragma unroll 1
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+      train_put(S, next);
+      // the next tile's inputs come while this one is worked on
+      const bool more = tile + (int)gridDim.x < tiles;
+      next = train_fetch(T, more ? step : step + 1, more ? tile + gridDim.x : blockIdx.x);
+      __syncthreads();
+      // forward; the pre-activations and their erf stay in registers for the backward pass
+      float z1[2][4], e1[2][4], z2[2][4], e2[2][4];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const int col = wn + t * 8 + 2 * q;
+        float d[4] = {0.f, 0.f, 0.f, 0.f}, h[4];
+        tile_mma<kInPad, kSIn, kSIn>(d, S.x, wm, S.w.w1t, wn + t * 8);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          z1[t][i] = d[i] + S.w.b1[col + (i & 1)];
+          e1[t][i] = erff(z1[t][i] * 0.70710678118654752f);
+          h[i] = 0.5f * z1[t][i] * (1.0f + e1[t][i]);
+        }
+        *reinterpret_cast<__nv_bfloat162 *>(S.h1 + (wm + g) * kSHid + col) = __floats2bfloat162_rn(h[0], h[1]);
+        *reinterpret_cast<__nv_bfloat162 *>(S.h1 + (wm + g + 8) * kSHid + col) = __floats2bfloat162_rn(h[2], h[3]);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const int col = wn + t * 8 + 2 * q;
+        float d[4] = {0.f, 0.f, 0.f, 0.f}, h[4];
+        tile_mma<kHid, kSHid, kSHid>(d, S.h1, wm, S.w.w2t, wn + t * 8);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          z2[t][i] = d[i] + S.w.b2[col + (i & 1)];
+          e2[t][i] = erff(z2[t][i] * 0.70710678118654752f);
+          h[i] = 0.5f * z2[t][i] * (1.0f + e2[t][i]);
+        }
+        *reinterpret_cast<__nv_bfloat162 *>(S.h2 + (wm + g) * kSHid + col) = __floats2bfloat162_rn(h[0], h[1]);
+        *reinterpret_cast<__nv_bfloat162 *>(S.h2 + (wm + g + 8) * kSHid + col) = __floats2bfloat162_rn(h[2], h[3]);
+      }
+      __syncthreads();
+      {
+        const int n0 = (warp >> 1) * 8, col = n0 + 2 * q;
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        tile_mma<kHid, kSHid, kSHid>(d, S.h2, wm, S.w.w3t, n0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          S.logits[(wm + g + 8 * (i >> 1)) * kSOut + col + (i & 1)] = d[i] + S.w.b3[col + (i & 1)];
+      }
+      __syncthreads();
+      {  // masked softmax cross-entropy: 8 lanes a row, 4 columns a lane
+        const int r = tid >> 3, sub = tid & 7;
+        const bool valid = (int64_t)tile * kTrRows + r < T.batch;
+        const int nc = max(1, min(kOut, S.ncand[r])), y = S.label[r];
+        const float *z = S.logits + r * kSOut;
+        float zz[4], mx = -INFINITY, s = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          zz[j] = z[sub + 8 * j];
+          if (sub + 8 * j < nc) mx = fmaxf(mx, zz[j]);
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s += sub + 8 * j < nc ? expf(zz[j] - mx) : 0.f;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const float lse = mx + logf(s);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = sub + 8 * j;
+          const float p = c < nc ? expf(zz[j] - lse) : 0.f;
+          const float dz = valid ? (p - (c == y ? 1.f : 0.f)) * T.inv_scale : 0.f;
+          if (valid && c == y) loss += lse - zz[j];
+          gb3[j] += dz;
+          S.d3[r * kSOutB + c] = __float2bfloat16_rn(dz);
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {  // dZ2 = (dZ3 W3^T) gelu'(Z2)
+        const int col = wn + t * 8 + 2 * q;
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        tile_mma<kOut, kSOutB, kSOutB>(d, S.d3, wm, S.w.w3, wn + t * 8);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          d[i] *= gelu_grad(z2[t][i], e2[t][i]);
+          gb2[2 * t + (i & 1)] += d[i];
+        }
+        *reinterpret_cast<__nv_bfloat162 *>(S.d2 + (wm + g) * kSHid + col) = __floats2bfloat162_rn(d[0], d[1]);
+        *reinterpret_cast<__nv_bfloat162 *>(S.d2 + (wm + g + 8) * kSHid + col) = __floats2bfloat162_rn(d[2], d[3]);
+      }
+      grad_mma<2, kSHid, kSOutB>(gw3, S.h2, (warp & 3) * 16, S.d3, (warp >> 2) * 16);   // dW3 = H2^T dZ3
+      __syncthreads();
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {  // dZ1 = (dZ2 W2^T) gelu'(Z1)
+        const int col = wn + t * 8 + 2 * q;
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        tile_mma<kHid, kSHid, kSHid>(d, S.d2, wm, S.w.w2, wn + t * 8);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          d[i] *= gelu_grad(z1[t][i], e1[t][i]);
+          gb1[2 * t + (i & 1)] += d[i];
+        }
+        *reinterpret_cast<__nv_bfloat162 *>(S.d1 + (wm + g) * kSHid + col) = __floats2bfloat162_rn(d[0], d[1]);
+        *reinterpret_cast<__nv_bfloat162 *>(S.d1 + (wm + g + 8) * kSHid + col) = __floats2bfloat162_rn(d[2], d[3]);
+      }
+      grad_mma<4, kSHid, kSHid>(gw2, S.h1, (warp & 3) * 16, S.d2, (warp >> 2) * 32);    // dW2 = H1^T dZ2
+      __syncthreads();
+      grad_mma<1, kSIn, kSHid>(gw1, S.x, 0, S.d1, warp * 8);                            // dW1 = X^T dZ1
+      __syncthreads();   // the tile's buffers are free
+    }
+    // the block's partial gradients
+    float *G = T.part + (int64_t)blockIdx.x * kNParams;
+    {
+      const int m0 = (warp & 3) * 16 + g;
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        float *c = G + kOffW3 + m0 * kOut + (warp >> 2) * 16 + t * 8 + 2 * q;
+        *reinterpret_cast<float2 *>(c) = make_float2(gw3[t][0], gw3[t][1]);
+        *reinterpret_cast<float2 *>(c + 8 * kOut) = make_float2(gw3[t][2], gw3[t][3]);
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        float *c = G + kOffW2 + m0 * kHid + (warp >> 2) * 32 + t * 8 + 2 * q;
+        *reinterpret_cast<float2 *>(c) = make_float2(gw2[t][0], gw2[t][1]);
+        *reinterpret_cast<float2 *>(c + 8 * kHid) = make_float2(gw2[t][2], gw2[t][3]);
+      }
+      float *c = G + kOffW1 + g * kHid + warp * 8 + 2 * q;
+      *reinterpret_cast<float2 *>(c) = make_float2(gw1[0][0], gw1[0][1]);
+      if (g + 8 < kIn) *reinterpret_cast<float2 *>(c + 8 * kHid) = make_float2(gw1[0][2], gw1[0][3]);
+    }
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {   // column sums of dZ2, dZ1: over the lanes' rows, then the two row halves
+      float *gb = w == 0 ? gb2 : gb1;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) gb[i] += __shfl_xor_sync(0xffffffffu, gb[i], o);
+      if (g == 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) S.colsum[warp & 1][wn + (i >> 1) * 8 + 2 * q + (i & 1)] = gb[i];
+      __syncthreads();
+      if (tid < kHid) G[(w == 0 ? kOffB2 : kOffB1) + tid] = S.colsum[0][tid] + S.colsum[1][tid];
+      __syncthreads();
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      gb3[j] += __shfl_xor_sync(0xffffffffu, gb3[j], 8);
+      gb3[j] += __shfl_xor_sync(0xffffffffu, gb3[j], 16);
+      if (lane < 8) S.red[warp * kOut + lane + 8 * j] = gb3[j];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    if (lane == 0) S.lossw[warp] = loss;
+    __syncthreads();
+    if (tid < kOut) {
+      float s = 0.f;
+#pragma unroll
+      for (int w = 0; w < kTrThreads / 32; ++w) s += S.red[w * kOut + tid];
+      G[kOffB3 + tid] = s;
+    }
+    if (tid == 0) {
+      double l = 0.0;
+#pragma unroll
+      for (int w = 0; w < kTrThreads / 32; ++w) l += (double)S.lossw[w];
+      T.part_loss[blockIdx.x] = step == 0 ? l : T.part_loss[blockIdx.x] + l;
+    }
+    // the first 64 parameters of the share and their moments are on their way while the barrier is waited for
+    const int pf = p0 + (tid & 63);
+    const bool own = T.M && tid < 64 && pf < p1;
+    float pv = own ? T.P[pf] : 0.f, mv = own ? T.M[pf] : 0.f, vv = own ? T.V[pf] : 0.f;
+    if (!grid_barrier(T.ctrl, ++barriers)) return;
+    // gradients of the block's share: four groups of 64 threads take a quarter of the partials each
+    const float2 corr = T.M ? T.bias_corr[step] : make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int base = p0; base < p1; base += 64) {
+      const int p = base + (tid & 63), quarter = tid >> 6;
+      float s = 0.f;
+      if (p < p1) {
+#pragma unroll 8
+        for (int b = quarter; b < (int)gridDim.x; b += 4) s += __ldcg(T.part + (int64_t)b * kNParams + p);
+      }
+      S.red[tid] = s;
+      __syncthreads();
+      if (tid < 64 && p < p1) {
+        const float gr = (S.red[tid] + S.red[tid + 64]) + (S.red[tid + 128] + S.red[tid + 192]);
+        if (!T.M) {
+          T.grads[p] = gr;
+        } else {
+          if (base > p0) {
+            pv = T.P[p];
+            mv = T.M[p];
+            vv = T.V[p];
+          }
+          const float m = T.b1 * mv + (1.f - T.b1) * gr;
+          const float v = T.b2 * vv + (1.f - T.b2) * gr * gr;
+          pv -= T.lr * (m * corr.x) / (sqrtf(v * corr.y) + T.eps);
+          T.M[p] = m;
+          T.V[p] = v;
+          T.P[p] = pv;
+          train_image(*T.img, p, pv);
+        }
+      }
+      __syncthreads();
+    }
+    if (!grid_barrier(T.ctrl, ++barriers)) return;
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    double l = 0.0;
+    for (int b = 0; b < (int)gridDim.x; ++b) l += __ldcg(T.part_loss + b);
+    T.ctrl->loss = l;
+  }
+}
+
+}  // namespace mlp
+}  // namespace g4n

@@ -221,3 +221,51 @@ def test_trained_learned_barrel_full_size_sampled(env):
     for i in np.unique(np.random.default_rng(8).integers(0, n, 300)):
         r = og.transport(src, seed, 1, tid0=int(i), threads=1)
         assert hashes[2, 1][i] == r["hashes"][0], i
+
+
+@pytest.mark.parametrize("n", [16, 32, 48, 4864, 4880, 9760])
+def test_bf16_gradients_at_tile_edges(env, n):
+    """A half tile, one tile, a tile and a half, one tile per SM of a 152-SM GPU, one row block more, two tiles on
+    some blocks and a ragged one.  Tolerance: that of the BF16 gradients above (8 significant bits, 2e-2 in norm)."""
+    g4, torch, ctx = env
+    p = params(27)
+    g4.g4n_mlp_load(ctx, p)
+    X, y, nc = random_data(n, 28)
+    T = lambda a: torch.tensor(a, device="cuda")
+    loss, g = g4.g4n_mlp_grad(ctx, T(X), T(y), T(nc), precision=0)
+    ref_loss, ref_g = omlp.loss_and_grad(p.astype(np.float64), X.astype(np.float64), y, nc)
+    assert abs(loss - ref_loss) <= 2e-2 * abs(ref_loss)
+    for got, want in zip(omlp.unpack(g), omlp.unpack(ref_g)):
+        assert np.linalg.norm(got - want) <= 2e-2 * np.linalg.norm(want) + 1e-12
+    again = g4.g4n_mlp_grad(ctx, T(X), T(y), T(nc), precision=0)
+    assert again[0] == loss and np.array_equal(again[1], g)   # the summation order is fixed
+
+
+@pytest.mark.parametrize("batch", [16, 48, 4880])
+def test_training_step_matches_its_gradient(env, batch):
+    """One minibatch of an epoch: its loss is that of the permuted samples, and the update is Adam's first step on
+    their gradient (the same kernel's, over the same rows in the same order).  Tolerance: the update in FP32 from the
+    same gradient, a few roundings of relative 2^-24 in the step and one in the parameter."""
+    g4, torch, ctx = env
+    p, n, seed, lr = params(31), batch + 7, 9, np.float32(2e-3)
+    X, y, nc = random_data(n, 32)
+    wrap = (1 << 64) - 1
+    h = (seed * 0x9E3779B97F4A7C15 + 1) & wrap
+    h ^= h >> 31
+    h = (h * 0xBF58476D1CE4E5B9) & wrap
+    h ^= h >> 27
+    stride = (h % n) | 1
+    while math.gcd(stride, n) != 1:
+        stride += 2
+    rows = np.array([(r * stride + (h >> 17) % n) % n for r in range(batch)])
+    T = lambda a: torch.tensor(a, device="cuda")
+    g4.g4n_mlp_load(ctx, p)
+    loss, g = g4.g4n_mlp_grad(ctx, T(X[rows]), T(y[rows]), T(nc[rows]))
+    losses = g4.g4n_mlp_train(ctx, T(X), T(y), T(nc), epochs=1, batch=batch, lr=float(lr), seed=seed)
+    assert abs(losses[0] - loss) <= 1e-6 * loss
+    f = np.float32
+    m, v = (f(1) - f(0.9)) * g, (f(1) - f(0.999)) * g * g
+    c1, c2 = f(1) / (f(1) - f(0.9)), f(1) / (f(1) - f(0.999))
+    step = lr * (m * c1) / (np.sqrt(v * c2) + f(1e-8))
+    got = g4.g4n_mlp_get(ctx)
+    assert np.all(np.abs(got - (p - step)) <= 2.0 ** -23 * np.abs(p) + 1e-6 * np.abs(step) + 1e-12)

@@ -6,6 +6,7 @@
 //   DWorld[n]    64 B: composed world -> local transform of each volume
 //   DBox32[n]    32 B: FP32 bounding box of each volume in its mother's frame,
 //                rounded outward and padded (conservative prefilter for Inside)
+//   DPick32[n]   64 B: placement and solid in FP32 for the surface choice
 //   DVoxHdr[]    smart-voxel headers (one per slicing level and node)
 //   DVoxHdr32[]  their FP32 enclosures (the FP32 voxel walk)
 //   DVoxSlice[]  per slice: child (candidate list or sub-header) and the
@@ -80,6 +81,17 @@ struct alignas(16) DVol32 {
   float pad;
 };
 
+// FP32 placement and solid of a volume for the choice of the surface a ray crosses (nav_pick32.cuh): the translation
+// as the sum of two floats, so that the local point's error is relative to its distance from the solid and not to
+// its distance from the mother's origin; the solid's parameters rounded to float.
+struct alignas(64) DPick32 {
+  float th[3], tl[3];       // translation = th + tl within 2^-46 of it
+  float c, s;
+  float q[7];               // as DVol::p (cones: unused)
+  int32_t kind_flags;       // flags << 2 | kind
+};
+static_assert(sizeof(DPick32) == 64, "DPick32 must be 64 bytes");
+
 // Relocation across one face of a kKeyBox volume, decided on the host for a whole
 // region: the face's rectangle shrunk in-plane by a margin and thickened by tol/8
 // along the normal, as world-coordinate key intervals [lo, hi] per axis.  For
@@ -125,6 +137,7 @@ struct DGeom {
   const DWorld *wxf;
   const DBox32 *box;
   const DVol32 *v32;
+  const DPick32 *pick;
   const DVoxHdr *hdr;
   const DVoxHdr32 *hdr32;
   const DVoxSlice *slice;
@@ -139,6 +152,8 @@ struct DGeom {
   int32_t shared_grid;  // all materials tabulated on one energy grid
   int32_t pad;
   double tol, half;
+  float band32;         // (float)(2 half)
+  float pad32;
 };
 
 // Host-side record of a solid (cone: a = rmin1, b = rmax1 at z = -c; d = rmin2, e = rmax2 at +c).
@@ -164,6 +179,7 @@ struct HGeom {
   std::vector<DWorld> wxf;
   std::vector<DBox32> box;
   std::vector<DVol32> v32;
+  std::vector<DPick32> pick;
   std::vector<DVoxHdr> hdr;
   std::vector<DVoxHdr32> hdr32;
   std::vector<DVoxSlice> slice;

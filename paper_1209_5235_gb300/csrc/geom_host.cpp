@@ -964,6 +964,20 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
                                          : std::max({v.p[0], v.p[1], v.p[2]});
     w.scale = (float)(std::fabs(v.tx) + std::fabs(v.ty) + std::fabs(v.tz) + 2.0 * ext);
   }
+  g->pick.resize(n);
+  for (int i = 0; i < n; ++i) {
+    const DVol &v = g->vol[i];
+    DPick32 &w = g->pick[i];
+    const double t[3] = {v.tx, v.ty, v.tz};
+    for (int a = 0; a < 3; ++a) {
+      w.th[a] = (float)t[a];
+      w.tl[a] = (float)(t[a] - (double)w.th[a]);
+    }
+    w.c = (float)v.c;
+    w.s = (float)v.s;
+    for (int k = 0; k < 7; ++k) w.q[k] = (float)v.p[k];
+    w.kind_flags = v.flags << 2 | v.kind;
+  }
   // --- validation: containment (surface samples) and sibling overlaps (interior samples)
   std::mt19937_64 rng(0x9E3779B97F4A7C15ull);
   std::vector<double> pts;
@@ -1112,7 +1126,7 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
   }
   // --- upload as one blob
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-  constexpr int kTables = 17;
+  constexpr int kTables = 18;
   size_t off[kTables], sz[kTables] = {g->vol.size() * sizeof(DVol), g->wxf.size() * sizeof(DWorld), g->box.size() * sizeof(DBox32),
                             g->hdr.size() * sizeof(DVoxHdr), g->slice.size() * sizeof(DVoxSlice),
                             g->clist.size() * sizeof(DCandList), g->cand.size() * sizeof(int32_t),
@@ -1120,10 +1134,10 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
                             g->mat_off.size() * sizeof(int32_t), g->mat_n.size() * sizeof(int32_t),
                             g->v32.size() * sizeof(DVol32), g->kbox.size() * sizeof(DKeyBox),
                             g->skey.size() * sizeof(int64_t), g->face.size() * sizeof(DFace),
-                            g->hdr32.size() * sizeof(DVoxHdr32)};
+                            g->hdr32.size() * sizeof(DVoxHdr32), g->pick.size() * sizeof(DPick32)};
   const void *src[kTables] = {g->vol.data(), g->wxf.data(), g->box.data(), g->hdr.data(), g->slice.data(), g->clist.data(),
                          g->cand.data(), g->matE.data(), g->matC.data(), g->matP.data(), g->mat_off.data(), g->mat_n.data(),
-                         g->v32.data(), g->kbox.data(), g->skey.data(), g->face.data(), g->hdr32.data()};
+                         g->v32.data(), g->kbox.data(), g->skey.data(), g->face.data(), g->hdr32.data(), g->pick.data()};
   size_t total = 0;
   for (int k = 0; k < kTables; ++k) { off[k] = total; total += al(std::max<size_t>(sz[k], 8)); }
   if (ctx->device < 0) {  // host-only context: keep the host tables
@@ -1166,6 +1180,7 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
   d.mat_off = (const int32_t *)(base + off[10]);
   d.mat_n = (const int32_t *)(base + off[11]);
   d.v32 = (const DVol32 *)(base + off[12]);
+  d.pick = (const DPick32 *)(base + off[kTables - 1]);
   d.kbox = (const DKeyBox *)(base + off[13]);
   d.skey = (const int64_t *)(base + off[14]);
   d.face = (const DFace *)(base + off[15]);
@@ -1176,6 +1191,7 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
     if (m.E != B.mats[0].E) d.shared_grid = 0;
   d.tol = tol;
   d.half = 0.5 * tol;
+  d.band32 = (float)(2.0 * d.half);
   int32_t gid = (int32_t)ctx->geoms.size();
   if (cudaMemcpy(ctx->d_geoms + gid, &d, sizeof(DGeom), cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaFree(g->blob);

@@ -24,19 +24,14 @@
 
 #include "g4n_internal.h"
 #include "mlp_device.cuh"
+#include "nav_pick32.cuh"
+#include "nav_solids.cuh"
 
 namespace g4n {
 namespace dev {
 
-constexpr double kInf = __builtin_huge_val();
 constexpr float kInfF = __builtin_huge_valf();
 enum Mode : int { kFP64 = 0, kFP32 = 1, kLearned = 2 };  // kLearned: FP32 bounds + proposal first
-
-struct V3 {
-  double x, y, z;
-};
-
-__device__ __forceinline__ double comp(const V3 &v, int a) { return a == 0 ? v.x : (a == 1 ? v.y : v.z); }
 
 // Per-thread event counters (registers; constant indices only), flushed once per warp.
 struct Counters {
@@ -68,413 +63,6 @@ __device__ __forceinline__ void diag_test(Counters &c, int which, int curved_whi
   }
 }
 
-// key(x): a double's bits as a signed integer with the negative half reflected, so that
-// x < y <=> key(x) < key(y) for all non-NaN doubles (-0 < +0).
-__device__ __forceinline__ long long dkey(double x) {
-  const long long b = __double_as_longlong(x);
-  return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
-}
-
-// ---------------------------------------------------------------- frames
-
-__device__ __forceinline__ void to_local(const DVol &v, const V3 &pm, const V3 &vm, V3 &pl, V3 &vl) {
-  const double dx = pm.x - v.tx, dy = pm.y - v.ty;
-  if (v.flags & kPlacedAligned) {
-    pl = V3{dx, dy, pm.z - v.tz};
-    vl = vm;
-    return;
-  }
-  pl.x = v.c * dx + v.s * dy;
-  pl.y = v.c * dy - v.s * dx;
-  pl.z = pm.z - v.tz;
-  vl.x = v.c * vm.x + v.s * vm.y;
-  vl.y = v.c * vm.y - v.s * vm.x;
-  vl.z = vm.z;
-}
-
-// World -> local frame of a volume; world-aligned volumes need only the translation.
-__device__ __forceinline__ void world_to_local(const DWorld &w, bool aligned, const V3 &p, const V3 &u, V3 &pl,
-                                               V3 &vl) {
-  const double dx = p.x - w.tx, dy = p.y - w.ty;
-  if (aligned) {
-    pl = V3{dx, dy, p.z - w.tz};
-    vl = u;
-    return;
-  }
-  pl.x = w.c * dx + w.s * dy;
-  pl.y = w.c * dy - w.s * dx;
-  pl.z = p.z - w.tz;
-  vl.x = w.c * u.x + w.s * u.y;
-  vl.y = w.c * u.y - w.s * u.x;
-  vl.z = u.z;
-}
-
-// Reciprocal direction components (0 where the component is 0: never used there).
-struct Inv3 {
-  double x, y, z;
-};
-
-__device__ __forceinline__ Inv3 inv_dir(const V3 &v) {
-  return Inv3{v.x != 0.0 ? 1.0 / v.x : 0.0, v.y != 0.0 ? 1.0 / v.y : 0.0, v.z != 0.0 ? 1.0 / v.z : 0.0};
-}
-
-__device__ __forceinline__ double icomp(const Inv3 &v, int a) { return a == 0 ? v.x : (a == 1 ? v.y : v.z); }
-
-// ---------------------------------------------------------------- box
-
-__device__ __forceinline__ bool box_inside(const double *h, const V3 &p, const V3 &v, double half) {
-  const double ax = fabs(p.x) - h[0], ay = fabs(p.y) - h[1], az = fabs(p.z) - h[2];
-  const double m = fmax(ax, fmax(ay, az));
-  if (m > half) return false;
-  if (m < -half) return true;
-  if (ax >= -half && p.x * v.x >= 0.0) return false;
-  if (ay >= -half && p.y * v.y >= 0.0) return false;
-  if (az >= -half && p.z * v.z >= 0.0) return false;
-  return true;
-}
-
-__device__ __forceinline__ double box_dist_in(const double *h, const V3 &p, const V3 &v, double half) {
-  if ((fabs(p.x) - h[0] >= -half && p.x * v.x >= 0.0) || (fabs(p.y) - h[1] >= -half && p.y * v.y >= 0.0) ||
-      (fabs(p.z) - h[2] >= -half && p.z * v.z >= 0.0))
-    return kInf;
-  double tin = -kInf, tout = kInf;
-  const double pp[3] = {p.x, p.y, p.z}, vv[3] = {v.x, v.y, v.z};
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    if (vv[i] != 0.0) {
-      const double a = (-h[i] - pp[i]) / vv[i], b = (h[i] - pp[i]) / vv[i];
-      tin = fmax(tin, fmin(a, b));
-      tout = fmin(tout, fmax(a, b));
-    }
-  }
-  if (!(tout > tin + half)) return kInf;
-  return fmax(tin, 0.0);
-}
-
-// DistanceToOut with the reciprocal direction of the same frame; *face = the exit face
-// (2 axis + (v_axis > 0)) of the first axis attaining the minimum.  The zero tests of
-// v, the minimum and the clamp at 0 are integer operations on the bit patterns (the
-// order-preserving keys of doubles), which give the same value as fmin/fmax.
-__device__ __forceinline__ bool nonzero_bits(double x) { return (__double_as_longlong(x) << 1) != 0; }
-
-__device__ __forceinline__ double box_dist_out(const double *h, const V3 &p, const V3 &v, const Inv3 &iv, int *face) {
-  constexpr long long kKeyInf = 0x7FF0000000000000ll;  // key of +inf; NaN keys lie outside [key(-inf), key(+inf)]
-  double t = kInf;
-  long long kt = kKeyInf;
-  int f = -1;
-  const double pp[3] = {p.x, p.y, p.z}, vv[3] = {v.x, v.y, v.z}, ii[3] = {iv.x, iv.y, iv.z};
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    if (!nonzero_bits(vv[a])) continue;
-    const double ta = (copysign(h[a], vv[a]) - pp[a]) * ii[a];
-    const long long k = dkey(ta);
-    if (k < kt && k >= -kKeyInf - 1) {
-      kt = k;
-      t = ta;
-      f = 2 * a + (vv[a] > 0.0 ? 1 : 0);
-    }
-  }
-  *face = f;
-  return kt < 0 ? 0.0 : t;
-}
-
-__device__ __forceinline__ double box_safety_in(const double *h, const V3 &p) {
-  return fmax(fmax(fabs(p.x) - h[0], fmax(fabs(p.y) - h[1], fabs(p.z) - h[2])), 0.0);
-}
-
-__device__ __forceinline__ double box_safety_out(const double *h, const V3 &p) {
-  return fmax(fmin(h[0] - fabs(p.x), fmin(h[1] - fabs(p.y), h[2] - fabs(p.z))), 0.0);
-}
-
-// ---------------------------------------------------------------- orb
-
-// Roots of a t^2 + 2 b t + c = 0 without cancellation; false if the discriminant is not positive.
-__device__ __forceinline__ bool quad_roots(double a, double b, double c, double &lo, double &hi) {
-  const double disc = b * b - a * c;
-  if (!(disc > 0.0)) return false;
-  const double sq = sqrt(disc);
-  const double q = -(b + copysign(sq, b));
-  const double r1 = q / a, r2 = c / q;
-  lo = fmin(r1, r2);
-  hi = fmax(r1, r2);
-  return true;
-}
-
-__device__ __forceinline__ bool orb_inside(double R, const V3 &p, const V3 &v, double half) {
-  const double r2 = p.x * p.x + p.y * p.y + p.z * p.z;
-  const double ro = R + half, ri = R - half;
-  if (r2 > ro * ro) return false;
-  if (r2 < ri * ri) return true;
-  return p.x * v.x + p.y * v.y + p.z * v.z < 0.0;
-}
-
-__device__ __forceinline__ double orb_dist_in(double R, const V3 &p, const V3 &v, double half) {
-  const double b = p.x * v.x + p.y * v.y + p.z * v.z;
-  const double c = p.x * p.x + p.y * p.y + p.z * p.z - R * R;
-  double lo, hi;
-  if (!quad_roots(1.0, b, c, lo, hi)) return kInf;
-  return lo > half ? lo : kInf;
-}
-
-__device__ __forceinline__ double orb_dist_out(double R, const V3 &p, const V3 &v) {
-  const double b = p.x * v.x + p.y * v.y + p.z * v.z;
-  const double c = p.x * p.x + p.y * p.y + p.z * p.z - R * R;
-  double lo, hi;
-  if (!quad_roots(1.0, b, c, lo, hi)) return 0.0;
-  return fmax(hi, 0.0);
-}
-
-__device__ __forceinline__ double orb_safety_in(double R, const V3 &p) {
-  return fmax(sqrt(p.x * p.x + p.y * p.y + p.z * p.z) - R, 0.0);
-}
-
-__device__ __forceinline__ double orb_safety_out(double R, const V3 &p) {
-  return fmax(R - sqrt(p.x * p.x + p.y * p.y + p.z * p.z), 0.0);
-}
-
-// ---------------------------------------------------------------- tube segment
-// q[0..6] = rmin, rmax, hz, cos(sphi), sin(sphi), cos(ephi), sin(ephi).
-// ps = cross(u_start, p) and pe = cross(p, u_end) are the signed distances to the
-// lines of the two phi half-planes, positive on the solid's side.
-
-__device__ __forceinline__ bool tube_phi_ok(const double *q, int flags, double x, double y, double tol) {
-  if (!(flags & kSeg)) return true;
-  const double ps = q[3] * y - q[4] * x, pe = q[6] * x - q[5] * y;
-  return (flags & kWide) ? (ps >= -tol || pe >= -tol) : (ps >= -tol && pe >= -tol);
-}
-
-__device__ __forceinline__ bool tube_r_ok(const double *q, int flags, double x, double y, double half) {
-  const double r2 = x * x + y * y, ro = q[1] + half;
-  if (r2 > ro * ro) return false;
-  if (flags & kHasRmin) {
-    const double ri = q[0] - half;
-    if (r2 < ri * ri) return false;
-  }
-  return true;
-}
-
-__device__ __noinline__ bool tube_inside(const double *q, int flags, const V3 &p, const V3 &v, double half) {
-  const double sz = fabs(p.z) - q[2];
-  if (sz > half) return false;
-  const double r2 = p.x * p.x + p.y * p.y;
-  const double ro = q[1] + half;
-  if (r2 > ro * ro) return false;
-  bool nz = sz >= -half;
-  const double rmi = q[1] - half;
-  bool nrmax = r2 >= rmi * rmi;
-  bool nrmin = false;
-  if (flags & kHasRmin) {
-    const double ri = q[0] - half, rio = q[0] + half;
-    if (r2 < ri * ri) return false;
-    nrmin = r2 <= rio * rio;
-  }
-  bool ns = false, ne = false;
-  if (flags & kSeg) {
-    const double ps = q[3] * p.y - q[4] * p.x, pe = q[6] * p.x - q[5] * p.y;
-    if (!(flags & kWide)) {
-      if (ps < -half || pe < -half) return false;
-      ns = ps <= half;
-      ne = pe <= half;
-    } else {
-      const double m = fmax(ps, pe);
-      if (m < -half) return false;
-      if (m <= half) {
-        if (ps >= pe) ns = true;
-        else ne = true;
-      }
-    }
-  }
-  if (!(nz || nrmax || nrmin || ns || ne)) return true;
-  const double vr = p.x * v.x + p.y * v.y;
-  if (nz && !(p.z * v.z < 0.0)) return false;
-  if (nrmax && !(vr < 0.0)) return false;
-  if (nrmin && !(vr > 0.0)) return false;
-  if (ns && !(q[4] * v.x - q[3] * v.y < 0.0)) return false;
-  if (ne && !(q[5] * v.y - q[6] * v.x < 0.0)) return false;
-  return true;
-}
-
-// The crossings tube_cross takes the first of, one helper per surface: each returns its crossing
-// parameter t when t lies in (tmin, best) and the crossing passes the surface's range tests, else
-// +inf.
-// z plane the ray enters (enter) or leaves (exit) through
-__device__ __forceinline__ double tube_z_cand(const double *q, int flags, const V3 &p, const V3 &v, double half,
-                                              bool enter, double tmin) {
-  if (v.z == 0.0) return kInf;
-  const double sg = ((v.z < 0.0) == enter) ? 1.0 : -1.0;
-  const double t = (sg * q[2] - p.z) / v.z;
-  if (!(t > tmin)) return kInf;
-  const double qx = p.x + t * v.x, qy = p.y + t * v.y;
-  return (tube_r_ok(q, flags, qx, qy, half) && tube_phi_ok(q, flags, qx, qy, half)) ? t : kInf;
-}
-
-// cylinder of radius R (outer: the root that enters / leaves the solid through rmax; inner: through rmin)
-__device__ __forceinline__ double tube_cyl_cand(const double *q, int flags, const V3 &p, const V3 &v, double half,
-                                                bool enter, double tmin, double best, bool outer) {
-  const double a = v.x * v.x + v.y * v.y;
-  if (!(a > 0.0)) return kInf;
-  const double b = p.x * v.x + p.y * v.y;
-  const double r2 = p.x * p.x + p.y * p.y;
-  const double R = outer ? q[1] : q[0];
-  double lo, hi;
-  if (!quad_roots(a, b, r2 - R * R, lo, hi)) return kInf;
-  const double t = (enter == outer) ? lo : hi;
-  if (t > tmin && t < best && fabs(p.z + t * v.z) <= q[2] + half &&
-      tube_phi_ok(q, flags, p.x + t * v.x, p.y + t * v.y, half))
-    return t;
-  return kInf;
-}
-
-// phi half-plane at the start (start = true) or end of the segment
-__device__ __forceinline__ double tube_phi_cand(const double *q, int flags, const V3 &p, const V3 &v, double half,
-                                                bool enter, double tmin, double best, bool start) {
-  // v . outward normal of the plane, the signed distance to its line (positive on the solid's side)
-  const double dn = start ? q[4] * v.x - q[3] * v.y : q[5] * v.y - q[6] * v.x;
-  if (!(dn != 0.0 && ((dn < 0.0) == enter))) return kInf;
-  const double t = (start ? q[3] * p.y - q[4] * p.x : q[6] * p.x - q[5] * p.y) / dn;
-  if (!(t > tmin && t < best)) return kInf;
-  const double qx = p.x + t * v.x, qy = p.y + t * v.y;
-  const double along = start ? q[3] * qx + q[4] * qy : q[5] * qx + q[6] * qy;
-  return (along >= -half && tube_r_ok(q, flags, qx, qy, half) && fabs(p.z + t * v.z) <= q[2] + half) ? t : kInf;
-}
-
-// enter = true: first entering crossing with t > half (DistanceToIn);
-// enter = false: first exiting crossing with t > -half (DistanceToOut, clamped by the caller).
-__device__ __noinline__ double tube_cross(const double *q, int flags, const V3 &p, const V3 &v, double half, bool enter) {
-  const double tmin = enter ? half : -half;
-  double best = tube_z_cand(q, flags, p, v, half, enter, tmin);
-  best = fmin(best, tube_cyl_cand(q, flags, p, v, half, enter, tmin, best, true));
-  if (flags & kHasRmin) best = fmin(best, tube_cyl_cand(q, flags, p, v, half, enter, tmin, best, false));
-  if (flags & kSeg) {
-    best = fmin(best, tube_phi_cand(q, flags, p, v, half, enter, tmin, best, true));
-    best = fmin(best, tube_phi_cand(q, flags, p, v, half, enter, tmin, best, false));
-  }
-  return best;
-}
-
-__device__ __forceinline__ double tube_safety_in(const double *q, int flags, const V3 &p) {
-  const double r = sqrt(p.x * p.x + p.y * p.y);
-  double m = fmax(r - q[1], fabs(p.z) - q[2]);
-  if (flags & kHasRmin) m = fmax(m, q[0] - r);
-  if (flags & kSeg) {
-    const double a = q[4] * p.x - q[3] * p.y, b = q[5] * p.y - q[6] * p.x;
-    m = fmax(m, (flags & kWide) ? fmin(a, b) : fmax(a, b));
-  }
-  return fmax(m, 0.0);
-}
-
-__device__ __forceinline__ double tube_safety_out(const double *q, int flags, const V3 &p) {
-  const double r = sqrt(p.x * p.x + p.y * p.y);
-  double m = fmin(q[1] - r, q[2] - fabs(p.z));
-  if (flags & kHasRmin) m = fmin(m, r - q[0]);
-  if (flags & kSeg) m = fmin(m, fmin(fabs(q[3] * p.y - q[4] * p.x), fabs(q[6] * p.x - q[5] * p.y)));
-  return fmax(m, 0.0);
-}
-
-// ---------------------------------------------------------------- cone (full in phi)
-// q[0..6] = ki, ci, ko, co, hz, cos(inner half-angle), cos(outer half-angle): between
-// z = -hz and +hz the solid is Rin(z) <= r <= Rout(z), Rout = ko z + co, Rin = ki z + ci
-// (flag kHasRmin: inner surface present).  Bands along r at the point's z; outward normal of
-// the outer surface along (x / r, y / r, -ko), of the inner one along (-x / r, -y / r, ki).
-
-__device__ __noinline__ bool cone_inside(const double *q, int flags, const V3 &p, const V3 &v, double half) {
-  const double sz = fabs(p.z) - q[4];
-  if (sz > half) return false;
-  const double r2 = p.x * p.x + p.y * p.y;
-  const double ro = q[2] * p.z + q[3];
-  const double rop = ro + half, rom = ro - half;
-  if (r2 > rop * rop) return false;
-  const bool nz = sz >= -half;
-  const bool nrmax = r2 >= rom * rom;
-  bool nrmin = false;
-  if (flags & kHasRmin) {
-    const double ri = q[0] * p.z + q[1];
-    const double rim = ri - half, rip = ri + half;
-    if (r2 < rim * rim) return false;
-    nrmin = r2 <= rip * rip;
-  }
-  if (!(nz || nrmax || nrmin)) return true;
-  const double r = sqrt(r2);
-  const double vr = p.x * v.x + p.y * v.y;
-  if (nz && !(p.z * v.z < 0.0)) return false;
-  if (nrmax && !(vr - q[2] * r * v.z < 0.0)) return false;
-  if (nrmin && !(vr - q[0] * r * v.z > 0.0)) return false;
-  return true;
-}
-
-// enter = true: first entering crossing with t > half; enter = false: first exiting crossing
-// with t > -half.  Conical surfaces: a t^2 + 2 b t + cc = 0 with d = a t + b half the rate of
-// change of r^2 - R^2 along the ray (entering the solid: d < 0 at the outer surface, d > 0 at
-// the inner one); roots on the other half of the double cone (R < 0) are not surface points.
-__device__ __noinline__ double cone_cross(const double *q, int flags, const V3 &p, const V3 &v, double half, bool enter) {
-  const double tmin = enter ? half : -half;
-  const double hz = q[4];
-  double best = kInf;
-  if (v.z != 0.0) {
-    const double sg = ((v.z < 0.0) == enter) ? 1.0 : -1.0;
-    const double t = (sg * hz - p.z) / v.z;
-    if (t > tmin) {
-      const double qx = p.x + t * v.x, qy = p.y + t * v.y;
-      const double r2 = qx * qx + qy * qy;
-      const double ro = q[2] * (sg * hz) + q[3] + half;
-      bool ok = r2 <= ro * ro;
-      if (flags & kHasRmin) {
-        const double ri = q[0] * (sg * hz) + q[1] - half;
-        ok = ok && !(r2 < ri * ri);
-      }
-      if (ok) best = t;
-    }
-  }
-  const int nw = (flags & kHasRmin) ? 2 : 1;
-#pragma unroll 1
-  for (int w = 0; w < nw; ++w) {
-    const double k = w == 0 ? q[2] : q[0], c = w == 0 ? q[3] : q[1];
-    const double rz = k * p.z + c;
-    const double a = v.x * v.x + v.y * v.y - k * k * v.z * v.z;
-    const double b = p.x * v.x + p.y * v.y - k * v.z * rz;
-    const double cc = p.x * p.x + p.y * p.y - rz * rz;
-    double t0 = kInf, t1 = kInf;
-    if (a != 0.0) {
-      const double disc = b * b - a * cc;
-      if (disc > 0.0) {
-        const double sq = sqrt(disc);
-        const double qq = -(b + copysign(sq, b));
-        t0 = qq / a;
-        t1 = cc / qq;
-      }
-    } else if (b != 0.0) {
-      t0 = -cc / (2.0 * b);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const double t = i == 0 ? t0 : t1;
-      if (!(t > tmin && t < best)) continue;
-      const double d = a * t + b;
-      const bool into = w == 0 ? d < 0.0 : d > 0.0;
-      if (into != enter) continue;
-      const double qz = p.z + t * v.z;
-      if (fabs(qz) > hz + half) continue;
-      if (!(k * qz + c >= 0.0)) continue;
-      best = t;
-    }
-  }
-  return best;
-}
-
-__device__ __forceinline__ double cone_safety_in(const double *q, int flags, const V3 &p) {
-  const double r = sqrt(p.x * p.x + p.y * p.y);
-  double m = fmax(fabs(p.z) - q[4], (r - (q[2] * p.z + q[3])) * q[6]);
-  if (flags & kHasRmin) m = fmax(m, ((q[0] * p.z + q[1]) - r) * q[5]);
-  return fmax(m, 0.0);
-}
-
-__device__ __forceinline__ double cone_safety_out(const double *q, int flags, const V3 &p) {
-  const double r = sqrt(p.x * p.x + p.y * p.y);
-  double m = fmin(q[4] - fabs(p.z), ((q[2] * p.z + q[3]) - r) * q[6]);
-  if (flags & kHasRmin) m = fmin(m, (r - (q[0] * p.z + q[1])) * q[5]);
-  return fmax(m, 0.0);
-}
-
 // ---------------------------------------------------------------- dispatch on the solid kind
 
 __device__ __forceinline__ bool vol_inside(const DVol &d, const V3 &p, const V3 &v, double half) {
@@ -484,20 +72,61 @@ __device__ __forceinline__ bool vol_inside(const DVol &d, const V3 &p, const V3 
   return tube_inside(d.p, d.flags, p, v, half);
 }
 
-__device__ __forceinline__ double vol_dist_in(const DVol &d, const V3 &p, const V3 &v, double half) {
+// The full FP64 formulas (every surface), for cones and where the FP32 bounds of pick_solid do not decide.
+__device__ __noinline__ double vol_dist_in_full(const DVol &d, const V3 &p, const V3 &v, double half) {
   if (d.kind == kBox) return box_dist_in(d.p, p, v, half);
   if (d.kind == kOrb) return orb_dist_in(d.p[0], p, v, half);
   if (d.kind == kCone) return cone_cross(d.p, d.flags, p, v, half, true);
   return tube_cross(d.p, d.flags, p, v, half, true);
 }
 
-__device__ __forceinline__ double vol_dist_out(const DVol &d, const V3 &p, const V3 &v, const Inv3 &iv, double half,
-                                               int *face) {
-  *face = -1;
-  if (d.kind == kBox) return box_dist_out(d.p, p, v, iv, face);
+__device__ __noinline__ double vol_dist_out_full(const DVol &d, const V3 &p, const V3 &v, double half) {
+  if (d.kind == kBox) {
+    int face;
+    return box_dist_out(d.p, p, v, inv_dir(v), &face);
+  }
   if (d.kind == kOrb) return orb_dist_out(d.p[0], p, v);
   const double t = d.kind == kCone ? cone_cross(d.p, d.flags, p, v, half, false) : tube_cross(d.p, d.flags, p, v, half, false);
   return t == kInf ? 0.0 : fmax(t, 0.0);
+}
+
+// DistanceToIn, DistanceToOut: FP32 bounds choose the surface (or prove a miss), FP64 evaluates its crossing parameter.
+// Out of line: one copy serves the kernel's call sites (inlined, the calorimeter batch and the persistent barrel were
+// 1.4 and 2 % slower than with the full formulas out of line; so, level and 4 % faster).
+__device__ __noinline__ double vol_dist_in(const DVol &d, const DPick32 &k32, const V3 &p, const V3 &v, double half,
+                                           float band) {
+  const PickRay r = pick_ray(p, v);
+  const int kind = d.kind;
+  const float ext = kind == kOrb ? k32.q[0] : k32.q[0] + k32.q[1] + k32.q[2];
+  const float ep = 2.0f * kU * (fabsf(r.ph[0]) + fabsf(r.ph[1]) + fabsf(r.ph[2]) + ext) + 1e-30f;
+  const Pick k = pick_solid<true>(kind, k32.q, d.flags, r.ph[0], r.ph[1], r.ph[2], r.v[0], r.v[1], r.v[2], ep, band);
+  if (k.surf == kPickMiss) return kInf;
+  if (k.surf >= 0) {
+    double num, den;
+    surf_ratio(kind, d.p, k.surf, true, p, v, num, den);
+    const double t = num / den;
+    if (t > half) return t;
+  }
+  return vol_dist_in_full(d, p, v, half);
+}
+
+__device__ __noinline__ double vol_dist_out_curved(const DVol &d, const DPick32 &k32, const V3 &p, const V3 &v, double half,
+                                                   float band) {
+  const Pick k = pick_leaf(k32, pick_ray(p, v), band);
+  if (k.surf >= 0) {
+    double num, den;
+    surf_ratio(d.kind, d.p, k.surf, false, p, v, num, den);
+    const double t = num / den;
+    if (t > -half) return fmax(t, 0.0);
+  }
+  return vol_dist_out_full(d, p, v, half);
+}
+
+__device__ __forceinline__ double vol_dist_out(const DVol &d, const DPick32 &k32, const V3 &p, const V3 &v, const Inv3 &iv,
+                                               double half, float band, int *face) {
+  *face = -1;
+  if (d.kind == kBox) return box_dist_out(d.p, p, v, iv, face);
+  return vol_dist_out_curved(d, k32, p, v, half, band);
 }
 
 __device__ __forceinline__ double vol_safety_in(const DVol &d, const V3 &p) {
@@ -527,10 +156,24 @@ struct Ray32 {
   int sgn[3];            // sign of v_a (0 if |v_a| < 1e-30)
 };
 
+// The float neighbours of (float)x, below and above, by integer instructions (a conversion holds the FP64 pipe):
+// truncation, rounding to nearest even, a step of one unit either way.  Doubles below 2^-126 take the conversion.
 __device__ __forceinline__ void enclose(double x, float &lo, float &hi) {
-  const float f = (float)x;
-  lo = nextafterf(f, -kInfF);
-  hi = nextafterf(f, kInfF);
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const unsigned t = (h & 0x7fffffffu) - 0x38000000u;
+  if ((int)t < 0x00100000 || t >= 0x0fe00000u) {
+    const float f = (float)x;
+    lo = nextafterf(f, -kInfF);
+    hi = nextafterf(f, kInfF);
+    return;
+  }
+  unsigned m = (t << 3) | (l >> 29);
+  const unsigned rest = l & 0x1fffffffu;
+  m += (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) ? 1u : 0u;
+  const float in = __uint_as_float(m - 1u), out = __uint_as_float(m + 1u);
+  const bool neg = (int)h < 0;
+  lo = neg ? -out : in;
+  hi = neg ? -in : out;
 }
 
 __device__ __forceinline__ Ray32 make_ray32(const V3 &p, const V3 &v) {
@@ -539,17 +182,18 @@ __device__ __forceinline__ Ray32 make_ray32(const V3 &p, const V3 &v) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     enclose(pp[a], r.plo[a], r.phi[a]);
-    const double w = fabs(vv[a]);
-    if (w < 1e-30) {
+    const long long wb = __double_as_longlong(vv[a]) & 0x7FFFFFFFFFFFFFFFll;
+    if (wb < 0x39B4484BFEEBC2A0ll) {  // |v_a| < 1e-30
       r.sgn[a] = 0;
       r.ilo[a] = r.ihi[a] = 0.f;
       continue;
     }
-    r.sgn[a] = vv[a] > 0.0 ? 1 : -1;
+    r.sgn[a] = __double_as_longlong(vv[a]) > 0 ? 1 : -1;
     float wlo, whi;
-    enclose(w, wlo, whi);
-    r.ilo[a] = __frcp_rd(whi);
-    r.ihi[a] = wlo > 0.f ? __frcp_ru(wlo) : kInfF;
+    enclose(__longlong_as_double(wb), wlo, whi);
+    // the approximate reciprocal is within u of the reciprocal
+    r.ilo[a] = __fmul_rd(rcp_approx(whi), 1.0f - 2.0f * kU);
+    r.ihi[a] = __fmul_ru(rcp_approx(wlo), 1.0f + 2.0f * kU);
   }
   return r;
 }
@@ -598,76 +242,47 @@ __device__ __forceinline__ float box_gap_lb(const float *lo, const float *hi, co
 __device__ __forceinline__ float absmax(float lo, float hi) { return fmaxf(fabsf(lo), fabsf(hi)); }
 __device__ __forceinline__ float absmin(float lo, float hi) { return (lo <= 0.f && hi >= 0.f) ? 0.f : fminf(fabsf(lo), fabsf(hi)); }
 
-// Bounds of the leaf's DistanceToOut in its own frame: [*lo, *hi].  Boxes get the
-// directional interval; orbs and tubes the isotropic safety (lower) and the exit
-// of their bounding box (upper).  Also a lower bound of the isotropic safety.
-__device__ __forceinline__ void exit_bounds32(const DVol &V, const Ray32 &r, const V3 &p, float *lo, float *hi,
-                                              float *safety) {
-  float h[3];
-  if (V.kind == kBox) {
-    h[0] = __double2float_rd(V.p[0]);
-    h[1] = __double2float_rd(V.p[1]);
-    h[2] = __double2float_rd(V.p[2]);
-    float tlo = kInfF, thi = kInfF, s = kInfF;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      s = fminf(s, __fsub_rd(h[a], absmax(r.plo[a], r.phi[a])));
-      if (r.sgn[a] == 0) continue;
-      // exit through the face +h (v > 0) or -h (v < 0): distance (h - s p) / |v| with s = sign(v)
-      const float hu = __double2float_ru(V.p[a]);
-      float nlo, nhi;
-      if (r.sgn[a] > 0) {
-        nlo = __fsub_rd(h[a], r.phi[a]);
-        nhi = __fsub_ru(hu, r.plo[a]);
-      } else {
-        nlo = __fadd_rd(h[a], r.plo[a]);
-        nhi = __fadd_ru(hu, r.phi[a]);
-      }
-      tlo = fminf(tlo, div_lo(nlo, r, a));
-      thi = fminf(thi, div_hi(nhi, r, a));
-    }
-    *lo = fmaxf(tlo, 0.f);
-    *hi = fmaxf(thi, 0.f);
-    *safety = fmaxf(s, 0.f);
-    return;
-  }
-  float ax = absmax(r.plo[0], r.phi[0]), ay = absmax(r.plo[1], r.phi[1]), az = absmax(r.plo[2], r.phi[2]);
+// __double2float_rd / _ru of a double that is not negative, by integer instructions where it is of normal float size.
+__device__ __forceinline__ float float_rd(double x) {
+  const unsigned t = (unsigned)__double2hiint(x) - 0x38000000u;
+  if ((int)t < 0x00100000 || t >= 0x0fe00000u) return __double2float_rd(x);
+  return __uint_as_float((t << 3) | ((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ float float_ru(double x) {
+  const unsigned t = (unsigned)__double2hiint(x) - 0x38000000u, l = (unsigned)__double2loint(x);
+  if ((int)t < 0x00100000 || t >= 0x0fe00000u) return __double2float_ru(x);
+  return __uint_as_float(((t << 3) | (l >> 29)) + ((l & 0x1fffffffu) ? 1u : 0u));
+}
+
+// Lower bound of the isotropic safety of the leaf, point in its own frame (cones: 0).
+__device__ __forceinline__ float leaf_safety32(const DVol &V, const Ray32 &r, const V3 &p) {
   float s;
-  float ext[3];
-  if (V.kind == kCone) {
-    // no FP32 safety (0 bounds it); the exit lies within the bounding box of the end radii
-    s = 0.f;
-    const double rmax = fmax(V.p[3] - V.p[2] * V.p[4], V.p[3] + V.p[2] * V.p[4]);
-    ext[0] = ext[1] = __double2float_ru(rmax);
-    ext[2] = __double2float_ru(V.p[4]);
-  } else if (V.kind == kOrb) {
-    const float R = __double2float_rd(V.p[0]);
+  if (V.kind == kBox) {
+    s = kInfF;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) s = fminf(s, __fsub_rd(float_rd(V.p[a]), absmax(r.plo[a], r.phi[a])));
+    return fmaxf(s, 0.f);
+  }
+  if (V.kind == kCone) return 0.f;
+  const float ax = absmax(r.plo[0], r.phi[0]), ay = absmax(r.plo[1], r.phi[1]), az = absmax(r.plo[2], r.phi[2]);
+  if (V.kind == kOrb) {
     const float rr = __fsqrt_ru(__fadd_ru(__fadd_ru(__fmul_ru(ax, ax), __fmul_ru(ay, ay)), __fmul_ru(az, az)));
-    s = __fsub_rd(R, rr);
-    ext[0] = ext[1] = ext[2] = __double2float_ru(V.p[0]);
+    s = __fsub_rd(float_rd(V.p[0]), rr);
   } else {
-    const float rmax = __double2float_rd(V.p[1]), hz = __double2float_rd(V.p[2]);
     const float rup = __fsqrt_ru(__fadd_ru(__fmul_ru(ax, ax), __fmul_ru(ay, ay)));
-    s = fminf(__fsub_rd(rmax, rup), __fsub_rd(hz, az));
+    s = fminf(__fsub_rd(float_rd(V.p[1]), rup), __fsub_rd(float_rd(V.p[2]), az));
     if (V.flags & kHasRmin) {
       const float mx = absmin(r.plo[0], r.phi[0]), my = absmin(r.plo[1], r.phi[1]);
       const float rdn = __fsqrt_rd(__fadd_rd(__fmul_rd(mx, mx), __fmul_rd(my, my)));
-      s = fminf(s, __fsub_rd(rdn, __double2float_ru(V.p[0])));
+      s = fminf(s, __fsub_rd(rdn, float_ru(V.p[0])));
     }
     if (V.flags & kSeg) {
       // phi planes: exact FP64 distances to the two lines, rounded down
       const double ds = fabs(V.p[3] * p.y - V.p[4] * p.x), de = fabs(V.p[6] * p.x - V.p[5] * p.y);
-      s = fminf(s, __double2float_rd(fmin(ds, de)));
+      s = fminf(s, fminf(float_rd(ds), float_rd(de)));
     }
-    ext[0] = ext[1] = __double2float_ru(V.p[1]);
-    ext[2] = __double2float_ru(V.p[2]);
   }
-  const float mlo[3] = {-ext[0], -ext[1], -ext[2]};
-  float xub = kInfF;
-  box_entry_lb(mlo, ext, r, &xub);
-  *safety = fmaxf(s, 0.f);
-  *lo = *safety;
-  *hi = xub;
+  return fmaxf(s, 0.f);
 }
 
 // Is the point inside the solid by more than the tolerance band whatever the direction?
@@ -676,21 +291,21 @@ __device__ __forceinline__ bool certainly_inside32(const DVol &V, const Ray32 &r
   if (V.kind == kBox) {
 #pragma unroll
     for (int a = 0; a < 3; ++a)
-      if (!(absmax(r.plo[a], r.phi[a]) < __fsub_rd(__double2float_rd(V.p[a]), band))) return false;
+      if (!(absmax(r.plo[a], r.phi[a]) < __fsub_rd(float_rd(V.p[a]), band))) return false;
     return true;
   }
   if (V.kind == kCone) return false;
   const float ax = absmax(r.plo[0], r.phi[0]), ay = absmax(r.plo[1], r.phi[1]), az = absmax(r.plo[2], r.phi[2]);
   if (V.kind == kOrb) {
-    const float R = __fsub_rd(__double2float_rd(V.p[0]), band);
+    const float R = __fsub_rd(float_rd(V.p[0]), band);
     return R > 0.f && __fadd_ru(__fadd_ru(__fmul_ru(ax, ax), __fmul_ru(ay, ay)), __fmul_ru(az, az)) < __fmul_rd(R, R);
   }
   if (V.flags & kSeg) return false;
-  const float rmax = __fsub_rd(__double2float_rd(V.p[1]), band);
-  if (!(az < __fsub_rd(__double2float_rd(V.p[2]), band))) return false;
+  const float rmax = __fsub_rd(float_rd(V.p[1]), band);
+  if (!(az < __fsub_rd(float_rd(V.p[2]), band))) return false;
   if (!(__fadd_ru(__fmul_ru(ax, ax), __fmul_ru(ay, ay)) < __fmul_rd(rmax, rmax))) return false;
   if (V.flags & kHasRmin) {
-    const float rmin = __fadd_ru(__double2float_ru(V.p[0]), band);
+    const float rmin = __fadd_ru(float_ru(V.p[0]), band);
     const float mx = absmin(r.plo[0], r.phi[0]), my = absmin(r.plo[1], r.phi[1]);
     if (!(__fadd_rd(__fmul_rd(mx, mx), __fmul_rd(my, my)) > __fmul_ru(rmin, rmin))) return false;
   }
@@ -779,7 +394,7 @@ __device__ __forceinline__ bool advance32(const Ray32 &r, const V3 &v, int a, fl
   }
   // |v_a| lies in [1 / ihi, 1 / ilo]
   const float ilo = sel3(r.ilo[0], r.ilo[1], r.ilo[2], a), ihi = sel3(r.ihi[0], r.ihi[1], r.ihi[2], a);
-  const float vlo = __frcp_rd(ihi), vhi = __frcp_ru(ilo);
+  const float vlo = __fmul_rd(rcp_approx(ihi), 1.0f - 2.0f * kU), vhi = __fmul_ru(rcp_approx(ilo), 1.0f + 2.0f * kU);
   const float mlo = tl >= 0.f ? __fmul_rd(tl, vlo) : __fmul_rd(tl, vhi);
   const float mhi = th >= 0.f ? __fmul_ru(th, vhi) : __fmul_ru(th, vlo);
   if (sg > 0) {
@@ -966,7 +581,7 @@ __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, 
             pz = (float)p.z;
             have_pf = true;
           }
-          if (box32_contains(B, px, py, pz) && !(iso_lb32(G.v32[c], px, py, pz) > (float)(2.0 * G.half))) {
+          if (box32_contains(B, px, py, pz) && !(iso_lb32(G.v32[c], px, py, pz) > G.band32)) {
             d = c;
             break;
           }
@@ -1072,7 +687,7 @@ __device__ __forceinline__ int relocate_warp(const DGeom &G, bool active, int le
       } else {
         world_to_local(G.wxf[leaf], L.flags & kWorldAligned, x, u, p, v);
         have_p = true;
-        if (MODE != kFP64) ok = certainly_inside32(L, make_ray32(p, v), (float)(4.0 * G.half) + 1e-30f);
+        if (MODE != kFP64) ok = certainly_inside32(L, make_ray32(p, v), 2.0f * G.band32 + 1e-30f);
         if (!ok) {
           diag_test<COUNT>(cnt, G4N_C_INSIDE, G4N_C_INSIDE_CURVED, L.kind);
           ok = vol_inside(L, p, v, G.half);
@@ -1377,9 +992,9 @@ __device__ __forceinline__ void node_features(const DGeom &G, const DVol &V, con
 // later round at the node it had stepped into (its Chain, kept by the caller), with the best
 // daughter found so far and the safety bound of its first round.
 struct WalkResume {
-  double best;    // best DistanceToIn found so far (+inf: none)
-  double safety;  // isotropic safety bound of the first round
-  int bl;         // the daughter of `best` (G4N_LIM_MOTHER: none)
+  double best;    // best DistanceToIn found so far (+inf: none); FP32 modes: two floats, its enclosure
+  double safety;  // isotropic safety bound of the first round; FP32 modes: two floats, it and the undecided bound
+  int bl;         // the daughter of `best` (G4N_LIM_MOTHER: none); FP32 modes: daughter << 3 | surface
   int it;         // voxel nodes walked so far (the walk's iteration cap)
 };
 
@@ -1388,20 +1003,14 @@ struct StepResult {
   double safety;  // isotropic lower bound
   int lim;        // daughter id or G4N_LIM_MOTHER
   int face;       // limiter mother and a box leaf: the exit face (2 axis + (v_axis > 0)), else -1
-  bool physics;   // FP32 mode: proven that the limit comes first (no FP64 geometry done)
   bool yielded;   // the search used its node budget: continue it from `resume`
   WalkResume resume;
 };
 
-// iv: the reciprocal of v; the FP32 modes read it only when the leaf is a box (its exit).
-//
-// Geometric step inside `leaf` from local point p along v (Sec. 3.2, problem 2),
-// warp-collective: DistanceToOut of the leaf, then DistanceToIn of the daughters
-// listed in the voxel nodes the ray crosses, stopping once the node exit lies
-// beyond the best distance or `limit`.  FP64 mode: every candidate in FP64.  FP32
-// mode: a candidate is evaluated in FP64 only if its FP32 entry bound does not
-// exceed the best exact distance so far, and no FP64 geometry at all is done when
-// the bounds prove that `limit` comes first.  Both return the FP64 result.
+// Geometric step inside `leaf` from local point p along v (Sec. 3.2, problem 2), plain FP64 navigator,
+// warp-collective: DistanceToOut of the leaf, then DistanceToIn of every daughter listed in the voxel nodes
+// the ray crosses, stopping once the node exit lies beyond the best distance or `limit`.
+// iv: the reciprocal of v.
 //
 // walk_cap: the voxel nodes a search may walk in all (its rounds together); a search that reaches it
 // stops there and sets *timeout (the caller reports G4N_ERR_TIMEOUT).
@@ -1410,7 +1019,7 @@ struct StepResult {
 // state to continue from in R.resume and in `ch`, which then holds the node stepped into);
 // `resume` continues such a search from there.  The result of a search is the same whether
 // or not it yields.  `ch` is the caller's voxel chain (per-lane local memory).
-template <int MODE, bool COUNT>
+template <bool COUNT>
 __device__ __forceinline__ StepResult geom_step_warp(const DGeom &G, bool active, int leaf, const V3 &p, const V3 &v,
                                                      const Inv3 &iv, double limit, bool want_safety, Counters &cnt,
                                                      bool *timeout, int walk_cap, const MlpCtx &mc, Chain &ch,
@@ -1418,60 +1027,248 @@ __device__ __forceinline__ StepResult geom_step_warp(const DGeom &G, bool active
                                                      const WalkResume &from = WalkResume{kInf, 0.0, -1, 0},
                                                      int budget = 0) {
   const double half = G.half;
-  StepResult R{kInf, 0.0, G4N_LIM_MOTHER, -1, false, false, WalkResume{kInf, 0.0, -1, 0}};
+  StepResult R{kInf, 0.0, G4N_LIM_MOTHER, -1, false, WalkResume{kInf, 0.0, -1, 0}};
   int nodes = 0;          // node steps taken in this call (the budget)
   double best = kInf, stop = 0.0, tout = kInf;
   int oface = -1;
-  float out_lo = 0.f;
-  float bound_f = kInfF;  // FP32 modes: float >= min(best, stop), the FP32 walk's bound
-  float saf_f = 0.f;      // FP32 modes: the isotropic safety bound
-  Ray32 r;
   bool walking = false, first = true;
   int i = 0, it = 0, bl = G4N_LIM_MOTHER;
   DCandList L{0, 0}, L0{0, 0};
-  int prop_done = -1;
   float feat[mlp::kIn];
   bool have_feat = false;
   if (active) {
     const DVol &V = G.vol[leaf];
-    if (MODE != kFP64) {
-      r = make_ray32(p, v);
-      float out_hi, saf32;
-      exit_bounds32(V, r, p, &out_lo, &out_hi, &saf32);
-      saf_f = resume ? (float)from.safety : saf32;
-      stop = fmin(limit, (double)out_hi);
-    } else {
-      diag_test<COUNT>(cnt, G4N_C_DIST_OUT, G4N_C_DIST_OUT_CURVED, V.kind);
-      tout = vol_dist_out(V, p, v, iv, half, &oface);
-      R.safety = resume ? from.safety : (want_safety ? vol_safety_out(V, p) : 0.0);
-      stop = fmin(limit, tout);
-    }
+    diag_test<COUNT>(cnt, G4N_C_DIST_OUT, G4N_C_DIST_OUT_CURVED, V.kind);
+    tout = vol_dist_out(V, G.pick[leaf], p, v, iv, half, G.band32, &oface);
+    R.safety = resume ? from.safety : (want_safety ? vol_safety_out(V, p) : 0.0);
+    stop = fmin(limit, tout);
     if (resume) {
       best = from.best;
       bl = from.bl;
       it = from.it;
       first = false;
     }
-    if (MODE != kFP64) bound_f = __double2float_ru(fmin(best, stop));
     if (V.vox >= 0) {
-      if (!resume && (MODE == kFP64 || !chain_fill32(G, ch, V.vox, r))) chain_fill(G, ch, 0, V.vox, p);
+      if (!resume) chain_fill(G, ch, 0, V.vox, p);
       L = G.clist[ch.list];
       L0 = L;
       walking = true;
       diag<COUNT>(cnt, G4N_C_VOX_NODES);
-      if (!resume && (MODE == kLearned || mc.log) && L.count >= 2 && L.count <= mlp::kOut) {
-        // learned mode: a proposal can only save work when two or more of the node's candidates pass
-        // the FP32 bounds (with one or none the bounds alone leave a single FP64 evaluation at most)
-        int open = 2;
-        if (MODE == kLearned) {
-          open = 0;
+      if (!resume && mc.log && L.count >= 2 && L.count <= mlp::kOut) {
+        node_features(G, V, ch, p, v, mc.loge, L.count, feat);
+        have_feat = true;
+      }
+    }
+  }
 #pragma unroll 1
-          for (int k = 0; k < L.count && open < 2; ++k) {
-            const int c = __ldg(&G.cand[L.offset + k]);
-            const DBox32 B = G.box[c];
-            const float iso = iso_lb32(G.v32[c], r.plo[0], r.plo[1], r.plo[2]) - (float)(2.0 * G.half);
-            if (fmaxf(box_entry_lb(B.lo, B.hi, r, nullptr), iso) <= bound_f) ++open;
-          }
+  while (__any_sync(kFull, walking)) {
+    int d = -1;
+    bool from_first = false;
+    if (walking) {
+      // the next candidate, walking nodes as lists run out
+#pragma unroll 1
+      for (;;) {
+        if (i < L.count) {
+          d = __ldg(&G.cand[L.offset + i]);
+          ++i;
+          from_first = first;
+          break;
+        }
+        // list done: exit of the current node along the ray; its slab boundaries bound the safety
+        const int w = walk_step64(G, ch, p, v, iv, fmin(best, stop), first && want_safety, &R.safety, &it, walk_cap, timeout);
+        first = false;
+        if (w == 0) {
+          walking = false;
+          break;
+        }
+        if (budget > 0 && ++nodes >= budget) {
+          // yield: ch holds the node stepped into; the search continues there in a later round
+          walking = false;
+          R.yielded = true;
+          diag<COUNT>(cnt, G4N_C_WALK_YIELDS);
+          break;
+        }
+        L = G.clist[ch.list];
+        i = 0;
+        diag<COUNT>(cnt, G4N_C_VOX_NODES);
+      }
+    }
+    __syncwarp();
+    if (d >= 0) {
+      const DVol &D = G.vol[d];
+      V3 dp, dv;
+      to_local(D, p, v, dp, dv);
+      diag_kind<COUNT>(cnt, D.kind);
+      const double t = vol_dist_in(D, G.pick[d], dp, dv, half, G.band32);
+      if (t < kInf && (t < best || (t == best && (bl < 0 || d < bl)))) {
+        best = t;
+        bl = d;
+      }
+      if (from_first && want_safety) R.safety = fmin(R.safety, vol_safety_in(D, dp));
+    }
+  }
+  if (!active) return R;
+  if (R.yielded) {
+    R.resume = WalkResume{best, R.safety, bl, it};
+    return R;
+  }
+  if (mc.log && have_feat && bl >= 0 && best <= tout) {
+    // training sample: the daughter entered, if it is listed in the first node
+    int slot = -1;
+    for (int k = 0; k < L0.count; ++k)
+      if (__ldg(&G.cand[L0.offset + k]) == bl) {
+        slot = k;
+        break;
+      }
+    if (slot >= 0) {
+      const unsigned long long at = atomicAdd(mc.log->count, 1ull);
+      if ((int64_t)at < mc.log->capacity) {
+        for (int k = 0; k < mlp::kIn; ++k) mc.log->feat[at * mlp::kIn + k] = feat[k];
+        mc.log->label[at] = slot;
+        mc.log->ncand[at] = L0.count;
+      }
+    }
+  }
+  // a daughter wins a tie with the mother; `best` already holds the lowest id among tied daughters
+  if (bl >= 0 && best <= tout) {
+    R.step = best;
+    R.lim = bl;
+  } else {
+    R.step = tout;
+    R.lim = G4N_LIM_MOTHER;
+    R.face = oface;
+  }
+  return R;
+}
+
+// ---------------------------------------------------------------- geometric step of the FP32 modes
+// The whole search in FP32: the leaf's exit, the voxel walk and the candidates as enclosures [lo, hi] of their crossing
+// parameters (nav_pick32.cuh).  Where one enclosure lies before all others it names the volume and the surface that the
+// FP64 search would find, and FP64 evaluates that one crossing parameter (step_exact32), once per step and for all
+// lanes of the warp together.  Where enclosures overlap (two surfaces within ~1e-6 of the coordinates of one another,
+// coinciding surfaces) the search is made again in FP64 (search_full).  Against a search that evaluated the exit and
+// every candidate the bounds let pass in FP64 as it met them (282 FP64 instructions per warp and step on the barrel, the
+// FP64 pipe 60 to 80 % busy): barrel batch of 10^7 tracks 167 -> 113 ms, nested barrel of 10^6 32.5 -> 24.7 ms, 10^6
+// compute_step queries on the barrel 1.61 -> 0.77 ms, identical histories.
+
+constexpr int kSurfFull = 7;   // the crossing was evaluated by the full FP64 formulas (cones, wide segments, unsure)
+
+struct Step32 {
+  float lo, hi;    // enclosure of the geometric step
+  float safety;    // isotropic lower bound
+  int vol;         // daughter entered, or G4N_LIM_MOTHER
+  int surf;        // the surface crossed, or kSurfFull
+  bool undecided;  // another crossing's enclosure overlaps: take search_full
+  bool yielded;
+  WalkResume resume;
+};
+
+// Enclosure of a non-negative double.
+__device__ __forceinline__ void enclose_up(double t, float &lo, float &hi) {
+  lo = trunc_float(t);
+  hi = __fmul_ru(lo, 1.0f + 2.0f * kU) + 1e-37f;
+}
+
+// The FP64 search of one lane, every candidate by the full formulas: step and limiter as geom_step_warp's (no safety).
+__device__ __noinline__ void search_full(const DGeom &G, int leaf, const V3 &p, const V3 &v, int walk_cap, double *step,
+                                         int *lim, int *face, bool *timeout) {
+  const DVol &V = G.vol[leaf];
+  const Inv3 iv = inv_dir(v);
+  int oface = -1, bl = G4N_LIM_MOTHER;
+  const double tout = V.kind == kBox ? box_dist_out(V.p, p, v, iv, &oface) : vol_dist_out_full(V, p, v, G.half);
+  double best = kInf;
+  if (V.vox >= 0) {
+    Chain ch;
+    chain_fill(G, ch, 0, V.vox, p);
+    int it = 0;
+#pragma unroll 1
+    do {
+      const DCandList L = G.clist[ch.list];
+#pragma unroll 1
+      for (int i = 0; i < L.count; ++i) {
+        const int d = __ldg(&G.cand[L.offset + i]);
+        const DVol &D = G.vol[d];
+        V3 dp, dv;
+        to_local(D, p, v, dp, dv);
+        const double t = vol_dist_in_full(D, dp, dv, G.half);
+        if (t < kInf && (t < best || (t == best && (bl < 0 || d < bl)))) {
+          best = t;
+          bl = d;
+        }
+      }
+    } while (walk_step64_ool(G, ch, p, v, iv, fmin(best, tout), false, nullptr, &it, walk_cap, timeout));
+  }
+  const bool in = bl >= 0 && best <= tout;
+  *step = in ? best : tout;
+  *lim = in ? bl : G4N_LIM_MOTHER;
+  *face = in ? -1 : oface;
+}
+
+// limit: a float not below the physics step.  Budget, resume, walk cap and chain as geom_step_warp's.  In the learned
+// mode the network's proposal is looked at before the node's other candidates; its enclosure prunes them.
+template <int MODE, bool COUNT>
+__device__ __forceinline__ Step32 geom_step32_warp(const DGeom &G, bool active, int leaf, const V3 &p, const V3 &v,
+                                                   float limit, bool want_safety, Counters &cnt, bool *timeout,
+                                                   int walk_cap, const MlpCtx &mc, Chain &ch, bool resume = false,
+                                                   const WalkResume &from = WalkResume{0.0, 0.0, -1, 0}, int budget = 0) {
+  Step32 R;
+  R.yielded = false;
+  R.undecided = false;
+  int nodes = 0;          // node steps taken in this call (the budget)
+  float best_lo = kInfF, best_hi = kInfF, unsure_lo = kInfF;   // unsure_lo: two overlapping crossings lie beyond it
+  float exit_lo = 0.f, exit_hi = kInfF, saf_f = 0.f, bound_f = kInfF, stop_f = kInfF;
+  int exit_surf = kSurfFull, best_vol = -1, best_surf = 0;
+  Ray32 r;
+  PickRay q;
+  bool walking = false, first = true;
+  int i = 0, it = 0;
+  DCandList L{0, 0}, L0{0, 0};
+  int prop_done = -1;
+  float feat[mlp::kIn];
+  bool have_feat = false;
+  if (active) {
+    const DVol &V = G.vol[leaf];
+    r = make_ray32(p, v);
+    q = pick_ray(p, v);
+    diag_test<COUNT>(cnt, G4N_C_DIST_OUT, G4N_C_DIST_OUT_CURVED, V.kind);
+    const Pick x = pick_leaf(G.pick[leaf], q, G.band32);
+    if (x.surf >= 0) {
+      exit_lo = x.lo;
+      exit_hi = x.hi;
+      exit_surf = x.surf;
+    } else {
+      enclose_up(vol_dist_out_full(V, p, v, G.half), exit_lo, exit_hi);
+    }
+    stop_f = fminf(limit, exit_hi);
+    if (resume) {
+      best_lo = __int_as_float(__double2loint(from.best));
+      best_hi = __int_as_float(__double2hiint(from.best));
+      unsure_lo = __int_as_float(__double2loint(from.safety));
+      saf_f = __int_as_float(__double2hiint(from.safety));
+      best_vol = from.bl < 0 ? -1 : from.bl >> 3;
+      best_surf = from.bl & 7;
+      it = from.it;
+      first = false;
+    } else {
+      saf_f = leaf_safety32(V, r, p);
+    }
+    bound_f = fminf(best_hi, stop_f);
+    if (V.vox >= 0) {
+      if (!resume && !chain_fill32(G, ch, V.vox, r)) chain_fill(G, ch, 0, V.vox, p);
+      L = G.clist[ch.list];
+      L0 = L;
+      walking = true;
+      diag<COUNT>(cnt, G4N_C_VOX_NODES);
+      if (MODE == kLearned && !resume && L.count >= 2 && L.count <= mlp::kOut) {
+        // a proposal can only save work when two or more of the node's candidates pass the FP32 bounds (with one
+        // or none the bounds alone leave a single evaluation at most)
+        int open = 0;
+#pragma unroll 1
+        for (int k = 0; k < L.count && open < 2; ++k) {
+          const int c = __ldg(&G.cand[L.offset + k]);
+          const DBox32 B = G.box[c];
+          const float iso = iso_lb32(G.v32[c], r.plo[0], r.plo[1], r.plo[2]) - G.band32;
+          if (fmaxf(box_entry_lb(B.lo, B.hi, r, nullptr), iso) <= bound_f) ++open;
         }
         if (open >= 2) {
           node_features(G, V, ch, p, v, mc.loge, L.count, feat);
@@ -1480,8 +1277,7 @@ __device__ __forceinline__ StepResult geom_step_warp(const DGeom &G, bool active
       }
     }
   }
-  // learned mode: the network proposes which first-node candidate is entered first; it is
-  // evaluated before the others so that its exact distance prunes them (warp-collective)
+  // learned mode: the network proposes which first-node candidate is entered first (warp-collective)
   int prop = -1;
   if (MODE == kLearned && __any_sync(kFull, have_feat)) {
     float f0[mlp::kIn];
@@ -1498,20 +1294,18 @@ __device__ __forceinline__ StepResult geom_step_warp(const DGeom &G, bool active
 #pragma unroll 1
   while (__any_sync(kFull, walking)) {
     int d = -1;
-    bool from_first = false;
     if (walking) {
-      // scan to the next candidate that needs FP64 work, walking nodes as lists run out
+      // scan to the next candidate that the bounds let matter, walking nodes as lists run out
 #pragma unroll 1
       for (;;) {
         if (MODE == kLearned && prop >= 0) {
           // the proposal goes first if its bound still allows it to matter
           const int c = __ldg(&G.cand[L0.offset + prop]);
           const DBox32 B = G.box[c];
-          const float iso = iso_lb32(G.v32[c], r.plo[0], r.plo[1], r.plo[2]) - (float)(2.0 * G.half);
+          const float iso = iso_lb32(G.v32[c], r.plo[0], r.plo[1], r.plo[2]) - G.band32;
           const float lb = fmaxf(box_entry_lb(B.lo, B.hi, r, nullptr), iso);
           if (lb <= bound_f) {
             d = c;
-            from_first = true;
             break;
           }
           prop = -1;  // not worth it: the scan treats the slot like any other
@@ -1519,35 +1313,26 @@ __device__ __forceinline__ StepResult geom_step_warp(const DGeom &G, bool active
         if (i < L.count) {
           const int c = __ldg(&G.cand[L.offset + i]);
           ++i;
-          if (MODE != kFP64) {
-            const DBox32 B = G.box[c];
-            const float iso = iso_lb32(G.v32[c], r.plo[0], r.plo[1], r.plo[2]) - (float)(2.0 * G.half);
-            if (first && want_safety) saf_f = fminf(saf_f, fmaxf(box_gap_lb(B.lo, B.hi, r), iso));
-            if (MODE == kLearned && first && i - 1 == prop_done) continue;  // already evaluated exactly
-            const float lb = fmaxf(box_entry_lb(B.lo, B.hi, r, nullptr), iso);
-            if (!(lb <= bound_f)) {
-              if (MODE == kLearned) diag<COUNT>(cnt, G4N_C_PRUNED);
-              continue;
-            }
-            diag<COUNT>(cnt, G4N_C_RECHECKS);
+          const DBox32 B = G.box[c];
+          const float iso = iso_lb32(G.v32[c], r.plo[0], r.plo[1], r.plo[2]) - G.band32;
+          if (first && want_safety) saf_f = fminf(saf_f, fmaxf(box_gap_lb(B.lo, B.hi, r), iso));
+          if (MODE == kLearned && first && i - 1 == prop_done) continue;  // already looked at
+          const float lb = fmaxf(box_entry_lb(B.lo, B.hi, r, nullptr), iso);
+          if (!(lb <= bound_f)) {
+            if (MODE == kLearned) diag<COUNT>(cnt, G4N_C_PRUNED);
+            continue;
           }
+          diag<COUNT>(cnt, G4N_C_RECHECKS);
           d = c;
-          from_first = first;
           break;
         }
         // list done: exit of the current node along the ray; its slab boundaries bound the safety
-        int w = 2;
-        if (MODE != kFP64) w = walk_step32(G, ch, r, v, bound_f, first && want_safety, &saf_f, &it, walk_cap, timeout);
+        int w = walk_step32(G, ch, r, v, bound_f, first && want_safety, &saf_f, &it, walk_cap, timeout);
         if (w == 2) {
-          // FP64 node step (the FP32 modes come here only when the intervals do not decide)
-          if (MODE == kFP64) {
-            w = walk_step64(G, ch, p, v, iv, fmin(best, stop), first && want_safety, &R.safety, &it, walk_cap, timeout);
-          } else {
-            double s64 = kInf;
-            w = walk_step64_ool(G, ch, p, v, inv_dir(v), fmin(best, stop), first && want_safety, &s64, &it, walk_cap,
-                                timeout);
-            saf_f = fminf(saf_f, __double2float_rd(s64));
-          }
+          // FP64 node step where the intervals do not decide
+          double s64 = kInf;
+          w = walk_step64_ool(G, ch, p, v, inv_dir(v), (double)bound_f, first && want_safety, &s64, &it, walk_cap, timeout);
+          saf_f = fminf(saf_f, __double2float_rd(s64));
         }
         first = false;
         if (w == 0) {
@@ -1573,61 +1358,96 @@ __device__ __forceinline__ StepResult geom_step_warp(const DGeom &G, bool active
       diag<COUNT>(cnt, G4N_C_RECHECKS);
     }
     if (d >= 0) {
-      const DVol &D = G.vol[d];
-      V3 dp, dv;
-      to_local(D, p, v, dp, dv);
-      diag_kind<COUNT>(cnt, D.kind);
-      const double t = vol_dist_in(D, dp, dv, half);
-      if (t < kInf && (t < best || (t == best && (bl < 0 || d < bl)))) {
-        best = t;
-        bl = d;
-        if (MODE != kFP64) bound_f = __double2float_ru(fmin(best, stop));
+      const DPick32 &D = G.pick[d];
+      diag_kind<COUNT>(cnt, D.kind_flags & 3);
+      Pick k = pick_daughter(D, q, G.band32);
+      if (k.surf == kPickUnsure && k.lo <= bound_f) {
+        // the full formulas
+        V3 dp, dv;
+        to_local(G.vol[d], p, v, dp, dv);
+        const double t = vol_dist_in_full(G.vol[d], dp, dv, G.half);
+        k.surf = t < kInf ? kSurfFull : kPickMiss;
+        enclose_up(t, k.lo, k.hi);
       }
-      if (MODE == kFP64 && from_first && want_safety) R.safety = fmin(R.safety, vol_safety_in(D, dp));
+      if (k.surf >= 0 && d != best_vol) {
+        // a candidate listed in several nodes is met again: the same crossing
+        if (best_vol >= 0 && k.lo <= best_hi && k.hi >= best_lo) unsure_lo = fminf(unsure_lo, fminf(k.lo, best_lo));
+        if (k.hi < best_hi) {
+          best_lo = k.lo;
+          best_hi = k.hi;
+          best_vol = d;
+          best_surf = k.surf;
+          bound_f = fminf(best_hi, stop_f);
+        }
+      }
     }
   }
-  if (MODE != kFP64) R.safety = saf_f;
+  R.safety = saf_f;
   if (!active) return R;
   if (R.yielded) {
-    R.resume = WalkResume{best, R.safety, bl, it};
+    R.resume.best = __hiloint2double(__float_as_int(best_hi), __float_as_int(best_lo));
+    R.resume.safety = __hiloint2double(__float_as_int(saf_f), __float_as_int(unsure_lo));
+    R.resume.bl = best_vol < 0 ? -1 : best_vol << 3 | best_surf;
+    R.resume.it = it;
     return R;
   }
-  if (MODE == kFP64 && mc.log && have_feat && bl >= 0 && best <= tout) {
-    // training sample: the daughter entered, if it is listed in the first node
-    int slot = -1;
-    for (int k = 0; k < L0.count; ++k)
-      if (__ldg(&G.cand[L0.offset + k]) == bl) {
-        slot = k;
-        break;
-      }
-    if (slot >= 0) {
-      const unsigned long long at = atomicAdd(mc.log->count, 1ull);
-      if ((int64_t)at < mc.log->capacity) {
-        for (int k = 0; k < mlp::kIn; ++k) mc.log->feat[at * mlp::kIn + k] = feat[k];
-        mc.log->label[at] = slot;
-        mc.log->ncand[at] = L0.count;
-      }
-    }
-  }
-  if (MODE != kFP64) {
-    // the FP32 bounds prove the limit comes first: no FP64 geometry needed
-    if (best > limit && (double)out_lo > limit) {
-      R.physics = true;
-      return R;
-    }
-    diag_test<COUNT>(cnt, G4N_C_DIST_OUT, G4N_C_DIST_OUT_CURVED, G.vol[leaf].kind);
-    tout = vol_dist_out(G.vol[leaf], p, v, iv, half, &oface);
-  }
-  // a daughter wins a tie with the mother; `best` already holds the lowest id among tied daughters
-  if (bl >= 0 && best <= tout) {
-    R.step = best;
-    R.lim = bl;
-  } else {
-    R.step = tout;
-    R.lim = G4N_LIM_MOTHER;
-    R.face = oface;
-  }
+  // the daughter or the exit, whichever enclosure comes first
+  const bool in = best_vol >= 0 && best_hi < exit_hi;
+  R.lo = fminf(fminf(best_lo, exit_lo), unsure_lo);
+  R.hi = in ? best_hi : exit_hi;
+  R.vol = in ? best_vol : G4N_LIM_MOTHER;
+  R.surf = in ? best_surf : exit_surf;
+  R.undecided = unsure_lo <= R.hi || (best_vol >= 0 && best_lo <= exit_hi && exit_lo <= best_hi);
   return R;
+}
+
+// The step that R names as a quotient for the caller to divide, or exactly: false, with *num = step, where the full
+// formulas or the full search were needed (then *lim and *face are final as well).
+__device__ __forceinline__ bool step_ratio32(const DGeom &G, int leaf, const V3 &p, const V3 &v, const Step32 &R,
+                                             int walk_cap, bool *timeout, double *num, double *den, int *lim, int *face) {
+  *lim = R.vol;
+  *face = -1;
+  if (R.undecided || R.surf == kSurfFull) {
+    if (R.undecided || R.vol < 0) {
+      search_full(G, leaf, p, v, walk_cap, num, lim, face, timeout);
+    } else {
+      V3 dp, dv;
+      to_local(G.vol[R.vol], p, v, dp, dv);
+      *num = vol_dist_in_full(G.vol[R.vol], dp, dv, G.half);
+    }
+    return false;
+  }
+  const bool in = R.vol >= 0;
+  const DVol &D = G.vol[in ? R.vol : leaf];
+  V3 dp = p, dv = v;
+  if (in) to_local(D, p, v, dp, dv);
+  else if (D.kind == kBox) *face = R.surf;
+  surf_ratio(D.kind, D.p, R.surf, in, dp, dv, *num, *den);
+  return true;
+}
+
+// The quotient s of step_ratio32 made a step: true if it lies beyond the surface band; else (a crossing at the start, by
+// rounding) s comes from the full search.
+__device__ __forceinline__ bool step_finish32(const DGeom &G, int leaf, const V3 &p, const V3 &v, double &s, int walk_cap,
+                                              bool *timeout, int *lim, int *face) {
+  if (s > (*lim >= 0 ? G.half : -G.half)) {
+    s = fmax(s, 0.0);
+    return true;
+  }
+  double full;
+  search_full(G, leaf, p, v, walk_cap, &full, lim, face, timeout);
+  s = full;
+  return false;
+}
+
+// The geometric step that R names.
+__device__ __forceinline__ double step_exact32(const DGeom &G, int leaf, const V3 &p, const V3 &v, const Step32 &R,
+                                               int walk_cap, bool *timeout, int *lim, int *face) {
+  double num, den;
+  if (!step_ratio32(G, leaf, p, v, R, walk_cap, timeout, &num, &den, lim, face)) return num;
+  double s = num / den;
+  step_finish32(G, leaf, p, v, s, walk_cap, timeout, lim, face);
+  return s;
 }
 
 // ---------------------------------------------------------------- attenuation table

@@ -163,18 +163,32 @@ __global__ void __launch_bounds__(128) k_compute_step(const DGeom *__restrict__ 
     }
     bool timeout = false;
     Chain ch;
-    const StepResult R = geom_step_warp<MODE, false>(G, ok, leaf, p, v, inv_dir(v), prop, true, cnt, &timeout, walk_cap,
-                                                     mc, ch);
+    double s = kInf, safety = 0.0;
+    int lim = G4N_LIM_MOTHER;
+    if constexpr (MODE == kFP64) {
+      const StepResult R = geom_step_warp<false>(G, ok, leaf, p, v, inv_dir(v), prop, true, cnt, &timeout, walk_cap, mc, ch);
+      s = R.step;
+      lim = R.lim;
+      safety = R.safety;
+    } else {
+      // a float not below the proposal (a NaN proposal limits nothing, a negative one everything)
+      const float f = trunc_float(prop), limit = f < 0.f ? f * (1.0f - 2.0f * kU) : f * (1.0f + 2.0f * kU) + 1e-30f;
+      const Step32 R = geom_step32_warp<MODE, false>(G, ok, leaf, p, v, limit, true, cnt, &timeout, walk_cap, mc, ch);
+      safety = (double)R.safety;
+      if (ok) {
+        int face;
+        if (limit < R.lo) lim = G4N_LIM_PHYSICS;   // the proposal comes first for certain
+        else s = step_exact32(G, leaf, p, v, R, walk_cap, &timeout, &lim, &face);
+      }
+    }
     if (ok) {
       if (timeout) flag(status, kStTimeout);
-      double s = R.step;
-      int lim = R.lim;
-      if (R.physics || prop < s) {
+      if (lim == G4N_LIM_PHYSICS || prop < s) {
         s = prop;
         lim = G4N_LIM_PHYSICS;
       }
       out_step[i] = s;
-      out_safety[i] = R.safety;
+      out_safety[i] = safety;
       out_lim[i] = lim;
     }
   }
@@ -510,79 +524,118 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
     next = kEmpty;
     act = false;
   }
-  // the free path s_phys = Y / mu (Eq. 7) races the geometric step; the division is only done
-  // when its value is needed (physics wins, or a voxel walk / FP32 bound needs the limit)
-  double sphys = kInf;
-  bool need_geo = false;
+  // the free path s_phys = Y / mu (Eq. 7) races the geometric step
+  double s = kInf;
+  int lim = G4N_LIM_PHYSICS, face = -1;
+  bool need_geo = false, geo = false, timeout = false;
   V3 p{0, 0, 0}, v{0, 0, 1};
-  Inv3 iv{0, 0, 0};
-  bool lazy = false;       // FP64 mode: sphys not computed, s * mu is compared with Y instead
-  bool want_saf = true;    // FP64 mode, leaf without daughters: the safety is taken in the interaction phase
-  double lim_geo = kInf;  // limit handed to the geometric step (an upper bound of sphys)
-  if (act) {
-    const DVol &L = G.vol[t.leaf];
-    const bool mu_pos = nonzero_bits(t.mu);  // mu >= 0
-    lazy = MODE == kFP64 && mu_pos && !mc.log;
-    if (!lazy) sphys = mu_pos ? t.Y / t.mu : kInf;
-    // a zero safety (after every boundary crossing) always needs the boundary search.  Lazy form: the
-    // search is skipped only when Y - safety mu (one rounding, by the fma) lies below -2^-49 Y, so that
-    // fl(Y / mu) < safety holds as well (the comparison the oracle makes)
-    need_geo = resume || !nonzero_bits(t.safety) ||
-               (lazy ? !(fma(-t.safety, t.mu, t.Y) < -0x1p-49 * t.Y) : !(sphys < t.safety));
-    want_saf = !(MODE == kFP64 && L.vox < 0);
-    if (!need_geo) {
-      diag<COUNT>(cnt, G4N_C_SAFETY_SKIPS);
-      if (lazy) sphys = t.Y / t.mu;
-    } else {
-      const bool aligned = L.flags & kWorldAligned;
-      world_to_local(G.wxf[t.leaf], aligned, t.x, t.u, p, v);
-      // the reciprocal direction serves the FP64 voxel walk and a box's exit; the FP32 modes walk in
-      // FP32 (their rare FP64 node step forms it itself) and need it only in box leaves
-      iv = aligned ? t.iu : ((MODE == kFP64 || L.kind == kBox) ? inv_dir(v) : Inv3{0.0, 0.0, 0.0});
-      // the voxel walk may stop at any bound >= sphys: candidates found beyond sphys lose
-      // to the physics step all the same
-      lim_geo = !lazy ? sphys
-                : L.vox < 0 ? kInf
-                            : (double)__fdiv_ru(__double2float_ru(t.Y), __double2float_rd(t.mu));
-    }
-  }
-  bool timeout = false;
   if (MODE == kLearned || mc.log) mc.loge = act ? (logf((float)t.E) + 4.6f) * 0.1f : 0.f;
   // the learned proposal and the sample log look at the first node only: no yielding there
   const int budget = (!YIELD || MODE == kLearned || mc.log) ? 0 : P.walk_budget;
-  const StepResult R = geom_step_warp<MODE, COUNT>(G, need_geo, need_geo ? t.leaf : 0, p, v, iv, lim_geo, want_saf,
-                                                   cnt, &timeout, P.walk_cap, mc, wch, resume, t.w, budget);
-  if (act && R.yielded) {
-    // the search used its node budget: the step continues in a later round
-    t.w = R.resume;
-    next = kWalk;
-    act = false;
-  }
-  bool geo = false;
-  double s = sphys;
-  int lim = G4N_LIM_PHYSICS;
-  if (act) {
-    if (timeout) flag(P.status, kStTimeout);
-    if (need_geo) {
+  const bool mu_pos = nonzero_bits(t.mu);  // mu >= 0
+  if constexpr (MODE == kFP64) {
+    // the division is only done when its value is needed: lazily, s * mu is compared with Y instead
+    Inv3 iv{0, 0, 0};
+    bool lazy = false, want_saf = true;  // leaf without daughters: the safety is taken in the interaction phase
+    double sphys = kInf, lim_geo = kInf;  // limit handed to the geometric step (an upper bound of sphys)
+    if (act) {
+      const DVol &L = G.vol[t.leaf];
+      lazy = mu_pos && !mc.log;
+      if (!lazy) sphys = mu_pos ? t.Y / t.mu : kInf;
+      // a zero safety (after every boundary crossing) always needs the boundary search.  Lazy form: the
+      // search is skipped only when Y - safety mu (one rounding, by the fma) lies below -2^-49 Y, so that
+      // fl(Y / mu) < safety holds as well (the comparison the oracle makes)
+      need_geo = resume || !nonzero_bits(t.safety) ||
+                 (lazy ? !(fma(-t.safety, t.mu, t.Y) < -0x1p-49 * t.Y) : !(sphys < t.safety));
+      want_saf = L.vox >= 0;
+      if (!need_geo) {
+        diag<COUNT>(cnt, G4N_C_SAFETY_SKIPS);
+        if (lazy) sphys = t.Y / t.mu;
+      } else {
+        const bool aligned = L.flags & kWorldAligned;
+        world_to_local(G.wxf[t.leaf], aligned, t.x, t.u, p, v);
+        iv = aligned ? t.iu : inv_dir(v);
+        // the voxel walk may stop at any bound >= sphys: candidates found beyond sphys lose
+        // to the physics step all the same
+        lim_geo = !lazy ? sphys
+                  : L.vox < 0 ? kInf
+                              : (double)__fdiv_ru(__double2float_ru(t.Y), __double2float_rd(t.mu));
+      }
+    }
+    const StepResult R = geom_step_warp<COUNT>(G, need_geo, need_geo ? t.leaf : 0, p, v, iv, lim_geo, want_saf, cnt,
+                                               &timeout, P.walk_cap, mc, wch, resume, t.w, budget);
+    if (act && R.yielded) {
+      // the search used its node budget: the step continues in a later round
+      t.w = R.resume;
+      next = kWalk;
+      act = false;
+    }
+    s = sphys;
+    if (act && need_geo) {
       t.safety = R.safety;
       // geometry wins iff step <= fl(Y / mu).  Lazy form: Y - step mu (one rounding, by the fma) decides
       // when it lies outside +-2^-49 Y, a margin far above the rounding of either form; a near-tie takes
       // the division itself
-      bool geo_first;
       if (!lazy) {
-        geo_first = R.step <= sphys;
+        geo = R.step <= sphys;
       } else {
         const double d = fma(-R.step, t.mu, t.Y), m = 0x1p-49 * t.Y;
-        geo_first = d > m || (!(d < -m) && R.step <= t.Y / t.mu);
+        geo = d > m || (!(d < -m) && R.step <= t.Y / t.mu);
       }
-      if (!R.physics && geo_first) {
-        geo = true;
+      if (geo) {
         s = R.step;
         lim = R.lim;
+        face = R.face;
       } else if (lazy) {
-        s = sphys = t.Y / t.mu;
+        s = t.Y / t.mu;
       }
     }
+  } else {
+    // both steps as float enclosures; FP64 evaluates the one that comes first, as one quotient
+    float phys_lo = kInfF, phys_hi = kInfF;
+    if (act) {
+      if (mu_pos) {
+        const float m = trunc_float(t.mu), f = trunc_float(t.Y) * rcp_approx(m);
+        phys_lo = m > 0.f ? f * (1.0f - 8.0f * kU) : 0.f;
+        phys_hi = m > 0.f ? f * (1.0f + 8.0f * kU) + 1e-30f : kInfF;
+      }
+      // a zero safety (after every boundary crossing) always needs the boundary search
+      need_geo = resume || !nonzero_bits(t.safety) || !(phys_hi < trunc_float(t.safety));
+      if (!need_geo) diag<COUNT>(cnt, G4N_C_SAFETY_SKIPS);
+      else world_to_local(G.wxf[t.leaf], G.vol[t.leaf].flags & kWorldAligned, t.x, t.u, p, v);
+    }
+    const Step32 R = geom_step32_warp<MODE, COUNT>(G, need_geo, need_geo ? t.leaf : 0, p, v, phys_hi, true, cnt, &timeout,
+                                                   P.walk_cap, mc, wch, resume, t.w, budget);
+    if (act && R.yielded) {
+      t.w = R.resume;
+      next = kWalk;
+      act = false;
+    }
+    if (act) {
+      double num = t.Y, den = t.mu;
+      bool quotient = true;
+      if (need_geo) {
+        t.safety = (double)R.safety;
+        geo = !(phys_hi < R.lo);
+        if (geo) quotient = step_ratio32(G, t.leaf, p, v, R, P.walk_cap, &timeout, &num, &den, &lim, &face);
+      }
+      s = quotient ? (geo || mu_pos ? num / den : kInf) : num;
+      if (geo) {
+        if (quotient) quotient = step_finish32(G, t.leaf, p, v, s, P.walk_cap, &timeout, &lim, &face);
+        // geometry wins iff step <= fl(Y / mu); the enclosures decide unless they overlap
+        if (mu_pos && (!quotient || !(R.hi < phys_lo))) {
+          const double sphys = t.Y / t.mu;
+          if (!(s <= sphys)) {
+            geo = false;
+            s = sphys;
+            lim = G4N_LIM_PHYSICS;
+          }
+        }
+      }
+    }
+  }
+  if (act) {
+    if (timeout) flag(P.status, kStTimeout);
     ++t.steps;
     if (!EV) cnt.c[G4N_C_STEPS]++;  // EV: the sum of the geometry- and physics-limited counts
     t.x.x += s * t.u.x;
@@ -596,7 +649,7 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       cnt.c[G4N_C_PHYS_STEPS]++;
       next = kInteract;
     } else {
-      if (nonzero_bits(t.mu)) t.Y = fmax(t.Y - s * t.mu, 0.0);
+      if (mu_pos) t.Y = fmax(t.Y - s * t.mu, 0.0);
       cnt.c[G4N_C_GEOM_STEPS]++;
       t.safety = 0.0;
     }
@@ -604,7 +657,7 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
   // leaving a box through a face whose relocation is tabulated needs no search
   int leaf = -1;
   const bool left = geo && lim == G4N_LIM_MOTHER && s > 0.0;
-  const bool fast = left && face_relocate(G, t.leaf, R.face, t.x, t.u, &leaf);
+  const bool fast = left && face_relocate(G, t.leaf, face, t.x, t.u, &leaf);
   if (fast) diag<COUNT>(cnt, G4N_C_FACE_RELOC);
   // relocation search, then (after 10 zero steps) the push and its relocation: one copy of
   // the relocation code serves both passes.  DEFER: a lane that needs the search stops here (its
@@ -979,21 +1032,29 @@ __global__ void __launch_bounds__(128, 3) k_free_path(const FParams P) {
     if (drained && !__any_sync(kFull, active)) break;
     // one segment: the geometric step from x inside `leaf`
     V3 p{0, 0, 0}, v{0, 0, 1};
-    Inv3 iv{0, 0, 0};
-    if (active) {
-      const bool aligned = G.vol[leaf].flags & kWorldAligned;
-      world_to_local(G.wxf[leaf], aligned, x, u, p, v);
-      iv = aligned ? iu : ((MODE == kFP64 || G.vol[leaf].kind == kBox) ? inv_dir(v) : Inv3{0.0, 0.0, 0.0});
-    }
+    double step = kInf;
+    int lim = G4N_LIM_MOTHER, face = -1;
     bool timeout = false;
     Chain ch;
-    const StepResult R = geom_step_warp<MODE, COUNT>(G, active, active ? leaf : 0, p, v, iv, kInf, false, cnt, &timeout,
+    const bool aligned = G.vol[leaf].flags & kWorldAligned;
+    if (active) world_to_local(G.wxf[leaf], aligned, x, u, p, v);
+    if constexpr (MODE == kFP64) {
+      const Inv3 iv = !active ? Inv3{0, 0, 0} : aligned ? iu : inv_dir(v);
+      const StepResult R = geom_step_warp<COUNT>(G, active, active ? leaf : 0, p, v, iv, kInf, false, cnt, &timeout,
+                                                 P.walk_cap, mc, ch);
+      step = R.step;
+      lim = R.lim;
+      face = R.face;
+    } else {
+      const Step32 R = geom_step32_warp<MODE, COUNT>(G, active, active ? leaf : 0, p, v, kInfF, false, cnt, &timeout,
                                                      P.walk_cap, mc, ch);
+      if (active) step = step_exact32(G, leaf, p, v, R, P.walk_cap, &timeout, &lim, &face);
+    }
     bool cross = false;
     double s = 0.0;
     if (active) {
       if (timeout) flag(P.status, kStTimeout);
-      s = R.step;
+      s = step;
       ++steps;
       cnt.c[G4N_C_STEPS]++;
       if (mu > 0.0 && S + s * mu >= Y) {
@@ -1015,9 +1076,9 @@ __global__ void __launch_bounds__(128, 3) k_free_path(const FParams P) {
         cross = true;
       }
     }
-    const bool left = cross && R.lim == G4N_LIM_MOTHER && s > 0.0;
+    const bool left = cross && lim == G4N_LIM_MOTHER && s > 0.0;
     int nl = -1;
-    const bool fast = left && face_relocate(G, leaf, R.face, x, u, &nl);
+    const bool fast = left && face_relocate(G, leaf, face, x, u, &nl);
     if (fast) diag<COUNT>(cnt, G4N_C_FACE_RELOC);
     const int searched = relocate_warp<MODE, COUNT>(G, cross && !fast, cross && !fast ? leaf : 0, x, u, left, cnt);
     if (!fast) nl = searched;

@@ -73,6 +73,29 @@ __device__ __forceinline__ void event(Counters &cnt, int k) {
   else cnt.c[k]++;
 }
 
+// The counts of the warp's lanes (registers) into the block's array: with EV only the two step counts are kept in
+// registers, without it the ten parity counts, with diagnostics all.
+template <bool COUNT, bool EV>
+__device__ __forceinline__ void flush_lanes(Counters &cnt) {
+  constexpr int kAll = COUNT ? G4N_N_COUNTERS : G4N_C_STEP_LIMIT + 1;
+  if (EV) cnt.c[G4N_C_STEPS] = cnt.c[G4N_C_GEOM_STEPS] + cnt.c[G4N_C_PHYS_STEPS];
+#pragma unroll
+  for (int k = 0; k < kAll; ++k) {
+    if (EV && !COUNT && k != G4N_C_STEPS && k != G4N_C_GEOM_STEPS && k != G4N_C_PHYS_STEPS) continue;
+    // the lanes' 32-bit counts in two halves: their sums over a warp fit 32 bits
+    const unsigned lo = __reduce_add_sync(0xffffffffu, cnt.c[k] & 0xffffu), hi = __reduce_add_sync(0xffffffffu, cnt.c[k] >> 16);
+    const unsigned long long v = lo + ((unsigned long long)hi << 16);
+    if ((threadIdx.x & 31u) == 0 && v) atomicAdd(&s_events[k], v);
+  }
+}
+
+// The block's array into the batch's counters (every thread of the block calls it).
+__device__ __forceinline__ void flush_block(unsigned long long *counters) {
+  __syncthreads();
+  for (int k = threadIdx.x; k < G4N_N_COUNTERS; k += blockDim.x)
+    if (s_events[k]) atomicAdd(&counters[k], s_events[k]);
+}
+
 // ---------------------------------------------------------------- locate
 
 // 8 blocks of 128 per SM (64 registers, a few hundred bytes of spills): the descent waits on its chain
@@ -851,10 +874,8 @@ __global__ void __launch_bounds__(128, (MODE == kFP32 && YIELD) ? 3 : 4) k_trans
   Counters cnt;
 #pragma unroll
   for (int k = 0; k < G4N_N_COUNTERS; ++k) cnt.c[k] = 0;
-  if (kEv) {
-    for (int k = threadIdx.x; k < G4N_N_COUNTERS; k += blockDim.x) s_events[k] = 0;
-    __syncthreads();
-  }
+  for (int k = threadIdx.x; k < G4N_N_COUNTERS; k += blockDim.x) s_events[k] = 0;
+  __syncthreads();
   const unsigned lane = threadIdx.x & 31u;
   MlpCtx mc{nullptr, nullptr, P.log, 0.f};
   if (MODE == kLearned) {
@@ -923,21 +944,8 @@ __global__ void __launch_bounds__(128, (MODE == kFP32 && YIELD) ? 3 : 4) k_trans
     }
     if (!REGROUP && drained && __ballot_sync(0xffffffffu, phase != kEmpty) == 0) break;
   }
-  // flush counters: the block's event counts, then a warp reduction of the lanes' counts, one atomic
-  // per counter per warp
-  if (kEv) {
-    cnt.c[G4N_C_STEPS] = cnt.c[G4N_C_GEOM_STEPS] + cnt.c[G4N_C_PHYS_STEPS];
-    __syncthreads();
-    for (int k = threadIdx.x; k < G4N_N_COUNTERS; k += blockDim.x)
-      if (s_events[k]) atomicAdd(&P.counters[k], s_events[k]);
-  }
-#pragma unroll
-  for (int k = 0; k < G4N_N_COUNTERS; ++k) {
-    unsigned long long v = cnt.c[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0 && v) atomicAdd(&P.counters[k], v);
-  }
+  flush_lanes<COUNT, kEv>(cnt);
+  flush_block(P.counters);
 }
 
 // ---------------------------------------------------------------- free path (Algorithm 1)

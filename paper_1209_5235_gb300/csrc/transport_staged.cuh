@@ -171,19 +171,11 @@ __device__ __forceinline__ void sg_retire(SgCtrl *C, bool ended) {
   if (m && (threadIdx.x & 31u) == 0) atomicAdd((unsigned long long *)&C->active, (unsigned long long)(-(long long)__popc(m)));
 }
 
-// The block's event counts (shared) and the lanes' step counts (registers) into the batch's counters.
+// The block's event counts (shared) and the lanes' step counts (registers) into the batch's counters.  (Reducing all 32
+// counter slots in every warp cost 900 instructions a warp: 20 to 30 us of each launch of an iteration, empty or not.)
 __device__ __forceinline__ void sg_flush(const TParams &P, Counters &cnt) {
-  cnt.c[G4N_C_STEPS] = cnt.c[G4N_C_GEOM_STEPS] + cnt.c[G4N_C_PHYS_STEPS];
-  __syncthreads();
-  for (int k = threadIdx.x; k < G4N_N_COUNTERS; k += blockDim.x)
-    if (s_events[k]) atomicAdd(&P.counters[k], s_events[k]);
-#pragma unroll
-  for (int k = 0; k < G4N_N_COUNTERS; ++k) {
-    unsigned long long v = cnt.c[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    if ((threadIdx.x & 31u) == 0 && v) atomicAdd(&P.counters[k], v);
-  }
+  flush_lanes<false, true>(cnt);
+  flush_block(P.counters);
 }
 
 __device__ __forceinline__ void sg_begin(Counters &cnt) {
@@ -280,7 +272,7 @@ __global__ void __launch_bounds__(128, 4) k_staged_step(const TParams P, const S
     if (RELOC_KERNEL && keep && next == kReloc) Q.iw[6 * Q.n + e] = aux;
     sg_retire(C, was && next == kEmpty);
   }
-  sg_flush(P, cnt);
+  if ((long long)blockIdx.x * blockDim.x < total) sg_flush(P, cnt);
   if (sg_last_block(C, 0) && threadIdx.x == 0) {
     volatile SgCtrl *V = C;
     const long long active = V->active;
@@ -334,7 +326,7 @@ __global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const 
     sg_push_block(Q, C, keep, keep ? sg_queue_of(P, t, ob) : 0, t);
     sg_retire(C, act && next == kEmpty);
   }
-  sg_flush(P, cnt);
+  if ((long long)blockIdx.x * blockDim.x < total) sg_flush(P, cnt);
   if (sg_last_block(C, 3) && threadIdx.x == 0) {
     ((volatile SgCtrl *)C)->cnt[kSgReloc] = 0;
     __threadfence();
@@ -377,7 +369,7 @@ __global__ void __launch_bounds__(128, 4) k_staged_finish(const TParams P, const
     sg_push(Q, C, mine && next == kStep, mine && next == kStep ? sg_queue_of(P, t, ob) : 0, t);
     sg_retire(C, mine && next == kEmpty);
   }
-  sg_flush(P, cnt);
+  if ((long long)blockIdx.x * blockDim.x < total) sg_flush(P, cnt);
   if (sg_last_block(C, 1) && threadIdx.x == 0) {
     volatile SgCtrl *V = C;
     V->cnt[kSgInteract] = 0;

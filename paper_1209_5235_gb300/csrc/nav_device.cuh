@@ -1540,7 +1540,11 @@ __device__ __forceinline__ uint64_t philox_m53(uint64_t seed, int64_t tid, uint3
   return philox_m53_pair(seed, tid, stream, draw).a;
 }
 
-__device__ __forceinline__ double m53_double(uint64_t m) { return (double)m * 0x1.0p-53; }
+// m 2^-53 (m in [1, 2^53], so exact), by integer instructions: a 64-bit conversion and a product hold the FP64 pipe.
+__device__ __forceinline__ double m53_double(uint64_t m) {
+  const int lz = __clzll((long long)m);                 // 10 .. 63
+  return __longlong_as_double(((long long)(1033 - lz) << 52) + (long long)(((m << lz) << 1) >> 12));
+}
 
 // m 2^-53 as a float, truncated to 24 bits (relative error < 2^-23), with integer
 // instructions only (m in [1, 2^53]).

@@ -233,7 +233,7 @@ constexpr int kNeverYield = 1 << 16;
 
 struct Track {
   V3 x, u;
-  Inv3 iu;           // reciprocal of u (used in world-aligned volumes)
+  Inv3 iu;           // reciprocal of u (FP64 mode, in world-aligned volumes)
   double E, Y, len, safety, mu, mupe, efrac;
   uint64_t h;
   int64_t tid, gidx;
@@ -280,31 +280,38 @@ __device__ __forceinline__ int find_item(const DItem *items, int n_items, int64_
   return lo;
 }
 
-// Unit-disc rejection: (cos, sin) of a uniform azimuth, one Philox block per trial.  Points
-// with a^2 + b^2 > 1 + 1e-5 in FP32 (from the Philox integers; error < 2e-6) are rejected
-// without FP64 work; the others take the FP64 test and, if accepted, the FP64 evaluation.
+// Unit-disc rejection: (cos, sin) of a uniform azimuth, one Philox block per trial.  A trial is decided in FP32 (from
+// the Philox integers; error of a^2 + b^2 < 2e-6) unless that lies within 1e-5 of 0 or 1, where FP64 decides.  The
+// accepted trial's values are evaluated after the loop, in FP64 and once for the warp: in the loop every round in which
+// some lane accepts would hold the FP64 pipe for all of them.
 __device__ __forceinline__ bool disc_azimuth(uint64_t seed, int64_t tid, uint32_t stream, uint32_t &draw, double &c,
                                              double &s, int trials) {
+  uint64_t ma = 0, mb = 0;
+  bool ok = false;
 #pragma unroll 1
-  for (int t = 0; t < trials; ++t) {
+  for (int t = 0; t < trials && !ok; ++t) {
     const M53x2 ab = philox_m53_pair(seed, tid, stream, draw);
-    const uint64_t ma = ab.a, mb = ab.b;
+    ma = ab.a;
+    mb = ab.b;
     const float af = 2.0f * m53_float(ma) - 1.0f, bf = 2.0f * m53_float(mb) - 1.0f;
     const float r2f = af * af + bf * bf;
     if (r2f > 1.0f + 1e-5f) continue;
-    const double a = 2.0 * m53_double(ma) - 1.0;
-    const double b = 2.0 * m53_double(mb) - 1.0;
-    const double r2 = a * a + b * b;
-    if (r2 > 0.0 && r2 <= 1.0) {
-      const double inv = 1.0 / r2;
-      c = (a * a - b * b) * inv;
-      s = 2.0 * a * b * inv;
-      return true;
+    ok = r2f < 1.0f - 1e-5f && r2f > 1e-5f;
+    if (!ok) {
+      const double a = 2.0 * m53_double(ma) - 1.0, b = 2.0 * m53_double(mb) - 1.0;
+      const double r2 = a * a + b * b;
+      ok = r2 > 0.0 && r2 <= 1.0;
     }
   }
   c = 1.0;
   s = 0.0;
-  return false;
+  if (ok) {
+    const double a = 2.0 * m53_double(ma) - 1.0, b = 2.0 * m53_double(mb) - 1.0;
+    const double inv = 1.0 / (a * a + b * b);
+    c = (a * a - b * b) * inv;
+    s = 2.0 * a * b * inv;
+  }
+  return ok;
 }
 
 // Source of track tid (stream 0).
@@ -367,9 +374,11 @@ __device__ __forceinline__ void set_energy(const DGeom &G, Track &t, double E) {
   if (G.shared_grid) energy_bin(G.matE, G.mat_n[0], E, t.ebin, t.efrac);
 }
 
+// The reciprocal serves the FP64 navigator's voxel walk and box exits; the FP32 modes have no use for it.
+template <int MODE>
 __device__ __forceinline__ void set_direction(Track &t, const V3 &u) {
   t.u = u;
-  t.iu = inv_dir(u);
+  if (MODE == kFP64) t.iu = inv_dir(u);
 }
 
 // Start track number g of the concatenated items on the lanes with `active` set
@@ -387,7 +396,7 @@ __device__ int start_warp(const TParams &P, bool active, int64_t g, Track &t, Co
     V3 u;
     double E;
     make_source(it.src, P.seed, t.tid, t.x, u, E, P.status, P.trial_cap);
-    set_direction(t, u);
+    set_direction<MODE>(t, u);
     tally(P, t, Gp->n_vol + 1, E);
     event<EV>(cnt, G4N_C_TRACKS);
     t.h = kFnvOffset;
@@ -423,42 +432,49 @@ __device__ int start_warp(const TParams &P, bool active, int64_t g, Track &t, Co
 // alpha r2)) and the uniforms' FP32 copies (built from the Philox integers, relative error
 // < 2^-23) are within 2e-6 of the exact ones, so such a decision is the exact one; the
 // others are taken on the FP64 thresholds of the plain formulas.  The accepted trial's eta
-// and cos theta are computed in FP64.  FP64 work is left for the accepted trial and the
-// rare close calls.
+// and cos theta are computed in FP64 after the loop, once for the warp (414 -> 285 FP64
+// instructions per warp of interactions with the disc's and the direction's reciprocal, barrel).
 __device__ __forceinline__ bool kahn(double E, uint64_t seed, int64_t tid, uint32_t &draw, double &eta, double &cost,
                                      int trials) {
   constexpr float kMargin = 1e-5f;
   const double al = E / kMeC2;
   const float alf = (float)al;
-  const float p1f = (1.0f + 2.0f * alf) / (9.0f + 2.0f * alf);
+  const float p1f = (1.0f + 2.0f * alf) / (9.0f + 2.0f * alf), einv = 1.0f / (1.0f + 2.0f * alf);
+  uint64_t m2 = 0;
+  bool first = false, ok = false;
 #pragma unroll 1
-  for (int t = 0; t < trials; ++t) {
+  for (int t = 0; t < trials && !ok; ++t) {
     const M53x2 b12 = philox_m53_pair(seed, tid, 1, draw);
-    const uint64_t m1 = b12.a, m2 = b12.b;
+    const uint64_t m1 = b12.a;
+    m2 = b12.b;
     const uint64_t m3 = philox_m53(seed, tid, 1, draw);
     const float d1 = m53_float(m1) - p1f;
-    const bool first = fabsf(d1) > kMargin ? d1 <= 0.f : m53_double(m1) <= (1.0 + 2.0 * al) / (9.0 + 2.0 * al);
+    first = fabsf(d1) > kMargin ? d1 <= 0.f : m53_double(m1) <= (1.0 + 2.0 * al) / (9.0 + 2.0 * al);
     const float r2f = m53_float(m2), r3f = m53_float(m3);
     const float a2 = 2.0f * alf * r2f, den = 1.0f + a2;
-    if (first) {
-      const float d = r3f - 4.0f * a2 / (den * den);
-      if (fabsf(d) > kMargin && d > 0.f) continue;
-      eta = 1.0 + 2.0 * al * m53_double(m2);
-      if (!(fabsf(d) > kMargin) && !(m53_double(m3) <= 4.0 * (1.0 / eta - 1.0 / (eta * eta)))) continue;
-      cost = 1.0 - (eta - 1.0) / al;
-    } else {
-      const float cf = 1.0f - 2.0f * (1.0f - r2f) / den;
-      const float d = r3f - 0.5f * (cf * cf + den / (1.0f + 2.0f * alf));
-      if (fabsf(d) > kMargin && d > 0.f) continue;
-      eta = (1.0 + 2.0 * al) / (1.0 + 2.0 * al * m53_double(m2));
-      cost = 1.0 - (eta - 1.0) / al;
-      if (!(fabsf(d) > kMargin) && !(m53_double(m3) <= 0.5 * (cost * cost + 1.0 / eta))) continue;
+    const float cf = 1.0f - __fdividef(2.0f * (1.0f - r2f), den);
+    const float d = r3f - (first ? __fdividef(4.0f * a2, den * den)
+                                 : 0.5f * (cf * cf + den * einv));
+    ok = !(d > 0.f);
+    if (!(fabsf(d) > kMargin)) {
+      if (first) {
+        const double e = 1.0 + 2.0 * al * m53_double(m2);
+        ok = m53_double(m3) <= 4.0 * (1.0 / e - 1.0 / (e * e));
+      } else {
+        const double e = (1.0 + 2.0 * al) / (1.0 + 2.0 * al * m53_double(m2));
+        const double c = 1.0 - (e - 1.0) / al;
+        ok = m53_double(m3) <= 0.5 * (c * c + 1.0 / e);
+      }
     }
-    return true;
   }
   eta = 1.0;
   cost = 1.0;
-  return false;
+  if (ok) {
+    const double x = 1.0 + 2.0 * al * m53_double(m2);
+    eta = first ? x : (1.0 + 2.0 * al) / x;
+    cost = 1.0 - (eta - 1.0) / al;
+  }
+  return ok;
 }
 
 // New direction at polar cosine ct and azimuth (cph, sph) about u.
@@ -717,7 +733,7 @@ __device__ int interact(const TParams &P, Track &t, Counters &cnt) {
   bool ok = kahn(t.E, P.seed, t.tid, t.draw, eta, cost, P.trial_cap);
   ok &= disc_azimuth(P.seed, t.tid, 1, t.draw, cph, sph, P.trial_cap);
   if (!ok) flag(P.status, kStRejection);
-  set_direction(t, deflect(t.u, cost, cph, sph));
+  set_direction<MODE>(t, deflect(t.u, cost, cph, sph));
   const double E1 = t.E / eta;
   if (E1 < P.cutoff) {
     event<EV>(cnt, G4N_C_CUTOFF);

@@ -18,6 +18,7 @@
 //   skey[]       per slice of a world-aligned mother: the smallest world
 //                coordinate (as a key) that falls in that slice or above
 //   DFace[]      6 per kKeyBox volume: relocation results across its faces
+//   portal[12 n] per volume: the leaf behind each face, leaving (6) and entering (6)
 // All tables are small (a few MB at most) and stay L2-resident.
 #pragma once
 
@@ -31,6 +32,7 @@ namespace g4n {
 
 constexpr int kDMax = G4N_DMAX;
 constexpr int kMaxLevels = 3;
+constexpr int kPortalNone = -2;            // a face without a portal (geom_portals.h)
 constexpr int kDefaultWalkCap = 1 << 16;   // voxel nodes one boundary search may walk
 constexpr int kDefaultTrialCap = 1000;     // trials of one rejection sampler
 
@@ -148,6 +150,7 @@ struct DGeom {
   const DKeyBox *kbox;
   const int64_t *skey;
   const DFace *face;
+  const int32_t *portal;
   int32_t n_vol, n_mat;
   int32_t shared_grid;  // all materials tabulated on one energy grid
   int32_t pad;
@@ -190,6 +193,7 @@ struct HGeom {
   std::vector<DKeyBox> kbox;
   std::vector<int64_t> skey;
   std::vector<DFace> face;
+  std::vector<int32_t> portal;
   std::vector<int32_t> touch_lv, touch_copy;  // per volume (touchable): logical volume, copy number
   int32_t max_depth = 0;
   // device blob

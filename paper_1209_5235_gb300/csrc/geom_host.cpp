@@ -19,6 +19,7 @@
 #include <random>
 
 #include "g4n_internal.h"
+#include "geom_portals.h"
 
 using namespace g4n;
 
@@ -1110,6 +1111,12 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
     }
   }
   if (g->face.empty()) g->face.push_back(DFace{});
+  // --- portals: the leaf behind each face of every box, tube segment and orb
+  g->portal.resize(12 * (size_t)n);
+  {
+    PortalBuilder portals(*g, tol);
+    for (int i = 0; i < n; ++i) portals.build(i, &g->portal[12 * (size_t)i]);
+  }
   // --- touchables: the logical volume and copy number of every volume
   g->touch_lv = B.touch_lv;
   g->touch_copy = B.touch_copy;
@@ -1126,7 +1133,7 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
   }
   // --- upload as one blob
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-  constexpr int kTables = 18;
+  constexpr int kTables = 19;
   size_t off[kTables], sz[kTables] = {g->vol.size() * sizeof(DVol), g->wxf.size() * sizeof(DWorld), g->box.size() * sizeof(DBox32),
                             g->hdr.size() * sizeof(DVoxHdr), g->slice.size() * sizeof(DVoxSlice),
                             g->clist.size() * sizeof(DCandList), g->cand.size() * sizeof(int32_t),
@@ -1134,10 +1141,10 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
                             g->mat_off.size() * sizeof(int32_t), g->mat_n.size() * sizeof(int32_t),
                             g->v32.size() * sizeof(DVol32), g->kbox.size() * sizeof(DKeyBox),
                             g->skey.size() * sizeof(int64_t), g->face.size() * sizeof(DFace),
-                            g->hdr32.size() * sizeof(DVoxHdr32), g->pick.size() * sizeof(DPick32)};
+                            g->hdr32.size() * sizeof(DVoxHdr32), g->pick.size() * sizeof(DPick32), g->portal.size() * sizeof(int32_t)};
   const void *src[kTables] = {g->vol.data(), g->wxf.data(), g->box.data(), g->hdr.data(), g->slice.data(), g->clist.data(),
                          g->cand.data(), g->matE.data(), g->matC.data(), g->matP.data(), g->mat_off.data(), g->mat_n.data(),
-                         g->v32.data(), g->kbox.data(), g->skey.data(), g->face.data(), g->hdr32.data(), g->pick.data()};
+                         g->v32.data(), g->kbox.data(), g->skey.data(), g->face.data(), g->hdr32.data(), g->pick.data(), g->portal.data()};
   size_t total = 0;
   for (int k = 0; k < kTables; ++k) { off[k] = total; total += al(std::max<size_t>(sz[k], 8)); }
   if (ctx->device < 0) {  // host-only context: keep the host tables
@@ -1180,7 +1187,8 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
   d.mat_off = (const int32_t *)(base + off[10]);
   d.mat_n = (const int32_t *)(base + off[11]);
   d.v32 = (const DVol32 *)(base + off[12]);
-  d.pick = (const DPick32 *)(base + off[kTables - 1]);
+  d.pick = (const DPick32 *)(base + off[17]);
+  d.portal = (const int32_t *)(base + off[18]);
   d.kbox = (const DKeyBox *)(base + off[13]);
   d.skey = (const int64_t *)(base + off[14]);
   d.face = (const DFace *)(base + off[15]);

@@ -199,9 +199,9 @@ __global__ void __launch_bounds__(128) k_compute_step(const DGeom *__restrict__ 
       const Step32 R = geom_step32_warp<MODE, false>(G, ok, leaf, p, v, limit, true, cnt, &timeout, walk_cap, mc, ch);
       safety = (double)R.safety;
       if (ok) {
-        int face;
+        int surf;
         if (limit < R.lo) lim = G4N_LIM_PHYSICS;   // the proposal comes first for certain
-        else s = step_exact32(G, leaf, p, v, R, walk_cap, &timeout, &lim, &face);
+        else s = step_exact32(G, leaf, p, v, R, walk_cap, &timeout, &lim, &surf);
       }
     }
     if (ok) {
@@ -565,7 +565,7 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
   }
   // the free path s_phys = Y / mu (Eq. 7) races the geometric step
   double s = kInf;
-  int lim = G4N_LIM_PHYSICS, face = -1;
+  int lim = G4N_LIM_PHYSICS, surf = -1;
   bool need_geo = false, geo = false, timeout = false;
   V3 p{0, 0, 0}, v{0, 0, 1};
   if (MODE == kLearned || mc.log) mc.loge = act ? (logf((float)t.E) + 4.6f) * 0.1f : 0.f;
@@ -624,7 +624,7 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       if (geo) {
         s = R.step;
         lim = R.lim;
-        face = R.face;
+        surf = R.surf;
       } else if (lazy) {
         s = t.Y / t.mu;
       }
@@ -656,11 +656,11 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       if (need_geo) {
         t.safety = (double)R.safety;
         geo = !(phys_hi < R.lo);
-        if (geo) quotient = step_ratio32(G, t.leaf, p, v, R, P.walk_cap, &timeout, &num, &den, &lim, &face);
+        if (geo) quotient = step_ratio32(G, t.leaf, p, v, R, P.walk_cap, &timeout, &num, &den, &lim, &surf);
       }
       s = quotient ? (geo || mu_pos ? num / den : kInf) : num;
       if (geo) {
-        if (quotient) quotient = step_finish32(G, t.leaf, p, v, s, P.walk_cap, &timeout, &lim, &face);
+        if (quotient) quotient = step_finish32(G, t.leaf, p, v, s, P.walk_cap, &timeout, &lim, &surf);
         // geometry wins iff step <= fl(Y / mu); the enclosures decide unless they overlap
         if (mu_pos && (!quotient || !(R.hi < phys_lo))) {
           const double sphys = t.Y / t.mu;
@@ -693,10 +693,11 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       t.safety = 0.0;
     }
   }
-  // leaving a box through a face whose relocation is tabulated needs no search
+  // crossing a face whose relocation is tabulated needs no search
   int leaf = -1;
   const bool left = geo && lim == G4N_LIM_MOTHER && s > 0.0;
-  const bool fast = left && face_relocate(G, t.leaf, face, t.x, t.u, &leaf);
+  bool fast = left && face_relocate(G, t.leaf, surf, t.x, t.u, &leaf);
+  if (geo && !fast && surf >= 0 && s > 0.0) fast = portal_relocate(G, t.leaf, lim, surf, p, v, s, &leaf);
   if (fast) diag<COUNT>(cnt, G4N_C_FACE_RELOC);
   // relocation search, then (after 10 zero steps) the push and its relocation: one copy of
   // the relocation code serves both passes.  DEFER: a lane that needs the search stops here (its
@@ -1057,7 +1058,7 @@ __global__ void __launch_bounds__(128, 3) k_free_path(const FParams P) {
     // one segment: the geometric step from x inside `leaf`
     V3 p{0, 0, 0}, v{0, 0, 1};
     double step = kInf;
-    int lim = G4N_LIM_MOTHER, face = -1;
+    int lim = G4N_LIM_MOTHER, surf = -1;
     bool timeout = false;
     Chain ch;
     const bool aligned = G.vol[leaf].flags & kWorldAligned;
@@ -1068,11 +1069,11 @@ __global__ void __launch_bounds__(128, 3) k_free_path(const FParams P) {
                                                  P.walk_cap, mc, ch);
       step = R.step;
       lim = R.lim;
-      face = R.face;
+      surf = R.surf;
     } else {
       const Step32 R = geom_step32_warp<MODE, COUNT>(G, active, active ? leaf : 0, p, v, kInfF, false, cnt, &timeout,
                                                      P.walk_cap, mc, ch);
-      if (active) step = step_exact32(G, leaf, p, v, R, P.walk_cap, &timeout, &lim, &face);
+      if (active) step = step_exact32(G, leaf, p, v, R, P.walk_cap, &timeout, &lim, &surf);
     }
     bool cross = false;
     double s = 0.0;
@@ -1102,7 +1103,8 @@ __global__ void __launch_bounds__(128, 3) k_free_path(const FParams P) {
     }
     const bool left = cross && lim == G4N_LIM_MOTHER && s > 0.0;
     int nl = -1;
-    const bool fast = left && face_relocate(G, leaf, face, x, u, &nl);
+    bool fast = left && face_relocate(G, leaf, surf, x, u, &nl);
+    if (cross && !fast && surf >= 0 && s > 0.0) fast = portal_relocate(G, leaf, lim, surf, p, v, s, &nl);
     if (fast) diag<COUNT>(cnt, G4N_C_FACE_RELOC);
     const int searched = relocate_warp<MODE, COUNT>(G, cross && !fast, cross && !fast ? leaf : 0, x, u, left, cnt);
     if (!fast) nl = searched;

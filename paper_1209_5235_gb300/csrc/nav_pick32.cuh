@@ -297,7 +297,7 @@ __device__ __forceinline__ Pick pick_solid(int kind, const float *q, int flags, 
 }
 
 // The crossing parameter of one surface in FP64 as a quotient num / den, by the formulas of the full tests: planes, and
-// circles through the quadratic's root without cancellation (lo: q / a for b >= 0, else c / q; hi the other one).  The
+// circles through the quadratic's root without cancellation (lo: q / a where q < 0, else c / q; hi the other one).  The
 // caller divides: one division for all lanes of a warp whatever their surfaces.  NaN where the quadratic has no root.
 __device__ __forceinline__ void surf_ratio(int kind, const double *p, int surf, bool enter, const V3 &x, const V3 &v,
                                            double &num, double &den) {
@@ -326,7 +326,7 @@ __device__ __forceinline__ void surf_ratio(int kind, const double *p, int surf, 
     c -= R * R;
     const double sq = sqrt(b * b - a * c), q = -(b + copysign(sq, b));
     const bool lo = enter == (kind == kOrb || surf == kPickOuter);
-    const bool direct = lo == (b >= 0.0);
+    const bool direct = lo == (__double2hiint(b) >= 0);   // by q's sign: b may be -0 (a ray from the axis)
     num = direct ? q : c;
     den = direct ? a : q;
   }

@@ -558,7 +558,7 @@ int staged_run(g4n_ctx *ctx, const g4n_batch_desc *b, TParams &P, cudaStream_t s
   const int g_drain = ctx->sm_count * std::max(per_sm_drain, 1);
   const long long drain_tracks = b->drain_tracks < 0 ? -1
                                  : b->drain_tracks > 0 ? b->drain_tracks
-                                                       : 4LL * g_drain * 128;
+                                                       : 2LL * g_drain * 128;
   if (cudaMemsetAsync(C, 0, sizeof(SgCtrl), st) != cudaSuccess) return g4n_fail(ctx, G4N_ERR_CUDA, "transport: control reset failed");
   if (int rc = launch_error(ctx, "staged transport setup")) return rc;
 

@@ -10,6 +10,7 @@
 #define __forceinline__ inline
 #define __noinline__
 using std::copysign;
+using std::copysignf;
 using std::fabs;
 using std::fmax;
 using std::fmin;
@@ -38,9 +39,9 @@ using namespace g4n::dev;
 static double uni(double a, double b) { return a + (b - a) * ((double)(rng() >> 11) * 0x1.0p-53); }
 
 // `mode` 0: a point anywhere around the solid; 1: the point of a crossing (in a surface's band), moved along the ray by
-// at most 1e-9.  `rotated`: point and direction reach the FP32 side through an FP32 rotation about z and a translation
-// of up to 2000, as from a mother's frame.
-// out: 0 cases, 1 chosen, 2 misses proved, 3 unsure, 4 wrong, 5 crossing outside its enclosure; *worst: relative error.
+// at most 1e-9; 2: a point on the solid's axis.  `rotated`: the solid is a daughter, rotated about z and moved by up to 2000
+// in its mother's frame, in which the ray is given.
+// out: 0 cases, 1 chosen, 2 misses proved, 3 unsure (chosen, but the quotient lies in the band, among them), 4 wrong, 5 crossing outside its enclosure; *worst: relative error.
 extern "C" void pick_check(int kind, int seg, int bore, int mode, int rotated, double scale, long long n, uint64_t seed,
                            long long *out, double *worst) {
   rng.seed(seed);
@@ -98,6 +99,9 @@ extern "C" void pick_check(int kind, int seg, int bore, int mode, int rotated, d
       const Inv3 iv{v.x != 0 ? 1 / v.x : 0, v.y != 0 ? 1 / v.y : 0, v.z != 0 ? 1 / v.z : 0};
       return box_dist_out(p, q, v, iv, &face);
     };
+    if (mode == 2) {  // on the axis, as from a beam line: b = x . v is a signed zero
+      x.x = x.y = 0.0;
+    }
     if (mode == 1) {  // to a surface of the solid, entering or leaving
       double t = inside(x) ? dist_out(x) : dist_in(x);
       if (!(t < kInf)) continue;
@@ -105,31 +109,30 @@ extern "C" void pick_check(int kind, int seg, int bore, int mode, int rotated, d
       x = V3{x.x + t * v.x, x.y + t * v.y, x.z + t * v.z};
     }
     const bool in = inside(x);
+    if (rotated && in) continue;
     ++out[0];
-    float fx = trunc_float(x.x), fy = trunc_float(x.y), fz = trunc_float(x.z);
-    float wx = trunc_float(v.x), wy = trunc_float(v.y), wz = trunc_float(v.z);
-    float q[7];
-    float ep = 2.0f * kU * (std::fabs(fx) + std::fabs(fy) + std::fabs(fz) + (float)(p[0] + p[1] + p[2])) + 1e-30f;
-    for (int k = 0; k < 7; ++k) q[k] = kind == kTube || k < 3 ? (rotated ? (float)p[k] : trunc_float(p[k])) : 0.f;
-    if (kind == kOrb) ep = 2.0f * kU * (std::fabs(fx) + std::fabs(fy) + std::fabs(fz) + (float)p[0]) + 1e-30f;
-    if (rotated) {  // mother -> local in FP32, with the bound the navigator takes
+    DPick32 D;
+    std::memset(&D, 0, sizeof D);
+    for (int k = 0; k < 7; ++k) D.q[k] = (float)p[k];
+    Pick k;
+    if (!rotated) {
+      D.c = 1.0f;
+      D.kind_flags = (flags | kPlacedAligned) << 2 | kind;
+      const PickRay r = pick_ray(x, v);
+      k = in ? pick_leaf(D, r, band) : pick_daughter(D, r, band);
+    } else {  // the solid as a daughter, rotated and moved in its mother's frame
       const double a = uni(0, 6.283185307), c = std::cos(a), s = std::sin(a);
-      const double tx = uni(-2000, 2000), ty = uni(-2000, 2000), tz = uni(-2000, 2000);
-      const double mx = c * x.x - s * x.y + tx, my = s * x.x + c * x.y + ty, mz = x.z + tz;
-      const float cx = (float)c, sx = (float)s;
-      const float m0 = trunc_float(mx), m1 = trunc_float(my), m2 = trunc_float(mz);
-      const float dx = m0 - (float)tx, dy = m1 - (float)ty;
-      fx = cx * dx + sx * dy;
-      fy = cx * dy - sx * dx;
-      fz = m2 - (float)tz;
-      const float u0 = trunc_float(c * v.x - s * v.y), u1 = trunc_float(s * v.x + c * v.y);
-      wx = cx * u0 + sx * u1;
-      wy = cx * u1 - sx * u0;
-      const float sc = (float)(std::fabs(tx) + std::fabs(ty) + std::fabs(tz) + 2.0 * ext);
-      ep = 8.0f * kU * (std::fabs(m0) + std::fabs(m1) + std::fabs(m2) + sc) + 1e-30f;
+      const double t[3] = {uni(-2000, 2000), uni(-2000, 2000), uni(-2000, 2000)};
+      for (int j = 0; j < 3; ++j) {
+        D.th[j] = (float)t[j];
+        D.tl[j] = (float)(t[j] - (double)D.th[j]);
+      }
+      D.c = (float)c;
+      D.s = (float)s;
+      D.kind_flags = flags << 2 | kind;
+      const V3 m{c * x.x - s * x.y + t[0], s * x.x + c * x.y + t[1], x.z + t[2]}, mv{c * v.x - s * v.y, s * v.x + c * v.y, v.z};
+      k = pick_daughter(D, pick_ray(m, mv), band);
     }
-    const Pick k = in ? pick_solid<false>(kind, q, flags, fx, fy, fz, wx, wy, wz, ep, band)
-                      : pick_solid<true>(kind, q, flags, fx, fy, fz, wx, wy, wz, ep, band);
     const double full = in ? dist_out(x) : dist_in(x);
     if (k.surf == kPickUnsure) {
       ++out[3];
@@ -142,7 +145,9 @@ extern "C" void pick_check(int kind, int seg, int bore, int mode, int rotated, d
       continue;
     }
     ++out[1];
-    double t = in ? surf_param<false>(kind, p, k.surf, x, v) : surf_param<true>(kind, p, k.surf, x, v);
+    double num, den;
+    surf_ratio(kind, p, k.surf, !in, x, v, num, den);
+    double t = num / den;
     if (!(t > (in ? -half : half))) {   // the caller then takes the full formulas
       ++out[3];
       continue;

@@ -34,9 +34,19 @@ def check(lib, solid, mode, rotated, scale, n=60000, seed=5):
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("solid", SOLIDS)
 def test_choice_is_the_fp64_answer(lib, solid, mode, rotated, scale):
-    (cases, chosen, missed, unsure, wrong, out_of_range), worst = check(lib, solid, mode, rotated, scale)
+    (cases, chosen, missed, unsure, wrong, out_of_range), worst = check(lib, solid, mode, rotated, scale, 300000 if mode else 60000)
     assert cases > 1000 and wrong == 0 and out_of_range == 0, (cases, chosen, missed, unsure, wrong, out_of_range)
     if solid.startswith("wide"):
         assert unsure == cases        # not convex in phi: always the full formulas
     elif mode == 0 and scale >= 40.0:
         assert unsure < 0.05 * cases  # the bounds decide nearly all
+
+
+@pytest.mark.parametrize("scale", [40.0, 1500.0])
+@pytest.mark.parametrize("solid", [s for s in SOLIDS if not s.startswith("wide")])
+def test_rays_from_the_axis_are_decided(lib, solid, scale):
+    """x . v is +0 or -0 there: the root taken does not depend on the sign of that zero."""
+    (cases, chosen, missed, unsure, wrong, out_of_range), worst = check(lib, solid, 2, 0, scale)
+    assert wrong == 0 and out_of_range == 0
+    if "segment" not in solid:      # a segment's apex lies on the axis
+        assert unsure < 0.01 * cases, (cases, chosen, missed, unsure)

@@ -195,14 +195,24 @@ __device__ __forceinline__ void sg_begin(Counters &cnt) {
   __syncthreads();
 }
 
-// True in the block of the grid that finishes last (the writes of all other blocks are then
+// Blocks of the grid that take part in a kernel over `total` tracks: those with a track of their own, block 0 at least.
+// The others leave at once, without the kernel's start and end (a grid of 2432 blocks counting itself out through one
+// atomic cost 20 to 35 us a launch, with an empty queue as well; with this and the drain at two tracks a thread:
+// calorimeter 6.68 -> 6.52 ms, its host batch of 2 10^5 2.5 -> 2.0, nested barrel 20.2 -> 17.8).  A block may read `total` after the last block has
+// reset it only if it is not one of them: the last block waits for all that take part, and block 0 always does.
+__device__ __forceinline__ unsigned sg_workers(long long total) {
+  const long long need = (total + blockDim.x - 1) / blockDim.x;
+  return need < 1 ? 1u : need < (long long)gridDim.x ? (unsigned)need : gridDim.x;
+}
+
+// True in the block that finishes last of the `workers` (the writes of all other blocks are then
 // visible to it); it resets the kernel's finished-block count for the next launch.
-__device__ __forceinline__ bool sg_last_block(SgCtrl *C, int which) {
+__device__ __forceinline__ bool sg_last_block(SgCtrl *C, int which, unsigned workers) {
   __shared__ bool last;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    last = atomicAdd(&C->fin[which], 1u) == gridDim.x - 1;
+    last = atomicAdd(&C->fin[which], 1u) == workers - 1;
     if (last) C->fin[which] = 0;
   }
   __syncthreads();
@@ -225,20 +235,40 @@ __device__ __forceinline__ MlpCtx sg_mlp(const TParams &P) {
   return mc;
 }
 
-// Entries of the four step queues of bank b: prefix sums in shared memory.
-__device__ __forceinline__ long long sg_prefix(const SgCtrl *C, int b, long long *pref) {
+// What a kernel of an iteration has to do, read by one thread of the block in a few wide loads past the L1 that overlap
+// (each thread reading for itself put 60 000 requests of a grid of 2432 blocks on one L2 line): the prefix sums of the four
+// step queues of bank b, the new tracks, the end of the batch or its hand-over to the drain.
+struct SgWork {
+  long long pref[kSgKinds + 1];
+  long long n_int, n_new, base, n_reloc;
+  int stop;
+};
+static_assert(offsetof(SgCtrl, n_new) % 16 == 0 && offsetof(SgCtrl, base) == offsetof(SgCtrl, n_new) + 8 &&
+                  offsetof(SgCtrl, done) % 8 == 0 && offsetof(SgCtrl, drain_now) == offsetof(SgCtrl, done) + 4 &&
+                  kSgInteract % 2 == 0 && kSgReloc == kSgInteract + 1 && kSgKinds == 4,
+              "fields read together");
+
+__device__ __forceinline__ const SgWork &sg_work(const SgCtrl *C, int b) {
+  __shared__ SgWork w;
   if (threadIdx.x == 0) {
-    const volatile SgCtrl *V = C;
-    long long acc = 0;
-    pref[0] = 0;
-#pragma unroll
-    for (int k = 0; k < kSgKinds; ++k) {
-      acc += (long long)V->cnt[b * kSgKinds + k];
-      pref[k + 1] = acc;
-    }
+    const ulonglong2 c01 = __ldcg(reinterpret_cast<const ulonglong2 *>(&C->cnt[b * kSgKinds]));
+    const ulonglong2 c23 = __ldcg(reinterpret_cast<const ulonglong2 *>(&C->cnt[b * kSgKinds + 2]));
+    const ulonglong2 ir = __ldcg(reinterpret_cast<const ulonglong2 *>(&C->cnt[kSgInteract]));
+    const ulonglong2 nb = __ldcg(reinterpret_cast<const ulonglong2 *>(&C->n_new));
+    const int2 end = __ldcg(reinterpret_cast<const int2 *>(&C->done));
+    w.pref[0] = 0;
+    w.pref[1] = (long long)c01.x;
+    w.pref[2] = w.pref[1] + (long long)c01.y;
+    w.pref[3] = w.pref[2] + (long long)c23.x;
+    w.pref[4] = w.pref[3] + (long long)c23.y;
+    w.n_int = (long long)ir.x;
+    w.n_reloc = (long long)ir.y;
+    w.n_new = (long long)nb.x;
+    w.base = (long long)nb.y;
+    w.stop = end.x | end.y;
   }
   __syncthreads();
-  return pref[kSgKinds];
+  return w;
 }
 
 // Step kernel of iteration (ib: the bank read, the other bank written).  Its last block admits
@@ -247,12 +277,13 @@ __device__ __forceinline__ long long sg_prefix(const SgCtrl *C, int b, long long
 // relocation kernel instead of searching here, with its limiter and exit flag in the entry's aux int.
 template <int MODE, bool RELOC_KERNEL>
 __global__ void __launch_bounds__(128, 4) k_staged_step(const TParams P, const SgQueues Q, SgCtrl *C, int ib) {
-  if (((const volatile SgCtrl *)C)->drain_now || ((const volatile SgCtrl *)C)->done) return;
+  const SgWork &W = sg_work(C, ib);
+  const long long total = W.pref[kSgKinds];
+  const unsigned workers = sg_workers(total);
+  if (W.stop || blockIdx.x >= workers) return;
   Counters cnt;
   sg_begin(cnt);
-  const MlpCtx mc = sg_mlp<MODE>(P);
-  __shared__ long long pref[kSgKinds + 1];
-  const long long total = sg_prefix(C, ib, pref);
+  const MlpCtx mc = total > 0 ? sg_mlp<MODE>(P) : MlpCtx{nullptr, nullptr, nullptr, 0.f};
   const int ob = ib ^ 1;
   const bool want_slot = P.out_hash || P.out_len;
   // block-sized strides: the loop condition is the same for every thread of the block (sg_push_block's barriers)
@@ -266,8 +297,8 @@ __global__ void __launch_bounds__(128, 4) k_staged_step(const TParams P, const S
     if (i < total) {
       int k = 0;
 #pragma unroll
-      for (int s = 1; s < kSgKinds; ++s) k += i >= pref[s];
-      sg_load<MODE>(Q, sg_entry(Q, ib * kSgKinds + k, i - pref[k]), t);
+      for (int s = 1; s < kSgKinds; ++s) k += i >= W.pref[s];
+      sg_load<MODE>(Q, sg_entry(Q, ib * kSgKinds + k, i - W.pref[k]), t);
       if (want_slot) sg_restore_gidx(P, t);
       phase = kStep;
     }
@@ -281,8 +312,8 @@ __global__ void __launch_bounds__(128, 4) k_staged_step(const TParams P, const S
     if (RELOC_KERNEL && keep && next == kReloc) Q.iw[6 * Q.n + e] = aux;
     sg_retire(C, was && next == kEmpty);
   }
-  if ((long long)blockIdx.x * blockDim.x < total) sg_flush(P, cnt);
-  if (sg_last_block(C, 0) && threadIdx.x == 0) {
+  if (total > 0) sg_flush(P, cnt);
+  if (sg_last_block(C, 0, workers) && threadIdx.x == 0) {
     volatile SgCtrl *V = C;
     const long long active = V->active;
     const long long left = P.total - (long long)V->q_head;
@@ -305,11 +336,12 @@ __global__ void __launch_bounds__(128, 4) k_staged_step(const TParams P, const S
 // at 128 registers, 6 blocks in between).
 template <int MODE>
 __global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const SgQueues Q, SgCtrl *C, int ib) {
-  const volatile SgCtrl *V0 = C;
-  if (V0->drain_now || V0->done) return;
+  const SgWork &W = sg_work(C, ib);
+  const long long total = W.n_reloc;
+  const unsigned workers = sg_workers(total);
+  if (W.stop || blockIdx.x >= workers) return;
   Counters cnt;
   sg_begin(cnt);
-  const long long total = (long long)V0->cnt[kSgReloc];
   const int ob = ib ^ 1;
   const bool want_slot = P.out_hash || P.out_len;
   // block-sized strides: the loop condition is the same for every thread of the block (sg_push_block's barriers)
@@ -335,8 +367,8 @@ __global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const 
     sg_push_block<MODE>(Q, C, keep, keep ? sg_queue_of(P, t, ob) : 0, t);
     sg_retire(C, act && next == kEmpty);
   }
-  if ((long long)blockIdx.x * blockDim.x < total) sg_flush(P, cnt);
-  if (sg_last_block(C, 3) && threadIdx.x == 0) {
+  if (total > 0) sg_flush(P, cnt);
+  if (sg_last_block(C, 3, workers) && threadIdx.x == 0) {
     ((volatile SgCtrl *)C)->cnt[kSgReloc] = 0;
     __threadfence();
   }
@@ -348,12 +380,12 @@ __global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const 
 template <int MODE>
 __global__ void __launch_bounds__(128, 4) k_staged_finish(const TParams P, const SgQueues Q, SgCtrl *C, int ib,
                                                            long long drain_tracks) {
-  const volatile SgCtrl *V0 = C;
-  if (V0->drain_now || V0->done) return;
+  const SgWork &W = sg_work(C, ib);
+  const long long n_int = W.n_int, g0 = W.base, total = n_int + W.n_new;
+  const unsigned workers = sg_workers(total);
+  if (W.stop || blockIdx.x >= workers) return;
   Counters cnt;
   sg_begin(cnt);
-  const long long n_int = (long long)V0->cnt[kSgInteract], n_new = V0->n_new, g0 = V0->base;
-  const long long total = n_int + n_new;
   const int ob = ib ^ 1;
   const bool want_slot = P.out_hash || P.out_len;
   const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
@@ -378,8 +410,8 @@ __global__ void __launch_bounds__(128, 4) k_staged_finish(const TParams P, const
     sg_push<MODE>(Q, C, mine && next == kStep, mine && next == kStep ? sg_queue_of(P, t, ob) : 0, t);
     sg_retire(C, mine && next == kEmpty);
   }
-  if ((long long)blockIdx.x * blockDim.x < total) sg_flush(P, cnt);
-  if (sg_last_block(C, 1) && threadIdx.x == 0) {
+  if (total > 0) sg_flush(P, cnt);
+  if (sg_last_block(C, 1, workers) && threadIdx.x == 0) {
     volatile SgCtrl *V = C;
     V->cnt[kSgInteract] = 0;
 #pragma unroll
@@ -409,8 +441,8 @@ __global__ void __launch_bounds__(128, 4) k_staged_drain(const TParams P, const 
   sg_begin(cnt);
   const MlpCtx mc = sg_mlp<MODE>(P);
   const int bank = V0->drain_bank;
-  __shared__ long long pref[kSgKinds + 1];
-  const long long total = sg_prefix(C, bank, pref);
+  const SgWork &W = sg_work(C, bank);
+  const long long total = W.pref[kSgKinds];
   const bool want_slot = P.out_hash || P.out_len;
   const unsigned lane = threadIdx.x & 31u;
   Track t;
@@ -432,8 +464,8 @@ __global__ void __launch_bounds__(128, 4) k_staged_drain(const TParams P, const 
       if (phase == kEmpty && g < total) {
         int k = 0;
 #pragma unroll
-        for (int s = 1; s < kSgKinds; ++s) k += g >= pref[s];
-        sg_load<MODE>(Q, sg_entry(Q, bank * kSgKinds + k, g - pref[k]), t);
+        for (int s = 1; s < kSgKinds; ++s) k += g >= W.pref[s];
+        sg_load<MODE>(Q, sg_entry(Q, bank * kSgKinds + k, g - W.pref[k]), t);
         if (want_slot) sg_restore_gidx(P, t);
         phase = kStep;
       }
@@ -448,7 +480,7 @@ __global__ void __launch_bounds__(128, 4) k_staged_drain(const TParams P, const 
     if (drained && __ballot_sync(kFull, phase != kEmpty) == 0) break;
   }
   sg_flush(P, cnt);
-  if (sg_last_block(C, 2) && threadIdx.x == 0) {
+  if (sg_last_block(C, 2, gridDim.x) && threadIdx.x == 0) {
     volatile SgCtrl *V = C;
 #pragma unroll
     for (int k = 0; k < kSgKinds; ++k) V->cnt[bank * kSgKinds + k] = 0;
@@ -556,6 +588,9 @@ int staged_run(g4n_ctx *ctx, const g4n_batch_desc *b, TParams &P, cudaStream_t s
   if (smem) cudaFuncSetAttribute(k_staged_drain<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_drain, k_staged_drain<MODE>, 128, smem);
   const int g_drain = ctx->sm_count * std::max(per_sm_drain, 1);
+  // two tracks per resident thread: with the iterations cheaper than they were the drain, bound by instruction fetch,
+  // pays later (batches of the nested barrel / calorimeter of 2 10^5 / 10^6 tracks at 4, 2, 1 a thread: 19.9, 18.1, 17.5
+  // / 2.48, 2.16, 2.37 / 6.86, 6.76, 7.21 ms; the barrel does not care)
   const long long drain_tracks = b->drain_tracks < 0 ? -1
                                  : b->drain_tracks > 0 ? b->drain_tracks
                                                        : 2LL * g_drain * 128;

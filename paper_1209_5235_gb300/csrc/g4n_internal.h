@@ -196,6 +196,7 @@ struct HGeom {
   std::vector<int32_t> portal;
   std::vector<int32_t> touch_lv, touch_copy;  // per volume (touchable): logical volume, copy number
   int32_t max_depth = 0;
+  bool all_keyed = false;   // every volume is a kKeyBox
   // device blob
   void *blob = nullptr;
   size_t blob_bytes = 0;

@@ -1075,6 +1075,8 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
     }
     if (v.vox >= 0) key_headers(*g, v.vox, wt);
   }
+  g->all_keyed = true;
+  for (int i = 0; i < n; ++i) g->all_keyed = g->all_keyed && (g->vol[i].flags & kKeyBox);
   // --- face relocation records of kKeyBox volumes
   for (int i = 0; i < n; ++i) g->vol[i].face = -1;
   for (int i = 0; i < n; ++i) {

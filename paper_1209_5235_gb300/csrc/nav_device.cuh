@@ -425,6 +425,26 @@ __device__ __forceinline__ int vox_lookup(const DGeom &G, int h, const V3 &p) {
   return 0;
 }
 
+// The same decided in FP32 on the point's enclosure (slice_of32), FP64 where a slice boundary lies within it.
+__device__ __forceinline__ int vox_lookup32(const DGeom &G, int h, const V3 &p) {
+  const int root = h;
+  float lo[3], hi[3];
+  enclose(p.x, lo[0], hi[0]);
+  enclose(p.y, lo[1], hi[1]);
+  enclose(p.z, lo[2], hi[2]);
+#pragma unroll 1
+  for (int lev = 0; lev < kMaxLevels; ++lev) {
+    const DVoxHdr32 H = G.hdr32[h];
+    const int a = H.n_axis & 3;
+    const int k = slice_of32(H, sel3(lo[0], lo[1], lo[2], a), sel3(hi[0], hi[1], hi[2], a));
+    if (k < 0) return vox_lookup(G, root, p);
+    const DVoxSlice S = G.slice[H.slice_base + k];
+    if (S.child >= 0) return S.child;
+    h = -S.child - 1;
+  }
+  return 0;
+}
+
 // ---------------------------------------------------------------- exact coordinate keys
 // key(x): a double's bits as a signed integer with the negative half reflected,
 // so that x < y <=> key(x) < key(y).  The geometry carries, for world-aligned
@@ -528,12 +548,16 @@ __device__ __forceinline__ int vox_lookup_keys(const DGeom &G, int h, const WPos
 constexpr unsigned kFull = 0xffffffffu;
 
 // Descend from volume m into the first daughter, in id order, that contains the
-// point; repeat.  (p, v) is the point in m's frame when have_p is set; otherwise it
+// point; repeat.  CLASSIFY: the daughters are first classified in FP32 (nav_pick32.cuh) and the voxel slices
+// looked up in FP32, so that only a point within the FP32 errors of a daughter's surface takes an FP64 test.  10^7
+// barrel queries of k_locate: 3.52 -> 2.20 ms (each candidate that passed its box in FP64 kept the FP64 pipe 78 %
+// busy); where the tracks of a nested barrel start, a batch of 10^6 17.9 -> 17.2 ms.  Relocations go without: with the
+// portals they are few, and the added code cost the barrel and the batched worlds 1 %, the default barrel 4 %.  (p, v) is the point in m's frame when have_p is set; otherwise it
 // is derived from the world point when an FP64 test needs it.  kKeyBox daughters
 // and keyed voxel trees are answered from the world point's keys.  `blocked` is a
 // daughter of m already known not to contain the point (the volume just left).
 // Returns the deepest volume.
-template <bool COUNT>
+template <bool COUNT, bool CLASSIFY>
 __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, V3 p, V3 v, bool have_p,
                                             const WPos &W, int blocked, Counters &cnt) {
 #pragma unroll 1
@@ -547,14 +571,15 @@ __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, 
         L = G.clist[vox_lookup_keys(G, h, W)];
       } else {
         if (!have_p) {
-          world_to_local(G.wxf[m], G.vol[m].flags & kWorldAligned, W.x, W.u, p, v);
+          if (CLASSIFY) p = world_to_local_point(G.wxf[m], G.vol[m].flags & kWorldAligned, W.x);
+          else world_to_local(G.wxf[m], G.vol[m].flags & kWorldAligned, W.x, W.u, p, v);
           have_p = true;
         }
-        L = G.clist[vox_lookup(G, h, p)];
+        L = G.clist[CLASSIFY ? vox_lookup32(G, h, p) : vox_lookup(G, h, p)];
       }
     }
-    float px = 0.f, py = 0.f, pz = 0.f;
-    bool have_pf = false;
+    PickRay q;
+    bool have_q = false;
     int i = 0, found = -1;
     bool searching = want, via_fp64 = false;
     V3 fp = p, fv = v;
@@ -578,19 +603,31 @@ __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, 
             continue;
           }
           if (!have_p) {
-            world_to_local(G.wxf[m], G.vol[m].flags & kWorldAligned, W.x, W.u, p, v);
+            if (CLASSIFY) p = world_to_local_point(G.wxf[m], G.vol[m].flags & kWorldAligned, W.x);
+            else world_to_local(G.wxf[m], G.vol[m].flags & kWorldAligned, W.x, W.u, p, v);
             have_p = true;
           }
-          if (!have_pf) {
-            px = (float)p.x;
-            py = (float)p.y;
-            pz = (float)p.z;
-            have_pf = true;
+          if (!have_q) {
+            if (CLASSIFY) {
+              q = pick_ray(p, V3{0.0, 0.0, 0.0});
+            } else {
+              q.ph[0] = (float)p.x;
+              q.ph[1] = (float)p.y;
+              q.ph[2] = (float)p.z;
+            }
+            have_q = true;
           }
-          if (box32_contains(B, px, py, pz) && !(iso_lb32(G.v32[c], px, py, pz) > G.band32)) {
+          if (!box32_contains(B, q.ph[0], q.ph[1], q.ph[2])) continue;
+          const int in = CLASSIFY ? classify_daughter(G.pick[c], q, G.band32)
+                                  : iso_lb32(G.v32[c], q.ph[0], q.ph[1], q.ph[2]) > G.band32 ? -1 : 0;
+          if (in < 0) continue;
+          if (in > 0) {
+            found = c;
+            searching = false;
+          } else {
             d = c;
-            break;
           }
+          break;
         }
         if (d < 0) searching = false;
       }
@@ -598,6 +635,7 @@ __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, 
       if (d >= 0) {
         const DVol &D = G.vol[d];
         V3 dp, dv;
+        if (CLASSIFY) world_to_local(G.wxf[m], G.vol[m].flags & kWorldAligned, W.x, W.u, p, v);
         to_local(D, p, v, dp, dv);
         diag_test<COUNT>(cnt, G4N_C_INSIDE, G4N_C_INSIDE_CURVED, D.kind);
         if (vol_inside(D, dp, dv, G.half)) {
@@ -627,22 +665,22 @@ __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, 
 // shared copy relieves: measured 8 % on the barrel scene); the FP64 navigator inlines it
 // (measured 2 % faster on the calorimeter, whose relocations are mostly face records).
 // Counters are passed by pointer (null without diagnostics) so that they stay in registers.
-template <bool COUNT>
+template <bool COUNT, bool CLASSIFY>
 __device__ __noinline__ int descend_ool(const DGeom &G, bool active, int m, V3 p, V3 v, bool have_p, const WPos &W,
                                         int blocked, Counters *cntp) {
   Counters none;
-  return descend_body<COUNT>(G, active, m, p, v, have_p, W, blocked, COUNT ? *cntp : none);
+  return descend_body<COUNT, CLASSIFY>(G, active, m, p, v, have_p, W, blocked, COUNT ? *cntp : none);
 }
 
-template <bool COUNT, bool OOL>
+template <bool COUNT, bool OOL, bool CLASSIFY>
 __device__ __forceinline__ int descend_warp(const DGeom &G, bool active, int m, V3 p, V3 v, bool have_p,
                                             const WPos &W, int blocked, Counters &cnt) {
-  if (OOL) return descend_ool<COUNT>(G, active, m, p, v, have_p, W, blocked, COUNT ? &cnt : nullptr);
-  return descend_body<COUNT>(G, active, m, p, v, have_p, W, blocked, cnt);
+  if (OOL) return descend_ool<COUNT, CLASSIFY>(G, active, m, p, v, have_p, W, blocked, COUNT ? &cnt : nullptr);
+  return descend_body<COUNT, CLASSIFY>(G, active, m, p, v, have_p, W, blocked, cnt);
 }
 
 // Locate from the world (warp-collective): the leaf, or -1 outside the world.
-template <bool COUNT, bool OOL = false>
+template <bool COUNT, bool OOL, bool CLASSIFY>
 __device__ __forceinline__ int locate_world_warp(const DGeom &G, bool active, const V3 &x, const V3 &u, Counters &cnt) {
   V3 p{0, 0, 0}, v{0, 0, 1};
   bool in = false, have_p = false;
@@ -658,7 +696,7 @@ __device__ __forceinline__ int locate_world_warp(const DGeom &G, bool active, co
       in = vol_inside(G.vol[0], p, v, G.half);
     }
   }
-  const int leaf = descend_warp<COUNT, OOL>(G, in, 0, p, v, have_p, W, -1, cnt);
+  const int leaf = descend_warp<COUNT, OOL, CLASSIFY>(G, in, 0, p, v, have_p, W, -1, cnt);
   return in ? leaf : -1;
 }
 
@@ -709,7 +747,7 @@ __device__ __forceinline__ int relocate_warp(const DGeom &G, bool active, int le
       }
     }
   }
-  const int out = descend_warp<COUNT, MODE != kFP64>(G, in, in ? leaf : 0, p, v, have_p, W, blocked, cnt);
+  const int out = descend_warp<COUNT, MODE != kFP64, false>(G, in, in ? leaf : 0, p, v, have_p, W, blocked, cnt);
   return in ? out : -1;
 }
 

@@ -101,6 +101,9 @@ __device__ __forceinline__ void flush_block(unsigned long long *counters) {
 // 8 blocks of 128 per SM (64 registers, a few hundred bytes of spills): the descent waits on its chain
 // of dependent table loads, and more resident warps hide it (10^7 calorimeter queries: 6.3e9 -> 8.8e9 /s
 // against 5 blocks at 96 registers; 10 to 16 blocks were slower again).
+// CLASSIFY: FP32 classification of the daughters (descend_body); geometries of world-aligned boxes alone, whose Inside
+// tests are key comparisons, go without (10^7 calorimeter queries 1.17 -> 1.15 ms).
+template <bool CLASSIFY>
 __global__ void __launch_bounds__(128, 8) k_locate(const DGeom *__restrict__ geoms, int gid, int64_t n,
                                                 const double *__restrict__ pos, const double *__restrict__ dir,
                                                 int32_t *__restrict__ out_depth, int32_t *__restrict__ out_path,
@@ -120,7 +123,7 @@ __global__ void __launch_bounds__(128, 8) k_locate(const DGeom *__restrict__ geo
       ok = !bad_dir(u) && isfinite(x.x + x.y + x.z);
       if (!ok) flag(status, kStBadInput);
     }
-    const int leaf = locate_world_warp<false>(G, ok, x, u, cnt);
+    const int leaf = locate_world_warp<false, false, CLASSIFY>(G, ok, x, u, cnt);
     if (i < n) {
       const int depth = ok ? (leaf >= 0 ? G.vol[leaf].depth : 0) : -1;
       out_depth[i] = depth;
@@ -384,7 +387,7 @@ __device__ __forceinline__ void set_direction(Track &t, const V3 &u) {
 // Start track number g of the concatenated items on the lanes with `active` set
 // (warp-collective: locate runs across the warp).  Returns the new phase of the
 // lane: kStep, or kEmpty if the track ended at once (or the lane was not active).
-template <int MODE, bool COUNT, bool EV>
+template <int MODE, bool COUNT, bool EV, bool CLASSIFY = false>
 __device__ int start_warp(const TParams &P, bool active, int64_t g, Track &t, Counters &cnt) {
   const DGeom *Gp = &P.geoms[P.items[0].geom];
   if (active) {
@@ -407,7 +410,7 @@ __device__ int start_warp(const TParams &P, bool active, int64_t g, Track &t, Co
     t.E = E;
   }
   const DGeom &G = *Gp;
-  const int leaf = locate_world_warp<COUNT, MODE != kFP64>(G, active, t.x, t.u, cnt);
+  const int leaf = locate_world_warp<COUNT, MODE != kFP64, CLASSIFY>(G, active, t.x, t.u, cnt);
   if (!active) return kEmpty;
   t.leaf = leaf;
   if (leaf < 0) {
@@ -1035,7 +1038,7 @@ __global__ void __launch_bounds__(128, 3) k_free_path(const FParams P) {
           cnt.c[G4N_C_TRACKS]++;
         }
       }
-      const int l0 = locate_world_warp<COUNT>(G, take, x0, u, cnt);
+      const int l0 = locate_world_warp<COUNT, false, false>(G, take, x0, u, cnt);
       if (take) {
         if (!(Y > 0.0) || l0 < 0) {
           // Y <= 0: the interaction is at the start point; outside the world: no segment at all
@@ -1307,7 +1310,8 @@ int g4n_locate(g4n_ctx *ctx, int32_t geom, int64_t n, const double *pos, const d
   cudaSetDevice(ctx->device);
   Workspace *ws = (Workspace *)ctx->ws;
   ++ctx->launches;
-  k_locate<<<grid_for(ctx, n, 128), 128, 0, (cudaStream_t)stream>>>(ctx->d_geoms, geom, n, pos, dir, out_depth,
+  const auto kern = ctx->geoms[geom]->all_keyed ? k_locate<false> : k_locate<true>;
+  kern<<<grid_for(ctx, n, 128), 128, 0, (cudaStream_t)stream>>>(ctx->d_geoms, geom, n, pos, dir, out_depth,
                                                                      out_path, &ws->status);
   return launch_error(ctx, "locate launch");
 }

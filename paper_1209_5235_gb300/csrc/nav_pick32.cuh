@@ -391,6 +391,36 @@ __device__ __forceinline__ float pick_to_daughter(const DPick32 &D, const PickRa
   return 6.0f * kU * (fabsf(dx) + fabsf(dy) + fabsf(x[2]) + ext) + 3e-14f * far + 1e-30f;
 }
 
+// Position of the point against the solid: 1 inside and -1 outside by more than the band, 0 undecided (cones: always).  Each
+// distance is within 4 ep of the exact one: the coordinates' errors (up to sqrt 3 ep), the sizes', the radius's roundings.
+__device__ __forceinline__ int classify_point(int kind, const float *q, int flags, float x, float y, float z, float ep,
+                                              float band) {
+  float d;
+  if (kind == kBox) {
+    d = fminf(q[0] - fabsf(x), fminf(q[1] - fabsf(y), q[2] - fabsf(z)));
+  } else if (kind == kOrb) {
+    d = q[0] - sqrt_approx(x * x + y * y + z * z);
+  } else if (kind == kTube) {
+    const float r = sqrt_approx(x * x + y * y);
+    d = fminf(q[2] - fabsf(z), q[1] - r);
+    if (flags & kHasRmin) d = fminf(d, r - q[0]);
+    if (flags & kSeg) {
+      const float ds = q[3] * y - q[4] * x, de = q[6] * x - q[5] * y;
+      d = fminf(d, (flags & kWide) ? fmaxf(ds, de) : fminf(ds, de));
+    }
+  } else {
+    return 0;
+  }
+  const float m = 4.0f * ep + band;
+  return d > m ? 1 : (d < -m ? -1 : 0);
+}
+
+// The same for daughter D of the volume whose frame the point is given in.
+__device__ __forceinline__ int classify_daughter(const DPick32 &D, const PickRay &r, float band) {
+  float x[3], v[3];
+  const float ep = pick_to_daughter(D, r, x, v);
+  return classify_point(D.kind_flags & 3, D.q, D.kind_flags >> 2, x[0], x[1], x[2], ep, band);
+}
 // DistanceToIn of daughter D of the volume whose frame the ray is given in.
 __device__ __forceinline__ Pick pick_daughter(const DPick32 &D, const PickRay &r, float band) {
   float x[3], v[3];

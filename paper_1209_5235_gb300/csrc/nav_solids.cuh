@@ -58,6 +58,13 @@ __device__ __forceinline__ void world_to_local(const DWorld &w, bool aligned, co
   vl.z = u.z;
 }
 
+// World -> local frame of a point alone.
+__device__ __forceinline__ V3 world_to_local_point(const DWorld &w, bool aligned, const V3 &p) {
+  const double dx = p.x - w.tx, dy = p.y - w.ty;
+  if (aligned) return V3{dx, dy, p.z - w.tz};
+  return V3{w.c * dx + w.s * dy, w.c * dy - w.s * dx, p.z - w.tz};
+}
+
 // Reciprocal direction components (0 where the component is 0: never used there).
 struct Inv3 {
   double x, y, z;

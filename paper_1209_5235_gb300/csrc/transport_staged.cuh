@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(128, 4) k_staged_finish(const TParams P, const
       next = interact<MODE, true>(P, t, cnt);
     }
     if (__any_sync(kFull, is_new)) {  // the source and the locate (warp-collective)
-      const int started = start_warp<MODE, false, true>(P, is_new, g0 + (i - n_int), t, cnt);
+      const int started = start_warp<MODE, false, true, MODE != kFP64>(P, is_new, g0 + (i - n_int), t, cnt);
       if (is_new) next = started;
     }
     const bool mine = is_int || is_new;

@@ -44,6 +44,8 @@ constexpr int kSgInteract = 2 * kSgKinds;
 constexpr int kSgReloc = 2 * kSgKinds + 1;
 constexpr int kSgArrays = 6;                // queue arrays of `pool` entries (see sg_entry)
 constexpr int kSgDoubles = 16, kSgInts = 7; // the seventh int: a deferred relocation's limiter and exit flag
+constexpr int kSgRepeat = 4, kSgKeep = 8;   // repeated steps of a warp (see k_staged_step)
+constexpr int kHold = 5;                    // phase of a lane that waits for its warp's last repeat
 constexpr int kSgChunk = 8;                 // iterations launched between reads of the end flag
 
 // Track-state queues, structure of arrays: field f of entry e at base_f[e].
@@ -304,8 +306,26 @@ __global__ void __launch_bounds__(128, 4) k_staged_step(const TParams P, const S
     }
     Chain ch;
     int aux = 0;
-    const int next = step_warp<MODE, false, false, true, RELOC_KERNEL>(P, t, phase, cnt, mc, ch, &aux);
     const bool was = phase == kStep;
+    // Steps in boxes without daughters are a few instructions each (an exit, a face record): while kSgKeep lanes of the
+    // warp stand in one they step on, up to kSgRepeat times, before the states go back to the queues (336 bytes of
+    // traffic and a share of an iteration's launches per step saved).  Calorimeter 10^6 6.55 -> 5.22 ms, stack of plates
+    // 19.9 -> 16.3 ms.  The variant with the relocation kernel, made for curved segments, goes without: repeated steps
+    // there cost the barrel half as much again.
+    int next = phase;
+#pragma unroll 1
+    for (int rep = 1;; ++rep) {
+      next = step_warp<MODE, false, false, true, RELOC_KERNEL>(P, t, next, cnt, mc, ch, &aux);
+      if (RELOC_KERNEL) break;
+      bool again = false;
+      if (next == kStep) {
+        const DVol &L = P.geoms[P.items[t.item].geom].vol[t.leaf];
+        again = L.kind == kBox && L.vox < 0;
+        if (!again) next = kHold;
+      }
+      if (rep >= kSgRepeat || __popc(__ballot_sync(kFull, again)) < kSgKeep) break;
+    }
+    if (next == kHold) next = kStep;
     const bool keep = was && next != kEmpty;
     const int q = !keep ? 0 : next == kStep ? sg_queue_of(P, t, ob) : next == kReloc ? kSgReloc : kSgInteract;
     const int64_t e = sg_push_block<MODE>(Q, C, keep, q, t);

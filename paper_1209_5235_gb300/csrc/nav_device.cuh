@@ -1314,7 +1314,14 @@ __device__ __noinline__ void search_full(const DGeom &G, int leaf, const V3 &p, 
 
 // limit: a float not below the physics step.  Budget, resume, walk cap and chain as geom_step_warp's.  In the learned
 // mode the network's proposal is looked at before the node's other candidates; its enclosure prunes them.
-template <int MODE, bool COUNT>
+//
+// SEEN: a daughter is listed in every node it reaches into, and a ray meets it again node after node; the last kSeen
+// candidates looked at are kept in registers and passed over (a second look could not change anything: the bound only
+// falls).  48 batched worlds 25.5 -> 20.0 ms, barrel 69.8 -> 64.9, nested barrel 17.0 -> 16.0.  The query kernel, whose
+// searches end in the first nodes, goes without.  Two
+// and eight candidates: barrel 67.2 and 66.4, worlds 22.6 and 20.2.
+constexpr int kSeen = 4;
+template <int MODE, bool COUNT, bool SEEN = true>
 __device__ __forceinline__ Step32 geom_step32_warp(const DGeom &G, bool active, int leaf, const V3 &p, const V3 &v,
                                                    float limit, bool want_safety, Counters &cnt, bool *timeout,
                                                    int walk_cap, const MlpCtx &mc, Chain &ch, bool resume = false,
@@ -1332,6 +1339,9 @@ __device__ __forceinline__ Step32 geom_step32_warp(const DGeom &G, bool active, 
   int i = 0, it = 0;
   DCandList L{0, 0}, L0{0, 0};
   int prop_done = -1;
+  int seen[kSeen];
+#pragma unroll
+  for (int k = 0; k < kSeen; ++k) seen[k] = -1;
   float feat[mlp::kIn];
   bool have_feat = false;
   if (active) {
@@ -1421,8 +1431,21 @@ __device__ __forceinline__ Step32 geom_step32_warp(const DGeom &G, bool active, 
         if (i < L.count) {
           const int c = __ldg(&G.cand[L.offset + i]);
           ++i;
+          if (SEEN) {
+            bool again = false;
+#pragma unroll
+            for (int k = 0; k < kSeen; ++k) again |= c == seen[k];
+            if (again) continue;
+#pragma unroll
+            for (int k = kSeen - 1; k > 0; --k) seen[k] = seen[k - 1];
+            seen[0] = c;
+          }
           const DBox32 B = G.box[c];
-          const float iso = iso_lb32(G.v32[c], r.plo[0], r.plo[1], r.plo[2]) - G.band32;
+          // the distance from the point bounds the entry as well; after the first node it prunes next to nothing that the
+          // box lets pass (barrel 1.4 %, worlds 3 % for leaving it out; the learned mode lost 3 % by that)
+          float iso = -kInfF;
+          if (MODE == kLearned || !SEEN || (first && want_safety))
+            iso = iso_lb32(G.v32[c], r.plo[0], r.plo[1], r.plo[2]) - G.band32;
           if (first && want_safety) saf_f = fminf(saf_f, fmaxf(box_gap_lb(B.lo, B.hi, r), iso));
           if (MODE == kLearned && first && i - 1 == prop_done) continue;  // already looked at
           const float lb = fmaxf(box_entry_lb(B.lo, B.hi, r, nullptr), iso);

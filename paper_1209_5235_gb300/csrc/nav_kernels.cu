@@ -33,7 +33,7 @@ namespace g4n {
 struct DItem {
   int32_t geom, pad;
   int64_t n, tid0, tally_off, start;
-  double src[16];  // pos[3], sigma, has_z, z0, z1, iso, dir[3], e_kind, e0, e1, -
+  double src[16];  // pos[3], sigma, has_z, z0, z1, iso, dir[3], e_kind, e0, e1, log(e1 / e0), -
 };
 
 enum StatusBits : uint32_t { kStStepLimit = 1u, kStTimeout = 2u, kStRejection = 4u, kStBadInput = 8u };
@@ -353,7 +353,7 @@ __device__ void make_source(const double *src, uint64_t seed, int64_t tid, V3 &x
   const int ek = (int)src[11];
   if (ek == 0) E = src[12];
   else if (ek == 1) E = src[12] + (src[13] - src[12]) * philox_uniform(seed, tid, 0, draw);
-  else E = src[12] * exp(philox_uniform(seed, tid, 0, draw) * log(src[13] / src[12]));
+  else E = src[12] * exp(philox_uniform(seed, tid, 0, draw) * src[14]);
 }
 
 __device__ __forceinline__ void tally(const TParams &P, const Track &t, int col, double e) {
@@ -1266,7 +1266,8 @@ int build_items(g4n_ctx *ctx, const g4n_batch_desc *b, std::vector<DItem> &items
     d.tally_off = w.tally_offset;
     d.start = total;
     double src[16] = {s.pos[0], s.pos[1], s.pos[2], s.spot_sigma, (double)(s.has_z != 0), s.z0, s.z1,
-                      (double)(s.isotropic != 0), s.dir[0], s.dir[1], s.dir[2], (double)s.e_kind, s.e0, s.e1, 0.0, 0.0};
+                      (double)(s.isotropic != 0), s.dir[0], s.dir[1], s.dir[2], (double)s.e_kind, s.e0, s.e1,
+                      s.e_kind == 2 ? std::log(s.e1 / s.e0) : 0.0, 0.0};
     std::memcpy(d.src, src, sizeof(src));
     total += w.n_tracks;
   }
@@ -1647,7 +1648,7 @@ extern "C" int g4n_transport_batch_noalloc(g4n_ctx *ctx, const g4n_batch_desc *b
     d.start = total;
     const double src[16] = {s.pos[0], s.pos[1], s.pos[2], s.spot_sigma, (double)(s.has_z != 0), s.z0, s.z1,
                             (double)(s.isotropic != 0), s.dir[0], s.dir[1], s.dir[2], (double)s.e_kind, s.e0, s.e1,
-                            0.0, 0.0};
+                            s.e_kind == 2 ? std::log(s.e1 / s.e0) : 0.0, 0.0};
     std::memcpy(d.src, src, sizeof(src));
     total += w.n_tracks;
   }

@@ -142,8 +142,13 @@ __global__ void __launch_bounds__(128, 8) k_locate(const DGeom *__restrict__ geo
 
 // ---------------------------------------------------------------- compute_step
 
-template <int MODE>
-__global__ void __launch_bounds__(128) k_compute_step(const DGeom *__restrict__ geoms, int gid, int64_t n,
+// SORT: a block takes tiles of 512 consecutive queries, sorts each by the kind of the leaf and whether it has
+// daughters (a counting sort of their indices in shared memory), and answers them in that order: unsorted queries had 7.2
+// lanes of a warp on the same instruction.  10^6 barrel queries 0.79 -> 0.68 ms (FP32 mode), 1.67 -> 1.25 ms (FP64).
+constexpr int kQueryTile = 4;   // queries per thread and sorted tile
+// 4 blocks per SM (128 registers): at the 147 the compiler takes otherwise the FP32 queries are 12 % slower.
+template <int MODE, bool SORT>
+__global__ void __launch_bounds__(128, 4) k_compute_step(const DGeom *__restrict__ geoms, int gid, int64_t n,
                                                       const double *__restrict__ pos, const double *__restrict__ dir,
                                                       const int32_t *__restrict__ depth, const int32_t *__restrict__ path,
                                                       const double *__restrict__ proposed, double *__restrict__ out_step,
@@ -152,7 +157,6 @@ __global__ void __launch_bounds__(128) k_compute_step(const DGeom *__restrict__ 
                                                       int walk_cap) {
   const DGeom &G = geoms[gid];
   Counters cnt;
-  const int64_t lane = threadIdx.x & 31;
   MlpCtx mc{nullptr, nullptr, nullptr, 0.f};
   if (MODE == kLearned) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -163,60 +167,99 @@ __global__ void __launch_bounds__(128) k_compute_step(const DGeom *__restrict__ 
     mc.scratch = reinterpret_cast<mlp::SmemWarp *>(smem + sizeof(mlp::SmemWeights)) + (threadIdx.x >> 5);
     mc.loge = 0.46f;  // log-energy feature at 1 MeV: the query carries no energy
   }
-  for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < n;
-       base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = base + lane;
-    bool ok = false;
-    int leaf = 0;
-    double prop = kInf;
-    V3 p{0, 0, 0}, v{0, 0, 1};
-    if (i < n) {
-      const V3 x{pos[i], pos[n + i], pos[2 * n + i]};
-      const V3 u{dir[i], dir[n + i], dir[2 * n + i]};
-      const int d = depth[i];
-      leaf = (d >= 1 && d <= kDMax) ? path[(int64_t)(d - 1) * n + i] : -1;
-      ok = !bad_dir(u) && leaf >= 0 && leaf < G.n_vol && G.vol[leaf].depth == d;
-      if (!ok) {
-        flag(status, kStBadInput);
-        out_step[i] = nan("");
-        out_safety[i] = nan("");
-        out_lim[i] = INT32_MIN;
-        leaf = 0;
+  __shared__ unsigned short order[SORT ? 128 * kQueryTile : 1];
+  __shared__ int count[16];
+  const int tid = threadIdx.x;
+  constexpr int kPer = SORT ? kQueryTile : 1;
+  constexpr int64_t kSpan = 128 * kPer;
+#pragma unroll 1
+  for (int64_t tile = blockIdx.x * kSpan; tile < n; tile += gridDim.x * kSpan) {
+    if (SORT) {
+      int key[kQueryTile], rank[kQueryTile];
+      if (tid < 16) count[tid] = 0;
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < kQueryTile; ++j) {
+        const int64_t i = tile + j * 128 + tid;
+        key[j] = 15;   // past the end: last
+        if (i < n) {
+          const int d = depth[i];
+          const int l = (d >= 1 && d <= kDMax) ? path[(int64_t)(d - 1) * n + i] : -1;
+          key[j] = l >= 0 && l < G.n_vol ? 2 * G.vol[l].kind + (G.vol[l].vox < 0) : 14;
+        }
+        rank[j] = atomicAdd(&count[key[j]], 1);
+      }
+      __syncthreads();
+      if (tid == 0) {
+        int acc = 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          const int c = count[k];
+          count[k] = acc;
+          acc += c;
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < kQueryTile; ++j) order[count[key[j]] + rank[j]] = (unsigned short)(j * 128 + tid);
+      __syncthreads();
+    }
+#pragma unroll 1
+    for (int j = 0; j < kPer; ++j) {
+      const int64_t i = tile + (SORT ? (int)order[j * 128 + tid] : tid);
+      bool ok = false;
+      int leaf = 0;
+      double prop = kInf;
+      V3 p{0, 0, 0}, v{0, 0, 1};
+      if (i < n) {
+        const V3 x{pos[i], pos[n + i], pos[2 * n + i]};
+        const V3 u{dir[i], dir[n + i], dir[2 * n + i]};
+        const int d = depth[i];
+        leaf = (d >= 1 && d <= kDMax) ? path[(int64_t)(d - 1) * n + i] : -1;
+        ok = !bad_dir(u) && leaf >= 0 && leaf < G.n_vol && G.vol[leaf].depth == d;
+        if (!ok) {
+          flag(status, kStBadInput);
+          out_step[i] = nan("");
+          out_safety[i] = nan("");
+          out_lim[i] = INT32_MIN;
+          leaf = 0;
+        } else {
+          prop = proposed ? proposed[i] : kInf;
+          world_to_local(G.wxf[leaf], G.vol[leaf].flags & kWorldAligned, x, u, p, v);
+        }
+      }
+      bool timeout = false;
+      Chain ch;
+      double s = kInf, safety = 0.0;
+      int lim = G4N_LIM_MOTHER;
+      if constexpr (MODE == kFP64) {
+        const StepResult R = geom_step_warp<false>(G, ok, leaf, p, v, inv_dir(v), prop, true, cnt, &timeout, walk_cap, mc, ch);
+        s = R.step;
+        lim = R.lim;
+        safety = R.safety;
       } else {
-        prop = proposed ? proposed[i] : kInf;
-        world_to_local(G.wxf[leaf], G.vol[leaf].flags & kWorldAligned, x, u, p, v);
+        // a float not below the proposal (a NaN proposal limits nothing, a negative one everything)
+        const float f = trunc_float(prop), limit = f < 0.f ? f * (1.0f - 2.0f * kU) : f * (1.0f + 2.0f * kU) + 1e-30f;
+        const Step32 R = geom_step32_warp<MODE, false, false>(G, ok, leaf, p, v, limit, true, cnt, &timeout, walk_cap, mc, ch);
+        safety = (double)R.safety;
+        if (ok) {
+          int surf;
+          if (limit < R.lo) lim = G4N_LIM_PHYSICS;   // the proposal comes first for certain
+          else s = step_exact32(G, leaf, p, v, R, walk_cap, &timeout, &lim, &surf);
+        }
       }
-    }
-    bool timeout = false;
-    Chain ch;
-    double s = kInf, safety = 0.0;
-    int lim = G4N_LIM_MOTHER;
-    if constexpr (MODE == kFP64) {
-      const StepResult R = geom_step_warp<false>(G, ok, leaf, p, v, inv_dir(v), prop, true, cnt, &timeout, walk_cap, mc, ch);
-      s = R.step;
-      lim = R.lim;
-      safety = R.safety;
-    } else {
-      // a float not below the proposal (a NaN proposal limits nothing, a negative one everything)
-      const float f = trunc_float(prop), limit = f < 0.f ? f * (1.0f - 2.0f * kU) : f * (1.0f + 2.0f * kU) + 1e-30f;
-      const Step32 R = geom_step32_warp<MODE, false, false>(G, ok, leaf, p, v, limit, true, cnt, &timeout, walk_cap, mc, ch);
-      safety = (double)R.safety;
       if (ok) {
-        int surf;
-        if (limit < R.lo) lim = G4N_LIM_PHYSICS;   // the proposal comes first for certain
-        else s = step_exact32(G, leaf, p, v, R, walk_cap, &timeout, &lim, &surf);
+        if (timeout) flag(status, kStTimeout);
+        if (lim == G4N_LIM_PHYSICS || prop < s) {
+          s = prop;
+          lim = G4N_LIM_PHYSICS;
+        }
+        out_step[i] = s;
+        out_safety[i] = safety;
+        out_lim[i] = lim;
       }
     }
-    if (ok) {
-      if (timeout) flag(status, kStTimeout);
-      if (lim == G4N_LIM_PHYSICS || prop < s) {
-        s = prop;
-        lim = G4N_LIM_PHYSICS;
-      }
-      out_step[i] = s;
-      out_safety[i] = safety;
-      out_lim[i] = lim;
-    }
+    if (SORT) __syncthreads();   // the tile's order has been read
   }
 }
 
@@ -1338,14 +1381,18 @@ int g4n_compute_step(g4n_ctx *ctx, int32_t geom, int64_t n, const double *pos, c
   if ((rc = ensure_ws(ctx, 0))) return rc;
   cudaSetDevice(ctx->device);
   Workspace *ws = (Workspace *)ctx->ws;
-  auto kern = mode == G4N_MODE_FP64 ? k_compute_step<kFP64>
-                                    : (mode == G4N_MODE_FP32_RECHECK ? k_compute_step<kFP32> : k_compute_step<kLearned>);
+  // sorted tiles once every SM gets a dozen of them (1.6 10^5 and 2 10^4 barrel queries: a half and 5 % slower sorted) and
+  // the leaves differ in more than having daughters (10^6 calorimeter queries: 6 % slower sorted)
+  const bool sorted = n >= (int64_t)ctx->sm_count * 12 * 128 * kQueryTile && !ctx->geoms[geom]->all_keyed;
+  auto kern = mode == G4N_MODE_FP64 ? (sorted ? k_compute_step<kFP64, true> : k_compute_step<kFP64, false>)
+              : mode == G4N_MODE_FP32_RECHECK ? (sorted ? k_compute_step<kFP32, true> : k_compute_step<kFP32, false>)
+                                              : (sorted ? k_compute_step<kLearned, true> : k_compute_step<kLearned, false>);
   const size_t smem = mlp_smem_bytes(mode, 128);
   if (smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   ++ctx->launches;
-  kern<<<grid_for(ctx, n, 128), 128, smem, (cudaStream_t)stream>>>(ctx->d_geoms, geom, n, pos, dir, depth, path,
-                                                                    proposed, out_step, out_safety, out_limiter,
-                                                                    &ws->status, g4n_mlp_image(ctx), ctx->walk_cap);
+  kern<<<grid_for(ctx, n, sorted ? 128 * kQueryTile : 128), 128, smem, (cudaStream_t)stream>>>(
+      ctx->d_geoms, geom, n, pos, dir, depth, path, proposed, out_step, out_safety, out_limiter, &ws->status,
+      g4n_mlp_image(ctx), ctx->walk_cap);
   return launch_error(ctx, "compute_step launch");
 }
 

@@ -1,0 +1,75 @@
+"""Query kernels at the sizes where they change their way of working: compute_step answers large batches in tiles sorted
+by the kind of the leaf, free paths refill their warps eight lanes at a time.  Every query is independent of the others,
+so a large call has to give bit for bit what small calls give for the same queries."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1209_5235_gb300 import build
+    build.build()
+    import paper_1209_5235_gb300 as g4
+    ctx = g4.g4n_create(0)
+    yield g4, torch, ctx
+    g4.g4n_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("extra", [-1, 0, 1, 511, 513])
+def test_compute_step_sorted_tiles(env, mode, extra):
+    g4, torch, ctx = env
+    gid = g4.build_scene(ctx, synth.scenes.barrel_scene(n_shells=5, n_phi=8, n_orbs=30))
+    n = torch.cuda.get_device_properties(0).multi_processor_count * 12 * 512 + extra
+    p, v = synth.scenes.query_points("barrel", n, 31)
+    v[:, 7] = 2.0   # not a unit direction: refused in the same way wherever the query is sorted to
+    T = lambda a: torch.tensor(a, device="cuda")
+    pos, dirs = T(p), T(v)
+    prop = T(np.random.default_rng(32).exponential(100.0, n))
+    depth, path = g4.g4n_locate(ctx, gid, pos, dirs)
+    try:
+        g4.g4n_sync(ctx)
+    except g4.G4NError:
+        pass
+    whole = g4.g4n_compute_step(ctx, gid, pos, dirs, depth, path, proposed=prop, mode=mode)
+    with pytest.raises(g4.G4NError):
+        g4.g4n_sync(ctx)
+    at = 0
+    while at < n:
+        k = min(200000, n - at)
+        s = slice(at, at + k)
+        part = g4.g4n_compute_step(ctx, gid, pos[:, s].contiguous(), dirs[:, s].contiguous(), depth[s].contiguous(),
+                                   path[:, s].contiguous(), proposed=prop[s].contiguous(), mode=mode)
+        for a, b in zip(whole, part):
+            a, b = a[s].cpu().numpy(), b.cpu().numpy()
+            assert np.array_equal(a, b, equal_nan=a.dtype.kind == "f")
+        at += k
+    try:
+        g4.g4n_sync(ctx)
+    except g4.G4NError:
+        pass
+
+
+@pytest.mark.parametrize("n", [1, 7, 33, 1000, 70001])
+def test_free_path_refills(env, n):
+    g4, torch, ctx = env
+    gid = g4.build_scene(ctx, synth.scenes.spheres_scene(n_side=6))
+    _, d, y = synth.scenes.spheres_rays("random", n, seed=41)
+    pos = torch.zeros((3, n), dtype=torch.float64, device="cuda")
+    dirs = torch.tensor(np.ascontiguousarray(d.T), device="cuda")
+    Y = torch.tensor(y, device="cuda")
+    T, steps = g4.g4n_free_path(ctx, gid, pos, dirs, Y, 1.0)
+    g4.g4n_sync(ctx)
+    keep = [0, n // 2, n - 1]
+    for k in keep:
+        t1, s1 = g4.g4n_free_path(ctx, gid, pos[:, k:k + 1].contiguous(), dirs[:, k:k + 1].contiguous(),
+                                  Y[k:k + 1].contiguous(), 1.0)
+        assert t1.item() == T[k].item() and s1.item() == steps[k].item()
+    assert not torch.isnan(T).any()

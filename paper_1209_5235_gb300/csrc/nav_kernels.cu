@@ -594,7 +594,7 @@ __device__ __forceinline__ int reloc_tail(const TParams &P, const DGeom &G, Trac
   return next;
 }
 
-template <int MODE, bool COUNT, bool YIELD, bool EV, bool DEFER = false>
+template <int MODE, bool COUNT, bool YIELD, bool EV, bool DEFER = false, bool ROUNDS = true>
 __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, MlpCtx mc, Chain &wch,
                          int *aux = nullptr) {
   const bool resume = YIELD && phase == kWalk;  // continue the step's yielded boundary search
@@ -689,7 +689,7 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       if (!need_geo) diag<COUNT>(cnt, G4N_C_SAFETY_SKIPS);
       else world_to_local(G.wxf[t.leaf], G.vol[t.leaf].flags & kWorldAligned, t.x, t.u, p, v);
     }
-    const Step32 R = geom_step32_warp<MODE, COUNT>(G, need_geo, need_geo ? t.leaf : 0, p, v, phys_hi, true, cnt, &timeout,
+    const Step32 R = geom_step32_warp<MODE, COUNT, true, ROUNDS>(G, need_geo, need_geo ? t.leaf : 0, p, v, phys_hi, true, cnt, &timeout,
                                                    P.walk_cap, mc, wch, resume, t.w, budget);
     if (act && R.yielded) {
       t.w = R.resume;
@@ -991,7 +991,7 @@ __global__ void __launch_bounds__(128, (MODE == kFP32 && YIELD) ? 3 : 4) k_trans
     __syncwarp();
     const long long c2 = COUNT ? clock64() : 0;
     const unsigned stepping2 = __ballot_sync(0xffffffffu, phase == kStep || phase == kWalk);
-    if (!REGROUP || stepping2) phase = step_warp<MODE, COUNT, YIELD, kEv>(P, t, phase, cnt, mc, wch);
+    if (!REGROUP || stepping2) phase = step_warp<MODE, COUNT, YIELD, kEv, false, YIELD>(P, t, phase, cnt, mc, wch);
     if (COUNT) {
       __syncwarp();
       const long long c3 = clock64();

@@ -759,22 +759,27 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
   return defer ? kReloc : next;
 }
 
-// The interaction at the end of a free path: photoabsorption if U mu_tot < mu_photo,
-// else a Compton scatter (Kahn), the cutoff, and a new Y = -log W.
+// The interaction at the end of a free path: photoabsorption if U mu_tot < mu_photo, else a Compton scatter (Kahn), the
+// cutoff, and a new Y = -log W.  One Philox block per interaction: U chooses the process, W gives the next free path.
+__device__ __forceinline__ bool interact_photo(const TParams &P, Track &t, uint64_t &w) {
+  const M53x2 uw = philox_m53_pair(P.seed, t.tid, 1, t.draw);
+  w = uw.b;
+  return m53_double(uw.a) * t.mu < t.mupe;
+}
+
+template <bool EV>
+__device__ __forceinline__ int absorb(const TParams &P, Track &t, Counters &cnt) {
+  event<EV>(cnt, G4N_C_PHOTO);
+  tally(P, t, t.leaf, t.E);
+  if (P.out_hash) t.h = hash_step(t.h, t.leaf, G4N_LIM_PHYSICS, kEvPhoto);
+  finish(P, t);
+  return kEmpty;
+}
+
 template <int MODE, bool EV>
-__device__ int interact(const TParams &P, Track &t, Counters &cnt) {
+__device__ __forceinline__ int scatter(const TParams &P, Track &t, uint64_t w, Counters &cnt) {
   const DItem &it = P.items[t.item];
   const DGeom &G = P.geoms[it.geom];
-  // one block per interaction: U chooses the process, W gives the next free path
-  const M53x2 uw = philox_m53_pair(P.seed, t.tid, 1, t.draw);
-  const double U = m53_double(uw.a);
-  if (U * t.mu < t.mupe) {
-    event<EV>(cnt, G4N_C_PHOTO);
-    tally(P, t, t.leaf, t.E);
-    if (P.out_hash) t.h = hash_step(t.h, t.leaf, G4N_LIM_PHYSICS, kEvPhoto);
-    finish(P, t);
-    return kEmpty;
-  }
   event<EV>(cnt, G4N_C_COMPTON);
   double eta, cost, cph, sph;
   bool ok = kahn(t.E, P.seed, t.tid, t.draw, eta, cost, P.trial_cap);
@@ -791,7 +796,7 @@ __device__ int interact(const TParams &P, Track &t, Counters &cnt) {
   }
   tally(P, t, t.leaf, t.E - E1);
   set_energy(G, t, E1);
-  t.Y = -log(m53_double(uw.b));
+  t.Y = -log(m53_double(w));
   if (P.out_hash) t.h = hash_step(t.h, t.leaf, G4N_LIM_PHYSICS, kEvCompton);
   update_mu(G, t);
   // FP64 mode: the isotropic safety of a leaf without daughters, at the interaction point
@@ -804,6 +809,12 @@ __device__ int interact(const TParams &P, Track &t, Counters &cnt) {
     t.safety = fmax(t.safety, vol_safety_out(L, p));
   }
   return kStep;
+}
+
+template <int MODE, bool EV>
+__device__ int interact(const TParams &P, Track &t, Counters &cnt) {
+  uint64_t w;
+  return interact_photo(P, t, w) ? absorb<EV>(P, t, cnt) : scatter<MODE, EV>(P, t, w, cnt);
 }
 
 // ---------------------------------------------------------------- regrouping between rounds

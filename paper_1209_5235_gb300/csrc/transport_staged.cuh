@@ -397,40 +397,88 @@ __global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const 
 // Finish kernel of the iteration: the interaction queue, then the admitted new tracks, all
 // written to bank ob.  Its last block ends the iteration: the queues just read are emptied, and it
 // decides the end of the batch or the hand-over of the last tracks to the drain kernel.
+//
+// A block takes tiles of 128 interactions.  Of each it first draws the processes, ends the absorbed tracks and lists the
+// scattered ones (their queue entries, in shared memory); whenever 128 are listed, or no more tiles come, their states are
+// loaded and they scatter, in full warps: FP64 work costs a warp the same for one lane as for 32, and about half of the
+// interactions are absorptions.  10^6 calorimeter tracks 5.21 -> 5.11 ms, barrel 10^7 62.5 -> 61.5 (FP64 mode 86.5 -> 84.8),
+// 2 10^5 nested barrel tracks 15.70 -> 15.62.
 template <int MODE>
 __global__ void __launch_bounds__(128, 4) k_staged_finish(const TParams P, const SgQueues Q, SgCtrl *C, int ib,
                                                            long long drain_tracks) {
   const SgWork &W = sg_work(C, ib);
-  const long long n_int = W.n_int, g0 = W.base, total = n_int + W.n_new;
-  const unsigned workers = sg_workers(total);
+  const long long n_int = W.n_int, n_new = W.n_new, g0 = W.base;
+  const long long t_int = (n_int + 127) >> 7, tiles = t_int + ((n_new + 127) >> 7);
+  const unsigned workers = sg_workers(tiles << 7);
   if (W.stop || blockIdx.x >= workers) return;
+  __shared__ unsigned list[256], n_list;
+  if (threadIdx.x == 0) n_list = 0;
   Counters cnt;
   sg_begin(cnt);
   const int ob = ib ^ 1;
   const bool want_slot = P.out_hash || P.out_len;
-  const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
+  const int tid = threadIdx.x;
+  int listed = 0;   // the same in every thread of the block
 #pragma unroll 1
-  for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w * 32 < total; w += nw) {
-    const long long i = w * 32 + (threadIdx.x & 31u);
-    const bool is_int = i < n_int, is_new = !is_int && i < total;
-    Track t;
-    t.item = 0;
-    t.leaf = 0;
-    int next = kEmpty;
-    if (is_int) {
-      sg_load<MODE>(Q, sg_entry(Q, kSgInteract, i), t);
-      if (want_slot) sg_restore_gidx(P, t);
-      next = interact<MODE, true>(P, t, cnt);
+  for (long long tile = blockIdx.x;; tile += gridDim.x) {
+    const bool drawing = tile < t_int;
+    if (drawing) {
+      const long long i = (tile << 7) + tid;
+      Track t;
+      bool absorbed = false, scattered = false;
+      if (i < n_int) {
+        sg_load<MODE>(Q, sg_entry(Q, kSgInteract, i), t);
+        uint64_t w;
+        absorbed = interact_photo(P, t, w);
+        scattered = !absorbed;
+        if (absorbed) {
+          if (want_slot) sg_restore_gidx(P, t);
+          absorb<true>(P, t, cnt);
+        }
+      }
+      const unsigned m = __ballot_sync(kFull, scattered);
+      unsigned at = 0;
+      if (m && (tid & 31) == 0) at = atomicAdd(&n_list, (unsigned)__popc(m));
+      at = __shfl_sync(kFull, at, 0);
+      if (scattered) list[at + __popc(m & ((1u << (tid & 31)) - 1u))] = (unsigned)i;
+      sg_retire(C, absorbed);
+      listed += __syncthreads_count(scattered);
     }
-    if (__any_sync(kFull, is_new)) {  // the source and the locate (warp-collective)
-      const int started = start_warp<MODE, false, true, MODE != kFP64>(P, is_new, g0 + (i - n_int), t, cnt);
-      if (is_new) next = started;
+    if (listed >= 128 || (!drawing && listed > 0)) {
+      const bool mine = tid < listed;
+      Track t;
+      t.item = 0;
+      t.leaf = 0;
+      int next = kEmpty;
+      if (mine) {
+        sg_load<MODE>(Q, sg_entry(Q, kSgInteract, list[tid]), t);
+        if (want_slot) sg_restore_gidx(P, t);
+        const M53x2 uw = philox_m53_pair(P.seed, t.tid, 1, t.draw);
+        next = scatter<MODE, true>(P, t, uw.b, cnt);
+      }
+      sg_push<MODE>(Q, C, mine && next == kStep, mine && next == kStep ? sg_queue_of(P, t, ob) : 0, t);
+      sg_retire(C, mine && next == kEmpty);
+      const int left = max(0, listed - 128);
+      const unsigned moved = tid < left ? list[128 + tid] : 0u;
+      __syncthreads();
+      if (tid < left) list[tid] = moved;
+      if (tid == 0) n_list = (unsigned)left;
+      listed = left;
+      __syncthreads();
     }
-    const bool mine = is_int || is_new;
-    sg_push<MODE>(Q, C, mine && next == kStep, mine && next == kStep ? sg_queue_of(P, t, ob) : 0, t);
-    sg_retire(C, mine && next == kEmpty);
+    if (!drawing && tile < tiles) {
+      const long long i = ((tile - t_int) << 7) + tid;
+      const bool is_new = i < n_new;
+      Track t;
+      t.item = 0;
+      t.leaf = 0;
+      const int next = start_warp<MODE, false, true, MODE != kFP64>(P, is_new, g0 + i, t, cnt);   // source and locate
+      sg_push<MODE>(Q, C, is_new && next == kStep, is_new && next == kStep ? sg_queue_of(P, t, ob) : 0, t);
+      sg_retire(C, is_new && next == kEmpty);
+    }
+    if (tile >= tiles && listed == 0) break;
   }
-  if (total > 0) sg_flush(P, cnt);
+  if (tiles > 0) sg_flush(P, cnt);
   if (sg_last_block(C, 1, workers) && threadIdx.x == 0) {
     volatile SgCtrl *V = C;
     V->cnt[kSgInteract] = 0;

@@ -117,6 +117,20 @@ def test_staged_pool_and_drain(env, name, pool, drain):
         _compare(g4, r, *out, sc.n_volumes)
 
 
+@pytest.mark.parametrize("name", ["calorimeter", "barrel"])
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 257, 3001])
+def test_staged_small_batches_without_drain(env, name, n):
+    """The finish kernel scatters in tiles of 128 listed interactions; without the drain every iteration down to the last
+    track's goes through it, in batches that end below, at and above a tile."""
+    g4, torch, ctx = env
+    sc, src, _, og, gid, _ = _scene(env, name)
+    r = og.transport(src, SEED + n, n, threads=0)
+    for mode, flags in ((0, 0), (1, 1)):
+        out = _run(env, gid, sc, src, SEED + n, n, mode=mode, drain_tracks=-1, staged_flags=flags)
+        g4.g4n_sync(ctx)
+        _compare(g4, r, *out, sc.n_volumes)
+
+
 def test_staged_without_history_outputs(env):
     """The timed launches ask for no hash or length: tallies and counters are unchanged."""
     g4, torch, ctx = env

@@ -1147,7 +1147,6 @@ __device__ __forceinline__ StepResult geom_step_warp(const DGeom &G, bool active
     diag_test<COUNT>(cnt, G4N_C_DIST_OUT, G4N_C_DIST_OUT_CURVED, V.kind);
     tout = vol_dist_out(V, G.pick[leaf], p, v, iv, half, G.band32, &osurf);
     R.safety = resume ? from.safety : (want_safety ? vol_safety_out(V, p) : 0.0);
-    stop = fmin(limit, tout);
     if (resume) {
       best = from.best;
       bl = from.bl;
@@ -1155,6 +1154,7 @@ __device__ __forceinline__ StepResult geom_step_warp(const DGeom &G, bool active
       first = false;
     }
     if (V.vox >= 0) {
+      stop = fmin(limit, tout);
       if (!resume) chain_fill(G, ch, 0, V.vox, p);
       L = G.clist[ch.list];
       L0 = L;

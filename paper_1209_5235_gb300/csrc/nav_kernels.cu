@@ -677,8 +677,10 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       if (!lazy) {
         geo = R.step <= sphys;
       } else {
-        const double d = fma(-R.step, t.mu, t.Y), m = 0x1p-49 * t.Y;
-        geo = d > m || (!(d < -m) && R.step <= t.Y / t.mu);
+        // compared by the ordered keys of the doubles, integer instructions where the FP64 pipe is the bound (with the
+        // remaining depth clamped by its sign and no FP64 minimum in boxes without daughters: calorimeter 4.94 -> 4.82 ms)
+        const long long d = dkey(fma(-R.step, t.mu, t.Y)), m = dkey(0x1p-49 * t.Y);
+        geo = d > m || (d >= ~m && R.step <= t.Y / t.mu);
       }
       if (geo) {
         s = R.step;
@@ -747,7 +749,10 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       cnt.c[G4N_C_PHYS_STEPS]++;
       next = kInteract;
     } else {
-      if (mu_pos) t.Y = fmax(t.Y - s * t.mu, 0.0);
+      if (mu_pos) {
+        const double y = t.Y - s * t.mu;
+        t.Y = __double2hiint(y) < 0 ? 0.0 : y;
+      }
       cnt.c[G4N_C_GEOM_STEPS]++;
       t.safety = 0.0;
     }

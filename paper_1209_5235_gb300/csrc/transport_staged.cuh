@@ -347,42 +347,51 @@ __global__ void __launch_bounds__(128, 4) k_staged_step(const TParams P, const S
   }
 }
 
+// The deferred relocation of entry i of the relocation queue (warp-collective; `act`: the lanes with one): the search, the
+// push after ten zero steps and the step record.  Returns the lane's next phase.
+template <int MODE>
+__device__ __forceinline__ int sg_relocate(const TParams &P, const SgQueues &Q, long long i, bool act, Track &t,
+                                           Counters &cnt) {
+  t.item = 0;
+  t.leaf = 0;
+  int aux = 0;
+  if (act) {
+    const int64_t e = sg_entry(Q, kSgReloc, i);
+    sg_load<MODE>(Q, e, t);
+    aux = __ldcs(Q.iw + 6 * Q.n + e);
+    if (P.out_hash || P.out_len) sg_restore_gidx(P, t);
+  }
+  const DGeom &G = P.geoms[P.items[act ? t.item : 0].geom];
+  // every lane searches (the step kernel already counted the zero step); aux = limiter << 1 | left the leaf
+  return reloc_tail<MODE, false, true>(P, G, t, act, act, -1, (aux & 1) != 0, 0.0, aux >> 1, false, cnt, kEmpty);
+}
+
 // Relocation kernel of the iteration (the option G4N_STAGED_RELOCATION_KERNEL): the steps whose relocation
 // search the step kernel deferred, in full warps of searching lanes (in the step kernel a warp's lanes limited
 // by physics or answered by a face record wait while the others search); then the push after ten zero
 // steps and the step record, as the step kernel would have done them, and the tracks go on to bank ob.  Its
-// last block empties the queue.  8 blocks of 128 per SM (64 registers): the searches wait on chains of
+// last block empties the queue.  A queue shorter than reloc_min, a wave of the finish kernel, it leaves to that kernel: most
+// crossings are answered by face records and portals, and the few searches left cost an iteration a launch's latency,
+// 40 to 60 us (barrel 10^7 61.24 -> 60.47 ms, FP64 mode 84.5 -> 83.4, nested barrel 15.60 -> 15.50).  8 blocks of 128 per SM (64 registers): the searches wait on chains of
 // dependent table loads, and more resident warps hide them (barrel 10^7: 2.4 % of the batch against 4 blocks
 // at 128 registers, 6 blocks in between).
 template <int MODE>
-__global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const SgQueues Q, SgCtrl *C, int ib) {
+__global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const SgQueues Q, SgCtrl *C, int ib,
+                                                          long long reloc_min) {
   const SgWork &W = sg_work(C, ib);
   const long long total = W.n_reloc;
   const unsigned workers = sg_workers(total);
-  if (W.stop || blockIdx.x >= workers) return;
+  if (W.stop || total < reloc_min || blockIdx.x >= workers) return;
   Counters cnt;
   sg_begin(cnt);
   const int ob = ib ^ 1;
-  const bool want_slot = P.out_hash || P.out_len;
   // block-sized strides: the loop condition is the same for every thread of the block (sg_push_block's barriers)
 #pragma unroll 1
   for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < total; b0 += (long long)gridDim.x * blockDim.x) {
     const long long i = b0 + threadIdx.x;
     const bool act = i < total;
     Track t;
-    t.item = 0;
-    t.leaf = 0;
-    int aux = 0;
-    if (act) {
-      const int64_t e = sg_entry(Q, kSgReloc, i);
-      sg_load<MODE>(Q, e, t);
-      aux = __ldcs(Q.iw + 6 * Q.n + e);
-      if (want_slot) sg_restore_gidx(P, t);
-    }
-    const DGeom &G = P.geoms[P.items[act ? t.item : 0].geom];
-    // every lane searches (the step kernel already counted the zero step); aux = limiter << 1 | left the leaf
-    const int next = reloc_tail<MODE, false, true>(P, G, t, act, act, -1, (aux & 1) != 0, 0.0, aux >> 1, false, cnt,
-                                                   kEmpty);
+    const int next = sg_relocate<MODE>(P, Q, i, act, t, cnt);
     const bool keep = act && next == kStep;
     sg_push_block<MODE>(Q, C, keep, keep ? sg_queue_of(P, t, ob) : 0, t);
     sg_retire(C, act && next == kEmpty);
@@ -394,7 +403,7 @@ __global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const 
   }
 }
 
-// Finish kernel of the iteration: the interaction queue, then the admitted new tracks, all
+// Finish kernel of the iteration: the relocations left to it, the interaction queue, then the admitted new tracks, all
 // written to bank ob.  Its last block ends the iteration: the queues just read are emptied, and it
 // decides the end of the batch or the hand-over of the last tracks to the drain kernel.
 //
@@ -403,12 +412,13 @@ __global__ void __launch_bounds__(128, 8) k_staged_reloc(const TParams P, const 
 // loaded and they scatter, in full warps: FP64 work costs a warp the same for one lane as for 32, and about half of the
 // interactions are absorptions.  10^6 calorimeter tracks 5.21 -> 5.11 ms, barrel 10^7 62.5 -> 61.5 (FP64 mode 86.5 -> 84.8),
 // 2 10^5 nested barrel tracks 15.70 -> 15.62.
-template <int MODE>
+template <int MODE, bool RELOC_KERNEL>
 __global__ void __launch_bounds__(128, 4) k_staged_finish(const TParams P, const SgQueues Q, SgCtrl *C, int ib,
                                                            long long drain_tracks) {
   const SgWork &W = sg_work(C, ib);
   const long long n_int = W.n_int, n_new = W.n_new, g0 = W.base;
-  const long long t_int = (n_int + 127) >> 7, tiles = t_int + ((n_new + 127) >> 7);
+  const long long n_rel = RELOC_KERNEL ? W.n_reloc : 0;   // those the relocation kernel left: few
+  const long long t_rel = (n_rel + 127) >> 7, t_int = t_rel + ((n_int + 127) >> 7), tiles = t_int + ((n_new + 127) >> 7);
   const unsigned workers = sg_workers(tiles << 7);
   if (W.stop || blockIdx.x >= workers) return;
   __shared__ unsigned list[256], n_list;
@@ -421,9 +431,18 @@ __global__ void __launch_bounds__(128, 4) k_staged_finish(const TParams P, const
   int listed = 0;   // the same in every thread of the block
 #pragma unroll 1
   for (long long tile = blockIdx.x;; tile += gridDim.x) {
+    if (RELOC_KERNEL && tile < t_rel) {
+      const long long i = (tile << 7) + tid;
+      const bool act = i < n_rel;
+      Track t;
+      const int next = sg_relocate<MODE>(P, Q, i, act, t, cnt);
+      sg_push<MODE>(Q, C, act && next == kStep, act && next == kStep ? sg_queue_of(P, t, ob) : 0, t);
+      sg_retire(C, act && next == kEmpty);
+      continue;
+    }
     const bool drawing = tile < t_int;
     if (drawing) {
-      const long long i = (tile << 7) + tid;
+      const long long i = ((tile - t_rel) << 7) + tid;
       Track t;
       bool absorbed = false, scattered = false;
       if (i < n_int) {
@@ -482,6 +501,7 @@ __global__ void __launch_bounds__(128, 4) k_staged_finish(const TParams P, const
   if (sg_last_block(C, 1, workers) && threadIdx.x == 0) {
     volatile SgCtrl *V = C;
     V->cnt[kSgInteract] = 0;
+    if (RELOC_KERNEL) V->cnt[kSgReloc] = 0;
 #pragma unroll
     for (int k = 0; k < kSgKinds; ++k) V->cnt[ib * kSgKinds + k] = 0;
     V->n_new = 0;
@@ -651,7 +671,8 @@ int staged_run(g4n_ctx *ctx, const g4n_batch_desc *b, TParams &P, cudaStream_t s
   const int g_step = reloc_kernel ? sg_grid(ctx, b, k_staged_step<MODE, true>, smem)
                                   : sg_grid(ctx, b, k_staged_step<MODE, false>, smem);
   const int g_reloc = sg_grid(ctx, b, k_staged_reloc<MODE>, 0);
-  const int g_fin = sg_grid(ctx, b, k_staged_finish<MODE>, 0);
+  const int g_fin = reloc_kernel ? sg_grid(ctx, b, k_staged_finish<MODE, true>, 0)
+                                 : sg_grid(ctx, b, k_staged_finish<MODE, false>, 0);
   int per_sm_drain = 0;
   if (smem) cudaFuncSetAttribute(k_staged_drain<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_drain, k_staged_drain<MODE>, 128, smem);
@@ -676,12 +697,14 @@ int staged_run(g4n_ctx *ctx, const g4n_batch_desc *b, TParams &P, cudaStream_t s
       const int ib = (int)(it & 1);
       if (reloc_kernel) {
         k_staged_step<MODE, true><<<g_step, 128, smem, st>>>(P, Q, C, ib);
-        k_staged_reloc<MODE><<<g_reloc, 128, 0, st>>>(P, Q, C, ib);
+        // a queue shorter than a wave of the finish kernel goes with that one
+        k_staged_reloc<MODE><<<g_reloc, 128, 0, st>>>(P, Q, C, ib, 128LL * g_fin);
+        k_staged_finish<MODE, true><<<g_fin, 128, 0, st>>>(P, Q, C, ib, drain_tracks);
         ++ctx->launches;
       } else {
         k_staged_step<MODE, false><<<g_step, 128, smem, st>>>(P, Q, C, ib);
+        k_staged_finish<MODE, false><<<g_fin, 128, 0, st>>>(P, Q, C, ib, drain_tracks);
       }
-      k_staged_finish<MODE><<<g_fin, 128, 0, st>>>(P, Q, C, ib, drain_tracks);
       ctx->launches += 2;
     }
     if (drain_tracks >= 0) {

@@ -55,6 +55,28 @@ __device__ __forceinline__ void mma_bf16(float &d0, float &d1, float &d2, float 
 
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
 
+// GELU for outputs that are rounded to BF16: max(x, 0) - |x| tail(|x|), the normal distribution's tail as 2^P with P of
+// degree 10, fitted to its logarithm on [0, 13] (least squares, reweighted towards equal errors of y tail(y): 3e-10) and
+// decreasing beyond.  No branches, 16 instructions, about half of the erf form's, and closer to 64 bits: largest error on
+// [-10, 10] 2.4e-7, root mean square 4.6e-8 (erf form 4.9e-7, 6.4e-8), on [-1, 1] 5.9e-8, 1.2e-8 (8.2e-8, 1.3e-8).
+// Stack of plates 13.25 -> 12.67 ms.
+__device__ __forceinline__ float gelu16(float x) {
+  const float y = fabsf(x);
+  float p = -5.68980263e-08f;
+  p = fmaf(p, y, 1.40031331e-06f);
+  p = fmaf(p, y, -1.52829445e-05f);
+  p = fmaf(p, y, 9.4810299e-05f);
+  p = fmaf(p, y, -0.000324589254f);
+  p = fmaf(p, y, 6.37534364e-05f);
+  p = fmaf(p, y, 0.00689659362f);
+  p = fmaf(p, y, -0.0524214247f);
+  p = fmaf(p, y, -0.459223877f);
+  p = fmaf(p, y, -1.15110412f);
+  p = fmaf(p, y, -1.0f);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(p));
+  return fmaf(-fminf(y, 3e38f), p, fmaxf(x, 0.f));
+}
+
 // Four 8 x 8 BF16 matrices; lane i gives the address of row i & 7 of matrix i >> 3.
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16 *p) {
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
@@ -63,7 +85,7 @@ __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16 *p) 
 }
 
 __device__ __forceinline__ uint32_t gelu_pair(float x, float y) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(gelu(x), gelu(y));
+  const __nv_bfloat162 h = __floats2bfloat162_rn(gelu16(x), gelu16(y));
   return *reinterpret_cast<const uint32_t *>(&h);
 }
 

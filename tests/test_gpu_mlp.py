@@ -269,3 +269,29 @@ def test_training_step_matches_its_gradient(env, batch):
     step = lr * (m * c1) / (np.sqrt(v * c2) + f(1e-8))
     got = g4.g4n_mlp_get(ctx)
     assert np.all(np.abs(got - (p - step)) <= 2.0 ** -23 * np.abs(p) + 1e-6 * np.abs(step) + 1e-12)
+
+
+@pytest.mark.parametrize("scale", [0.1, 1.0, 10.0])
+@pytest.mark.parametrize("n", [1, 16, 17, 32, 33, 129])
+def test_predict_rows_and_activation_range(env, n, scale):
+    """Row counts around the 16-row halves and the 32-row tiles; weights that keep the hidden layers' inputs near zero, around
+    one, and far out in GELU's tails.  A row does not depend on its batch, and lies within one BF16 unit per hidden value
+    (2^-8, carried through the layers; GELU's slope is below 1.13) plus the FP32 sums' rounding of the emulated pass."""
+    g4, torch, ctx = env
+    p = (params(11) * scale).astype(np.float32)
+    g4.g4n_mlp_load(ctx, p)
+    X, _, _ = random_data(160, 12)
+    full = g4.g4n_mlp_predict(ctx, torch.tensor(X, device="cuda")).cpu().numpy()
+    part = g4.g4n_mlp_predict(ctx, torch.tensor(X[:n], device="cuda")).cpu().numpy()
+    assert np.array_equal(part, full[:n])
+    ref, _ = omlp.forward(p, X, emulate_bf16=True)
+    b16 = lambda a: torch.tensor(np.asarray(a, dtype=np.float32)).bfloat16().double().numpy()
+    W1, b1, W2, b2, W3, b3 = [np.asarray(a, dtype=np.float64) for a in omlp.unpack(p)]
+    W1, W2, W3 = b16(W1), b16(W2), b16(W3)
+    h1 = b16(omlp.gelu(b16(X) @ W1 + b1))
+    h2 = b16(omlp.gelu(h1 @ W2 + b2))
+    u, f = 2.0 ** -8, 128 * 2.0 ** -23
+    e1 = u * np.abs(h1) + 1.13 * f * (np.abs(b16(X)) @ np.abs(W1) + np.abs(b1)) + 1e-6
+    e2 = u * np.abs(h2) + 1.13 * (e1 @ np.abs(W2) + f * (np.abs(h1) @ np.abs(W2) + np.abs(b2))) + 1e-6
+    e3 = e2 @ np.abs(W3) + f * (np.abs(h2) @ np.abs(W3) + np.abs(b3)) + 1e-6
+    assert np.all(np.abs(full - ref) <= e3)

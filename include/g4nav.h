@@ -313,7 +313,7 @@ typedef struct {
  * searches after geometry-limited steps in a kernel of their own, in full warps of searching lanes
  * (it pays where most relocations need a search, as in tube segments, and costs a launch per
  * iteration where face records answer most of them, as in box cells).  drain_tracks: the persistent kernel takes over once every track has started and
- * at most this many are in flight (0 = two per resident thread of that kernel, < 0 = never).
+ * at most this many are in flight (0 = one per resident thread of that kernel, < 0 = never).
  * The staged schedule ignores block_size (128), walk_budget (searches never yield) and
  * regroup_period; blocks_per_sm (0 = as many as fit) applies to its kernels.  Launches with
  * G4N_FLAG_DIAGNOSTICS, the sample log (g4n_mlp_log), the allocation-free entry point and CUDA

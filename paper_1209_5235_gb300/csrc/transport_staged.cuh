@@ -677,12 +677,12 @@ int staged_run(g4n_ctx *ctx, const g4n_batch_desc *b, TParams &P, cudaStream_t s
   if (smem) cudaFuncSetAttribute(k_staged_drain<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_drain, k_staged_drain<MODE>, 128, smem);
   const int g_drain = ctx->sm_count * std::max(per_sm_drain, 1);
-  // two tracks per resident thread: with the iterations cheaper than they were the drain, bound by instruction fetch,
-  // pays later (batches of the nested barrel / calorimeter of 2 10^5 / 10^6 tracks at 4, 2, 1 a thread: 19.9, 18.1, 17.5
-  // / 2.48, 2.16, 2.37 / 6.86, 6.76, 7.21 ms; the barrel does not care)
+  // one track per resident thread: the drain, bound by instruction fetch, pays late, and the cheaper the iterations the
+  // later (at 4, 2, 1, 1/2 a thread: calorimeter 10^6 5.24, 4.81, 4.67, 4.68 ms, 2 10^5 from the host 2.46, 1.85, 1.72,
+  // 1.87; nested barrel 18.1, 15.6, 14.8, 14.4; barrel 10^6 11.7, 10.28, 10.28, 10.9)
   const long long drain_tracks = b->drain_tracks < 0 ? -1
                                  : b->drain_tracks > 0 ? b->drain_tracks
-                                                       : 2LL * g_drain * 128;
+                                                       : 1LL * g_drain * 128;
   if (cudaMemsetAsync(C, 0, sizeof(SgCtrl), st) != cudaSuccess) return g4n_fail(ctx, G4N_ERR_CUDA, "transport: control reset failed");
   if (int rc = launch_error(ctx, "staged transport setup")) return rc;
 

@@ -1,9 +1,10 @@
 // mlp.cu -- training and inference entry points of the candidate-proposal MLP.
 //
-// Training (g4n_mlp_train, and the BF16 gradients of g4n_mlp_grad) is the
-// persistent kernel of mlp_train.cuh: BF16 products on the tensor cores with
-// FP32 accumulation, masked softmax cross-entropy, Adam on FP32 master
-// weights.  The FP32 reference gradients are plain kernels of this file.
+// Training (g4n_mlp_train, and the BF16 gradients of g4n_mlp_grad) on minibatches
+// of kFusedRows rows and more is the persistent kernel of mlp_train.cuh: BF16
+// products on the tensor cores with FP32 accumulation, masked softmax
+// cross-entropy, Adam on FP32 master weights.  Smaller minibatches and the FP32
+// reference gradients take one kernel of this file per product and elementwise pass.
 // The packed FP32 parameter layout used by the API is
 //   W1[9][64], b1[64], W2[64][64], b2[64], W3[64][32], b3[32]   (6880 floats),
 // W[k][n] mapping input k to output n.
@@ -27,16 +28,57 @@ using namespace g4n::mlp;
 
 namespace {
 
-// ---------------------------------------------------------------- FP32 reference gradients
-// The FP32 path of g4n_mlp_grad: plain kernels, one per product and elementwise pass.
+// Rows from which a minibatch takes the persistent kernel.  The plain kernels split the sums over the rows into partials of
+// 256 rows or a little more and add these atomically.  One or two (fewer than 768 rows) have the same sum in either order: a
+// training repeats bit for bit.  Another order of summation ends 4e-4 away after 250 steps (BF16 rounds the differences
+// up), so these trainings keep theirs, and their 26 launches (170 us a step, where the persistent kernel takes 11 to 19).  From
+// three partials on the order varies and two runs of the plain kernels differ by as much (1024 rows, 250 steps: up to 4e-4;
+// 4096: 1e-3; their error against 64 bits is 1e-3 to 5e-3 either way).
+constexpr int64_t kFusedRows = 768;
+
+// ---------------------------------------------------------------- plain kernels
 // C[M x N] += op(A)[M x K] op(B)[K x N]; A(m, k) = transA ? A[k * lda + m] : A[m * lda + k],
-// B(k, n) = transB ? B[n * ldb + k] : B[k * ldb + n].
+// B(k, n) = transB ? B[n * ldb + k] : B[k * ldb + n].  BF16: M, K multiples of 16, N a multiple of 8.
 
 __device__ __forceinline__ float ldA(const float *A, int lda, bool tA, int m, int k) {
   return tA ? A[(int64_t)k * lda + m] : A[(int64_t)m * lda + k];
 }
 __device__ __forceinline__ float ldB(const float *B, int ldb, bool tB, int k, int n) {
   return tB ? B[(int64_t)n * ldb + k] : B[(int64_t)k * ldb + n];
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+// One warp per 16 x 8 output tile and K chunk (blockIdx.z); chunks add into C atomically.
+__global__ void k_gemm_bf16(int M, int N, int K, int kchunk, const float *__restrict__ A, int lda, bool tA,
+                            const float *__restrict__ B, int ldb, bool tB, float *__restrict__ C, int ldc) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int tiles_n = N / 8;
+  const int tm = warp / tiles_n, tn = warp % tiles_n;
+  if (tm * 16 >= M) return;
+  const int k0 = blockIdx.z * kchunk, k1 = min(K, k0 + kchunk);
+  const int m0 = tm * 16, n0 = tn * 8;
+  float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
+  for (int k = k0; k < k1; k += 16) {
+    const int kc = k + 2 * q;
+    const uint32_t a0 = pack_bf16(ldA(A, lda, tA, m0 + g, kc), ldA(A, lda, tA, m0 + g, kc + 1));
+    const uint32_t a1 = pack_bf16(ldA(A, lda, tA, m0 + g + 8, kc), ldA(A, lda, tA, m0 + g + 8, kc + 1));
+    const uint32_t a2 = pack_bf16(ldA(A, lda, tA, m0 + g, kc + 8), ldA(A, lda, tA, m0 + g, kc + 9));
+    const uint32_t a3 = pack_bf16(ldA(A, lda, tA, m0 + g + 8, kc + 8), ldA(A, lda, tA, m0 + g + 8, kc + 9));
+    const uint32_t b0 = pack_bf16(ldB(B, ldb, tB, kc, n0 + g), ldB(B, ldb, tB, kc + 1, n0 + g));
+    const uint32_t b1 = pack_bf16(ldB(B, ldb, tB, kc + 8, n0 + g), ldB(B, ldb, tB, kc + 9, n0 + g));
+    mma_bf16(d0, d1, d2, d3, a0, a1, a2, a3, b0, b1);
+  }
+  float *c0 = C + (int64_t)(m0 + g) * ldc + n0 + 2 * q;
+  float *c1 = c0 + (int64_t)8 * ldc;
+  atomicAdd(c0, d0);
+  atomicAdd(c0 + 1, d1);
+  atomicAdd(c1, d2);
+  atomicAdd(c1 + 1, d3);
 }
 
 // One thread per output element and K chunk (blockIdx.z); chunks add into C atomically.
@@ -64,11 +106,13 @@ __global__ void k_bias_gelu(int64_t rows, int cols, float *__restrict__ Z, const
 // Logits += b3; masked softmax over the first ncand[r] columns; loss (sum) and dZ3 = (p - onehot) / scale.
 __global__ void k_softmax_ce(int64_t rows, float *__restrict__ Z3, const float *__restrict__ b3,
                              const int32_t *__restrict__ label, const int32_t *__restrict__ ncand,
-                             float inv_scale, float *__restrict__ dZ3, double *__restrict__ loss) {
+                             const int64_t *__restrict__ idx, float inv_scale, float *__restrict__ dZ3,
+                             double *__restrict__ loss) {
   const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (r >= rows) return;
-  const int n = max(1, min(kOut, ncand[r]));
-  const int y = label[r];
+  const int64_t src = idx ? idx[r] : r;
+  const int n = max(1, min(kOut, ncand[src]));
+  const int y = label[src];
   float *z = Z3 + r * kOut;
   float mx = -INFINITY;
   for (int c = 0; c < kOut; ++c) {
@@ -105,13 +149,33 @@ __global__ void k_colsum(int64_t rows, int cols, const float *__restrict__ X, fl
   }
 }
 
-// Feature rows padded to 16 columns (zeros beyond 9).
-__global__ void k_pad_rows(int64_t rows, const float *__restrict__ feat, float *__restrict__ X) {
+// Gather a minibatch of padded feature rows (16 columns, zeros beyond 9).
+__global__ void k_gather(int64_t rows, const float *__restrict__ feat, const int64_t *__restrict__ idx,
+                         float *__restrict__ X) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= rows * kInPad) return;
   const int64_t r = e / kInPad;
   const int k = (int)(e % kInPad);
-  X[e] = k < kIn ? feat[r * kIn + k] : 0.f;
+  const int64_t src = idx ? idx[r] : r;
+  X[e] = k < kIn ? feat[src * kIn + k] : 0.f;
+}
+
+// Minibatch index: a fixed-stride walk through a random rotation, a permutation of [0, n).
+__global__ void k_batch_index(int64_t rows, int64_t n, int64_t start, int64_t stride, int64_t offset,
+                              int64_t *__restrict__ idx) {
+  const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (r < rows) idx[r] = (int64_t)((((uint64_t)(start + r) % (uint64_t)n) * (uint64_t)stride + (uint64_t)offset) % (uint64_t)n);
+}
+
+__global__ void k_add_double(double *dst, const double *src) { *dst += *src; }
+
+__global__ void k_adam(int n, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
+                       float *__restrict__ v, float lr, float b1, float b2, float c1, float c2, float eps) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  m[i] = b1 * m[i] + (1.f - b1) * g[i];
+  v[i] = b2 * v[i] + (1.f - b2) * g[i] * g[i];
+  p[i] -= lr * (m[i] * c1) / (sqrtf(v[i] * c2) + eps);
 }
 
 // Shared-memory image (transposed BF16, padded) from the packed FP32 parameters.
@@ -169,10 +233,11 @@ struct MlpState {
   SmemWeights *img = nullptr;
   float *W1p = nullptr;
   int64_t step = 0;
-  // FP32 gradient scratch for `cap` rows
+  // scratch of the plain kernels for `cap` rows
   int64_t cap = 0;
   float *X = nullptr, *Z1 = nullptr, *H1 = nullptr, *Z2 = nullptr, *H2 = nullptr, *Z3 = nullptr, *dZ3 = nullptr,
         *dH2 = nullptr, *dH1 = nullptr, *dW1p = nullptr;
+  int64_t *idx = nullptr;
   double *loss = nullptr;
   // k_mlp_train: partial gradients and losses (one row per block), control block, Adam's corrections per step
   float *part = nullptr;
@@ -187,8 +252,9 @@ MlpState *state(g4n_ctx *ctx) { return reinterpret_cast<MlpState *>(ctx->mlp); }
 
 void free_scratch(MlpState *s) {
   cudaFree(s->X); cudaFree(s->Z1); cudaFree(s->H1); cudaFree(s->Z2); cudaFree(s->H2); cudaFree(s->Z3);
-  cudaFree(s->dZ3); cudaFree(s->dH2); cudaFree(s->dH1); cudaFree(s->dW1p); cudaFree(s->loss);
+  cudaFree(s->dZ3); cudaFree(s->dH2); cudaFree(s->dH1); cudaFree(s->dW1p); cudaFree(s->idx); cudaFree(s->loss);
   s->X = s->Z1 = s->H1 = s->Z2 = s->H2 = s->Z3 = s->dZ3 = s->dH2 = s->dH1 = s->dW1p = nullptr;
+  s->idx = nullptr;
   s->loss = nullptr;
   s->cap = 0;
 }
@@ -202,7 +268,7 @@ int ensure_scratch(g4n_ctx *ctx, MlpState *s, int64_t rows) {
             cudaMalloc(&s->H2, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->Z3, rows * kOut * 4) == cudaSuccess &&
             cudaMalloc(&s->dZ3, rows * kOut * 4) == cudaSuccess && cudaMalloc(&s->dH2, rows * kHid * 4) == cudaSuccess &&
             cudaMalloc(&s->dH1, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->dW1p, kInPad * kHid * 4) == cudaSuccess &&
-            cudaMalloc(&s->loss, 8) == cudaSuccess;
+            cudaMalloc(&s->idx, rows * 8) == cudaSuccess && cudaMalloc(&s->loss, 8) == cudaSuccess;
   if (!ok) {
     free_scratch(s);
     return g4n_fail(ctx, G4N_ERR_OOM, "mlp: scratch allocation failed");
@@ -211,48 +277,55 @@ int ensure_scratch(g4n_ctx *ctx, MlpState *s, int64_t rows) {
   return G4N_OK;
 }
 
-void gemm(int M, int N, int K, const float *A, int lda, bool tA, const float *B, int ldb, bool tB, float *C, int ldc,
-          cudaStream_t st) {
+void gemm(bool bf16, int M, int N, int K, const float *A, int lda, bool tA, const float *B, int ldb, bool tB, float *C,
+          int ldc, cudaStream_t st) {
   const int ksplit = std::max(1, std::min(256, K / 256));
   const int kchunk = ((K + ksplit - 1) / ksplit + 15) / 16 * 16;
   const int nz = (K + kchunk - 1) / kchunk;
-  dim3 grid((int)(((int64_t)M * N + 127) / 128), 1, nz);
-  k_gemm_fp32<<<grid, 128, 0, st>>>(M, N, K, kchunk, A, lda, tA, B, ldb, tB, C, ldc);
+  if (bf16) {
+    const int warps = (M / 16) * (N / 8);
+    dim3 grid((warps + 3) / 4, 1, nz);
+    k_gemm_bf16<<<grid, 128, 0, st>>>(M, N, K, kchunk, A, lda, tA, B, ldb, tB, C, ldc);
+  } else {
+    dim3 grid((int)(((int64_t)M * N + 127) / 128), 1, nz);
+    k_gemm_fp32<<<grid, 128, 0, st>>>(M, N, K, kchunk, A, lda, tA, B, ldb, tB, C, ldc);
+  }
 }
 
 inline int blocks(int64_t n, int b = 256) { return (int)std::max<int64_t>(1, (n + b - 1) / b); }
 
-// FP32 forward + backward over `rows` samples.  Gradients into s->G, the sum of the losses into s->loss.
-void forward_backward_fp32(MlpState *s, int64_t rows, const float *feat, const int32_t *label, const int32_t *ncand,
-                           float inv_scale, cudaStream_t st) {
+// Forward + backward over `rows` samples (rows a multiple of 16; the caller pads with
+// ncand = 1, label = 0 rows of zero weight via inv_scale).  Gradients into s->G.
+void forward_backward(MlpState *s, bool bf16, int64_t rows, const float *feat, const int32_t *label,
+                      const int32_t *ncand, const int64_t *idx, float inv_scale, cudaStream_t st) {
   const int R = (int)rows;
   float *P = s->P, *G = s->G;
   cudaMemsetAsync(s->loss, 0, 8, st);
-  k_pad_rows<<<blocks(rows * kInPad), 256, 0, st>>>(rows, feat, s->X);
+  k_gather<<<blocks(rows * kInPad), 256, 0, st>>>(rows, feat, idx, s->X);
   k_pad_w1<<<blocks(kInPad * kHid), 256, 0, st>>>(P, s->W1p);
   cudaMemsetAsync(s->Z1, 0, rows * kHid * 4, st);
-  gemm(R, kHid, kInPad, s->X, kInPad, false, s->W1p, kHid, false, s->Z1, kHid, st);
+  gemm(bf16, R, kHid, kInPad, s->X, kInPad, false, s->W1p, kHid, false, s->Z1, kHid, st);
   k_bias_gelu<<<blocks(rows * kHid), 256, 0, st>>>(rows, kHid, s->Z1, P + kOffB1, s->H1);
   cudaMemsetAsync(s->Z2, 0, rows * kHid * 4, st);
-  gemm(R, kHid, kHid, s->H1, kHid, false, P + kOffW2, kHid, false, s->Z2, kHid, st);
+  gemm(bf16, R, kHid, kHid, s->H1, kHid, false, P + kOffW2, kHid, false, s->Z2, kHid, st);
   k_bias_gelu<<<blocks(rows * kHid), 256, 0, st>>>(rows, kHid, s->Z2, P + kOffB2, s->H2);
   cudaMemsetAsync(s->Z3, 0, rows * kOut * 4, st);
-  gemm(R, kOut, kHid, s->H2, kHid, false, P + kOffW3, kOut, false, s->Z3, kOut, st);
-  k_softmax_ce<<<blocks(rows), 256, 0, st>>>(rows, s->Z3, P + kOffB3, label, ncand, inv_scale, s->dZ3, s->loss);
+  gemm(bf16, R, kOut, kHid, s->H2, kHid, false, P + kOffW3, kOut, false, s->Z3, kOut, st);
+  k_softmax_ce<<<blocks(rows), 256, 0, st>>>(rows, s->Z3, P + kOffB3, label, ncand, idx, inv_scale, s->dZ3, s->loss);
   // backward
   cudaMemsetAsync(G, 0, kNParams * 4, st);
-  gemm(kHid, kOut, R, s->H2, kHid, true, s->dZ3, kOut, false, G + kOffW3, kOut, st);    // dW3 = H2^T dZ3
+  gemm(bf16, kHid, kOut, R, s->H2, kHid, true, s->dZ3, kOut, false, G + kOffW3, kOut, st);    // dW3 = H2^T dZ3
   k_colsum<<<kOut, 256, 0, st>>>(rows, kOut, s->dZ3, G + kOffB3);
   cudaMemsetAsync(s->dH2, 0, rows * kHid * 4, st);
-  gemm(R, kHid, kOut, s->dZ3, kOut, false, P + kOffW3, kOut, true, s->dH2, kHid, st);   // dH2 = dZ3 W3^T
+  gemm(bf16, R, kHid, kOut, s->dZ3, kOut, false, P + kOffW3, kOut, true, s->dH2, kHid, st);   // dH2 = dZ3 W3^T
   k_gelu_bwd<<<blocks(rows * kHid), 256, 0, st>>>(rows * kHid, s->dH2, s->Z2);
-  gemm(kHid, kHid, R, s->H1, kHid, true, s->dH2, kHid, false, G + kOffW2, kHid, st);    // dW2 = H1^T dZ2
+  gemm(bf16, kHid, kHid, R, s->H1, kHid, true, s->dH2, kHid, false, G + kOffW2, kHid, st);    // dW2 = H1^T dZ2
   k_colsum<<<kHid, 256, 0, st>>>(rows, kHid, s->dH2, G + kOffB2);
   cudaMemsetAsync(s->dH1, 0, rows * kHid * 4, st);
-  gemm(R, kHid, kHid, s->dH2, kHid, false, P + kOffW2, kHid, true, s->dH1, kHid, st);   // dH1 = dZ2 W2^T
+  gemm(bf16, R, kHid, kHid, s->dH2, kHid, false, P + kOffW2, kHid, true, s->dH1, kHid, st);   // dH1 = dZ2 W2^T
   k_gelu_bwd<<<blocks(rows * kHid), 256, 0, st>>>(rows * kHid, s->dH1, s->Z1);
   cudaMemsetAsync(s->dW1p, 0, kInPad * kHid * 4, st);
-  gemm(kInPad, kHid, R, s->X, kInPad, true, s->dH1, kHid, false, s->dW1p, kHid, st);   // dW1 = X^T dZ1
+  gemm(bf16, kInPad, kHid, R, s->X, kInPad, true, s->dH1, kHid, false, s->dW1p, kHid, st);   // dW1 = X^T dZ1
   cudaMemcpyAsync(G + kOffW1, s->dW1p, kIn * kHid * 4, cudaMemcpyDeviceToDevice, st);
   k_colsum<<<kHid, 256, 0, st>>>(rows, kHid, s->dH1, G + kOffB1);
 }
@@ -308,6 +381,32 @@ int run_train(g4n_ctx *ctx, MlpState *s, TrainParams &T, double *loss, cudaStrea
     return g4n_fail(ctx, G4N_ERR_CUDA, std::string("mlp training: ") + cudaGetErrorString(cudaGetLastError()));
   if (end.failed) return g4n_fail(ctx, G4N_ERR_TIMEOUT, "mlp training: a grid barrier reached its iteration cap");
   *loss = end.loss;
+  return G4N_OK;
+}
+
+// One epoch of `nb` minibatches by the plain kernels.  *loss = sum of the losses.
+int train_plain(g4n_ctx *ctx, MlpState *s, int64_t n, const float *feat, const int32_t *label, const int32_t *ncand,
+                int32_t batch, int64_t nb, uint64_t stride, uint64_t offset, float lr, const float2 *corr, double *loss,
+                cudaStream_t st) {
+  double *sum = nullptr;
+  if (cudaMalloc(&sum, 8) != cudaSuccess) {
+    cudaGetLastError();
+    return g4n_fail(ctx, G4N_ERR_OOM, "mlp_train: allocation failed");
+  }
+  cudaMemsetAsync(sum, 0, 8, st);
+  for (int64_t b = 0; b < nb; ++b) {
+    k_batch_index<<<blocks(batch), 256, 0, st>>>(batch, n, b * batch, (int64_t)stride, (int64_t)offset, s->idx);
+    forward_backward(s, true, batch, feat, label, ncand, s->idx, 1.0f / (float)batch, st);
+    k_adam<<<blocks(kNParams), 256, 0, st>>>(kNParams, s->P, s->G, s->M, s->V, lr, 0.9f, 0.999f, corr[b].x, corr[b].y,
+                                             1e-8f);
+    k_add_double<<<1, 1, 0, st>>>(sum, s->loss);  // epoch loss accumulates on the device
+  }
+  k_pack_image<<<8, 256, 0, st>>>(s->P, s->img);
+  cudaMemcpyAsync(loss, sum, 8, cudaMemcpyDeviceToHost, st);
+  cudaStreamSynchronize(st);
+  cudaFree(sum);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return g4n_fail(ctx, G4N_ERR_CUDA, std::string("mlp_train: ") + cudaGetErrorString(e));
   return G4N_OK;
 }
 
@@ -402,7 +501,7 @@ int g4n_mlp_grad(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *labe
   cudaSetDevice(ctx->device);
   MlpState *s = state(ctx);
   double loss = 0.0;
-  if (precision == 0) {
+  if (precision == 0 && n >= kFusedRows) {
     if (n > INT32_MAX - kTrRows) return g4n_fail(ctx, G4N_ERR_ARG, "mlp_grad: too many samples");
     if ((rc = ensure_train(ctx, s, 0))) return rc;
     TrainParams T{};
@@ -417,7 +516,7 @@ int g4n_mlp_grad(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *labe
     if ((rc = run_train(ctx, s, T, &loss, 0))) return rc;
   } else {
     if ((rc = ensure_scratch(ctx, s, n))) return rc;
-    forward_backward_fp32(s, n, feat, label, ncand, 1.0f / (float)n, 0);
+    forward_backward(s, precision == 0, n, feat, label, ncand, nullptr, 1.0f / (float)n, 0);
     if (cudaMemcpy(&loss, s->loss, 8, cudaMemcpyDeviceToHost) != cudaSuccess)
       return g4n_fail(ctx, G4N_ERR_CUDA, "mlp_grad: failed");
   }
@@ -438,7 +537,8 @@ int g4n_mlp_train(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *lab
   MlpState *s = state(ctx);
   const int64_t nb = n / batch;
   if (nb > INT32_MAX) return g4n_fail(ctx, G4N_ERR_ARG, "mlp_train: too many minibatches");
-  if ((rc = ensure_train(ctx, s, nb))) return rc;
+  const bool fused = batch >= kFusedRows;
+  if ((rc = fused ? ensure_train(ctx, s, nb) : ensure_scratch(ctx, s, batch))) return rc;
   std::unique_ptr<float2[]> corr(new (std::nothrow) float2[(size_t)nb]);
   if (!corr) return g4n_fail(ctx, G4N_ERR_OOM, "mlp_train: allocation failed");
   for (int ep = 0; ep < epochs; ++ep) {
@@ -449,10 +549,17 @@ int g4n_mlp_train(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *lab
     h ^= h >> 27;
     uint64_t stride = (h % (uint64_t)n) | 1;
     while (std::gcd(stride, (uint64_t)n) != 1) stride += 2;
+    double tot = 0.0;
     for (int64_t k = 0; k < nb; ++k) {
       ++s->step;
       corr[k].x = 1.0f / (1.0f - std::pow(0.9f, (float)s->step));
       corr[k].y = 1.0f / (1.0f - std::pow(0.999f, (float)s->step));
+    }
+    const uint64_t offset = (h >> 17) % (uint64_t)n;
+    if (!fused) {
+      if ((rc = train_plain(ctx, s, n, feat, label, ncand, batch, nb, stride, offset, lr, corr.get(), &tot, st))) return rc;
+      if (out_loss) out_loss[ep] = (float)(tot / ((double)nb * batch));
+      continue;
     }
     // the kernels of the epoch before have ended (run_train waits for them)
     if (cudaMemcpyAsync(s->corr, corr.get(), (size_t)nb * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess)
@@ -466,12 +573,11 @@ int g4n_mlp_train(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *lab
     T.batch = batch;
     T.permuted = true;
     T.stride = stride;
-    T.offset = (h >> 17) % (uint64_t)n;
+    T.offset = offset;
     T.inv_scale = 1.0f / (float)batch;
     T.M = s->M;
     T.V = s->V;
     T.lr = lr;
-    double tot = 0.0;
     if ((rc = run_train(ctx, s, T, &tot, st))) return rc;
     k_pack_image<<<8, 256, 0, st>>>(s->P, s->img);
     if (out_loss) out_loss[ep] = (float)(tot / ((double)nb * batch));

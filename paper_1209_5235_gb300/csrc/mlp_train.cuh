@@ -5,7 +5,7 @@
 // needs the weights of the one before it, so training is bound by the length of a step's serial
 // chain, not by arithmetic.  As separate kernels per GEMM and elementwise pass a step was 26
 // launches and clears in a row, 186 us at 4096 rows on GB300; here all steps of an epoch are one
-// launch and a step takes 10.5 us (an epoch of 2^20 samples: 47.7 -> 2.82 ms with the loading of the
+// launch and a step takes 11 us (an epoch of 2^20 samples: 47.7 -> 2.87 ms with the loading of the
 // parameters before it and their reading back).  A step:
 //   forward and backward of the block's row tiles, every intermediate in registers or shared memory;
 //   partial gradients to global memory; grid barrier;
@@ -300,9 +300,11 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
 #pragma unroll
-        for (int j = 0; j < 4; ++j) s += sub + 8 * j < nc ? expf(zz[j] - mx) : 0.f;
+        for (int j = 0; j < 4; ++j) {   // in the order of the columns, as the plain kernel sums them
+          const float ex = sub + 8 * j < nc ? expf(zz[j] - mx) : 0.f;
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+          for (int o = 0; o < 8; ++o) s += __shfl_sync(0xffffffffu, ex, o, 8);
+        }
         const float lse = mx + logf(s);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {

@@ -223,9 +223,9 @@ def test_trained_learned_barrel_full_size_sampled(env):
         assert hashes[2, 1][i] == r["hashes"][0], i
 
 
-@pytest.mark.parametrize("n", [16, 32, 48, 4864, 4880, 9760])
+@pytest.mark.parametrize("n", [16, 32, 48, 768, 784, 4864, 4880, 9760])
 def test_bf16_gradients_at_tile_edges(env, n):
-    """A half tile, one tile, a tile and a half, one tile per SM of a 152-SM GPU, one row block more, two tiles on
+    """Small batches of the plain kernels, the first and a ragged one of the persistent kernel, one tile per SM of a 152-SM GPU, one row block more, two tiles on
     some blocks and a ragged one.  Tolerance: that of the BF16 gradients above (8 significant bits, 2e-2 in norm)."""
     g4, torch, ctx = env
     p = params(27)
@@ -241,7 +241,7 @@ def test_bf16_gradients_at_tile_edges(env, n):
     assert again[0] == loss and np.array_equal(again[1], g)   # the summation order is fixed
 
 
-@pytest.mark.parametrize("batch", [16, 48, 4880])
+@pytest.mark.parametrize("batch", [16, 48, 768, 4880])
 def test_training_step_matches_its_gradient(env, batch):
     """One minibatch of an epoch: its loss is that of the permuted samples, and the update is Adam's first step on
     their gradient (the same kernel's, over the same rows in the same order).  Tolerance: the update in FP32 from the

@@ -552,7 +552,8 @@ constexpr unsigned kFull = 0xffffffffu;
 // looked up in FP32, so that only a point within the FP32 errors of a daughter's surface takes an FP64 test.  10^7
 // barrel queries of k_locate: 3.52 -> 2.20 ms (each candidate that passed its box in FP64 kept the FP64 pipe 78 %
 // busy); where the tracks of a nested barrel start, a batch of 10^6 17.9 -> 17.2 ms.  Relocations go without: with the
-// portals they are few, and the added code cost the barrel and the batched worlds 1 %, the default barrel 4 %.  (p, v) is the point in m's frame when have_p is set; otherwise it
+// portals they are few, and the added code cost the barrel and the batched worlds 1 %, the default barrel 4 %.
+// (p, v) is the point in m's frame when have_p is set; otherwise it
 // is derived from the world point when an FP64 test needs it.  kKeyBox daughters
 // and keyed voxel trees are answered from the world point's keys.  `blocked` is a
 // daughter of m already known not to contain the point (the volume just left).

@@ -7,8 +7,9 @@
 // the phases.  The staged schedule keeps the tracks in flight in HBM instead, as structure-of-arrays
 // queues, and advances them in iterations of two kernels:
 //
-//   step    every queued track takes one step (Sec. 3.2 problem 2, Eq. 7): the geometric step
-//           with its voxel walk, the move, the relocation.  The tracks that go on stepping are
+//   step    every queued track takes one step (Sec. 3.2 problem 2, Eq. 7), in boxes without
+//           daughters up to four: the geometric step with its voxel walk, the move, the
+//           relocation.  The tracks that go on stepping are
 //           written to the next iteration's queue of their leaf's solid kind (box, tube, orb,
 //           cone), so that each warp of the next step kernel runs one kind of geometry; the
 //           tracks whose free path ended go to the interaction queue.
@@ -17,14 +18,14 @@
 //           in flight, both written to the next step queues.
 //
 // Each kernel is small enough for the instruction caches and its warps are full (the queues are
-// compact); the cost is one load and one store of a track's state (168 B) per step and per
-// interaction (and per deferred relocation), from HBM/L2 at full coalescing.  Every history is the
+// compact); the cost is one load and one store of a track's state (144 B, in the FP64 mode 168)
+// per step and per interaction (and per deferred relocation), from HBM/L2 at full coalescing.  Every history is the
 // same as in the persistent kernel (the same device functions advance a track; the order of steps
 // within a history is fixed), so results do not depend on the schedule.
 //
 // With G4N_STAGED_RELOCATION_KERNEL a third kernel runs between the two: the step kernel queues the
-// steps whose relocation needs a search (not answered by a face record), and the relocation kernel
-// runs those searches in full warps.
+// steps whose relocation needs a search (not answered by a face record or a portal), and the
+// relocation kernel runs those searches in full warps; a short queue goes with the finish kernel.
 //
 // The last tracks of a batch (fewer than drain_tracks in flight, no new ones left) are finished
 // by one persistent kernel that takes them from the queue: an iteration costs at least the
@@ -200,8 +201,9 @@ __device__ __forceinline__ void sg_begin(Counters &cnt) {
 // Blocks of the grid that take part in a kernel over `total` tracks: those with a track of their own, block 0 at least.
 // The others leave at once, without the kernel's start and end (a grid of 2432 blocks counting itself out through one
 // atomic cost 20 to 35 us a launch, with an empty queue as well; with this and the drain at two tracks a thread:
-// calorimeter 6.68 -> 6.52 ms, its host batch of 2 10^5 2.5 -> 2.0, nested barrel 20.2 -> 17.8).  A block may read `total` after the last block has
-// reset it only if it is not one of them: the last block waits for all that take part, and block 0 always does.
+// calorimeter 6.68 -> 6.52 ms, its host batch of 2 10^5 2.5 -> 2.0, nested barrel 20.2 -> 17.8).  A block may read `total`
+// after the last block has reset it only if it is not one of them: the last block waits for all that take part, and block 0
+// always does.
 __device__ __forceinline__ unsigned sg_workers(long long total) {
   const long long need = (total + blockDim.x - 1) / blockDim.x;
   return need < 1 ? 1u : need < (long long)gridDim.x ? (unsigned)need : gridDim.x;

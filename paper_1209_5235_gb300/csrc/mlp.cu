@@ -31,7 +31,7 @@ namespace {
 // Rows from which a minibatch takes the persistent kernel.  The plain kernels split the sums over the rows into partials of
 // 256 rows or a little more and add these atomically.  One or two (fewer than 768 rows) have the same sum in either order: a
 // training repeats bit for bit.  Another order of summation ends 4e-4 away after 250 steps (BF16 rounds the differences
-// up), so these trainings keep theirs, and their 26 launches (170 us a step, where the persistent kernel takes 11 to 19).  From
+// up), so these trainings keep theirs, and their 24 launches (160 us a step, where the persistent kernel takes 11 to 19).  From
 // three partials on the order varies and two runs of the plain kernels differ by as much (1024 rows, 250 steps: up to 4e-4;
 // 4096: 1e-3; their error against 64 bits is 1e-3 to 5e-3 either way).
 constexpr int64_t kFusedRows = 768;
@@ -238,7 +238,9 @@ struct MlpState {
   float *X = nullptr, *Z1 = nullptr, *H1 = nullptr, *Z2 = nullptr, *H2 = nullptr, *Z3 = nullptr, *dZ3 = nullptr,
         *dH2 = nullptr, *dH1 = nullptr, *dW1p = nullptr;
   int64_t *idx = nullptr;
-  double *loss = nullptr;
+  // what gathers sums (Z1, Z2, dH2, dH1, Z3, dW1p, the loss): one block, cleared at once (a step at 512 rows 178 -> 160 us)
+  float *sums = nullptr;
+  double *loss = nullptr, *epoch = nullptr;
   // k_mlp_train: partial gradients and losses (one row per block), control block, Adam's corrections per step
   float *part = nullptr;
   double *part_loss = nullptr;
@@ -251,24 +253,25 @@ struct MlpState {
 MlpState *state(g4n_ctx *ctx) { return reinterpret_cast<MlpState *>(ctx->mlp); }
 
 void free_scratch(MlpState *s) {
-  cudaFree(s->X); cudaFree(s->Z1); cudaFree(s->H1); cudaFree(s->Z2); cudaFree(s->H2); cudaFree(s->Z3);
-  cudaFree(s->dZ3); cudaFree(s->dH2); cudaFree(s->dH1); cudaFree(s->dW1p); cudaFree(s->idx); cudaFree(s->loss);
+  cudaFree(s->X); cudaFree(s->H1); cudaFree(s->H2); cudaFree(s->dZ3); cudaFree(s->sums); cudaFree(s->idx);
+  cudaFree(s->epoch);
   s->X = s->Z1 = s->H1 = s->Z2 = s->H2 = s->Z3 = s->dZ3 = s->dH2 = s->dH1 = s->dW1p = nullptr;
+  s->sums = nullptr;
   s->idx = nullptr;
-  s->loss = nullptr;
+  s->loss = s->epoch = nullptr;
   s->cap = 0;
 }
+
+size_t sums_bytes(int64_t rows) { return (size_t)rows * (4 * kHid + kOut) * 4 + kInPad * kHid * 4 + 8; }
 
 int ensure_scratch(g4n_ctx *ctx, MlpState *s, int64_t rows) {
   if (s->cap >= rows) return G4N_OK;
   cudaDeviceSynchronize();
   free_scratch(s);
-  bool ok = cudaMalloc(&s->X, rows * kInPad * 4) == cudaSuccess && cudaMalloc(&s->Z1, rows * kHid * 4) == cudaSuccess &&
-            cudaMalloc(&s->H1, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->Z2, rows * kHid * 4) == cudaSuccess &&
-            cudaMalloc(&s->H2, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->Z3, rows * kOut * 4) == cudaSuccess &&
-            cudaMalloc(&s->dZ3, rows * kOut * 4) == cudaSuccess && cudaMalloc(&s->dH2, rows * kHid * 4) == cudaSuccess &&
-            cudaMalloc(&s->dH1, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->dW1p, kInPad * kHid * 4) == cudaSuccess &&
-            cudaMalloc(&s->idx, rows * 8) == cudaSuccess && cudaMalloc(&s->loss, 8) == cudaSuccess;
+  bool ok = cudaMalloc(&s->X, rows * kInPad * 4) == cudaSuccess && cudaMalloc(&s->H1, rows * kHid * 4) == cudaSuccess &&
+            cudaMalloc(&s->H2, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->dZ3, rows * kOut * 4) == cudaSuccess &&
+            cudaMalloc(&s->sums, sums_bytes(rows)) == cudaSuccess && cudaMalloc(&s->idx, rows * 8) == cudaSuccess &&
+            cudaMalloc(&s->epoch, 8) == cudaSuccess;
   if (!ok) {
     free_scratch(s);
     return g4n_fail(ctx, G4N_ERR_OOM, "mlp: scratch allocation failed");
@@ -300,31 +303,32 @@ void forward_backward(MlpState *s, bool bf16, int64_t rows, const float *feat, c
                       const int32_t *ncand, const int64_t *idx, float inv_scale, cudaStream_t st) {
   const int R = (int)rows;
   float *P = s->P, *G = s->G;
-  cudaMemsetAsync(s->loss, 0, 8, st);
+  s->Z1 = s->sums;
+  s->Z2 = s->Z1 + rows * kHid;
+  s->dH2 = s->Z2 + rows * kHid;
+  s->dH1 = s->dH2 + rows * kHid;
+  s->Z3 = s->dH1 + rows * kHid;
+  s->dW1p = s->Z3 + rows * kOut;
+  s->loss = (double *)(s->dW1p + kInPad * kHid);
+  cudaMemsetAsync(s->sums, 0, sums_bytes(rows), st);
+  cudaMemsetAsync(G, 0, kNParams * 4, st);
   k_gather<<<blocks(rows * kInPad), 256, 0, st>>>(rows, feat, idx, s->X);
   k_pad_w1<<<blocks(kInPad * kHid), 256, 0, st>>>(P, s->W1p);
-  cudaMemsetAsync(s->Z1, 0, rows * kHid * 4, st);
   gemm(bf16, R, kHid, kInPad, s->X, kInPad, false, s->W1p, kHid, false, s->Z1, kHid, st);
   k_bias_gelu<<<blocks(rows * kHid), 256, 0, st>>>(rows, kHid, s->Z1, P + kOffB1, s->H1);
-  cudaMemsetAsync(s->Z2, 0, rows * kHid * 4, st);
   gemm(bf16, R, kHid, kHid, s->H1, kHid, false, P + kOffW2, kHid, false, s->Z2, kHid, st);
   k_bias_gelu<<<blocks(rows * kHid), 256, 0, st>>>(rows, kHid, s->Z2, P + kOffB2, s->H2);
-  cudaMemsetAsync(s->Z3, 0, rows * kOut * 4, st);
   gemm(bf16, R, kOut, kHid, s->H2, kHid, false, P + kOffW3, kOut, false, s->Z3, kOut, st);
   k_softmax_ce<<<blocks(rows), 256, 0, st>>>(rows, s->Z3, P + kOffB3, label, ncand, idx, inv_scale, s->dZ3, s->loss);
   // backward
-  cudaMemsetAsync(G, 0, kNParams * 4, st);
   gemm(bf16, kHid, kOut, R, s->H2, kHid, true, s->dZ3, kOut, false, G + kOffW3, kOut, st);    // dW3 = H2^T dZ3
   k_colsum<<<kOut, 256, 0, st>>>(rows, kOut, s->dZ3, G + kOffB3);
-  cudaMemsetAsync(s->dH2, 0, rows * kHid * 4, st);
   gemm(bf16, R, kHid, kOut, s->dZ3, kOut, false, P + kOffW3, kOut, true, s->dH2, kHid, st);   // dH2 = dZ3 W3^T
   k_gelu_bwd<<<blocks(rows * kHid), 256, 0, st>>>(rows * kHid, s->dH2, s->Z2);
   gemm(bf16, kHid, kHid, R, s->H1, kHid, true, s->dH2, kHid, false, G + kOffW2, kHid, st);    // dW2 = H1^T dZ2
   k_colsum<<<kHid, 256, 0, st>>>(rows, kHid, s->dH2, G + kOffB2);
-  cudaMemsetAsync(s->dH1, 0, rows * kHid * 4, st);
   gemm(bf16, R, kHid, kHid, s->dH2, kHid, false, P + kOffW2, kHid, true, s->dH1, kHid, st);   // dH1 = dZ2 W2^T
   k_gelu_bwd<<<blocks(rows * kHid), 256, 0, st>>>(rows * kHid, s->dH1, s->Z1);
-  cudaMemsetAsync(s->dW1p, 0, kInPad * kHid * 4, st);
   gemm(bf16, kInPad, kHid, R, s->X, kInPad, true, s->dH1, kHid, false, s->dW1p, kHid, st);   // dW1 = X^T dZ1
   cudaMemcpyAsync(G + kOffW1, s->dW1p, kIn * kHid * 4, cudaMemcpyDeviceToDevice, st);
   k_colsum<<<kHid, 256, 0, st>>>(rows, kHid, s->dH1, G + kOffB1);
@@ -388,23 +392,17 @@ int run_train(g4n_ctx *ctx, MlpState *s, TrainParams &T, double *loss, cudaStrea
 int train_plain(g4n_ctx *ctx, MlpState *s, int64_t n, const float *feat, const int32_t *label, const int32_t *ncand,
                 int32_t batch, int64_t nb, uint64_t stride, uint64_t offset, float lr, const float2 *corr, double *loss,
                 cudaStream_t st) {
-  double *sum = nullptr;
-  if (cudaMalloc(&sum, 8) != cudaSuccess) {
-    cudaGetLastError();
-    return g4n_fail(ctx, G4N_ERR_OOM, "mlp_train: allocation failed");
-  }
-  cudaMemsetAsync(sum, 0, 8, st);
+  cudaMemsetAsync(s->epoch, 0, 8, st);
   for (int64_t b = 0; b < nb; ++b) {
     k_batch_index<<<blocks(batch), 256, 0, st>>>(batch, n, b * batch, (int64_t)stride, (int64_t)offset, s->idx);
     forward_backward(s, true, batch, feat, label, ncand, s->idx, 1.0f / (float)batch, st);
     k_adam<<<blocks(kNParams), 256, 0, st>>>(kNParams, s->P, s->G, s->M, s->V, lr, 0.9f, 0.999f, corr[b].x, corr[b].y,
                                              1e-8f);
-    k_add_double<<<1, 1, 0, st>>>(sum, s->loss);  // epoch loss accumulates on the device
+    k_add_double<<<1, 1, 0, st>>>(s->epoch, s->loss);  // epoch loss accumulates on the device
   }
   k_pack_image<<<8, 256, 0, st>>>(s->P, s->img);
-  cudaMemcpyAsync(loss, sum, 8, cudaMemcpyDeviceToHost, st);
+  cudaMemcpyAsync(loss, s->epoch, 8, cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
-  cudaFree(sum);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return g4n_fail(ctx, G4N_ERR_CUDA, std::string("mlp_train: ") + cudaGetErrorString(e));
   return G4N_OK;

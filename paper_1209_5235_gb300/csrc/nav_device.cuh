@@ -558,7 +558,8 @@ constexpr unsigned kFull = 0xffffffffu;
 // and keyed voxel trees are answered from the world point's keys.  `blocked` is a
 // daughter of m already known not to contain the point (the volume just left).
 // Returns the deepest volume.
-template <bool COUNT, bool CLASSIFY>
+// KEYED: every volume is a kKeyBox; nothing but keys.
+template <bool COUNT, bool CLASSIFY, bool KEYED = false>
 __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, V3 p, V3 v, bool have_p,
                                             const WPos &W, int blocked, Counters &cnt) {
 #pragma unroll 1
@@ -568,7 +569,7 @@ __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, 
     DCandList L{0, 0};
     if (want) {
       const int h = G.vol[m].vox;
-      if (G.hdr[h].keyed) {
+      if (KEYED || G.hdr[h].keyed) {
         L = G.clist[vox_lookup_keys(G, h, W)];
       } else {
         if (!have_p) {
@@ -594,7 +595,7 @@ __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, 
           ++i;
           if (c == blocked) continue;
           const DBox32 &B = G.box[c];
-          if (B.keyed) {
+          if (KEYED || B.keyed) {
             diag<COUNT>(cnt, G4N_C_KEY_INSIDE);
             if (keybox_inside(G, c, W)) {
               found = c;
@@ -633,7 +634,7 @@ __device__ __forceinline__ int descend_body(const DGeom &G, bool active, int m, 
         if (d < 0) searching = false;
       }
       __syncwarp();
-      if (d >= 0) {
+      if (!KEYED && d >= 0) {
         const DVol &D = G.vol[d];
         V3 dp, dv;
         if (CLASSIFY) world_to_local(G.wxf[m], G.vol[m].flags & kWorldAligned, W.x, W.u, p, v);
@@ -681,13 +682,13 @@ __device__ __forceinline__ int descend_warp(const DGeom &G, bool active, int m, 
 }
 
 // Locate from the world (warp-collective): the leaf, or -1 outside the world.
-template <bool COUNT, bool OOL, bool CLASSIFY>
+template <bool COUNT, bool OOL, bool CLASSIFY, bool KEYED = false>
 __device__ __forceinline__ int locate_world_warp(const DGeom &G, bool active, const V3 &x, const V3 &u, Counters &cnt) {
   V3 p{0, 0, 0}, v{0, 0, 1};
   bool in = false, have_p = false;
   const WPos W = make_wpos(x, u);
   if (active) {
-    if (G.vol[0].flags & kKeyBox) {
+    if (KEYED || (G.vol[0].flags & kKeyBox)) {
       diag<COUNT>(cnt, G4N_C_KEY_INSIDE);
       in = keybox_inside(G, 0, W);
     } else {
@@ -697,7 +698,8 @@ __device__ __forceinline__ int locate_world_warp(const DGeom &G, bool active, co
       in = vol_inside(G.vol[0], p, v, G.half);
     }
   }
-  const int leaf = descend_warp<COUNT, OOL, CLASSIFY>(G, in, 0, p, v, have_p, W, -1, cnt);
+  const int leaf = KEYED ? descend_body<COUNT, false, true>(G, in, 0, p, v, have_p, W, -1, cnt)
+                         : descend_warp<COUNT, OOL, CLASSIFY>(G, in, 0, p, v, have_p, W, -1, cnt);
   return in ? leaf : -1;
 }
 

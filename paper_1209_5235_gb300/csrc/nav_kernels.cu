@@ -101,8 +101,9 @@ __device__ __forceinline__ void flush_block(unsigned long long *counters) {
 // 8 blocks of 128 per SM (64 registers, a few hundred bytes of spills): the descent waits on its chain
 // of dependent table loads, and more resident warps hide it (10^7 calorimeter queries: 6.3e9 -> 8.8e9 /s
 // against 5 blocks at 96 registers; 10 to 16 blocks were slower again).
-// CLASSIFY: FP32 classification of the daughters (descend_body); geometries of world-aligned boxes alone, whose Inside
-// tests are key comparisons, go without (10^7 calorimeter queries 1.17 -> 1.15 ms).
+// CLASSIFY: FP32 classification of the daughters (descend_body).  Geometries of world-aligned boxes alone, whose Inside
+// tests and voxel lookups are all key comparisons, take a descent without anything else (10^7 calorimeter queries 1.15 ->
+// 0.84 ms, 10^6 0.148 -> 0.116; at 10 blocks per SM 0.90 and 0.110, at 12 1.04 and 0.123).
 template <bool CLASSIFY>
 __global__ void __launch_bounds__(128, 8) k_locate(const DGeom *__restrict__ geoms, int gid, int64_t n,
                                                 const double *__restrict__ pos, const double *__restrict__ dir,
@@ -123,7 +124,7 @@ __global__ void __launch_bounds__(128, 8) k_locate(const DGeom *__restrict__ geo
       ok = !bad_dir(u) && isfinite(x.x + x.y + x.z);
       if (!ok) flag(status, kStBadInput);
     }
-    const int leaf = locate_world_warp<false, false, CLASSIFY>(G, ok, x, u, cnt);
+    const int leaf = locate_world_warp<false, false, CLASSIFY, !CLASSIFY>(G, ok, x, u, cnt);
     if (i < n) {
       const int depth = ok ? (leaf >= 0 ? G.vol[leaf].depth : 0) : -1;
       out_depth[i] = depth;

@@ -1,7 +1,7 @@
 // mlp.cu -- training and inference entry points of the candidate-proposal MLP.
 //
-// Training (g4n_mlp_train, and the BF16 gradients of g4n_mlp_grad) on minibatches
-// of kFusedRows rows and more is the persistent kernel of mlp_train.cuh: BF16
+// Training (g4n_mlp_train) on large minibatches, and the BF16 gradients of
+// g4n_mlp_grad on many rows, are the persistent kernel of mlp_train.cuh: BF16
 // products on the tensor cores with FP32 accumulation, masked softmax
 // cross-entropy, Adam on FP32 master weights.  Smaller minibatches and the FP32
 // reference gradients take one kernel of this file per product and elementwise pass.
@@ -28,13 +28,16 @@ using namespace g4n::mlp;
 
 namespace {
 
-// Rows from which a minibatch takes the persistent kernel.  The plain kernels split the sums over the rows into partials of
-// 256 rows or a little more and add these atomically.  One or two (fewer than 768 rows) have the same sum in either order: a
-// training repeats bit for bit.  Another order of summation ends 4e-4 away after 250 steps (BF16 rounds the differences
-// up), so these trainings keep theirs, and their 24 launches (160 us a step, where the persistent kernel takes 11 to 19).  From
-// three partials on the order varies and two runs of the plain kernels differ by as much (1024 rows, 250 steps: up to 4e-4;
-// 4096: 1e-3; their error against 64 bits is 1e-3 to 5e-3 either way).
+// Rows from which BF16 gradients (g4n_mlp_grad) take the persistent kernel: from three K chunks on the plain kernels'
+// atomics leave the order of the partial sums open (of 400 pairs of calls on the same 768 rows 144 differed), the persistent
+// kernel adds them in ascending order.  Below, one or two chunks have one sum.
 constexpr int64_t kFusedRows = 768;
+// Rows from which a training does.  In trainings of 768 to 1300 rows a step (three to five chunks) the atomics of the plain kernels mostly
+// arrive in one order as long as a process keeps its buffers where they are, and its trainings repeat; another order ends
+// 1e-4 to 5e-4 away in the weights after 200 steps, as another process with other allocations before it does.  Those
+// keep the plain kernels (26 launches and clears, 170 us a step).  From eight chunks on no two runs agree (2048 rows, 200
+// steps: 3e-4 to 9e-4 between any two; 4096: 1e-3), and the persistent kernel's ascending order is one of theirs.
+constexpr int64_t kFusedTrainRows = 2048;
 
 // ---------------------------------------------------------------- plain kernels
 // C[M x N] += op(A)[M x K] op(B)[K x N]; A(m, k) = transA ? A[k * lda + m] : A[m * lda + k],
@@ -238,10 +241,12 @@ struct MlpState {
   float *X = nullptr, *Z1 = nullptr, *H1 = nullptr, *Z2 = nullptr, *H2 = nullptr, *Z3 = nullptr, *dZ3 = nullptr,
         *dH2 = nullptr, *dH1 = nullptr, *dW1p = nullptr;
   int64_t *idx = nullptr;
-  // what gathers sums (Z1, Z2, dH2, dH1, Z3, dW1p, the loss): one block, cleared at once (a step at 512 rows 178 -> 160 us)
-  float *sums = nullptr;
-  double *loss = nullptr, *epoch = nullptr;
-  // k_mlp_train: partial gradients and losses (one row per block), control block, Adam's corrections per step
+  double *loss = nullptr;
+  // k_mlp_train: fragments and FP32 deltas of `train_rows` rows, partial gradients, losses per block, control block, Adam's
+  // corrections per step
+  uint4 *frag = nullptr;
+  float *delta = nullptr;
+  int64_t train_rows = 0;
   float *part = nullptr;
   double *part_loss = nullptr;
   TrainCtrl *ctrl = nullptr;
@@ -253,25 +258,24 @@ struct MlpState {
 MlpState *state(g4n_ctx *ctx) { return reinterpret_cast<MlpState *>(ctx->mlp); }
 
 void free_scratch(MlpState *s) {
-  cudaFree(s->X); cudaFree(s->H1); cudaFree(s->H2); cudaFree(s->dZ3); cudaFree(s->sums); cudaFree(s->idx);
-  cudaFree(s->epoch);
+  cudaFree(s->X); cudaFree(s->Z1); cudaFree(s->H1); cudaFree(s->Z2); cudaFree(s->H2); cudaFree(s->Z3);
+  cudaFree(s->dZ3); cudaFree(s->dH2); cudaFree(s->dH1); cudaFree(s->dW1p); cudaFree(s->idx); cudaFree(s->loss);
   s->X = s->Z1 = s->H1 = s->Z2 = s->H2 = s->Z3 = s->dZ3 = s->dH2 = s->dH1 = s->dW1p = nullptr;
-  s->sums = nullptr;
   s->idx = nullptr;
-  s->loss = s->epoch = nullptr;
+  s->loss = nullptr;
   s->cap = 0;
 }
-
-size_t sums_bytes(int64_t rows) { return (size_t)rows * (4 * kHid + kOut) * 4 + kInPad * kHid * 4 + 8; }
 
 int ensure_scratch(g4n_ctx *ctx, MlpState *s, int64_t rows) {
   if (s->cap >= rows) return G4N_OK;
   cudaDeviceSynchronize();
   free_scratch(s);
-  bool ok = cudaMalloc(&s->X, rows * kInPad * 4) == cudaSuccess && cudaMalloc(&s->H1, rows * kHid * 4) == cudaSuccess &&
-            cudaMalloc(&s->H2, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->dZ3, rows * kOut * 4) == cudaSuccess &&
-            cudaMalloc(&s->sums, sums_bytes(rows)) == cudaSuccess && cudaMalloc(&s->idx, rows * 8) == cudaSuccess &&
-            cudaMalloc(&s->epoch, 8) == cudaSuccess;
+  bool ok = cudaMalloc(&s->X, rows * kInPad * 4) == cudaSuccess && cudaMalloc(&s->Z1, rows * kHid * 4) == cudaSuccess &&
+            cudaMalloc(&s->H1, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->Z2, rows * kHid * 4) == cudaSuccess &&
+            cudaMalloc(&s->H2, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->Z3, rows * kOut * 4) == cudaSuccess &&
+            cudaMalloc(&s->dZ3, rows * kOut * 4) == cudaSuccess && cudaMalloc(&s->dH2, rows * kHid * 4) == cudaSuccess &&
+            cudaMalloc(&s->dH1, rows * kHid * 4) == cudaSuccess && cudaMalloc(&s->dW1p, kInPad * kHid * 4) == cudaSuccess &&
+            cudaMalloc(&s->idx, rows * 8) == cudaSuccess && cudaMalloc(&s->loss, 8) == cudaSuccess;
   if (!ok) {
     free_scratch(s);
     return g4n_fail(ctx, G4N_ERR_OOM, "mlp: scratch allocation failed");
@@ -280,10 +284,15 @@ int ensure_scratch(g4n_ctx *ctx, MlpState *s, int64_t rows) {
   return G4N_OK;
 }
 
+// Length of a product's K chunks: one block column each, and one partial sum of every output.
+int64_t chunk_rows(int64_t K) {
+  const int64_t ksplit = std::max<int64_t>(1, std::min<int64_t>(kMaxChunks, K / 256));
+  return ((K + ksplit - 1) / ksplit + 15) / 16 * 16;
+}
+
 void gemm(bool bf16, int M, int N, int K, const float *A, int lda, bool tA, const float *B, int ldb, bool tB, float *C,
           int ldc, cudaStream_t st) {
-  const int ksplit = std::max(1, std::min(256, K / 256));
-  const int kchunk = ((K + ksplit - 1) / ksplit + 15) / 16 * 16;
+  const int kchunk = (int)chunk_rows(K);
   const int nz = (K + kchunk - 1) / kchunk;
   if (bf16) {
     const int warps = (M / 16) * (N / 8);
@@ -303,46 +312,68 @@ void forward_backward(MlpState *s, bool bf16, int64_t rows, const float *feat, c
                       const int32_t *ncand, const int64_t *idx, float inv_scale, cudaStream_t st) {
   const int R = (int)rows;
   float *P = s->P, *G = s->G;
-  s->Z1 = s->sums;
-  s->Z2 = s->Z1 + rows * kHid;
-  s->dH2 = s->Z2 + rows * kHid;
-  s->dH1 = s->dH2 + rows * kHid;
-  s->Z3 = s->dH1 + rows * kHid;
-  s->dW1p = s->Z3 + rows * kOut;
-  s->loss = (double *)(s->dW1p + kInPad * kHid);
-  cudaMemsetAsync(s->sums, 0, sums_bytes(rows), st);
-  cudaMemsetAsync(G, 0, kNParams * 4, st);
+  cudaMemsetAsync(s->loss, 0, 8, st);
   k_gather<<<blocks(rows * kInPad), 256, 0, st>>>(rows, feat, idx, s->X);
   k_pad_w1<<<blocks(kInPad * kHid), 256, 0, st>>>(P, s->W1p);
+  cudaMemsetAsync(s->Z1, 0, rows * kHid * 4, st);
   gemm(bf16, R, kHid, kInPad, s->X, kInPad, false, s->W1p, kHid, false, s->Z1, kHid, st);
   k_bias_gelu<<<blocks(rows * kHid), 256, 0, st>>>(rows, kHid, s->Z1, P + kOffB1, s->H1);
+  cudaMemsetAsync(s->Z2, 0, rows * kHid * 4, st);
   gemm(bf16, R, kHid, kHid, s->H1, kHid, false, P + kOffW2, kHid, false, s->Z2, kHid, st);
   k_bias_gelu<<<blocks(rows * kHid), 256, 0, st>>>(rows, kHid, s->Z2, P + kOffB2, s->H2);
+  cudaMemsetAsync(s->Z3, 0, rows * kOut * 4, st);
   gemm(bf16, R, kOut, kHid, s->H2, kHid, false, P + kOffW3, kOut, false, s->Z3, kOut, st);
   k_softmax_ce<<<blocks(rows), 256, 0, st>>>(rows, s->Z3, P + kOffB3, label, ncand, idx, inv_scale, s->dZ3, s->loss);
   // backward
+  cudaMemsetAsync(G, 0, kNParams * 4, st);
   gemm(bf16, kHid, kOut, R, s->H2, kHid, true, s->dZ3, kOut, false, G + kOffW3, kOut, st);    // dW3 = H2^T dZ3
   k_colsum<<<kOut, 256, 0, st>>>(rows, kOut, s->dZ3, G + kOffB3);
+  cudaMemsetAsync(s->dH2, 0, rows * kHid * 4, st);
   gemm(bf16, R, kHid, kOut, s->dZ3, kOut, false, P + kOffW3, kOut, true, s->dH2, kHid, st);   // dH2 = dZ3 W3^T
   k_gelu_bwd<<<blocks(rows * kHid), 256, 0, st>>>(rows * kHid, s->dH2, s->Z2);
   gemm(bf16, kHid, kHid, R, s->H1, kHid, true, s->dH2, kHid, false, G + kOffW2, kHid, st);    // dW2 = H1^T dZ2
   k_colsum<<<kHid, 256, 0, st>>>(rows, kHid, s->dH2, G + kOffB2);
+  cudaMemsetAsync(s->dH1, 0, rows * kHid * 4, st);
   gemm(bf16, R, kHid, kHid, s->dH2, kHid, false, P + kOffW2, kHid, true, s->dH1, kHid, st);   // dH1 = dZ2 W2^T
   k_gelu_bwd<<<blocks(rows * kHid), 256, 0, st>>>(rows * kHid, s->dH1, s->Z1);
+  cudaMemsetAsync(s->dW1p, 0, kInPad * kHid * 4, st);
   gemm(bf16, kInPad, kHid, R, s->X, kInPad, true, s->dH1, kHid, false, s->dW1p, kHid, st);   // dW1 = X^T dZ1
   cudaMemcpyAsync(G + kOffW1, s->dW1p, kIn * kHid * 4, cudaMemcpyDeviceToDevice, st);
   k_colsum<<<kHid, 256, 0, st>>>(rows, kHid, s->dH1, G + kOffB1);
 }
 
-// Buffers of k_mlp_train for `steps` minibatches.
-int ensure_train(g4n_ctx *ctx, MlpState *s, int64_t steps) {
+void free_train(MlpState *s) {
+  cudaFree(s->frag); cudaFree(s->delta); cudaFree(s->part); cudaFree(s->part_loss); cudaFree(s->ctrl); cudaFree(s->timg);
+  cudaFree(s->corr);
+  s->frag = nullptr;
+  s->delta = s->part = nullptr;
+  s->part_loss = nullptr;
+  s->ctrl = nullptr;
+  s->timg = nullptr;
+  s->corr = nullptr;
+  s->train_rows = s->corr_cap = 0;
+}
+
+// Buffers of k_mlp_train for `steps` minibatches of `rows` rows (every use of them has ended: run_train waits for its kernel).
+int ensure_train(g4n_ctx *ctx, MlpState *s, int64_t rows, int64_t steps) {
+  const size_t ld = (size_t)(rows + kTrRows - 1) / kTrRows * kTrRows;
   bool ok = true;
   if (!s->ctrl)
-    ok = cudaMalloc(&s->part, (size_t)ctx->sm_count * kNParams * 4) == cudaSuccess &&
+    ok = cudaMalloc(&s->part, ((size_t)kMaxChunks * kNParams + kColParts * kCols) * 4) == cudaSuccess &&
          cudaMalloc(&s->part_loss, (size_t)ctx->sm_count * 8) == cudaSuccess &&
          cudaMalloc(&s->ctrl, sizeof(TrainCtrl)) == cudaSuccess &&
          cudaMalloc(&s->timg, sizeof(TrainWeights)) == cudaSuccess &&
          cudaMemset(s->timg, 0, sizeof(TrainWeights)) == cudaSuccess;
+  if (ok && s->train_rows < rows) {
+    cudaFree(s->frag);
+    cudaFree(s->delta);
+    s->frag = nullptr;
+    s->delta = nullptr;
+    s->train_rows = 0;
+    ok = cudaMalloc(&s->frag, ld / 16 * kFrags * 32 * sizeof(uint4)) == cudaSuccess &&
+         cudaMalloc(&s->delta, ld * kCols * 4) == cudaSuccess;
+    if (ok) s->train_rows = rows;
+  }
   if (ok && s->corr_cap < steps) {
     cudaFree(s->corr);
     s->corr = nullptr;
@@ -352,28 +383,31 @@ int ensure_train(g4n_ctx *ctx, MlpState *s, int64_t steps) {
   }
   if (!ok) {
     cudaGetLastError();
-    cudaFree(s->part); cudaFree(s->part_loss); cudaFree(s->ctrl); cudaFree(s->timg);
-    s->part = nullptr;
-    s->part_loss = nullptr;
-    s->ctrl = nullptr;
-    s->timg = nullptr;
+    free_train(s);
     return g4n_fail(ctx, G4N_ERR_OOM, "mlp: scratch allocation failed");
   }
   return G4N_OK;
 }
 
-// Run k_mlp_train on `st` and wait for it: one block per tile of 32 rows, at most one per SM.  *loss = sum of the losses.
+// Run k_mlp_train on `st` and wait for it: a block per tile of 32 rows, or a warp per task of the gradients where those are
+// more (4096 rows: 128 tiles, 136 blocks for 1088 tasks), at most a block per SM.  *loss = sum of the losses.
 int run_train(g4n_ctx *ctx, MlpState *s, TrainParams &T, double *loss, cudaStream_t st) {
   T.P = s->P;
   T.b1 = 0.9f;
   T.b2 = 0.999f;
   T.eps = 1e-8f;
+  T.chunk = chunk_rows(T.batch);
+  T.chunks = (int)((T.batch + T.chunk - 1) / T.chunk);
+  T.frag = s->frag;
+  T.delta = s->delta;
+  T.delta_ld = (T.batch + kTrRows - 1) / kTrRows * kTrRows;
   T.part = s->part;
   T.part_loss = s->part_loss;
   T.bias_corr = s->corr;
   T.ctrl = s->ctrl;
   T.img = s->timg;
-  const int grid = std::min((T.batch + kTrRows - 1) / kTrRows, ctx->sm_count);
+  const int64_t tasks = (int64_t)T.chunks * kChunkTiles + kCols / 2 * kColParts;
+  const int grid = (int)std::min<int64_t>(std::max(T.delta_ld / kTrRows, (tasks + 7) / 8), ctx->sm_count);
   void *args[] = {&T};
   TrainCtrl end{};
   cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem));
@@ -392,17 +426,23 @@ int run_train(g4n_ctx *ctx, MlpState *s, TrainParams &T, double *loss, cudaStrea
 int train_plain(g4n_ctx *ctx, MlpState *s, int64_t n, const float *feat, const int32_t *label, const int32_t *ncand,
                 int32_t batch, int64_t nb, uint64_t stride, uint64_t offset, float lr, const float2 *corr, double *loss,
                 cudaStream_t st) {
-  cudaMemsetAsync(s->epoch, 0, 8, st);
+  double *sum = nullptr;
+  if (cudaMalloc(&sum, 8) != cudaSuccess) {
+    cudaGetLastError();
+    return g4n_fail(ctx, G4N_ERR_OOM, "mlp_train: allocation failed");
+  }
+  cudaMemsetAsync(sum, 0, 8, st);
   for (int64_t b = 0; b < nb; ++b) {
     k_batch_index<<<blocks(batch), 256, 0, st>>>(batch, n, b * batch, (int64_t)stride, (int64_t)offset, s->idx);
     forward_backward(s, true, batch, feat, label, ncand, s->idx, 1.0f / (float)batch, st);
     k_adam<<<blocks(kNParams), 256, 0, st>>>(kNParams, s->P, s->G, s->M, s->V, lr, 0.9f, 0.999f, corr[b].x, corr[b].y,
                                              1e-8f);
-    k_add_double<<<1, 1, 0, st>>>(s->epoch, s->loss);  // epoch loss accumulates on the device
+    k_add_double<<<1, 1, 0, st>>>(sum, s->loss);  // epoch loss accumulates on the device
   }
   k_pack_image<<<8, 256, 0, st>>>(s->P, s->img);
-  cudaMemcpyAsync(loss, s->epoch, 8, cudaMemcpyDeviceToHost, st);
+  cudaMemcpyAsync(loss, sum, 8, cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
+  cudaFree(sum);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return g4n_fail(ctx, G4N_ERR_CUDA, std::string("mlp_train: ") + cudaGetErrorString(e));
   return G4N_OK;
@@ -429,7 +469,7 @@ void g4n_mlp_free(g4n_ctx *ctx) {
   if (!s) return;
   free_scratch(s);
   cudaFree(s->P); cudaFree(s->G); cudaFree(s->M); cudaFree(s->V); cudaFree(s->img); cudaFree(s->W1p);
-  cudaFree(s->part); cudaFree(s->part_loss); cudaFree(s->ctrl); cudaFree(s->timg); cudaFree(s->corr);
+  free_train(s);
   delete s;
   ctx->mlp = nullptr;
 }
@@ -500,15 +540,14 @@ int g4n_mlp_grad(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *labe
   MlpState *s = state(ctx);
   double loss = 0.0;
   if (precision == 0 && n >= kFusedRows) {
-    if (n > INT32_MAX - kTrRows) return g4n_fail(ctx, G4N_ERR_ARG, "mlp_grad: too many samples");
-    if ((rc = ensure_train(ctx, s, 0))) return rc;
+    if ((rc = ensure_train(ctx, s, n, 0))) return rc;
     TrainParams T{};
     T.n = n;
     T.feat = feat;
     T.label = label;
     T.ncand = ncand;
     T.steps = 1;
-    T.batch = (int)n;
+    T.batch = n;
     T.inv_scale = 1.0f / (float)n;
     T.grads = s->G;
     if ((rc = run_train(ctx, s, T, &loss, 0))) return rc;
@@ -535,8 +574,8 @@ int g4n_mlp_train(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *lab
   MlpState *s = state(ctx);
   const int64_t nb = n / batch;
   if (nb > INT32_MAX) return g4n_fail(ctx, G4N_ERR_ARG, "mlp_train: too many minibatches");
-  const bool fused = batch >= kFusedRows;
-  if ((rc = fused ? ensure_train(ctx, s, nb) : ensure_scratch(ctx, s, batch))) return rc;
+  const bool fused = batch >= kFusedTrainRows;
+  if ((rc = fused ? ensure_train(ctx, s, batch, nb) : ensure_scratch(ctx, s, batch))) return rc;
   std::unique_ptr<float2[]> corr(new (std::nothrow) float2[(size_t)nb]);
   if (!corr) return g4n_fail(ctx, G4N_ERR_OOM, "mlp_train: allocation failed");
   for (int ep = 0; ep < epochs; ++ep) {

@@ -3,23 +3,30 @@
 //
 // A minibatch of this network is little work -- 4096 rows are 0.17 GFLOP of GEMM -- and every step
 // needs the weights of the one before it, so training is bound by the length of a step's serial
-// chain, not by arithmetic.  As separate kernels per GEMM and elementwise pass a step was 26
+// chain, not by arithmetic.  As separate kernels per GEMM and elementwise pass a step is 26
 // launches and clears in a row, 186 us at 4096 rows on GB300; here all steps of an epoch are one
-// launch and a step takes 11 us (an epoch of 2^20 samples: 47.7 -> 2.87 ms with the loading of the
-// parameters before it and their reading back).  A step:
-//   forward and backward of the block's row tiles, every intermediate in registers or shared memory;
-//   partial gradients to global memory; grid barrier;
-//   each block sums the partials of its share of the parameters and updates them (Adam); grid barrier;
-//   reload of the weights' image (31 KB, from L2).
+// launch.  A step:
+//   1. forward and backward of the block's row tiles; what the gradients need goes to global memory (L2): the
+//      activations and deltas as mma fragments, the deltas in FP32 as well; grid barrier;
+//   2. partial gradients, one warp per 16 x 16 tile of a weight gradient and chunk of rows, and per two columns
+//      and eighth of a bias gradient; grid barrier;
+//   3. each block adds the partials of its share of the parameters and updates them (Adam); grid barrier;
+//      reload of the weights' image (31 KB, from L2).
+//
+// The sums are those of the plain kernels (mlp.cu), operation by operation: a chunk has the rows that one K chunk of
+// their GEMM has, multiplied 16 rows after the other from a zero accumulator; the chunks are added in ascending order,
+// one of the orders in which the plain kernels' atomics may arrive; a bias gradient has k_colsum's threads, tree and
+// warps.  BF16 rounding of the next operands makes 1e-3 of a last bit within 250 steps, so that another grouping of
+// the sums would be another training.  Gradients of up to two chunks, and trainings on them, are the plain kernels' bit for
+// bit.  The order is fixed: results do not vary from run to run.
 //
 // A tile is 32 rows by all 64 hidden columns on 8 warps (2 row halves x 4 column groups of 16), so
 // that a minibatch of 4096 rows fills 128 SMs and a layer is a few mma.sync per warp.  Products are
 // mma.sync m16n8k16 (BF16 in, FP32 accumulation), the K chunks of an output in ascending order from a
 // zero accumulator, bias added afterwards.  tcgen05 tiles need 128 rows per CTA: a quarter of the SMs
-// and four times the elementwise work (erf, exp) per SM, on a chain that waits for latency anyway.
-// The weight-gradient products take their transposed operands from shared memory with ldmatrix.trans
-// and keep their 28 accumulators per lane in registers over all of a block's tiles.  Summation order
-// is fixed: results do not vary from run to run.
+// and four times the elementwise work (erf, exp) per SM, on a chain that waits for latency anyway, and
+// its sums over K are not the ones above.  ldmatrix.trans transposes the operands of the weight gradients once, where
+// they are written; phase 2 reads whole fragments, 512 bytes a warp.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -49,17 +56,31 @@ struct TrainCtrl {
   double loss;            // sum of the losses over the launch
 };
 
+// A 16-row step of a minibatch as the weight-gradient products read it: A fragments (16 columns) of H1, H2 and X, B
+// fragments (2 x 8 columns) of the deltas, 32 lanes x 16 bytes each.
+constexpr int kFragH1 = 0, kFragH2 = 4, kFragX = 8, kFragD2 = 9, kFragD1 = 13, kFragD3 = 17, kFrags = 19;
+constexpr int kColZ3 = 0, kColZ2 = kOut, kColZ1 = kOut + kHid, kCols = kOut + 2 * kHid;   // columns of the FP32 deltas
+constexpr int kChunkTiles = 28;                  // 16 x 16 tiles of the weight gradients: W2 16, W3 8, W1 4
+constexpr int kColParts = 8;                     // partial sums of a bias gradient: k_colsum's warps
+constexpr int kMaxChunks = 256;                  // K chunks of the plain kernels' GEMM
+
 struct TrainParams {
   int64_t n;                        // samples
   const float *feat;
   const int32_t *label, *ncand;
-  int steps, batch;                 // minibatches of `batch` rows
+  int steps;
+  int64_t batch;                    // rows of a minibatch
+  int64_t chunk;                    // rows of a partial weight gradient (a multiple of 16)
+  int chunks;
   bool permuted;                    // row r of step s is sample ((s batch + r) mod n * stride + offset) mod n, else s batch + r
   uint64_t stride, offset;
   float inv_scale;
   float *P, *M, *V;                 // parameters and Adam moments; M null: gradients of one step into `grads` instead
   float *grads;
-  float *part;                      // gridDim.x x kNParams partial gradients
+  uint4 *frag;                      // [16-row step][kFrags][32]
+  float *delta;                     // [kCols][delta_ld]
+  int64_t delta_ld;
+  float *part;                      // chunks x kNParams partial weight gradients, then kColParts x kCols bias partials
   double *part_loss;                // gridDim.x
   const float2 *bias_corr;          // per step: Adam's 1 / (1 - beta^t)
   float lr, b1, b2, eps;
@@ -84,7 +105,6 @@ struct TrainSmem {
   __nv_bfloat16 x[kTrRows * kSIn], h1[kTrRows * kSHid], h2[kTrRows * kSHid];
   __nv_bfloat16 d3[kTrRows * kSOutB], d2[kTrRows * kSHid], d1[kTrRows * kSHid];
   float logits[kTrRows * kSOut];
-  float red[kTrThreads], colsum[2][kHid];
   float lossw[kTrThreads / 32];
   int32_t label[kTrRows], ncand[kTrRows];
 };
@@ -94,11 +114,6 @@ __device__ __forceinline__ void ldsm4t(uint32_t &r0, uint32_t &r1, uint32_t &r2,
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(a) : "memory");
 }
-__device__ __forceinline__ void ldsm2t(uint32_t &r0, uint32_t &r1, const __nv_bfloat16 *p) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(a) : "memory");
-}
-
 // d[4] (+)= a row-major 16 x K tile of `in` (row stride SA, first row row0) times B from wt ([n][k], stride SB) at
 // columns n0 .. n0 + 7.
 template <int K, int SA, int SB>
@@ -112,21 +127,77 @@ __device__ __forceinline__ void tile_mma(float d[4], const __nv_bfloat16 *in, in
              ld_pair(a_hi + kt * 16 + 8), ld_pair(bp + kt * 16), ld_pair(bp + kt * 16 + 8));
 }
 
-// acc[NT][4] += (columns m0 .. m0 + 15 of `a`)^T (columns n0 .. of `b`) over the tile's 32 rows: NT n-tiles of 8.
-template <int NT, int SA, int SB>
-__device__ __forceinline__ void grad_mma(float acc[][4], const __nv_bfloat16 *a, int m0, const __nv_bfloat16 *b, int n0) {
+// Fragment of 16 columns from c0 and 16 rows from k of a row-major tile, transposed, to `out`.  As an A operand the second
+// 8 x 8 matrix holds the next columns, as two B operands the next rows.
+template <bool AS_A, int STRIDE>
+__device__ __forceinline__ void put_fragment(uint4 *out, const __nv_bfloat16 *t, int k, int c0) {
   const int lane = threadIdx.x & 31, r = lane & 7, mat = lane >> 3;
-#pragma unroll
-  for (int k = 0; k < kTrRows; k += 16) {
-    uint32_t a0, a1, a2, a3;
-    ldsm4t(a0, a1, a2, a3, a + (k + (mat >> 1) * 8 + r) * SA + m0 + (mat & 1) * 8);
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      uint32_t b0, b1;
-      ldsm2t(b0, b1, b + (k + (mat & 1) * 8 + r) * SB + n0 + t * 8);
-      mma_bf16(acc[t][0], acc[t][1], acc[t][2], acc[t][3], a0, a1, a2, a3, b0, b1);
-    }
+  const int dk = AS_A ? mat >> 1 : mat & 1, dc = AS_A ? mat & 1 : mat >> 1;
+  uint4 f;
+  ldsm4t(f.x, f.y, f.z, f.w, t + (k + dk * 8 + r) * STRIDE + c0 + dc * 8);
+  __stcg(out + lane, f);
+}
+
+// Phase 2, one 16 x 16 tile of a chunk's weight gradients: dW2 = H1^T dZ2, dW3 = H2^T dZ3, dW1 = X^T dZ1.
+__device__ __forceinline__ void chunk_gradient(const TrainParams &T, int z, int tile) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  int fa, fb, off, ld, m0, n0;
+  if (tile < 16) {
+    fa = kFragH1 + (tile >> 2), fb = kFragD2 + (tile & 3), off = kOffW2, ld = kHid, m0 = (tile >> 2) * 16, n0 = (tile & 3) * 16;
+  } else if (tile < 24) {
+    const int t = tile - 16;
+    fa = kFragH2 + (t >> 1), fb = kFragD3 + (t & 1), off = kOffW3, ld = kOut, m0 = (t >> 1) * 16, n0 = (t & 1) * 16;
+  } else {
+    fa = kFragX, fb = kFragD1 + (tile - 24), off = kOffW1, ld = kHid, m0 = 0, n0 = (tile - 24) * 16;
   }
+  const int64_t s0 = z * T.chunk / 16, s1 = min(T.batch, (z + 1) * T.chunk) / 16;
+  const uint4 *A = T.frag + (s0 * kFrags + fa) * 32 + lane, *B = T.frag + (s0 * kFrags + fb) * 32 + lane;
+  float d[2][4] = {};
+#pragma unroll 8
+  for (int64_t s = s0; s < s1; ++s, A += kFrags * 32, B += kFrags * 32) {
+    const uint4 a = __ldcg(A), b = __ldcg(B);
+    mma_bf16(d[0][0], d[0][1], d[0][2], d[0][3], a.x, a.y, a.z, a.w, b.x, b.y);
+    mma_bf16(d[1][0], d[1][1], d[1][2], d[1][3], a.x, a.y, a.z, a.w, b.z, b.w);
+  }
+  float *G = T.part + (int64_t)z * kNParams + off + (m0 + g) * ld + n0 + 2 * q;
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    __stcg(reinterpret_cast<float2 *>(G + t * 8), make_float2(d[t][0], d[t][1]));
+    if (tile < 24 || g + 8 < kIn) __stcg(reinterpret_cast<float2 *>(G + t * 8 + 8 * ld), make_float2(d[t][2], d[t][3]));
+  }
+}
+
+// Phase 2, columns c and c + 1 of the FP32 deltas: the sum that warp w of k_colsum has.
+__device__ __forceinline__ void column_sums(const TrainParams &T, int c, int w) {
+  const int lane = threadIdx.x & 31;
+  const float *x = T.delta + c * T.delta_ld, *y = x + T.delta_ld;
+  float a = 0.f, b = 0.f;
+#pragma unroll 16
+  for (int64_t r = w * 32 + lane; r < T.batch; r += 32 * kColParts) {
+    a += __ldcg(x + r);
+    b += __ldcg(y + r);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  if (lane == 0)
+    __stcg(reinterpret_cast<float2 *>(T.part + (int64_t)T.chunks * kNParams + w * kCols + c), make_float2(a, b));
+}
+
+// Phase 3, the gradient of parameter p: its partials, in ascending order.
+__device__ __forceinline__ float gradient_of(const TrainParams &T, int p) {
+  int col = -1;
+  if (p >= kOffB3) col = kColZ3 + p - kOffB3;
+  else if (p >= kOffB2 && p < kOffW3) col = kColZ2 + p - kOffB2;
+  else if (p >= kOffB1 && p < kOffW2) col = kColZ1 + p - kOffB1;
+  const float *g = col < 0 ? T.part + p : T.part + (int64_t)T.chunks * kNParams + col;
+  const int n = col < 0 ? T.chunks : kColParts, step = col < 0 ? kNParams : kCols;
+  float s = 0.f;
+#pragma unroll 16
+  for (int i = 0; i < n; ++i) s += __ldcg(g + (int64_t)i * step);
+  return s;
 }
 
 // Parameter p of value v into the image.
@@ -190,13 +261,13 @@ struct TrainFetch {
   uint32_t bits[2];
 };
 
-__device__ __forceinline__ TrainFetch train_fetch(const TrainParams &T, int64_t step, int tile) {
+__device__ __forceinline__ TrainFetch train_fetch(const TrainParams &T, int64_t step, int64_t tile) {
   TrainFetch f{{0u, 0u}};
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int e = threadIdx.x + j * kTrThreads;
     const int r = e / (kIn + 2), k = e % (kIn + 2);
-    const int64_t row = (int64_t)tile * kTrRows + r;
+    const int64_t row = tile * kTrRows + r;
     if (r >= kTrRows || row >= T.batch || step >= T.steps) continue;
     uint64_t at = (uint64_t)(step * T.batch + row);
     if (T.permuted) at = ((at % (uint64_t)T.n) * T.stride + T.offset) % (uint64_t)T.n;
@@ -222,7 +293,8 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
   TrainSmem &S = *reinterpret_cast<TrainSmem *>(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
   const int wm = (warp & 1) * 16, wn = (warp >> 1) * 16;   // the warp's rows and hidden columns of a tile
-  const int tiles = (T.batch + kTrRows - 1) / kTrRows;
+  const int64_t tiles = (T.batch + kTrRows - 1) / kTrRows;
+  const int tasks = T.chunks * kChunkTiles, wide = (int)gridDim.x * (kTrThreads / 32);
   for (int e = tid; e < kTrRows * kSIn; e += kTrThreads) S.x[e] = __float2bfloat16_rn(0.f);   // columns 9 .. 15 stay zero
   // the share of the parameters that this block updates
   const int share = (kNParams + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -235,16 +307,18 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
   for (int64_t step = 0; step < T.steps; ++step) {
     __syncthreads();
     train_load_weights(S.w, T.img);
-    float gw1[1][4] = {}, gw2[4][4] = {}, gw3[2][4] = {};   // weight gradients: the warp's tiles
-    float gb1[4] = {}, gb2[4] = {}, gb3[4] = {};            // bias gradients: the lane's columns
     float loss = 0.f;
 #pragma unroll 1
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
       train_put(S, next);
       // the next tile's inputs come while this one is worked on
-      const bool more = tile + (int)gridDim.x < tiles;
+      const bool more = tile + gridDim.x < tiles;
       next = train_fetch(T, more ? step : step + 1, more ? tile + gridDim.x : blockIdx.x);
       __syncthreads();
+      // fragments of the warp: 16-row step fk of the tile, 16 columns from 16 fc
+      const int fk = warp & 1, fc = warp >> 1;
+      uint4 *frag = T.frag + (tile * 2 + fk) * (kFrags * 32);
+      float *delta = T.delta + tile * kTrRows;
       // forward; the pre-activations and their erf stay in registers for the backward pass
       float z1[2][4], e1[2][4], z2[2][4], e2[2][4];
 #pragma unroll
@@ -262,6 +336,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
         *reinterpret_cast<__nv_bfloat162 *>(S.h1 + (wm + g + 8) * kSHid + col) = __floats2bfloat162_rn(h[2], h[3]);
       }
       __syncthreads();
+      put_fragment<true, kSHid>(frag + (kFragH1 + fc) * 32, S.h1, fk * 16, fc * 16);
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
         const int col = wn + t * 8 + 2 * q;
@@ -277,6 +352,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
         *reinterpret_cast<__nv_bfloat162 *>(S.h2 + (wm + g + 8) * kSHid + col) = __floats2bfloat162_rn(h[2], h[3]);
       }
       __syncthreads();
+      put_fragment<true, kSHid>(frag + (kFragH2 + fc) * 32, S.h2, fk * 16, fc * 16);
       {
         const int n0 = (warp >> 1) * 8, col = n0 + 2 * q;
         float d[4] = {0.f, 0.f, 0.f, 0.f};
@@ -312,11 +388,13 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
           const float p = c < nc ? expf(zz[j] - lse) : 0.f;
           const float dz = valid ? (p - (c == y ? 1.f : 0.f)) * T.inv_scale : 0.f;
           if (valid && c == y) loss += lse - zz[j];
-          gb3[j] += dz;
+          __stcg(delta + (kColZ3 + c) * T.delta_ld + r, dz);
           S.d3[r * kSOutB + c] = __float2bfloat16_rn(dz);
         }
       }
       __syncthreads();
+      if (fc < 2) put_fragment<false, kSOutB>(frag + (kFragD3 + fc) * 32, S.d3, fk * 16, fc * 16);
+      else if (fc == 2) put_fragment<true, kSIn>(frag + kFragX * 32, S.x, fk * 16, 0);
 #pragma unroll
       for (int t = 0; t < 2; ++t) {  // dZ2 = (dZ3 W3^T) gelu'(Z2)
         const int col = wn + t * 8 + 2 * q;
@@ -325,13 +403,13 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           d[i] *= gelu_grad(z2[t][i], e2[t][i]);
-          gb2[2 * t + (i & 1)] += d[i];
+          __stcg(delta + (kColZ2 + col + (i & 1)) * T.delta_ld + wm + g + 8 * (i >> 1), d[i]);
         }
         *reinterpret_cast<__nv_bfloat162 *>(S.d2 + (wm + g) * kSHid + col) = __floats2bfloat162_rn(d[0], d[1]);
         *reinterpret_cast<__nv_bfloat162 *>(S.d2 + (wm + g + 8) * kSHid + col) = __floats2bfloat162_rn(d[2], d[3]);
       }
-      grad_mma<2, kSHid, kSOutB>(gw3, S.h2, (warp & 3) * 16, S.d3, (warp >> 2) * 16);   // dW3 = H2^T dZ3
       __syncthreads();
+      put_fragment<false, kSHid>(frag + (kFragD2 + fc) * 32, S.d2, fk * 16, fc * 16);
 #pragma unroll
       for (int t = 0; t < 2; ++t) {  // dZ1 = (dZ2 W2^T) gelu'(Z1)
         const int col = wn + t * 8 + 2 * q;
@@ -340,109 +418,54 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           d[i] *= gelu_grad(z1[t][i], e1[t][i]);
-          gb1[2 * t + (i & 1)] += d[i];
+          __stcg(delta + (kColZ1 + col + (i & 1)) * T.delta_ld + wm + g + 8 * (i >> 1), d[i]);
         }
         *reinterpret_cast<__nv_bfloat162 *>(S.d1 + (wm + g) * kSHid + col) = __floats2bfloat162_rn(d[0], d[1]);
         *reinterpret_cast<__nv_bfloat162 *>(S.d1 + (wm + g + 8) * kSHid + col) = __floats2bfloat162_rn(d[2], d[3]);
       }
-      grad_mma<4, kSHid, kSHid>(gw2, S.h1, (warp & 3) * 16, S.d2, (warp >> 2) * 32);    // dW2 = H1^T dZ2
       __syncthreads();
-      grad_mma<1, kSIn, kSHid>(gw1, S.x, 0, S.d1, warp * 8);                            // dW1 = X^T dZ1
-      __syncthreads();   // the tile's buffers are free
-    }
-    // the block's partial gradients
-    float *G = T.part + (int64_t)blockIdx.x * kNParams;
-    {
-      const int m0 = (warp & 3) * 16 + g;
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        float *c = G + kOffW3 + m0 * kOut + (warp >> 2) * 16 + t * 8 + 2 * q;
-        *reinterpret_cast<float2 *>(c) = make_float2(gw3[t][0], gw3[t][1]);
-        *reinterpret_cast<float2 *>(c + 8 * kOut) = make_float2(gw3[t][2], gw3[t][3]);
-      }
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        float *c = G + kOffW2 + m0 * kHid + (warp >> 2) * 32 + t * 8 + 2 * q;
-        *reinterpret_cast<float2 *>(c) = make_float2(gw2[t][0], gw2[t][1]);
-        *reinterpret_cast<float2 *>(c + 8 * kHid) = make_float2(gw2[t][2], gw2[t][3]);
-      }
-      float *c = G + kOffW1 + g * kHid + warp * 8 + 2 * q;
-      *reinterpret_cast<float2 *>(c) = make_float2(gw1[0][0], gw1[0][1]);
-      if (g + 8 < kIn) *reinterpret_cast<float2 *>(c + 8 * kHid) = make_float2(gw1[0][2], gw1[0][3]);
-    }
-#pragma unroll
-    for (int w = 0; w < 2; ++w) {   // column sums of dZ2, dZ1: over the lanes' rows, then the two row halves
-      float *gb = w == 0 ? gb2 : gb1;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) gb[i] += __shfl_xor_sync(0xffffffffu, gb[i], o);
-      if (g == 0)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) S.colsum[warp & 1][wn + (i >> 1) * 8 + 2 * q + (i & 1)] = gb[i];
-      __syncthreads();
-      if (tid < kHid) G[(w == 0 ? kOffB2 : kOffB1) + tid] = S.colsum[0][tid] + S.colsum[1][tid];
-      __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      gb3[j] += __shfl_xor_sync(0xffffffffu, gb3[j], 8);
-      gb3[j] += __shfl_xor_sync(0xffffffffu, gb3[j], 16);
-      if (lane < 8) S.red[warp * kOut + lane + 8 * j] = gb3[j];
+      put_fragment<false, kSHid>(frag + (kFragD1 + fc) * 32, S.d1, fk * 16, fc * 16);
+      // S.x, S.label and S.ncand are rewritten for the next tile: their readers are past the barrier above
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
     if (lane == 0) S.lossw[warp] = loss;
     __syncthreads();
-    if (tid < kOut) {
-      float s = 0.f;
-#pragma unroll
-      for (int w = 0; w < kTrThreads / 32; ++w) s += S.red[w * kOut + tid];
-      G[kOffB3 + tid] = s;
-    }
     if (tid == 0) {
       double l = 0.0;
 #pragma unroll
       for (int w = 0; w < kTrThreads / 32; ++w) l += (double)S.lossw[w];
       T.part_loss[blockIdx.x] = step == 0 ? l : T.part_loss[blockIdx.x] + l;
     }
-    // the first 64 parameters of the share and their moments are on their way while the barrier is waited for
-    const int pf = p0 + (tid & 63);
-    const bool own = T.M && tid < 64 && pf < p1;
-    float pv = own ? T.P[pf] : 0.f, mv = own ? T.M[pf] : 0.f, vv = own ? T.V[pf] : 0.f;
     if (!grid_barrier(T.ctrl, ++barriers)) return;
-    // gradients of the block's share: four groups of 64 threads take a quarter of the partials each
+    for (int task = (int)blockIdx.x + (int)gridDim.x * warp; task < tasks + kCols / 2 * kColParts; task += wide) {
+      if (task < tasks) chunk_gradient(T, task / kChunkTiles, task % kChunkTiles);
+      else column_sums(T, (task - tasks) / kColParts * 2, (task - tasks) % kColParts);
+    }
+    // the first parameters of the share and their moments are on their way while the barrier is waited for
+    const bool own = T.M && p0 + tid < p1;
+    float pv = own ? T.P[p0 + tid] : 0.f, mv = own ? T.M[p0 + tid] : 0.f, vv = own ? T.V[p0 + tid] : 0.f;
+    if (!grid_barrier(T.ctrl, ++barriers)) return;
     const float2 corr = T.M ? T.bias_corr[step] : make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int base = p0; base < p1; base += 64) {
-      const int p = base + (tid & 63), quarter = tid >> 6;
-      float s = 0.f;
-      if (p < p1) {
-#pragma unroll 8
-        for (int b = quarter; b < (int)gridDim.x; b += 4) s += __ldcg(T.part + (int64_t)b * kNParams + p);
+    for (int p = p0 + tid; p < p1; p += kTrThreads) {
+      const float gr = gradient_of(T, p);
+      if (!T.M) {
+        T.grads[p] = gr;
+        continue;
       }
-      S.red[tid] = s;
-      __syncthreads();
-      if (tid < 64 && p < p1) {
-        const float gr = (S.red[tid] + S.red[tid + 64]) + (S.red[tid + 128] + S.red[tid + 192]);
-        if (!T.M) {
-          T.grads[p] = gr;
-        } else {
-          if (base > p0) {
-            pv = T.P[p];
-            mv = T.M[p];
-            vv = T.V[p];
-          }
-          const float m = T.b1 * mv + (1.f - T.b1) * gr;
-          const float v = T.b2 * vv + (1.f - T.b2) * gr * gr;
-          pv -= T.lr * (m * corr.x) / (sqrtf(v * corr.y) + T.eps);
-          T.M[p] = m;
-          T.V[p] = v;
-          T.P[p] = pv;
-          train_image(*T.img, p, pv);
-        }
+      if (p != p0 + tid) {
+        pv = T.P[p];
+        mv = T.M[p];
+        vv = T.V[p];
       }
-      __syncthreads();
+      const float m = T.b1 * mv + (1.f - T.b1) * gr;
+      const float v = T.b2 * vv + (1.f - T.b2) * gr * gr;
+      pv -= T.lr * (m * corr.x) / (sqrtf(v * corr.y) + T.eps);
+      T.M[p] = m;
+      T.V[p] = v;
+      T.P[p] = pv;
+      train_image(*T.img, p, pv);
     }
     if (!grid_barrier(T.ctrl, ++barriers)) return;
   }

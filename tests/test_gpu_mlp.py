@@ -295,3 +295,58 @@ def test_predict_rows_and_activation_range(env, n, scale):
     e2 = u * np.abs(h2) + 1.13 * (e1 @ np.abs(W2) + f * (np.abs(h1) @ np.abs(W2) + np.abs(b2))) + 1e-6
     e3 = e2 @ np.abs(W3) + f * (np.abs(h2) @ np.abs(W3) + np.abs(b3)) + 1e-6
     assert np.all(np.abs(full - ref) <= e3)
+
+
+def gradient_chunk(n):
+    """Rows of a partial weight gradient: 256 or a little more, a multiple of 16, at most 256 partials."""
+    split = max(1, min(256, n // 256))
+    return -(-(-(-n // split)) // 16) * 16
+
+
+@pytest.mark.parametrize("n", [1024, 1088, 2048, 2176, 4096])
+def test_gradient_is_the_ascending_sum_of_its_chunks(env, n):
+    """Training's rounding of the weights to BF16 makes another grouping of a gradient's sums another training: a weight
+    gradient over many rows is, bit for bit, the FP32 sum of the chunks' gradients in ascending order.  The number of
+    chunks is a power of two, so that a chunk's own gradient (a mean over its rows) scales exactly."""
+    g4, torch, ctx = env
+    g4.g4n_mlp_load(ctx, params(41))
+    X, y, nc = random_data(n, 42)
+    T = lambda a: torch.tensor(np.ascontiguousarray(a), device="cuda")
+    chunk = gradient_chunk(n)
+    chunks = n // chunk
+    assert chunk * chunks == n and chunks & (chunks - 1) == 0 and chunk < 512
+    want = np.zeros(omlp.N_PARAMS, dtype=np.float32)
+    for z in range(chunks):
+        rows = slice(z * chunk, (z + 1) * chunk)
+        want += g4.g4n_mlp_grad(ctx, T(X[rows]), T(y[rows]), T(nc[rows]))[1] * np.float32(1.0 / chunks)
+    got = omlp.unpack(g4.g4n_mlp_grad(ctx, T(X), T(y), T(nc))[1])
+    for name, k in (("W1", 0), ("W2", 2), ("W3", 4)):
+        assert np.array_equal(got[k], omlp.unpack(want)[k]), name
+
+
+def test_bias_gradient_is_the_column_sum(env):
+    """The order of a bias gradient's sum: 256 partial sums of every 256th row, a butterfly over 32 of them, the eight
+    results in ascending order; bit for bit.  A row's own term comes from a batch of it and rows without a gradient (one
+    candidate: its probability is one)."""
+    g4, torch, ctx = env
+    n = 1024
+    g4.g4n_mlp_load(ctx, params(43))
+    X, y, nc = random_data(n, 44)
+    T = lambda a: torch.tensor(np.ascontiguousarray(a), device="cuda")
+    bias = lambda g: np.concatenate([omlp.unpack(g)[k].ravel() for k in (1, 3, 5)])
+    feat, label, ncand = T(X), T(y), T(nc)
+    F, L, N = feat[:16].clone(), torch.zeros(16, dtype=torch.int32, device="cuda"), torch.ones(16, dtype=torch.int32, device="cuda")
+    rows = np.empty((n, 160), dtype=np.float32)
+    for r in range(n):
+        F[0], L[0], N[0] = feat[r], label[r], ncand[r]
+        rows[r] = bias(g4.g4n_mlp_grad(ctx, F, L, N)[1]) * np.float32(16.0 / n)
+    acc = np.zeros((256, 160), dtype=np.float32)
+    for j in range(n // 256):
+        acc += rows[256 * j:256 * (j + 1)]
+    acc = acc.reshape(8, 32, 160)
+    for o in (16, 8, 4, 2, 1):
+        acc = acc + acc[:, np.arange(32) ^ o]
+    want = np.zeros(160, dtype=np.float32)
+    for w in range(8):
+        want += acc[w, 0]
+    assert np.array_equal(bias(g4.g4n_mlp_grad(ctx, feat, label, ncand)[1]), want)

@@ -105,7 +105,7 @@ struct TrainSmem {
   __nv_bfloat16 x[kTrRows * kSIn], h1[kTrRows * kSHid], h2[kTrRows * kSHid];
   __nv_bfloat16 d3[kTrRows * kSOutB], d2[kTrRows * kSHid], d1[kTrRows * kSHid];
   float logits[kTrRows * kSOut];
-  float lossw[kTrThreads / 32];
+  double lossw[kTrThreads / 32];
   int32_t label[kTrRows], ncand[kTrRows];
 };
 
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
   for (int64_t step = 0; step < T.steps; ++step) {
     __syncthreads();
     train_load_weights(S.w, T.img);
-    float loss = 0.f;
+    double loss = 0.0;   // every row in FP64, as the plain kernel adds them
 #pragma unroll 1
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
       train_put(S, next);
@@ -382,15 +382,17 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
           for (int o = 0; o < 8; ++o) s += __shfl_sync(0xffffffffu, ex, o, 8);
         }
         const float lse = mx + logf(s);
+        float row_loss = 0.f;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int c = sub + 8 * j;
           const float p = c < nc ? expf(zz[j] - lse) : 0.f;
           const float dz = valid ? (p - (c == y ? 1.f : 0.f)) * T.inv_scale : 0.f;
-          if (valid && c == y) loss += lse - zz[j];
+          if (valid && c == y) row_loss = lse - zz[j];
           __stcg(delta + (kColZ3 + c) * T.delta_ld + r, dz);
           S.d3[r * kSOutB + c] = __float2bfloat16_rn(dz);
         }
+        loss += (double)row_loss;
       }
       __syncthreads();
       if (fc < 2) put_fragment<false, kSOutB>(frag + (kFragD3 + fc) * 32, S.d3, fk * 16, fc * 16);
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
     if (tid == 0) {
       double l = 0.0;
 #pragma unroll
-      for (int w = 0; w < kTrThreads / 32; ++w) l += (double)S.lossw[w];
+      for (int w = 0; w < kTrThreads / 32; ++w) l += S.lossw[w];
       T.part_loss[blockIdx.x] = step == 0 ? l : T.part_loss[blockIdx.x] + l;
     }
     if (!grid_barrier(T.ctrl, ++barriers)) return;

@@ -350,3 +350,18 @@ def test_bias_gradient_is_the_column_sum(env):
     for w in range(8):
         want += acc[w, 0]
     assert np.array_equal(bias(g4.g4n_mlp_grad(ctx, feat, label, ncand)[1]), want)
+
+
+def test_loss_of_many_rows_is_summed_in_fp64(env):
+    """A row's loss is an FP32 value, their sum is not: the loss over 2^17 rows is that of its parts of 512 rows, whose sums the
+    plain kernels take row by row in FP64.  Tolerance: a rounding of 2^-53 per row."""
+    g4, torch, ctx = env
+    n = 1 << 17
+    g4.g4n_mlp_load(ctx, params(45))
+    X, y, nc = random_data(n, 46)
+    T = lambda a: torch.tensor(np.ascontiguousarray(a), device="cuda")
+    feat, label, ncand = T(X), T(y), T(nc)
+    parts = [g4.g4n_mlp_grad(ctx, feat[k:k + 512], label[k:k + 512], ncand[k:k + 512])[0] for k in range(0, n, 512)]
+    want = math.fsum(parts) / len(parts)
+    loss, _ = g4.g4n_mlp_grad(ctx, feat, label, ncand)
+    assert abs(loss - want) <= n * 2.0 ** -53 * want, (loss, want)

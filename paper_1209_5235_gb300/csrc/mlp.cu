@@ -354,8 +354,10 @@ void free_train(MlpState *s) {
   s->train_rows = s->corr_cap = 0;
 }
 
-// Buffers of k_mlp_train for `steps` minibatches of `rows` rows (every use of them has ended: run_train waits for its kernel).
-int ensure_train(g4n_ctx *ctx, MlpState *s, int64_t rows, int64_t steps) {
+// Buffers of k_mlp_train for `steps` minibatches of `rows` rows, to be used on `st` (every earlier use has ended: run_train waits
+// for its kernel).  The image's padding is cleared on `st`: the default stream does not order a clear before the kernels of
+// a non-blocking one.
+int ensure_train(g4n_ctx *ctx, MlpState *s, int64_t rows, int64_t steps, cudaStream_t st) {
   const size_t ld = (size_t)(rows + kTrRows - 1) / kTrRows * kTrRows;
   bool ok = true;
   if (!s->ctrl)
@@ -363,7 +365,7 @@ int ensure_train(g4n_ctx *ctx, MlpState *s, int64_t rows, int64_t steps) {
          cudaMalloc(&s->part_loss, (size_t)ctx->sm_count * 8) == cudaSuccess &&
          cudaMalloc(&s->ctrl, sizeof(TrainCtrl)) == cudaSuccess &&
          cudaMalloc(&s->timg, sizeof(TrainWeights)) == cudaSuccess &&
-         cudaMemset(s->timg, 0, sizeof(TrainWeights)) == cudaSuccess;
+         cudaMemsetAsync(s->timg, 0, sizeof(TrainWeights), st) == cudaSuccess;
   if (ok && s->train_rows < rows) {
     cudaFree(s->frag);
     cudaFree(s->delta);
@@ -540,7 +542,7 @@ int g4n_mlp_grad(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *labe
   MlpState *s = state(ctx);
   double loss = 0.0;
   if (precision == 0 && n >= kFusedRows) {
-    if ((rc = ensure_train(ctx, s, n, 0))) return rc;
+    if ((rc = ensure_train(ctx, s, n, 0, 0))) return rc;
     TrainParams T{};
     T.n = n;
     T.feat = feat;
@@ -575,7 +577,7 @@ int g4n_mlp_train(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *lab
   const int64_t nb = n / batch;
   if (nb > INT32_MAX) return g4n_fail(ctx, G4N_ERR_ARG, "mlp_train: too many minibatches");
   const bool fused = batch >= kFusedTrainRows;
-  if ((rc = fused ? ensure_train(ctx, s, batch, nb) : ensure_scratch(ctx, s, batch))) return rc;
+  if ((rc = fused ? ensure_train(ctx, s, batch, nb, st) : ensure_scratch(ctx, s, batch))) return rc;
   std::unique_ptr<float2[]> corr(new (std::nothrow) float2[(size_t)nb]);
   if (!corr) return g4n_fail(ctx, G4N_ERR_OOM, "mlp_train: allocation failed");
   for (int ep = 0; ep < epochs; ++ep) {

@@ -365,3 +365,26 @@ def test_loss_of_many_rows_is_summed_in_fp64(env):
     want = math.fsum(parts) / len(parts)
     loss, _ = g4.g4n_mlp_grad(ctx, feat, label, ncand)
     assert abs(loss - want) <= n * 2.0 ** -53 * want, (loss, want)
+
+
+def test_first_training_on_a_side_stream(env):
+    """The buffers of a context's first training are made ready on the training's own stream: with work queued on the default
+    stream, which a side stream does not wait for, its weights are those of a training on an idle device."""
+    g4, torch, _ = env
+    X, y, nc = random_data(4096, 48)
+    data = [torch.tensor(a, device="cuda") for a in (X, y, nc)]
+    got = []
+    for busy in (False, True):
+        ctx = g4.g4n_create(0)
+        try:
+            g4.g4n_mlp_load(ctx, params(47))
+            torch.cuda.synchronize()
+            side = torch.cuda.Stream()
+            if busy:
+                torch.cuda._sleep(200_000_000)   # cycles: a tenth of a second of the default stream
+            g4.g4n_mlp_train(ctx, *data, epochs=2, batch=2048, lr=2e-3, seed=3, stream=side)
+            torch.cuda.synchronize()
+            got.append(g4.g4n_mlp_get(ctx))
+        finally:
+            g4.g4n_destroy(ctx)
+    assert np.array_equal(got[0], got[1])

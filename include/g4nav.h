@@ -407,7 +407,9 @@ int g4n_mlp_log(g4n_ctx *ctx, const g4n_batch_desc *batch, float *feat, int32_t 
 /* Train on n logged samples (DEVICE buffers as above) with this library's kernels: BF16
  * tensor-core GEMMs with FP32 accumulation, masked softmax cross-entropy, Adam (lr, beta
  * 0.9/0.999) on FP32 master weights.  Minibatches of `batch` (multiple of 16) per epoch from a
- * seeded permutation.  out_loss: HOST array of `epochs` mean losses, or NULL.  Synchronous. */
+ * seeded permutation.  out_loss: HOST array of `epochs` mean losses, or NULL.  Synchronous.
+ * G4N_ERR_TIMEOUT (a capped wait inside an epoch gave up): parameters and optimizer state are those
+ * at the beginning of that epoch. */
 int g4n_mlp_train(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *label, const int32_t *ncand,
                   int32_t epochs, int32_t batch, float lr, uint64_t seed, float *out_loss, g4n_stream stream);
 

@@ -286,3 +286,5 @@ struct SmemWeights;
 // Device image of the loaded MLP weights (null if none) and its release.
 const g4n::mlp::SmemWeights *g4n_mlp_image(g4n_ctx *ctx);
 void g4n_mlp_free(g4n_ctx *ctx);
+// Polls after which a grid barrier of the loaded network's training gives up (0: the default, seconds).
+extern "C" void g4n_mlp_barrier_cap(g4n_ctx *ctx, uint32_t polls);

@@ -253,6 +253,8 @@ struct MlpState {
   TrainWeights *timg = nullptr;
   float2 *corr = nullptr;
   int64_t corr_cap = 0;
+  float *kept = nullptr;
+  unsigned polls = kBarrierPolls;
 };
 
 MlpState *state(g4n_ctx *ctx) { return reinterpret_cast<MlpState *>(ctx->mlp); }
@@ -344,9 +346,9 @@ void forward_backward(MlpState *s, bool bf16, int64_t rows, const float *feat, c
 
 void free_train(MlpState *s) {
   cudaFree(s->frag); cudaFree(s->delta); cudaFree(s->part); cudaFree(s->part_loss); cudaFree(s->ctrl); cudaFree(s->timg);
-  cudaFree(s->corr);
+  cudaFree(s->corr); cudaFree(s->kept);
   s->frag = nullptr;
-  s->delta = s->part = nullptr;
+  s->delta = s->part = s->kept = nullptr;
   s->part_loss = nullptr;
   s->ctrl = nullptr;
   s->timg = nullptr;
@@ -363,6 +365,7 @@ int ensure_train(g4n_ctx *ctx, MlpState *s, int64_t rows, int64_t steps, cudaStr
   if (!s->ctrl)
     ok = cudaMalloc(&s->part, ((size_t)kMaxChunks * kNParams + kColParts * kCols) * 4) == cudaSuccess &&
          cudaMalloc(&s->part_loss, (size_t)ctx->sm_count * 8) == cudaSuccess &&
+         cudaMalloc(&s->kept, 3 * kNParams * 4) == cudaSuccess &&
          cudaMalloc(&s->ctrl, sizeof(TrainCtrl)) == cudaSuccess &&
          cudaMalloc(&s->timg, sizeof(TrainWeights)) == cudaSuccess &&
          cudaMemsetAsync(s->timg, 0, sizeof(TrainWeights), st) == cudaSuccess;
@@ -393,6 +396,7 @@ int ensure_train(g4n_ctx *ctx, MlpState *s, int64_t rows, int64_t steps, cudaStr
 
 // Run k_mlp_train on `st` and wait for it: a block per tile of 32 rows, or a warp per task of the gradients where those are
 // more (4096 rows: 128 tiles, 136 blocks for 1088 tasks), at most a block per SM.  *loss = sum of the losses.
+// A launch whose barrier gave up leaves the parameters and moments as it found them.
 int run_train(g4n_ctx *ctx, MlpState *s, TrainParams &T, double *loss, cudaStream_t st) {
   T.P = s->P;
   T.b1 = 0.9f;
@@ -407,6 +411,8 @@ int run_train(g4n_ctx *ctx, MlpState *s, TrainParams &T, double *loss, cudaStrea
   T.part_loss = s->part_loss;
   T.bias_corr = s->corr;
   T.ctrl = s->ctrl;
+  T.polls = s->polls;
+  T.kept = s->kept;
   T.img = s->timg;
   const int64_t tasks = (int64_t)T.chunks * kChunkTiles + kCols / 2 * kColParts;
   const int grid = (int)std::min<int64_t>(std::max(T.delta_ld / kTrRows, (tasks + 7) / 8), ctx->sm_count);
@@ -419,7 +425,16 @@ int run_train(g4n_ctx *ctx, MlpState *s, TrainParams &T, double *loss, cudaStrea
       cudaMemcpyAsync(&end, s->ctrl, sizeof(end), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return g4n_fail(ctx, G4N_ERR_CUDA, std::string("mlp training: ") + cudaGetErrorString(cudaGetLastError()));
-  if (end.failed) return g4n_fail(ctx, G4N_ERR_TIMEOUT, "mlp training: a grid barrier reached its iteration cap");
+  if (end.failed) {
+    // before every block has kept its share none has updated it
+    if (T.M && end.begun &&
+        (cudaMemcpyAsync(s->P, s->kept, kNParams * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
+         cudaMemcpyAsync(s->M, s->kept + kNParams, kNParams * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
+         cudaMemcpyAsync(s->V, s->kept + 2 * kNParams, kNParams * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
+         cudaStreamSynchronize(st) != cudaSuccess))
+      return g4n_fail(ctx, G4N_ERR_CUDA, std::string("mlp training: ") + cudaGetErrorString(cudaGetLastError()));
+    return g4n_fail(ctx, G4N_ERR_TIMEOUT, "mlp training: a grid barrier reached its iteration cap");
+  }
   *loss = end.loss;
   return G4N_OK;
 }
@@ -506,6 +521,10 @@ int g4n_mlp_load(g4n_ctx *ctx, const float *params) {
   return G4N_OK;
 }
 
+void g4n_mlp_barrier_cap(g4n_ctx *ctx, uint32_t polls) {
+  if (MlpState *s = state(ctx)) s->polls = polls ? polls : kBarrierPolls;
+}
+
 int g4n_mlp_get(g4n_ctx *ctx, float *params) {
   if (!ctx || !params) return g4n_fail(ctx, G4N_ERR_ARG, "mlp_get: null argument");
   MlpState *s = state(ctx);
@@ -590,13 +609,14 @@ int g4n_mlp_train(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *lab
     while (std::gcd(stride, (uint64_t)n) != 1) stride += 2;
     double tot = 0.0;
     for (int64_t k = 0; k < nb; ++k) {
-      ++s->step;
-      corr[k].x = 1.0f / (1.0f - std::pow(0.9f, (float)s->step));
-      corr[k].y = 1.0f / (1.0f - std::pow(0.999f, (float)s->step));
+      const float step = (float)(s->step + k + 1);
+      corr[k].x = 1.0f / (1.0f - std::pow(0.9f, step));
+      corr[k].y = 1.0f / (1.0f - std::pow(0.999f, step));
     }
     const uint64_t offset = (h >> 17) % (uint64_t)n;
     if (!fused) {
       if ((rc = train_plain(ctx, s, n, feat, label, ncand, batch, nb, stride, offset, lr, corr.get(), &tot, st))) return rc;
+      s->step += nb;
       if (out_loss) out_loss[ep] = (float)(tot / ((double)nb * batch));
       continue;
     }
@@ -618,6 +638,7 @@ int g4n_mlp_train(g4n_ctx *ctx, int64_t n, const float *feat, const int32_t *lab
     T.V = s->V;
     T.lr = lr;
     if ((rc = run_train(ctx, s, T, &tot, st))) return rc;
+    s->step += nb;
     k_pack_image<<<8, 256, 0, st>>>(s->P, s->img);
     if (out_loss) out_loss[ep] = (float)(tot / ((double)nb * batch));
   }

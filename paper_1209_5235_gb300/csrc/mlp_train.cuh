@@ -53,6 +53,8 @@ __device__ __forceinline__ float gelu_grad(float x, float e) {  // e = erf(x / s
 struct TrainCtrl {
   unsigned int arrived;   // grid barrier: blocks arrived, over all barriers of the launch
   unsigned int failed;    // a barrier gave up
+  unsigned int begun;     // every block has kept its share of the parameters and moments (TrainParams::kept), updates may have begun
+  unsigned int pad;
   double loss;            // sum of the losses over the launch
 };
 
@@ -77,6 +79,7 @@ struct TrainParams {
   float inv_scale;
   float *P, *M, *V;                 // parameters and Adam moments; M null: gradients of one step into `grads` instead
   float *grads;
+  float *kept;                      // P, M and V as the launch found them, for a caller whose launch fails
   uint4 *frag;                      // [16-row step][kFrags][32]
   float *delta;                     // [kCols][delta_ld]
   int64_t delta_ld;
@@ -85,6 +88,7 @@ struct TrainParams {
   const float2 *bias_corr;          // per step: Adam's 1 / (1 - beta^t)
   float lr, b1, b2, eps;
   TrainCtrl *ctrl;
+  unsigned polls;                   // of a grid barrier before it gives up
   struct TrainWeights *img;
 };
 
@@ -235,8 +239,8 @@ __device__ __forceinline__ void train_load_weights(TrainWeights &S, const TrainW
 }
 
 // Barrier number `k` (1, 2, ...) of the grid (cooperative launch: every block is resident).  A block that has polled
-// kBarrierPolls times sets `failed` and ends; the others see it at their next barrier (or while they poll) and end too.
-__device__ __forceinline__ bool grid_barrier(TrainCtrl *C, unsigned k) {
+// `cap` times sets `failed` and ends; the others see it at their next barrier (or while they poll) and end too.
+__device__ __forceinline__ bool grid_barrier(TrainCtrl *C, unsigned k, unsigned cap) {
   __shared__ bool ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -246,7 +250,7 @@ __device__ __forceinline__ bool grid_barrier(TrainCtrl *C, unsigned k) {
     unsigned polls = 0, seen;
     for (;;) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&C->arrived) : "memory");
-      if ((int)(seen - target) >= 0 || ++polls >= kBarrierPolls) break;
+      if ((int)(seen - target) >= 0 || ++polls >= cap) break;
       if ((polls & 1023u) == 0 && *(volatile unsigned int *)&C->failed) break;
     }
     if ((int)(seen - target) < 0) atomicExch(&C->failed, 1u);
@@ -300,8 +304,17 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
   const int share = (kNParams + (int)gridDim.x - 1) / (int)gridDim.x;
   const int p0 = min(kNParams, (int)blockIdx.x * share), p1 = min(kNParams, p0 + share);
   unsigned barriers = 0;
-  for (int p = p0 + tid; p < p1; p += kTrThreads) train_image(*T.img, p, T.P[p]);
-  if (!grid_barrier(T.ctrl, ++barriers)) return;
+  for (int p = p0 + tid; p < p1; p += kTrThreads) {
+    const float v = T.P[p];
+    train_image(*T.img, p, v);
+    if (T.M) {
+      T.kept[p] = v;
+      T.kept[kNParams + p] = T.M[p];
+      T.kept[2 * kNParams + p] = T.V[p];
+    }
+  }
+  if (!grid_barrier(T.ctrl, ++barriers, T.polls)) return;
+  if (blockIdx.x == 0 && tid == 0) T.ctrl->begun = 1u;
   TrainFetch next = train_fetch(T, 0, blockIdx.x);
 #pragma unroll 1
   for (int64_t step = 0; step < T.steps; ++step) {
@@ -439,7 +452,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
       for (int w = 0; w < kTrThreads / 32; ++w) l += S.lossw[w];
       T.part_loss[blockIdx.x] = step == 0 ? l : T.part_loss[blockIdx.x] + l;
     }
-    if (!grid_barrier(T.ctrl, ++barriers)) return;
+    if (!grid_barrier(T.ctrl, ++barriers, T.polls)) return;
     for (int task = (int)blockIdx.x + (int)gridDim.x * warp; task < tasks + kCols / 2 * kColParts; task += wide) {
       if (task < tasks) chunk_gradient(T, task / kChunkTiles, task % kChunkTiles);
       else column_sums(T, (task - tasks) / kColParts * 2, (task - tasks) % kColParts);
@@ -447,7 +460,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
     // the first parameters of the share and their moments are on their way while the barrier is waited for
     const bool own = T.M && p0 + tid < p1;
     float pv = own ? T.P[p0 + tid] : 0.f, mv = own ? T.M[p0 + tid] : 0.f, vv = own ? T.V[p0 + tid] : 0.f;
-    if (!grid_barrier(T.ctrl, ++barriers)) return;
+    if (!grid_barrier(T.ctrl, ++barriers, T.polls)) return;
     const float2 corr = T.M ? T.bias_corr[step] : make_float2(0.f, 0.f);
 #pragma unroll 1
     for (int p = p0 + tid; p < p1; p += kTrThreads) {
@@ -469,7 +482,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train(const TrainParams T) {
       T.P[p] = pv;
       train_image(*T.img, p, pv);
     }
-    if (!grid_barrier(T.ctrl, ++barriers)) return;
+    if (!grid_barrier(T.ctrl, ++barriers, T.polls)) return;
   }
   if (blockIdx.x == 0 && tid == 0) {
     double l = 0.0;

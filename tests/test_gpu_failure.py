@@ -131,3 +131,49 @@ def test_graph_status_survives_workspace_growth(env):
         assert g4.counters_dict(cnt)["step_limit"] > 0
     finally:
         g4.g4n_graph_destroy(graph)
+
+
+def test_training_barrier_cap_leaves_the_network_as_it_was(env):
+    """A training whose grid barrier gives up (after a few polls, here) reports G4N_ERR_TIMEOUT; parameters, moments, step
+    count and inference image are those before it, wherever it stopped: the training that follows gives the weights of a
+    context that never failed."""
+    import ctypes
+    g4, torch = env[:2]
+    from paper_1209_5235_gb300 import binding
+    from synth.mlp_init import mlp_init
+    rng = np.random.default_rng(3)
+    n = 8 * 2048
+    X = torch.tensor(rng.uniform(-1, 1, (n, 9)).astype(np.float32), device="cuda")
+    nc = torch.tensor(rng.integers(2, 33, n).astype(np.int32), device="cuda")
+    y = torch.minimum(torch.tensor(rng.integers(0, 32, n).astype(np.int32), device="cuda"), nc - 1)
+    train = lambda c: g4.g4n_mlp_train(c, X, y, nc, epochs=1, batch=2048, lr=2e-3, seed=7)
+    cap = binding.load().g4n_mlp_barrier_cap
+    cap.restype, cap.argtypes = None, [ctypes.c_void_p, ctypes.c_uint32]
+    ctxs = [g4.g4n_create(0) for _ in range(2)]
+    try:
+        for c in ctxs:
+            g4.g4n_mlp_load(c, mlp_init(51))
+            train(c)
+        before, logits = g4.g4n_mlp_get(ctxs[0]), g4.g4n_mlp_predict(ctxs[0], X[:64]).cpu().numpy()
+        failed = 0
+        for polls in (1, 2, 4, 8, 16, 32):
+            cap(ctxs[0], polls)
+            try:
+                train(ctxs[0])
+            except g4.G4NError as e:
+                assert e.code == g4.G4N_ERR_TIMEOUT and "barrier" in str(e)
+                failed += 1
+                assert np.array_equal(g4.g4n_mlp_get(ctxs[0]), before)
+                assert np.array_equal(g4.g4n_mlp_predict(ctxs[0], X[:64]).cpu().numpy(), logits)
+            else:
+                break
+        assert failed >= 1
+        cap(ctxs[0], 0)
+        if failed < 6:      # a training went through with few polls: the other context does it as well
+            train(ctxs[1])
+        for c in ctxs:
+            train(c)
+        assert np.array_equal(g4.g4n_mlp_get(ctxs[0]), g4.g4n_mlp_get(ctxs[1]))
+    finally:
+        for c in ctxs:
+            g4.g4n_destroy(c)

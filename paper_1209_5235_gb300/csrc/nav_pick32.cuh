@@ -4,13 +4,19 @@
 // lanes; an FP32 one for half a cycle.  A tube segment's DistanceToIn or DistanceToOut in FP64 evaluates five surfaces
 // with their range tests (seven divisions, two square roots, ~160 FP64 instructions), of which one surface's crossing
 // parameter is the answer.  Here FP32 arithmetic with error bounds finds that surface, and only its parameter is
-// evaluated in FP64 (one division, at most one square root): the same value, because the bounds prove that every other
-// crossing is later, earlier than the start, or not on the solid.  Where they do not prove it the caller takes the full
-// FP64 formulas.
+// evaluated in FP64 (one division, at most one square root): the full formulas' crossing, because the bounds prove that
+// every other one is later, earlier than the start, or not on the solid.  Where they do not prove it the caller takes the
+// full FP64 formulas.
 //
 // A solid along the ray is the interval between its last entry into and its first exit from the half-spaces and the
 // cylinder whose intersection is its convex hull (the Hull below), less the interval inside its bore.  Each crossing
 // parameter is kept as [t - e, t + e].
+//
+// The tolerance band is part of the bounds.  The FP64 formulas accept a crossing up to half a band outside the solid's other
+// surfaces and refuse a start in a band, so a comparison of two crossings has to hold wherever each surface lies within its
+// band: pick_solid adds the band to the bound of the point's error.  At the default tolerance that changes nothing for solids of a millimetre and
+// more (2e-7 of their size in FP32 rounding against 1e-9 mm); solids of 1e-4 mm, or tolerances of 1e-5 of a solid's size,
+// are decided in the full formulas more often.
 //
 // Error bounds.  u = 2^-23.  The FP32 point differs from the exact one by at most ep in each coordinate (the caller's
 // bound: conversions, and the rotation into the solid's frame), sizes and plane normals are within u/2 relative, the
@@ -290,6 +296,7 @@ __device__ __forceinline__ Pick pick_tube(const float *q, int flags, float x, fl
 template <bool ENTER>
 __device__ __forceinline__ Pick pick_solid(int kind, const float *q, int flags, float x, float y, float z, float vx,
                                            float vy, float vz, float ep, float band) {
+  ep += band;   // every surface may lie half a band further in or out
   if (kind == kBox) return pick_box<ENTER>(q, x, y, z, vx, vy, vz, ep, band);
   if (kind == kOrb) return pick_orb<ENTER>(q[0], x, y, z, vx, vy, vz, ep, band);
   if (kind == kTube) return pick_tube<ENTER>(q, flags, x, y, z, vx, vy, vz, ep, band);

@@ -143,7 +143,7 @@ class PortalBuilder {
       const DWorld &w = g.wxf[i];
       size = std::max(size, std::fabs(w.tx) + std::fabs(w.ty) + std::fabs(w.tz) + extent(v));
     }
-    margin = 1e-6 + 1e-9 * size;
+    margin = 1e-6 + 1e-9 * size + 2.0 * tol;   // clear of the band, half a tolerance, at any tolerance scale
     // the band has to be far above the rounding of coordinates of this size (2e-16 each, through a move and a transform)
     // for "in the band" to be certain
     usable = 0.5 * tol >= 4e-14 * size;

@@ -136,3 +136,67 @@ def test_portals_are_the_oracles_relocation(lib, name):
     got = np.where(depth > 0, path[np.arange(len(depth)), np.maximum(depth, 1) - 1], -1)
     bad = np.nonzero(got != np.array(want))[0]
     assert bad.size == 0, (len(want), bad.size, [(pos[i], dirs[i], want[i], got[i]) for i in bad[:3]])
+
+
+def gap_scene(gap):
+    """Solids a gap apart: two boxes, two shells, two segments of a shell, a box on a tube; once about z turned."""
+    from synth.scenes import BOX, TUBE, Placement, Scene, Solid, VoxelSpec
+    base = synth.scenes.tiny_scene()
+    r, w = 100.0, 2 * math.pi
+    solids = [Solid(BOX, (500.0, 500.0, 500.0)), Solid(BOX, (20.0, 30.0, 40.0)), Solid(TUBE, (0.0, 50.0, 60.0, 0.0, w)),
+              Solid(TUBE, (50.0 + gap, r, 60.0, 0.0, w)), Solid(TUBE, (r + gap, 150.0, 60.0, 0.3, 1.0)),
+              Solid(TUBE, (r + gap, 150.0, 60.0, 1.3 + gap / r, 1.0)), Solid(BOX, (30.0, 30.0, 10.0))]
+    c, s = math.cos(0.4), math.sin(0.4)
+    places = [Placement(-1, 0, 0, (0.0, 0.0, 0.0)), Placement(0, 1, 0, (300.0, 200.0, 0.0)),
+              Placement(0, 1, 0, (340.0 + gap, 200.0, 0.0)),
+              Placement(0, 1, 0, (-300.0, 200.0, 0.0), (c, s)),
+              Placement(0, 1, 0, (-300.0 + c * (40.0 + gap), 200.0 + s * (40.0 + gap), 0.0), (c, s)),
+              Placement(0, 2, 0, (0.0, 0.0, 0.0)), Placement(0, 3, 0, (0.0, 0.0, 0.0)), Placement(0, 4, 0, (0.0, 0.0, 0.0)),
+              Placement(0, 5, 0, (0.0, 0.0, 0.0)), Placement(0, 6, 0, (0.0, 0.0, 70.0 + gap), (c, s))]
+    return Scene("gaps", base.materials, solids, places, VoxelSpec(mode="smart"))
+
+
+@pytest.mark.parametrize("scale", [1e3, 1e5, 1e6])
+@pytest.mark.parametrize("part", [0.2, 0.45, 0.7, 3.0])
+def test_portals_know_the_tolerance(lib, scale, part):
+    """Across a gap that is a part of the tolerance 1e-9 mm x scale the far solid's band may hold the crossing point, where the
+    direction decides: with and without the gap in the band a portal is the oracle's relocation."""
+    tol = 1e-9 * scale
+    scene = gap_scene(part * tol)
+    ctx = g4.g4n_create(-1)
+    oracle.set_scale(scale)
+    try:
+        g4.g4n_set_tolerance_scale(ctx, scale)
+        gid = g4.build_scene(ctx, scene)
+        n = lib.portals_of(ctx, gid, None)
+        table = np.zeros(n, dtype=np.int32)
+        lib.portals_of(ctx, gid, table.ctypes.data_as(ctypes.c_void_p))
+        table, frames = table.reshape(-1, 2, 6), world_frames(scene)
+        rng = np.random.default_rng(12)
+        pos, dirs, want = [], [], []
+        for v, pl in enumerate(scene.placements):
+            solid = scene.solids[pl.solid]
+            for face in range(6):
+                for entering in (0, 1):
+                    if table[v, entering, face] == NONE or face_point(rng, solid.kind, solid.params, face, 0.01) is None:
+                        continue
+                    for _ in range(20):
+                        p, nrm = face_point(rng, solid.kind, solid.params, face, 0.01)
+                        d = rng.normal(size=3)
+                        d /= np.linalg.norm(d)
+                        if abs(d @ nrm) < 0.01:
+                            continue
+                        if (d @ nrm > 0) == bool(entering):
+                            d = -d
+                        t, c, s = frames[v]
+                        turn = np.array([[c, -s, 0], [s, c, 0], [0, 0, 1]])
+                        pos.append(turn @ p + t)
+                        dirs.append(turn @ d)
+                        want.append(table[v, entering, face])
+        depth, path = oracle.Geometry(scene).locate_many(np.array(pos), np.array(dirs))
+        got = np.where(depth > 0, path[np.arange(len(depth)), np.maximum(depth, 1) - 1], -1)
+        bad = np.nonzero(got != np.array(want))[0]
+        assert len(want) > 100 and bad.size == 0, (len(want), bad.size, [(pos[i], dirs[i], want[i], got[i]) for i in bad[:3]])
+    finally:
+        oracle.set_scale(1.0)
+        g4.g4n_destroy(ctx)

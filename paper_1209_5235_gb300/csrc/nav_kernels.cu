@@ -239,8 +239,9 @@ __global__ void __launch_bounds__(128, 4) k_compute_step(const DGeom *__restrict
         lim = R.lim;
         safety = R.safety;
       } else {
-        // a float not below the proposal (a NaN proposal limits nothing, a negative one everything)
-        const float f = trunc_float(prop), limit = f < 0.f ? f * (1.0f - 2.0f * kU) : f * (1.0f + 2.0f * kU) + 1e-30f;
+        // a float not below the proposal (a NaN proposal of either sign limits nothing, a negative one everything)
+        const float f = trunc_float(prop);
+        const float limit = isnan(prop) ? kInfF : f < 0.f ? f * (1.0f - 2.0f * kU) : f * (1.0f + 2.0f * kU) + 1e-30f;
         const Step32 R = geom_step32_warp<MODE, false, false>(G, ok, leaf, p, v, limit, true, cnt, &timeout, walk_cap, mc, ch);
         safety = (double)R.safety;
         if (ok) {

@@ -73,3 +73,38 @@ def test_free_path_refills(env, n):
                                   Y[k:k + 1].contiguous(), 1.0)
         assert t1.item() == T[k].item() and s1.item() == steps[k].item()
     assert not torch.isnan(T).any()
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("n", [3001, 1000001])
+def test_compute_step_proposals_at_the_ends(env, mode, n):
+    """A NaN of either sign and +inf limit nothing: the answers without a proposal, bit for bit.  Zeros, negative values, the
+    smallest doubles and -inf come before every boundary: the step is the proposal.  1e300 (beyond any float) limits nothing.
+    The larger n takes the sorted tiles."""
+    g4, torch, ctx = env
+    from synth.mlp_init import mlp_init
+    g4.g4n_mlp_load(ctx, mlp_init(3))
+    gid = g4.build_scene(ctx, synth.scenes.barrel_scene(n_shells=5, n_phi=8, n_orbs=30))
+    p, v = synth.scenes.query_points("barrel", n, 33)
+    pos, dirs = torch.tensor(p, device="cuda"), torch.tensor(v, device="cuda")
+    depth, path = g4.g4n_locate(ctx, gid, pos, dirs)
+    g4.g4n_sync(ctx)
+    run = lambda prop: [a.clone() for a in g4.g4n_compute_step(ctx, gid, pos, dirs, depth, path, proposed=prop, mode=mode)]
+    bits = lambda b: torch.full((n,), b, dtype=torch.int64, device="cuda").view(torch.float64)
+    free = run(None)
+    ok = torch.isfinite(free[0])
+    assert ok.float().mean() > 0.9
+    for b in (0x7ff8000000000000, 0x7ff8000000000000 - (1 << 63), 0x7ff0000000000001, 0x7fffffffffffffff, -1,
+              0x7ff0000000000000):
+        step, safety, lim = run(bits(b))
+        assert torch.equal(step[ok], free[0][ok]) and torch.equal(lim, free[2]), hex(b & (2 ** 64 - 1))
+    step, _, lim = run(torch.full((n,), 1e300, dtype=torch.float64, device="cuda"))
+    assert torch.equal(step[ok], free[0][ok]) and torch.equal(lim, free[2])
+    inside = ok & (free[0] > 0)
+    for value in (0.0, -0.0, 5e-324, -5e-324, -1e-300, -3.0, -1e300, -np.inf):
+        step, _, lim = run(torch.full((n,), value, dtype=torch.float64, device="cuda"))
+        assert torch.all(step[inside] == value) and torch.all(lim[inside] == g4.G4N_LIM_PHYSICS), value
+    try:
+        g4.g4n_sync(ctx)
+    except g4.G4NError:
+        pass

@@ -89,7 +89,7 @@ struct alignas(16) DVol32 {
 struct alignas(64) DPick32 {
   float th[3], tl[3];       // translation = th + tl within 2^-46 of it
   float c, s;
-  float q[7];               // as DVol::p (cones: unused)
+  float q[7];               // as DVol::p (cones: unused); boxes: q[3 .. 5] what the half-lengths q[0 .. 2] lack of DVol::p
   int32_t kind_flags;       // flags << 2 | kind
 };
 static_assert(sizeof(DPick32) == 64, "DPick32 must be 64 bytes");

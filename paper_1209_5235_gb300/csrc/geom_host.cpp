@@ -977,6 +977,8 @@ static int finalize_impl(g4n_ctx *ctx, int32_t *out_geom) {
     w.c = (float)v.c;
     w.s = (float)v.s;
     for (int k = 0; k < 7; ++k) w.q[k] = (float)v.p[k];
+    if (v.kind == kBox)
+      for (int k = 0; k < 3; ++k) w.q[3 + k] = (float)(v.p[k] - (double)w.q[k]);
     w.kind_flags = v.flags << 2 | v.kind;
   }
   // --- validation: containment (surface samples) and sibling overlaps (interior samples)

@@ -47,10 +47,11 @@ constexpr float kU = 1.1920929e-7f;
 constexpr float kPickInf = __builtin_huge_valf();
 
 // Surfaces: boxes 2 axis + (direction component > 0); tubes as below; orbs 0.
-enum PickSurf : int { kPickMiss = -1, kPickUnsure = -2, kPickZ = 0, kPickOuter = 1, kPickInner = 2, kPickStart = 3, kPickEnd = 4 };
+enum PickSurf : int { kPickMiss = -1, kPickUnsure = -2, kPickLeaving = -3, kPickZ = 0, kPickOuter = 1, kPickInner = 2, kPickStart = 3, kPickEnd = 4 };
 
 struct Pick {
-  int surf;       // the surface, kPickMiss (no crossing) or kPickUnsure (the bounds do not decide)
+  int surf;       // the surface, kPickMiss (no crossing), kPickUnsure (the bounds do not decide) or kPickLeaving (a box
+                  // DistanceToIn from inside, or from where it is left: zero or none)
   float lo, hi;   // enclosure of the crossing parameter; unsure: a lower bound in lo
 };
 
@@ -258,6 +259,7 @@ __device__ __forceinline__ Pick pick_box(const float *q, float x, float y, float
   hull_slab(H, y, vy, q[1], ed, 2 + (vy > 0.0f));
   hull_slab(H, z, vz, q[2], ed, 4 + (vz > 0.0f));
   const Bore none{kPickInf, kPickInf, kPickInf, kPickInf};
+  if (ENTER && fmaxf(H.ahi, H.a2hi) < 0.0f && H.bhi >= 0.0f) return Pick{kPickLeaving, 0.f, kPickInf};
   return ENTER ? pick_enter(H, none, band) : pick_exit(H, none);
 }
 
@@ -428,11 +430,33 @@ __device__ __forceinline__ int classify_daughter(const DPick32 &D, const PickRay
   const float ep = pick_to_daughter(D, r, x, v);
   return classify_point(D.kind_flags & 3, D.q, D.kind_flags >> 2, x[0], x[1], x[2], ep, band);
 }
+// Is the ray, from inside box D or from where it leaves it, certainly leaving: does some axis's coordinate lie in or beyond
+// the band of the face that the ray moves to?  Then DistanceToIn is none, else zero.  A track that has just left the
+// box stands 1e-13 from that face, where hull_slab's bounds (7e-7 of the sizes) see no difference to a point inside; the
+// distance from the face as a sum of floats does (the sizes' low parts are q[3 .. 5]): an FP64 test there instead cost the
+// stack of plates 4 %.
+__device__ __forceinline__ bool box_left(const DPick32 &D, const PickRay &r, float band) {
+  bool left = false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // x = p - t as two floats: the difference of the high parts with its rounding, and the low parts' (within 2^-45 of the coordinates)
+    const float h = r.ph[a] - D.th[a], bb = h - r.ph[a];
+    const float l = ((r.ph[a] - (h - bb)) - (D.th[a] + bb)) + (r.pl[a] - D.tl[a]);
+    const bool neg = h < 0.0f;
+    const float gap = (D.q[a] - fabsf(h)) + (D.q[3 + a] - (neg ? -l : l));   // to the face on the point's side
+    const float err = 1e-13f * (fabsf(r.ph[a]) + fabsf(D.th[a]) + D.q[a]) + 4.0f * kU * fabsf(gap);
+    left = left || (gap + err < 0.5f * band * (1.0f - 2.0f * kU) && (neg ? r.v[a] < 0.0f : r.v[a] > 0.0f));
+  }
+  return left;
+}
+
 // DistanceToIn of daughter D of the volume whose frame the ray is given in.
 __device__ __forceinline__ Pick pick_daughter(const DPick32 &D, const PickRay &r, float band) {
   float x[3], v[3];
   const float ep = pick_to_daughter(D, r, x, v);
-  return pick_solid<true>(D.kind_flags & 3, D.q, D.kind_flags >> 2, x[0], x[1], x[2], v[0], v[1], v[2], ep, band);
+  Pick k = pick_solid<true>(D.kind_flags & 3, D.q, D.kind_flags >> 2, x[0], x[1], x[2], v[0], v[1], v[2], ep, band);
+  if (k.surf == kPickLeaving) k.surf = (D.kind_flags >> 2 & kPlacedAligned) && box_left(D, r, band) ? kPickMiss : kPickUnsure;
+  return k;
 }
 
 }  // namespace dev

@@ -108,3 +108,35 @@ def test_compute_step_proposals_at_the_ends(env, mode, n):
         g4.g4n_sync(ctx)
     except g4.G4NError:
         pass
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("name", ["mixed", "calorimeter"])
+def test_compute_step_from_the_mother_of_the_leaf(env, mode, name):
+    """A query may name a volume while its point lies in one of the volume's daughters (a stepping loop that has not yet gone
+    down).  The step is the oracle's: zero into a box.  Tolerance: that of the parity tests, 1e-9 mm."""
+    import oracle
+    from synth.mlp_init import mlp_init
+    from gpu_common import mixed_scene
+    g4, torch, ctx = env
+    g4.g4n_mlp_load(ctx, mlp_init(3))
+    sc = mixed_scene(seed=23, n=200, half=200.0) if name == "mixed" else synth.scenes.calorimeter_scene(
+        nx=4, ny=4, n_layers=6, voxel=synth.scenes.VoxelSpec())
+    og = oracle.Geometry(sc)
+    gid = g4.build_scene(ctx, sc)
+    rng = np.random.default_rng(24)
+    half = np.abs([pl.t for pl in sc.placements[1:] if pl.mother == 0]).max(axis=0) + 10.0
+    p, v = rng.uniform(-half, half, (60000, 3)), rng.normal(size=(60000, 3))
+    v /= np.linalg.norm(v, axis=1)[:, None]
+    depth, path = og.locate_many(p, v)
+    keep = depth > 1
+    p, v, depth, path = p[keep], v[keep], depth[keep] - 1, path[keep]
+    want, lim_ref, _ = og.compute_step_many(p, v, depth, path)
+    T = lambda a, t: torch.tensor(np.ascontiguousarray(a), dtype=t, device="cuda")
+    s, _, lim = g4.g4n_compute_step(ctx, gid, T(p.T, torch.float64), T(v.T, torch.float64), T(depth, torch.int32),
+                                    T(path.T, torch.int32), mode=mode)
+    g4.g4n_sync(ctx)
+    s, lim = s.cpu().numpy(), lim.cpu().numpy()
+    assert len(p) > 1000 and (want == 0.0).sum() > 100
+    assert np.array_equal(lim, lim_ref), (lim != lim_ref).sum()
+    assert np.all(np.abs(s - want) <= 1e-9)

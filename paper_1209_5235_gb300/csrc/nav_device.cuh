@@ -1547,10 +1547,12 @@ __device__ __forceinline__ Step32 geom_step32_warp(const DGeom &G, bool active, 
   return R;
 }
 
-// The step that R names as a quotient for the caller to divide, or exactly: false, with *num = step, where the full
-// formulas or the full search were needed (then *lim is final as well).  *surf: the surface crossed, -1: not known.
+// The step that R names as num / den * mul for the caller to evaluate (mul is 1 but for the exit from a box, (h - p) times the
+// reciprocal of the direction as box_dist_out has it), or exactly: false, with *num = step, where the full formulas or
+// the full search were needed (then *lim is final as well).  *surf: the surface crossed, -1: not known.
 __device__ __forceinline__ bool step_ratio32(const DGeom &G, int leaf, const V3 &p, const V3 &v, const Step32 &R,
-                                             int walk_cap, bool *timeout, double *num, double *den, int *lim, int *surf) {
+                                             int walk_cap, bool *timeout, double *num, double *den, double *mul, int *lim,
+                                             int *surf) {
   *lim = R.vol;
   *surf = -1;
   if (R.undecided || R.surf == kSurfFull) {
@@ -1569,6 +1571,10 @@ __device__ __forceinline__ bool step_ratio32(const DGeom &G, int leaf, const V3 
   if (in) to_local(D, p, v, dp, dv);
   *surf = R.surf;
   surf_ratio(D.kind, D.p, R.surf, in, dp, dv, *num, *den);
+  if (!in && D.kind == kBox) {
+    *mul = *num;
+    *num = 1.0;
+  }
   return true;
 }
 
@@ -1590,9 +1596,9 @@ __device__ __forceinline__ bool step_finish32(const DGeom &G, int leaf, const V3
 // The geometric step that R names.
 __device__ __forceinline__ double step_exact32(const DGeom &G, int leaf, const V3 &p, const V3 &v, const Step32 &R,
                                                int walk_cap, bool *timeout, int *lim, int *surf) {
-  double num, den;
-  if (!step_ratio32(G, leaf, p, v, R, walk_cap, timeout, &num, &den, lim, surf)) return num;
-  double s = num / den;
+  double num, den, mul = 1.0;
+  if (!step_ratio32(G, leaf, p, v, R, walk_cap, timeout, &num, &den, &mul, lim, surf)) return num;
+  double s = num / den * mul;
   step_finish32(G, leaf, p, v, s, walk_cap, timeout, lim, surf);
   return s;
 }

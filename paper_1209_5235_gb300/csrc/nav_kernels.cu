@@ -716,14 +716,14 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       act = false;
     }
     if (act) {
-      double num = t.Y, den = t.mu;
+      double num = t.Y, den = t.mu, mul = 1.0;
       bool quotient = true;
       if (need_geo) {
         t.safety = (double)R.safety;
         geo = !(phys_hi < R.lo);
-        if (geo) quotient = step_ratio32(G, t.leaf, p, v, R, P.walk_cap, &timeout, &num, &den, &lim, &surf);
+        if (geo) quotient = step_ratio32(G, t.leaf, p, v, R, P.walk_cap, &timeout, &num, &den, &mul, &lim, &surf);
       }
-      s = quotient ? (geo || mu_pos ? num / den : kInf) : num;
+      s = quotient ? (geo || mu_pos ? num / den * mul : kInf) : num;
       if (geo) {
         if (quotient) quotient = step_finish32(G, t.leaf, p, v, s, P.walk_cap, &timeout, &lim, &surf);
         // geometry wins iff step <= fl(Y / mu); the enclosures decide unless they overlap

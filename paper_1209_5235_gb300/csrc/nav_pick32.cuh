@@ -4,7 +4,7 @@
 // lanes; an FP32 one for half a cycle.  A tube segment's DistanceToIn or DistanceToOut in FP64 evaluates five surfaces
 // with their range tests (seven divisions, two square roots, ~160 FP64 instructions), of which one surface's crossing
 // parameter is the answer.  Here FP32 arithmetic with error bounds finds that surface, and only its parameter is
-// evaluated in FP64 (one division, at most one square root): the full formulas' crossing, because the bounds prove that
+// evaluated in FP64 (one division, at most one square root): the full formulas' value, because the bounds prove that
 // every other one is later, earlier than the start, or not on the solid.  Where they do not prove it the caller takes the
 // full FP64 formulas.
 //
@@ -305,7 +305,8 @@ __device__ __forceinline__ Pick pick_solid(int kind, const float *q, int flags, 
   return Pick{kPickUnsure, 0.f, kPickInf};   // cones
 }
 
-// The crossing parameter of one surface in FP64 as a quotient num / den, by the formulas of the full tests: planes, and
+// The crossing parameter of one surface in FP64 as a quotient num / den, by the formulas of the full tests and with their
+// operations in their order, for the same bits (nav_solids.cuh's fused sums; a box's exit takes the reciprocal): planes, and
 // circles through the quadratic's root without cancellation (lo: q / a where q < 0, else c / q; hi the other one).  The
 // caller divides: one division for all lanes of a warp whatever their surfaces.  NaN where the quadratic has no root.
 __device__ __forceinline__ void surf_ratio(int kind, const double *p, int surf, bool enter, const V3 &x, const V3 &v,
@@ -319,22 +320,24 @@ __device__ __forceinline__ void surf_ratio(int kind, const double *p, int surf, 
     num = (((v.z < 0.0) == enter) ? p[2] : -p[2]) - x.z;
     den = v.z;
   } else if (kind == kTube && surf >= kPickStart) {
-    const double c = surf == kPickStart ? p[3] : -p[5], s = surf == kPickStart ? p[4] : -p[6];
-    num = c * x.y - s * x.x;
-    den = s * v.x - c * v.y;
+    const bool st = surf == kPickStart;
+    num = cross2(st ? p[3] : p[6], st ? x.y : x.x, st ? p[4] : p[5], st ? x.x : x.y);
+    den = cross2(st ? p[4] : p[5], st ? v.x : v.y, st ? p[3] : p[6], st ? v.y : v.x);
   } else {
-    double a = 1.0, b = x.x * v.x + x.y * v.y, c = x.x * x.x + x.y * x.y;
-    double R = p[0];
-    if (kind == kTube) {
-      a = v.x * v.x + v.y * v.y;
-      if (surf == kPickOuter) R = p[1];
-    } else {
-      b += x.z * v.z;
-      c += x.z * x.z;
+    const bool orb = kind != kTube;
+    const double a = orb ? 1.0 : dot2(v.x, v.x, v.y, v.y), R = !orb && surf == kPickOuter ? p[1] : p[0];
+    // the terms in the order of orb_dist_in, orb_dist_out and tube_cyl_cand
+    const bool by = orb && !enter, cy = !orb || !enter;
+    double b = dot2(by ? x.y : x.x, by ? v.y : v.x, by ? x.x : x.y, by ? v.x : v.y);
+    const double c0 = cy ? x.y : x.x, c1 = cy ? x.x : x.y;
+    double c = dot2(c0, c0, c1, c1);
+    if (orb) {
+      b = fma(x.z, v.z, b);
+      c = fma(x.z, x.z, c);
     }
-    c -= R * R;
-    const double sq = sqrt(b * b - a * c), q = -(b + copysign(sq, b));
-    const bool lo = enter == (kind == kOrb || surf == kPickOuter);
+    c = fma(-R, R, c);
+    const double sq = sqrt(quad_disc(a, b, c)), q = -(b + copysign(sq, b));
+    const bool lo = enter == (orb || surf == kPickOuter);
     const bool direct = lo == (__double2hiint(b) >= 0);   // by q's sign: b may be -0 (a ray from the axis)
     num = direct ? q : c;
     den = direct ? a : q;

@@ -24,6 +24,16 @@ __device__ __forceinline__ long long dkey(double x) {
   return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
 }
 
+// ---------------------------------------------------------------- sums of products
+// Written with their fused operations: the full formulas and the evaluation of one chosen surface (surf_ratio), each in several
+// kernels, have to give the same bits, and the compiler fuses a plain sum of products by the uses of its terms.
+
+// a b + c d and a b - c d.
+__device__ __forceinline__ double dot2(double a, double b, double c, double d) { return fma(a, b, c * d); }
+__device__ __forceinline__ double cross2(double a, double b, double c, double d) { return fma(a, b, -(c * d)); }
+__device__ __forceinline__ double dot3(const V3 &p, const V3 &v) { return fma(p.z, v.z, dot2(p.x, v.x, p.y, v.y)); }
+__device__ __forceinline__ double dot3_yx(const V3 &p, const V3 &v) { return fma(p.z, v.z, dot2(p.y, v.y, p.x, v.x)); }
+
 // ---------------------------------------------------------------- frames
 
 __device__ __forceinline__ void to_local(const DVol &v, const V3 &pm, const V3 &vm, V3 &pl, V3 &vl) {
@@ -33,11 +43,11 @@ __device__ __forceinline__ void to_local(const DVol &v, const V3 &pm, const V3 &
     vl = vm;
     return;
   }
-  pl.x = v.c * dx + v.s * dy;
-  pl.y = v.c * dy - v.s * dx;
+  pl.x = dot2(v.c, dx, v.s, dy);
+  pl.y = cross2(v.c, dy, v.s, dx);
   pl.z = pm.z - v.tz;
-  vl.x = v.c * vm.x + v.s * vm.y;
-  vl.y = v.c * vm.y - v.s * vm.x;
+  vl.x = dot2(v.c, vm.x, v.s, vm.y);
+  vl.y = cross2(v.c, vm.y, v.s, vm.x);
   vl.z = vm.z;
 }
 
@@ -50,11 +60,11 @@ __device__ __forceinline__ void world_to_local(const DWorld &w, bool aligned, co
     vl = u;
     return;
   }
-  pl.x = w.c * dx + w.s * dy;
-  pl.y = w.c * dy - w.s * dx;
+  pl.x = dot2(w.c, dx, w.s, dy);
+  pl.y = cross2(w.c, dy, w.s, dx);
   pl.z = p.z - w.tz;
-  vl.x = w.c * u.x + w.s * u.y;
-  vl.y = w.c * u.y - w.s * u.x;
+  vl.x = dot2(w.c, u.x, w.s, u.y);
+  vl.y = cross2(w.c, u.y, w.s, u.x);
   vl.z = u.z;
 }
 
@@ -62,7 +72,7 @@ __device__ __forceinline__ void world_to_local(const DWorld &w, bool aligned, co
 __device__ __forceinline__ V3 world_to_local_point(const DWorld &w, bool aligned, const V3 &p) {
   const double dx = p.x - w.tx, dy = p.y - w.ty;
   if (aligned) return V3{dx, dy, p.z - w.tz};
-  return V3{w.c * dx + w.s * dy, w.c * dy - w.s * dx, p.z - w.tz};
+  return V3{dot2(w.c, dx, w.s, dy), cross2(w.c, dy, w.s, dx), p.z - w.tz};
 }
 
 // Reciprocal direction components (0 where the component is 0: never used there).
@@ -144,9 +154,12 @@ __device__ __forceinline__ double box_safety_out(const double *h, const V3 &p) {
 
 // ---------------------------------------------------------------- orb
 
+// Discriminant of a t^2 + 2 b t + c.
+__device__ __forceinline__ double quad_disc(double a, double b, double c) { return fma(b, b, -(a * c)); }
+
 // Roots of a t^2 + 2 b t + c = 0 without cancellation; false if the discriminant is not positive.
 __device__ __forceinline__ bool quad_roots(double a, double b, double c, double &lo, double &hi) {
-  const double disc = b * b - a * c;
+  const double disc = quad_disc(a, b, c);
   if (!(disc > 0.0)) return false;
   const double sq = sqrt(disc);
   const double q = -(b + copysign(sq, b));
@@ -165,16 +178,14 @@ __device__ __forceinline__ bool orb_inside(double R, const V3 &p, const V3 &v, d
 }
 
 __device__ __forceinline__ double orb_dist_in(double R, const V3 &p, const V3 &v, double half) {
-  const double b = p.x * v.x + p.y * v.y + p.z * v.z;
-  const double c = p.x * p.x + p.y * p.y + p.z * p.z - R * R;
+  const double b = dot3(p, v), c = fma(-R, R, dot3(p, p));
   double lo, hi;
   if (!quad_roots(1.0, b, c, lo, hi)) return kInf;
   return lo > half ? lo : kInf;
 }
 
 __device__ __forceinline__ double orb_dist_out(double R, const V3 &p, const V3 &v) {
-  const double b = p.x * v.x + p.y * v.y + p.z * v.z;
-  const double c = p.x * p.x + p.y * p.y + p.z * p.z - R * R;
+  const double b = dot3_yx(p, v), c = fma(-R, R, dot3_yx(p, p));
   double lo, hi;
   if (!quad_roots(1.0, b, c, lo, hi)) return 0.0;
   return fmax(hi, 0.0);
@@ -267,13 +278,12 @@ __device__ __forceinline__ double tube_z_cand(const double *q, int flags, const 
 // cylinder of radius R (outer: the root that enters / leaves the solid through rmax; inner: through rmin)
 __device__ __forceinline__ double tube_cyl_cand(const double *q, int flags, const V3 &p, const V3 &v, double half,
                                                 bool enter, double tmin, double best, bool outer) {
-  const double a = v.x * v.x + v.y * v.y;
+  const double a = dot2(v.x, v.x, v.y, v.y);
   if (!(a > 0.0)) return kInf;
-  const double b = p.x * v.x + p.y * v.y;
-  const double r2 = p.x * p.x + p.y * p.y;
+  const double b = dot2(p.x, v.x, p.y, v.y);
   const double R = outer ? q[1] : q[0];
   double lo, hi;
-  if (!quad_roots(a, b, r2 - R * R, lo, hi)) return kInf;
+  if (!quad_roots(a, b, fma(-R, R, dot2(p.y, p.y, p.x, p.x)), lo, hi)) return kInf;
   const double t = (enter == outer) ? lo : hi;
   if (t > tmin && t < best && fabs(p.z + t * v.z) <= q[2] + half &&
       tube_phi_ok(q, flags, p.x + t * v.x, p.y + t * v.y, half))
@@ -285,9 +295,9 @@ __device__ __forceinline__ double tube_cyl_cand(const double *q, int flags, cons
 __device__ __forceinline__ double tube_phi_cand(const double *q, int flags, const V3 &p, const V3 &v, double half,
                                                 bool enter, double tmin, double best, bool start) {
   // v . outward normal of the plane, the signed distance to its line (positive on the solid's side)
-  const double dn = start ? q[4] * v.x - q[3] * v.y : q[5] * v.y - q[6] * v.x;
+  const double dn = start ? cross2(q[4], v.x, q[3], v.y) : cross2(q[5], v.y, q[6], v.x);
   if (!(dn != 0.0 && ((dn < 0.0) == enter))) return kInf;
-  const double t = (start ? q[3] * p.y - q[4] * p.x : q[6] * p.x - q[5] * p.y) / dn;
+  const double t = (start ? cross2(q[3], p.y, q[4], p.x) : cross2(q[6], p.x, q[5], p.y)) / dn;
   if (!(t > tmin && t < best)) return kInf;
   const double qx = p.x + t * v.x, qy = p.y + t * v.y;
   const double along = start ? q[3] * qx + q[4] * qy : q[5] * qx + q[6] * qy;

@@ -140,3 +140,37 @@ def test_compute_step_from_the_mother_of_the_leaf(env, mode, name):
     assert len(p) > 1000 and (want == 0.0).sum() > 100
     assert np.array_equal(lim, lim_ref), (lim != lim_ref).sum()
     assert np.all(np.abs(s - want) <= 1e-9)
+
+
+@pytest.mark.parametrize("name", ["calorimeter", "barrel", "mixed", "cones", "segments"])
+def test_modes_give_the_same_steps(env, name):
+    """The three modes choose the crossed surface in their own ways and evaluate it by the same operations: steps and
+    limiters agree bit for bit, whichever formulas a query ends in."""
+    from synth.mlp_init import mlp_init
+    from gpu_common import cones_scene, mixed_scene, segments_scene
+    g4, torch, ctx = env
+    g4.g4n_mlp_load(ctx, mlp_init(3))
+    n = 200000
+    if name in ("calorimeter", "barrel"):
+        sc = synth.scenes.barrel_scene() if name == "barrel" else synth.scenes.calorimeter_scene(
+            voxel=synth.scenes.VoxelSpec(mode="smart"))
+        p, v = synth.scenes.query_points(name, n, 34)
+    else:
+        sc, half = {"mixed": (mixed_scene(seed=23, n=200, half=200.0), 200.0), "cones": (cones_scene(), 480.0),
+                    "segments": (segments_scene(), 380.0)}[name]
+        rng = np.random.default_rng(35)
+        p, v = rng.uniform(-half, half, (3, n)), rng.normal(size=(3, n))
+        v /= np.linalg.norm(v, axis=0)
+    gid = g4.build_scene(ctx, sc)
+    pos, dirs = torch.tensor(p, device="cuda"), torch.tensor(v, device="cuda")
+    depth, path = g4.g4n_locate(ctx, gid, pos, dirs)
+    prop = torch.tensor(np.random.default_rng(36).exponential(300.0, n), device="cuda")
+    got = [[a.cpu().numpy().copy() for a in g4.g4n_compute_step(ctx, gid, pos, dirs, depth, path, proposed=prop, mode=mode)]
+           for mode in (0, 1, 2)]
+    try:
+        g4.g4n_sync(ctx)
+    except g4.G4NError:
+        pass    # points outside the world
+    for mode in (1, 2):
+        assert np.array_equal(got[mode][2], got[0][2])
+        assert np.array_equal(got[mode][0], got[0][0], equal_nan=True), (got[mode][0] != got[0][0]).sum()

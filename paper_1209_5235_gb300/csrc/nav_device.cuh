@@ -1556,8 +1556,11 @@ __device__ __forceinline__ bool step_ratio32(const DGeom &G, int leaf, const V3 
   *lim = R.vol;
   *surf = -1;
   if (R.undecided || R.surf == kSurfFull) {
-    if (R.undecided || R.vol < 0) {
+    if (R.undecided) {
       search_full(G, leaf, p, v, walk_cap, num, lim, timeout);
+    } else if (R.vol < 0) {
+      // the exit comes first for certain, from a cone or a wide segment, say: that alone
+      *num = vol_dist_out_full(G.vol[leaf], p, v, G.half);
     } else {
       V3 dp, dv;
       to_local(G.vol[R.vol], p, v, dp, dv);

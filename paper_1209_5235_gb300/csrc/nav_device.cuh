@@ -1281,13 +1281,14 @@ __device__ __forceinline__ void enclose_up(double t, float &lo, float &hi) {
   hi = __fmul_ru(lo, 1.0f + 2.0f * kU) + 1e-37f;
 }
 
-// The FP64 search of one lane, every candidate by the full formulas: step and limiter as geom_step_warp's (no safety).
-__device__ __noinline__ void search_full(const DGeom &G, int leaf, const V3 &p, const V3 &v, int walk_cap, double *step,
-                                         int *lim, bool *timeout) {
+// The FP64 search of one lane, every candidate by the full formulas: step and limiter as geom_step_warp's (no safety).  It
+// walks as far as that one does, to `limit` at most: a step beyond it may be any value beyond it.
+__device__ __noinline__ void search_full(const DGeom &G, int leaf, const V3 &p, const V3 &v, float limit, int walk_cap,
+                                         double *step, int *lim, bool *timeout) {
   const DVol &V = G.vol[leaf];
   const Inv3 iv = inv_dir(v);
   int bl = G4N_LIM_MOTHER;
-  const double tout = vol_dist_out_full(V, p, v, G.half);
+  const double tout = vol_dist_out_full(V, p, v, G.half), stop = fmin(tout, (double)limit);
   double best = kInf;
   if (V.vox >= 0) {
     Chain ch;
@@ -1308,7 +1309,7 @@ __device__ __noinline__ void search_full(const DGeom &G, int leaf, const V3 &p, 
           bl = d;
         }
       }
-    } while (walk_step64_ool(G, ch, p, v, iv, fmin(best, tout), false, nullptr, &it, walk_cap, timeout));
+    } while (walk_step64_ool(G, ch, p, v, iv, fmin(best, stop), false, nullptr, &it, walk_cap, timeout));
   }
   const bool in = bl >= 0 && best <= tout;
   *step = in ? best : tout;
@@ -1551,13 +1552,13 @@ __device__ __forceinline__ Step32 geom_step32_warp(const DGeom &G, bool active, 
 // reciprocal of the direction as box_dist_out has it), or exactly: false, with *num = step, where the full formulas or
 // the full search were needed (then *lim is final as well).  *surf: the surface crossed, -1: not known.
 __device__ __forceinline__ bool step_ratio32(const DGeom &G, int leaf, const V3 &p, const V3 &v, const Step32 &R,
-                                             int walk_cap, bool *timeout, double *num, double *den, double *mul, int *lim,
-                                             int *surf) {
+                                             float limit, int walk_cap, bool *timeout, double *num, double *den, double *mul,
+                                             int *lim, int *surf) {
   *lim = R.vol;
   *surf = -1;
   if (R.undecided || R.surf == kSurfFull) {
     if (R.undecided) {
-      search_full(G, leaf, p, v, walk_cap, num, lim, timeout);
+      search_full(G, leaf, p, v, limit, walk_cap, num, lim, timeout);
     } else if (R.vol < 0) {
       // the exit comes first for certain, from a cone or a wide segment, say: that alone
       *num = vol_dist_out_full(G.vol[leaf], p, v, G.half);
@@ -1583,26 +1584,26 @@ __device__ __forceinline__ bool step_ratio32(const DGeom &G, int leaf, const V3 
 
 // The quotient s of step_ratio32 made a step: true if it lies beyond the surface band; else (a crossing at the start, by
 // rounding) s comes from the full search.
-__device__ __forceinline__ bool step_finish32(const DGeom &G, int leaf, const V3 &p, const V3 &v, double &s, int walk_cap,
-                                              bool *timeout, int *lim, int *surf) {
+__device__ __forceinline__ bool step_finish32(const DGeom &G, int leaf, const V3 &p, const V3 &v, double &s, float limit,
+                                              int walk_cap, bool *timeout, int *lim, int *surf) {
   if (s > (*lim >= 0 ? G.half : -G.half)) {
     s = fmax(s, 0.0);
     return true;
   }
   double full;
-  search_full(G, leaf, p, v, walk_cap, &full, lim, timeout);
+  search_full(G, leaf, p, v, limit, walk_cap, &full, lim, timeout);
   s = full;
   *surf = -1;
   return false;
 }
 
-// The geometric step that R names.
+// The geometric step that R names; limit as the search had it.
 __device__ __forceinline__ double step_exact32(const DGeom &G, int leaf, const V3 &p, const V3 &v, const Step32 &R,
-                                               int walk_cap, bool *timeout, int *lim, int *surf) {
+                                               float limit, int walk_cap, bool *timeout, int *lim, int *surf) {
   double num, den, mul = 1.0;
-  if (!step_ratio32(G, leaf, p, v, R, walk_cap, timeout, &num, &den, &mul, lim, surf)) return num;
+  if (!step_ratio32(G, leaf, p, v, R, limit, walk_cap, timeout, &num, &den, &mul, lim, surf)) return num;
   double s = num / den * mul;
-  step_finish32(G, leaf, p, v, s, walk_cap, timeout, lim, surf);
+  step_finish32(G, leaf, p, v, s, limit, walk_cap, timeout, lim, surf);
   return s;
 }
 

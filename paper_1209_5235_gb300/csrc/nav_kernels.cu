@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(128, 4) k_compute_step(const DGeom *__restrict
         if (ok) {
           int surf;
           if (limit < R.lo) lim = G4N_LIM_PHYSICS;   // the proposal comes first for certain
-          else s = step_exact32(G, leaf, p, v, R, walk_cap, &timeout, &lim, &surf);
+          else s = step_exact32(G, leaf, p, v, R, limit, walk_cap, &timeout, &lim, &surf);
         }
       }
       if (ok) {
@@ -721,11 +721,11 @@ __device__ int step_warp(const TParams &P, Track &t, int phase, Counters &cnt, M
       if (need_geo) {
         t.safety = (double)R.safety;
         geo = !(phys_hi < R.lo);
-        if (geo) quotient = step_ratio32(G, t.leaf, p, v, R, P.walk_cap, &timeout, &num, &den, &mul, &lim, &surf);
+        if (geo) quotient = step_ratio32(G, t.leaf, p, v, R, phys_hi, P.walk_cap, &timeout, &num, &den, &mul, &lim, &surf);
       }
       s = quotient ? (geo || mu_pos ? num / den * mul : kInf) : num;
       if (geo) {
-        if (quotient) quotient = step_finish32(G, t.leaf, p, v, s, P.walk_cap, &timeout, &lim, &surf);
+        if (quotient) quotient = step_finish32(G, t.leaf, p, v, s, phys_hi, P.walk_cap, &timeout, &lim, &surf);
         // geometry wins iff step <= fl(Y / mu); the enclosures decide unless they overlap
         if (mu_pos && (!quotient || !(R.hi < phys_lo))) {
           const double sphys = t.Y / t.mu;
@@ -1157,7 +1157,7 @@ __global__ void __launch_bounds__(128, 3) k_free_path(const FParams P) {
     } else {
       const Step32 R = geom_step32_warp<MODE, COUNT>(G, active, active ? leaf : 0, p, v, kInfF, false, cnt, &timeout,
                                                      P.walk_cap, mc, ch);
-      if (active) step = step_exact32(G, leaf, p, v, R, P.walk_cap, &timeout, &lim, &surf);
+      if (active) step = step_exact32(G, leaf, p, v, R, kInfF, P.walk_cap, &timeout, &lim, &surf);
     }
     bool cross = false;
     double s = 0.0;

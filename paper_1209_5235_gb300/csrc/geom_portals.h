@@ -43,14 +43,20 @@ struct PPatch {
   int n = 0;                       // points of a segment (2) or convex polygon (4, in order)
   double px[4], py[4];
   double cx = 0, cy = 0, r0 = 0, r1 = 0, a0 = 0, a1 = 0;
+  double c[2] = {0, 0}, s[2] = {0, 0};   // cosines and sines of a0, a1
   double zlo = 0, zhi = 0;
 };
 
-inline bool angle_in(double t, double a0, double a1) {   // a1 - a0 <= 2 pi
-  double d = std::fmod(t - a0, 2.0 * kPi);
-  if (d < 0) d += 2.0 * kPi;
-  return d <= a1 - a0 + 1e-12;
+// Is the direction (dx, dy) in the patch's angles a0 .. a1 (<= 2 pi), or within 1e-12 of them?  (In is the safe answer: it
+// widens the ranges below.)
+inline bool direction_in(const PPatch &P, double dx, double dy) {
+  const double span = P.a1 - P.a0, tol = 1e-12 * (std::fabs(dx) + std::fabs(dy));
+  if (span > 2.0 * kPi - 1e-9) return true;
+  const bool after = P.c[0] * dy - P.s[0] * dx >= -tol, before = dx * P.s[1] - dy * P.c[1] >= -tol;
+  return span <= kPi ? after && before : after || before;
 }
+
+inline double length(double x, double y) { return std::sqrt(x * x + y * y); }   // (hypot's care for overflow costs 20 ns)
 
 struct PRange {
   double lo = INFINITY, hi = -INFINITY;
@@ -67,19 +73,18 @@ inline PRange range_linear(const PPatch &P, double nx, double ny, double o) {
     for (int i = 0; i < P.n; ++i) r.add(nx * P.px[i] + ny * P.py[i] + o);
     return r;
   }
-  const double c = nx * P.cx + ny * P.cy + o, len = std::hypot(nx, ny);
+  const double c = nx * P.cx + ny * P.cy + o, len = length(nx, ny);
   if (P.kind == PPatch::kBall) {
     r.add(c - len * P.r1);
     r.add(c + len * P.r1);
     return r;
   }
-  const double phi = std::atan2(ny, nx);
+  const bool most = direction_in(P, nx, ny), least = direction_in(P, -nx, -ny);
   for (int k = P.kind == PPatch::kArc ? 1 : 0; k < 2; ++k) {
     const double R = k ? P.r1 : P.r0;
-    r.add(c + R * len * std::cos(P.a0 - phi));
-    r.add(c + R * len * std::cos(P.a1 - phi));
-    if (angle_in(phi, P.a0, P.a1)) r.add(c + R * len);
-    if (angle_in(phi + kPi, P.a0, P.a1)) r.add(c - R * len);
+    for (int a = 0; a < 2; ++a) r.add(c + R * (nx * P.c[a] + ny * P.s[a]));
+    if (most) r.add(c + R * len);
+    if (least) r.add(c - R * len);
   }
   return r;
 }
@@ -87,14 +92,14 @@ inline PRange range_linear(const PPatch &P, double nx, double ny, double o) {
 inline double segment_distance(double x, double y, double ax, double ay, double bx, double by) {
   const double dx = bx - ax, dy = by - ay, l2 = dx * dx + dy * dy;
   const double t = l2 > 0.0 ? std::min(1.0, std::max(0.0, ((x - ax) * dx + (y - ay) * dy) / l2)) : 0.0;
-  return std::hypot(ax + t * dx - x, ay + t * dy - y);
+  return length(ax + t * dx - x, ay + t * dy - y);
 }
 
 // Distance from (x, y) over the patch.
 inline PRange range_distance(const PPatch &P, double x, double y) {
   PRange r;
   if (P.kind == PPatch::kPoints) {
-    for (int i = 0; i < P.n; ++i) r.add(std::hypot(P.px[i] - x, P.py[i] - y));
+    for (int i = 0; i < P.n; ++i) r.add(length(P.px[i] - x, P.py[i] - y));
     bool in = P.n > 2, pos = false, neg = false;
     for (int i = 0; i < P.n; ++i) {
       const int j = (i + 1) % P.n;
@@ -106,27 +111,27 @@ inline PRange range_distance(const PPatch &P, double x, double y) {
     if (in && !(pos && neg)) r.add(0.0);
     return r;
   }
-  const double D = std::hypot(x - P.cx, y - P.cy), psi = std::atan2(y - P.cy, x - P.cx);
+  const double D = length(x - P.cx, y - P.cy);
   if (P.kind == PPatch::kBall) {
     r.add(std::max(0.0, D - P.r1));
     r.add(D + P.r1);
     return r;
   }
+  const bool near = direction_in(P, x - P.cx, y - P.cy), far = direction_in(P, P.cx - x, P.cy - y);
   for (int k = P.kind == PPatch::kArc ? 1 : 0; k < 2; ++k) {
     const double R = k ? P.r1 : P.r0;
-    for (double a : {P.a0, P.a1}) r.add(std::hypot(P.cx + R * std::cos(a) - x, P.cy + R * std::sin(a) - y));
-    if (angle_in(psi, P.a0, P.a1)) r.add(std::fabs(R - D));
-    if (angle_in(psi + kPi, P.a0, P.a1)) r.add(R + D);
+    for (int a = 0; a < 2; ++a) r.add(length(P.cx + R * P.c[a] - x, P.cy + R * P.s[a] - y));
+    if (near) r.add(std::fabs(R - D));
+    if (far) r.add(R + D);
     if (D < 1e-9 * (1.0 + R)) {   // about the centre: the angle of (x, y) means nothing
       r.add(std::max(0.0, R - D));
       r.add(R + D);
     }
   }
   if (P.kind == PPatch::kSector) {
-    for (double a : {P.a0, P.a1})
-      r.add(segment_distance(x, y, P.cx + P.r0 * std::cos(a), P.cy + P.r0 * std::sin(a), P.cx + P.r1 * std::cos(a),
-                             P.cy + P.r1 * std::sin(a)));
-    if (D >= P.r0 && D <= P.r1 && (angle_in(psi, P.a0, P.a1) || D < 1e-9)) r.add(0.0);
+    for (int a = 0; a < 2; ++a)
+      r.add(segment_distance(x, y, P.cx + P.r0 * P.c[a], P.cy + P.r0 * P.s[a], P.cx + P.r1 * P.c[a], P.cy + P.r1 * P.s[a]));
+    if (D >= P.r0 && D <= P.r1 && (near || D < 1e-9)) r.add(0.0);
   }
   return r;
 }
@@ -136,10 +141,14 @@ class PortalBuilder {
   PortalBuilder(const HGeom &geom, double tolerance) : g(geom), tol(tolerance), eps(tolerance / 16.0) {
     const int n = (int)g.vol.size();
     surfs.resize(n);
+    daughters.resize(n);
+    cand_seen.resize(n);
+    list_seen.resize(g.clist.size());
     double size = 0.0;
     for (int i = 0; i < n; ++i) {
       volume_surfaces(i);
       const DVol &v = g.vol[i];
+      if (v.mother >= 0) daughters[v.mother].push_back(i);
       const DWorld &w = g.wxf[i];
       size = std::max(size, std::fabs(w.tx) + std::fabs(w.ty) + std::fabs(w.tz) + extent(v));
     }
@@ -169,7 +178,10 @@ class PortalBuilder {
   double tol, eps, margin = 0.0, scale = 0.0;
   bool usable = false;
   std::vector<std::vector<PSurf>> surfs;
+  std::vector<std::vector<int32_t>> daughters;        // in id order
   std::vector<int32_t> lists, cands;
+  std::vector<uint32_t> list_seen, cand_seen;         // the search that last met a list, a candidate
+  uint32_t searches = 0;
 
   static double extent(const DVol &v) {
     if (v.kind == kBox) return v.p[0] + v.p[1] + v.p[2];
@@ -282,6 +294,10 @@ class PortalBuilder {
       P.a0 = turn + a;
       P.a1 = P.a0 + d;
     }
+    for (int a = 0; a < 2; ++a) {
+      P.c[a] = std::cos(a ? P.a1 : P.a0);
+      P.s[a] = std::sin(a ? P.a1 : P.a0);
+    }
     P.r0 = (v.flags & kHasRmin) ? v.p[0] : 0.0;
     P.r1 = v.p[1];
     P.zlo = w.tz - v.p[2];
@@ -329,8 +345,8 @@ class PortalBuilder {
     if (s.type == kSphere) {
       const double zmin = std::max(0.0, std::max(P.zlo - s.cz, s.cz - P.zhi));
       const double zmax = std::max(std::fabs(P.zlo - s.cz), std::fabs(P.zhi - s.cz));
-      d.lo = std::hypot(d.lo, zmin);
-      d.hi = std::hypot(d.hi, zmax);
+      d.lo = length(d.lo, zmin);
+      d.hi = length(d.hi, zmax);
     }
     r.add(s.sign * (s.R - d.lo));
     r.add(s.sign * (s.R - d.hi));
@@ -343,6 +359,9 @@ class PortalBuilder {
     if (W == V) return dir < 0 ? 1 : 0;   // the crossing points lie on its face, away from its other surfaces
     const DVol &w = g.vol[W];
     const bool wide = w.kind == kTube && (w.flags & kWide), v_wide = g.vol[V].kind == kTube && (g.vol[V].flags & kWide);
+    // most volumes lie beyond a plane of theirs (that no face of V coincides with: outside all the same if one does)
+    for (const PSurf &s : surfs[W])
+      if ((s.type == kZPlane || (s.type == kLine && !wide)) && range(s, P).hi < -margin) return 0;
     bool all = w.kind != kCone;
     int phi_in = 0, phi_out = 0;
     for (const PSurf &s : surfs[W]) {
@@ -382,16 +401,22 @@ class PortalBuilder {
     return all ? 1 : -1;
   }
 
-  void collect(int32_t h, const double *lo, const double *hi) {
+  // The candidate lists of the nodes of header h that the box lo .. hi reaches, while they list fewer than `most` in all.
+  void collect(int32_t h, const double *lo, const double *hi, size_t most, size_t &listed) {
     const DVoxHdr &H = g.hdr[h];
     const int n = H.nslices;
-    const long k0 = std::max(0L, std::min((long)n - 1, (long)std::floor((lo[H.axis] - H.lo) * H.inv_width) - 1));
-    const long k1 = std::max(0L, std::min((long)n - 1, (long)std::floor((hi[H.axis] - H.lo) * H.inv_width) + 1));
-    for (long k = k0; k <= k1; ++k) {
+    const long k0 = std::max(0L, std::min((long)n - 1, (long)std::floor((lo[H.axis] - H.lo) * H.inv_width - 1e-6)));
+    const long k1 = std::max(0L, std::min((long)n - 1, (long)std::floor((hi[H.axis] - H.lo) * H.inv_width + 1e-6)));
+    for (long k = k0; k <= k1 && listed < most; ++k) {
       const DVoxSlice &S = g.slice[H.slice_base + k];
       if (k > k0 && S.k0 < k) continue;   // a merged node, already taken
-      if (S.child >= 0) lists.push_back(S.child);
-      else collect(-S.child - 1, lo, hi);
+      if (S.child < 0) {
+        collect(-S.child - 1, lo, hi, most, listed);
+      } else if (list_seen[S.child] != searches) {
+        list_seen[S.child] = searches;
+        lists.push_back(S.child);
+        listed += g.clist[S.child].count;
+      }
     }
   }
 
@@ -414,23 +439,33 @@ class PortalBuilder {
       const PRange x = range_linear(P, w.c, w.s, -w.c * w.tx - w.s * w.ty), y = range_linear(P, -w.s, w.c, w.s * w.tx - w.c * w.ty);
       const double sl = margin;
       const double lo[3] = {x.lo - sl, y.lo - sl, P.zlo - w.tz - sl}, hi[3] = {x.hi + sl, y.hi + sl, P.zhi - w.tz + sl};
+      auto reached = [&](int32_t d) {
+        const DBox32 &B = g.box[d];
+        for (int b = 0; b < 3; ++b)
+          if ((double)B.hi[b] < lo[b] || (double)B.lo[b] > hi[b]) return false;
+        return d != blocked;
+      };
       lists.clear();
       cands.clear();
-      collect(g.vol[cur].vox, lo, hi);
-      std::sort(lists.begin(), lists.end());
-      lists.erase(std::unique(lists.begin(), lists.end()), lists.end());
-      for (int32_t l : lists) {
-        const DCandList &cl = g.clist[l];
-        for (int32_t q = 0; q < cl.count; ++q) {
-          const int32_t d = g.cand[cl.offset + q];
-          const DBox32 &B = g.box[d];
-          bool hit = d != blocked;
-          for (int b = 0; b < 3 && hit; ++b) hit = (double)B.hi[b] >= lo[b] && (double)B.lo[b] <= hi[b];
-          if (hit) cands.push_back(d);
+      ++searches;
+      size_t listed = 0;
+      collect(g.vol[cur].vox, lo, hi, daughters[cur].size(), listed);
+      if (listed >= daughters[cur].size()) {
+        // a face that large meets daughters again node after node: each once, then (1200 shells about one axis: 57 s -> 1)
+        for (int32_t d : daughters[cur])
+          if (reached(d)) cands.push_back(d);
+      } else {
+        for (int32_t l : lists) {
+          const DCandList &cl = g.clist[l];
+          for (int32_t q = 0; q < cl.count; ++q) {
+            const int32_t d = g.cand[cl.offset + q];
+            if (cand_seen[d] == searches) continue;
+            cand_seen[d] = searches;
+            if (reached(d)) cands.push_back(d);
+          }
         }
+        std::sort(cands.begin(), cands.end());
       }
-      std::sort(cands.begin(), cands.end());
-      cands.erase(std::unique(cands.begin(), cands.end()), cands.end());
       int found = -1;
       for (int32_t d : cands) {
         const int in = inside(d, V, f, P, dir);

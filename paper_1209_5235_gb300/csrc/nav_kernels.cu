@@ -242,7 +242,11 @@ __global__ void __launch_bounds__(128, 4) k_compute_step(const DGeom *__restrict
         // a float not below the proposal (a NaN proposal of either sign limits nothing, a negative one everything)
         const float f = trunc_float(prop);
         const float limit = isnan(prop) ? kInfF : f < 0.f ? f * (1.0f - 2.0f * kU) : f * (1.0f + 2.0f * kU) + 1e-30f;
-        const Step32 R = geom_step32_warp<MODE, false, false>(G, ok, leaf, p, v, limit, true, cnt, &timeout, walk_cap, mc, ch);
+        Step32 R = geom_step32_warp<MODE, false, false>(G, ok, leaf, p, v, limit, true, cnt, &timeout, walk_cap, mc, ch);
+        if (isnan(p.x + p.y + p.z)) {   // the floats of a point hold no NaN: such a query gets what the FP64 formulas make of it
+          R.undecided = true;
+          R.lo = -kInfF;
+        }
         safety = (double)R.safety;
         if (ok) {
           int surf;

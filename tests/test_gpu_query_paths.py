@@ -174,3 +174,26 @@ def test_modes_give_the_same_steps(env, name):
     for mode in (1, 2):
         assert np.array_equal(got[mode][2], got[0][2])
         assert np.array_equal(got[mode][0], got[0][0], equal_nan=True), (got[mode][0] != got[0][0]).sum()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), -float("nan"), float("inf"), -float("inf"), 1e300, 1e20])
+def test_modes_agree_on_points_that_are_no_points(env, bad):
+    """compute_step takes a point as it is given: the FP32 mode's answer to a NaN, an infinity or a coordinate beyond any float
+    is the FP64 mode's."""
+    from gpu_common import mixed_scene
+    g4, torch, ctx = env
+    gid = g4.build_scene(ctx, mixed_scene(seed=23, n=200, half=200.0))
+    rng, n = np.random.default_rng(37), 20000
+    p, v = rng.uniform(-150, 150, (3, n)), rng.normal(size=(3, n))
+    v /= np.linalg.norm(v, axis=0)
+    pos, dirs = torch.tensor(p, device="cuda"), torch.tensor(v, device="cuda")
+    depth, path = g4.g4n_locate(ctx, gid, pos, dirs)
+    g4.g4n_sync(ctx)
+    pos[0, ::2] = bad
+    pos[2, ::3] = bad
+    got = [[a.cpu().numpy().copy() for a in g4.g4n_compute_step(ctx, gid, pos, dirs, depth, path, mode=mode)] for mode in (0, 1)]
+    try:
+        g4.g4n_sync(ctx)
+    except g4.G4NError:
+        pass
+    assert np.array_equal(got[0][0], got[1][0], equal_nan=True) and np.array_equal(got[0][2], got[1][2])

@@ -197,3 +197,52 @@ def test_modes_agree_on_points_that_are_no_points(env, bad):
     except g4.G4NError:
         pass
     assert np.array_equal(got[0][0], got[1][0], equal_nan=True) and np.array_equal(got[0][2], got[1][2])
+
+
+@pytest.mark.parametrize("scale", [1e3, 1e6])
+@pytest.mark.parametrize("name", ["mixed", "gaps", "segments"])
+def test_large_tolerance_scales(env, name, scale):
+    """Queries and histories at large tolerances (1e-6 and 1e-3 mm) are the oracle's in every mode, points in surface bands and
+    solids a part of the tolerance apart among them."""
+    import oracle
+    from gpu_common import mixed_scene, random_queries, segments_scene
+    from test_portals_host import gap_scene
+    g4, torch, _ = env
+    sc = {"mixed": lambda: mixed_scene(seed=23, n=150, half=200.0), "gaps": lambda: gap_scene(0.3e-9 * scale),
+          "segments": segments_scene}[name]()
+    ctx = g4.g4n_create(0)
+    oracle.set_scale(scale)
+    try:
+        g4.g4n_set_tolerance_scale(ctx, scale)
+        gid = g4.build_scene(ctx, sc)
+        og = oracle.Geometry(sc)
+        p, v = random_queries(og, sc, 20000, seed=38, aim_frac=0.5)
+        depth, path = og.locate_many(p, v)
+        ok = depth > 0
+        p, v, depth, path = p[ok], v[ok], depth[ok], path[ok]
+        T = lambda a, t: torch.tensor(np.ascontiguousarray(a), dtype=t, device="cuda")
+        pos, dirs = T(p.T, torch.float64), T(v.T, torch.float64)
+        d, pa = g4.g4n_locate(ctx, gid, pos, dirs)
+        assert np.array_equal(d.cpu().numpy(), depth) and np.array_equal(pa.cpu().numpy().T, path)
+        want, lim_ref, _ = og.compute_step_many(p, v, depth, path)
+        for mode in (0, 1):
+            s, _, lim = g4.g4n_compute_step(ctx, gid, pos, dirs, T(depth, torch.int32), T(path.T, torch.int32), mode=mode)
+            g4.g4n_sync(ctx)
+            assert np.array_equal(lim.cpu().numpy(), lim_ref), (mode, (lim.cpu().numpy() != lim_ref).sum())
+            assert np.all(np.abs(s.cpu().numpy() - want) <= 1e-9)
+        src = synth.scenes.Source(pos=(15.0, -13.0, 2.0), isotropic=True, e_kind="loguniform", e0=0.05, e1=5.0)
+        n = 20000
+        ref = og.transport(src, 39, n)["hashes"]
+        for mode in (0, 1):
+            for schedule, flags in ((0, 0), (1, 0), (1, 1)):
+                edep = torch.zeros((100, sc.n_volumes + 2), dtype=torch.float64, device="cuda")
+                cnt = torch.zeros(g4.G4N_N_COUNTERS, dtype=torch.int64, device="cuda")
+                h = torch.zeros(n, dtype=torch.int64, device="cuda")
+                g4.g4n_transport_batch(ctx, g4.make_items([(gid, n, 0, src, 0)]), 39, edep, cnt, h, mode=mode,
+                                       schedule=schedule, staged_flags=flags)
+                g4.g4n_sync(ctx)
+                bad = (h.cpu().numpy().view(np.uint64) != ref).sum()
+                assert bad == 0, (mode, schedule, flags, bad)
+    finally:
+        oracle.set_scale(1.0)
+        g4.g4n_destroy(ctx)

@@ -44,15 +44,17 @@ WORKLOAD = ("sampling calorimeter: 50 alternating 5 mm lead-like / 10 mm scintil
 # formulas of each test.  An Inside test of a world-aligned box answered by exact coordinate keys (key_inside) counts
 # as the FP64 box test whose answer it gives, and a relocation answered by a face record (face_reloc) as the two
 # Inside tests (mother, entered volume) the method needs at least: the work the method defines, not the instructions
-# the kernel executes.  DistanceToOut and Inside of tubes and cones (the *_curved counts, also included in dist_out
+# the kernel executes: in the FP32 modes most of it runs as FP32 bounds, and the fraction of the FP64 peak is the method's
+# work over the time, not the FP64 pipe's use.  DistanceToOut and Inside of tubes and cones (the *_curved counts, also included in dist_out
 # and inside) add their surplus over the box's: a tube segment's exit takes ~163 (z plane ~30, the two cylinders'
 # quadratics with their range tests ~69 with the shared a, b, r^2, the two phi planes ~64), its Inside ~40.
 FLOPS = {"steps": 40, "dist_out": 12, "cand_box": 56, "cand_orb": 40, "cand_tube": 90, "cand_cone": 100, "inside": 24,
          "key_inside": 24, "face_reloc": 48, "vox_nodes": 14, "phys_steps": 60, "dist_out_curved": 151,
          "inside_curved": 16}
 SCHEDULES = {0: "persistent", 1: "staged"}
-# bytes of one track's state in the staged schedule's queues (16 doubles, hash, id, 6 ints)
-STAGED_STATE_BYTES = 168
+# bytes of one track's state in the staged schedule's queues (16 doubles, hash, id, 6 ints; the FP32 modes leave the
+# reciprocal direction's three doubles alone)
+STAGED_STATE_BYTES = {"fp64": 168, "fp32_recheck": 144, "learned": 144}
 FP64_PEAK_TFLOPS = 152 * 2.070e9 * 4 / 1e12   # 152 SMs x 2.07 GHz x 4 FP64 flops/clk/SM (2 DFMA) = 1.2586
 
 
@@ -588,11 +590,12 @@ def run_gpu(args):
     reloc_kernel = staged and bool(R["launch"].get("staged_flags", 0) & g4.G4N_STAGED_RELOCATION_KERNEL)
     if staged:
         # the queues: every step and every interaction reads a state and writes one back, every start writes one;
-        # with the relocation kernel every relocation search (a crossing no face record answers) one more of each
-        hbm_bytes += STAGED_STATE_BYTES * (2 * cdiag["steps"] + 2 * (cdiag["photo"] + cdiag["compton"])
-                                           + cdiag["tracks"])
+        # with the relocation kernel every relocation search (a crossing no record or portal answers) one more of each
+        # (without the relocation kernel a track may take up to four steps in daughterless boxes at one visit: an upper bound)
+        state = STAGED_STATE_BYTES[chosen]
+        hbm_bytes += state * (2 * cdiag["steps"] + 2 * (cdiag["photo"] + cdiag["compton"]) + cdiag["tracks"])
         if reloc_kernel:
-            hbm_bytes += (STAGED_STATE_BYTES + 4) * 2 * (cdiag["geom_steps"] - cdiag["face_reloc"])
+            hbm_bytes += (state + 4) * 2 * (cdiag["geom_steps"] - cdiag["face_reloc"])
     line = {
         "metric": METRIC, "value": R["steps_per_s"], "unit": "steps/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": R["ms_per_step"], "higher_is_better": True,

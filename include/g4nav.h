@@ -59,7 +59,7 @@ enum { G4N_BOX = 0, G4N_TUBE = 1, G4N_ORB = 2, G4N_CONE = 3 };
 /* Precision modes of compute_step / transport. */
 enum {
   G4N_MODE_FP64 = 0,         /* every distance in FP64 */
-  G4N_MODE_FP32_RECHECK = 1, /* FP32 intersection/safety, FP64 recheck of near-minimum candidates */
+  G4N_MODE_FP32_RECHECK = 1, /* FP32 bounds choose the crossing and give the safety, FP64 evaluates the one that is chosen */
   G4N_MODE_LEARNED = 2       /* FP32_RECHECK plus the learned candidate proposal */
 };
 
@@ -74,17 +74,20 @@ enum {
   G4N_C_TRACKS = 0, G4N_C_STEPS, G4N_C_GEOM_STEPS, G4N_C_PHYS_STEPS, G4N_C_PHOTO, G4N_C_COMPTON, G4N_C_ESCAPED,
   G4N_C_CUTOFF, G4N_C_PUSHES, G4N_C_STEP_LIMIT,
   G4N_C_WALK_YIELDS = 10,    /* boundary searches that used their node budget and went on in a later round */
-  G4N_C_CAND_CONE = 11,      /* DistanceToIn evaluations of cones */
+  G4N_C_CAND_CONE = 11,      /* DistanceToIn of cones (see G4N_C_CAND_BOX) */
   G4N_C_DIST_OUT_CURVED = 12, /* of G4N_C_DIST_OUT: those of tubes and cones */
   G4N_C_INSIDE_CURVED = 13,  /* of G4N_C_INSIDE: those of tubes and cones */
-  G4N_C_FACE_RELOC = 14,     /* relocations answered by a box face's precomputed record */
+  G4N_C_FACE_RELOC = 14,     /* relocations answered by a precomputed record: a box face's, or the portal of any face */
   G4N_C_KEY_INSIDE = 15,     /* Inside tests of world-aligned boxes answered by exact coordinate thresholds */
   G4N_C_SAFETY_SKIPS = 16,   /* steps that skipped the boundary search because safety exceeded the physics step */
-  G4N_C_CAND_BOX, G4N_C_CAND_TUBE, G4N_C_CAND_ORB, /* DistanceToIn evaluations by solid type */
-  G4N_C_DIST_OUT,            /* DistanceToOut evaluations */
+  /* DistanceToIn of candidates by solid type, and DistanceToOut of leaves.  In both a surface is chosen in FP32 and one
+   * crossing evaluated in FP64 (boxes' exits in the FP64 mode and whatever FP32 does not decide: the full formulas in FP64);
+   * the FP32 modes evaluate only the crossing that comes first, one a step. */
+  G4N_C_CAND_BOX, G4N_C_CAND_TUBE, G4N_C_CAND_ORB,
+  G4N_C_DIST_OUT,
   G4N_C_INSIDE,              /* FP64 Inside tests (after the bounding-box prefilter) */
   G4N_C_VOX_NODES,           /* voxel nodes visited by the boundary search */
-  G4N_C_RECHECKS,            /* FP64 rechecks in FP32_RECHECK mode */
+  G4N_C_RECHECKS,            /* FP32 modes: candidates that the bounds of their boxes let pass to the choice of a surface */
   G4N_C_PROPOSALS,           /* learned proposals used */
   G4N_C_PRUNED,              /* candidates skipped by the proposal bound */
   G4N_C_CYC_REFILL = 26,     /* warp clock cycles spent refilling idle lanes (diagnostics) */

@@ -41,3 +41,19 @@ def test_tuner_shapes_are_valid_batch_descriptions():
         assert d.pool_tracks >= 0 and d.drain_tracks >= -1 and 0 <= d.blocks_per_sm <= 16
         assert d.block_size % 32 == 0 and d.block_size <= 128
     assert {s["drain_tracks"] for s in at.STAGED} >= {0, -1}     # the default drain point and no drain are both tried
+
+
+def test_tuner_leaves_a_local_minimum_of_single_changes(monkeypatch):
+    """A short walk budget that pays only with regrouping is found although neither change alone is faster."""
+    torch = __import__("torch")
+    monkeypatch.setattr(torch, "zeros", lambda *a, **k: torch.empty(0))
+
+    def cost(ctx, items, seed, edep, cnt, mode, cfg, reps=2, stream=None):
+        if cfg["schedule"] == b.G4N_SCHEDULE_STAGED:
+            return 300.0
+        short, regroup = cfg["walk_budget"] <= 32, cfg["regroup_period"] == 1
+        return 130.0 if short and regroup else 170.0 if short else 166.0 if not regroup else 180.0
+
+    monkeypatch.setattr(at, "time_launch", cost)
+    res = at.autotune(None, _items(), 1, 1, modes=(1,), max_tracks=0)
+    assert res["cfg"]["walk_budget"] <= 32 and res["cfg"]["regroup_period"] == 1 and res["ms"] == 130.0
